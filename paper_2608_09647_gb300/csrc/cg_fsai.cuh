@@ -33,11 +33,15 @@ struct FsaiData {
   int noffs = 0, ntslots = 0;      // their count; count of those <= 0
   int32_t* trow = nullptr;         // row of each tril entry
   double* work = nullptr;          // training work vectors
+  int work_k = 0;                  // residual vectors it holds at a time
   double* rpart = nullptr;         // block partial sums of the loss kernels
+  double* rsums = nullptr;         // the sums: quad, log-diag, then e.e, r.r of every residual vector
+  unsigned* rctr = nullptr;        // blocks finished, per residual vector of a launch
+  int sums_k = 0;                  // pairs of sums rsums holds
   float* dout = nullptr;           // dLoss/do per tril entry
   float* gpart = nullptr;          // per-CTA partial parameter gradients
   float* mlp_o = nullptr;          // MLP output per tril entry
-  float* a32 = nullptr;            // A's values in fp32 (feature inputs)
+  void* rowf = nullptr;            // every row's scaled entries in bf16 (RowFeatures, cg_mlp.cu)
   float* d32 = nullptr;            // A_ii in fp32
   float* rs32 = nullptr;           // 1 / sqrt(A_ii) in fp32
   double* rs64 = nullptr;          // 1 / sqrt(A_ii) in fp64 (G from the outputs)

@@ -42,20 +42,21 @@ constexpr int kTileE = 64;               // entries per CTA step
 constexpr int kW1S = kIn + 8;            // padded smem row strides (bf16 elements)
 constexpr int kW2S = kHid + 8;
 constexpr int kTS = kTileE + 8;          // transposed tiles: [feature][entry]
+static_assert(kHid * kIn % (4 * kMlpThreads) == 0 && kHid * kHid % (4 * kMlpThreads) == 0, "whole 16-byte loads");
+
+// The scaled entries s(i, i + o_m) of one row over the offsets' slots, as the network
+// reads them: bf16, 0 where absent, in two 16-byte words.
+struct __align__(16) RowFeatures {
+  __nv_bfloat16 s[16];
+};
 
 struct MlpArgs {
   int64_t n, ntril;
-  const int32_t* __restrict__ rowptr;
-  const int32_t* __restrict__ colind;
-  const double* __restrict__ vals;
-  const double* __restrict__ diag;
   const int32_t* __restrict__ trow;      // row of each tril entry
   const int32_t* __restrict__ tci;       // column of each tril entry
-  const int32_t* __restrict__ tsrc;      // index of each tril entry in A's arrays
   const float* __restrict__ params;      // fp32 parameters (rounded to bf16 on load)
-  const float* __restrict__ a32;         // A's values, A_ii and 1 / sqrt(A_ii) in fp32
-  const float* __restrict__ d32;
-  const float* __restrict__ rs32;
+  const RowFeatures* __restrict__ rf;    // every row's scaled entries
+  const float* __restrict__ d32;         // A_ii in fp32
   int offs[kMaxOffs];
   int noffs, ntslots;
   double c0;
@@ -79,48 +80,50 @@ __device__ __forceinline__ uint32_t lds32(const __nv_bfloat16* p) {
   return *reinterpret_cast<const uint32_t*>(p);
 }
 
-__device__ __forceinline__ int offset_slot(const MlpArgs& M, int off) {
-  for (int m = 0; m < M.noffs; ++m)
-    if (M.offs[m] == off) return m;
-  return -1;
+__device__ __forceinline__ int offset_slot(const int (&offs)[kMaxOffs], int noffs, int off) {
+  int m = -1;
+#pragma unroll
+  for (int k = 0; k < kMaxOffs; ++k)
+    if (k < noffs && offs[k] == off) m = k;
+  return m;
 }
 
-// Features of tril entry e into a 32-wide bf16 row: lanes 0-15 write the
-// entry part and row i's entries, lanes 16-31 row j's entries and the tail.
-__device__ void entry_features(const MlpArgs& M, int64_t e, bool upper_half, __nv_bfloat16* xr) {
-  if (e >= M.ntril) {
-    const int a = upper_half ? 16 : 0;
-    for (int f = a; f < a + 16; ++f) xr[f] = __float2bfloat16_rn(0.0f);
-    return;
-  }
-  // formed in fp32 from fp32 copies of A's values and diagonal (GB300 runs
-  // fp64, conversions included, at 1/64 of the fp32 rate) and rounded to
-  // bf16, the network's input precision
-  const int i = M.trow[e], j = M.tci[e];
-  const float si = M.rs32[i], sj = M.rs32[j];
-  float f[19];
+// Features of tril entry e into a 32-wide bf16 row: lanes 0-15 write the entry part
+// and row i's entries, lanes 16-31 row j's entries and the tail.  Both rows' entries
+// come from the per-row table (row_features_kernel), two 16-byte loads a row, all in
+// flight together: each row is needed by ~10 entries, and forming its entries from
+// the CSR here, a chain of column, slot search, value and scale per stored entry
+// through an array in local memory, was most of both MLP kernels' time.
+__device__ __forceinline__ void entry_features(const MlpArgs& M, int64_t e, bool upper_half, __nv_bfloat16* xr) {
+  const bool live = e < M.ntril;
+  const int i = live ? M.trow[e] : 0, j = live ? M.tci[e] : 0;
+  union {
+    uint4 q[2];
+    __nv_bfloat16 s[16];
+  } r;
+  const uint4* src = reinterpret_cast<const uint4*>(M.rf + (upper_half ? j : i));
+  r.q[0] = __ldg(src);
+  r.q[1] = __ldg(src + 1);
+  const __nv_bfloat16 zero = __float2bfloat16_rn(0.0f);
   if (!upper_half) {
-    for (int k = 0; k < 19; ++k) f[k] = 0.0f;
-    const int slot = offset_slot(M, j - i);  // always one of the first ntslots
-    if (slot >= 0 && slot < 8) f[slot] = 1.0f;
-    f[8] = M.a32[M.tsrc[e]] * si * sj;
-    f[9] = logf(M.d32[j] / M.d32[i]);
-    for (int k = M.rowptr[i]; k < M.rowptr[i + 1]; ++k) {
-      const int c = M.colind[k];
-      const int s = offset_slot(M, c - i);
-      if (s >= 0) f[10 + s] = M.a32[k] * si * M.rs32[c];
+    const float di = __ldg(M.d32 + i), dj = __ldg(M.d32 + j);
+    const int slot = offset_slot(M.offs, M.noffs, j - i);  // always one of the first ntslots
+    __nv_bfloat16 sij = zero;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const bool on = live && slot == k;
+      xr[k] = __float2bfloat16_rn(on ? 1.0f : 0.0f);
+      if (on) sij = r.s[k];
     }
-    for (int k = 0; k < 19; ++k) xr[k] = __float2bfloat16_rn(f[k]);
+    xr[8] = sij;
+    xr[9] = live ? __float2bfloat16_rn(logf(dj / di)) : zero;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) xr[10 + k] = live ? r.s[k] : zero;
   } else {
-    for (int k = 0; k < 9; ++k) f[k] = 0.0f;
-    for (int k = M.rowptr[j]; k < M.rowptr[j + 1]; ++k) {
-      const int c = M.colind[k];
-      const int s = offset_slot(M, c - j);
-      if (s >= 0) f[s] = M.a32[k] * sj * M.rs32[c];
-    }
-    for (int k = 0; k < 9; ++k) xr[19 + k] = __float2bfloat16_rn(f[k]);
-    xr[28] = __float2bfloat16_rn(1.0f);
-    for (int k = 29; k < 32; ++k) xr[k] = __float2bfloat16_rn(0.0f);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) xr[19 + k] = live ? r.s[k] : zero;
+    xr[28] = __float2bfloat16_rn(live ? 1.0f : 0.0f);
+    for (int k = 29; k < 32; ++k) xr[k] = zero;
   }
 }
 
@@ -133,13 +136,38 @@ struct __align__(16) SmemW {
   float b3;
 };
 
-__device__ void load_weights(const MlpArgs& M, SmemW& S, __nv_bfloat16* w2t) {
-  for (int k = threadIdx.x; k < kHid * kIn; k += blockDim.x)
-    S.w1[(k / kIn) * kW1S + k % kIn] = __float2bfloat16_rn(M.params[kOffW1 + k]);
-  for (int k = threadIdx.x; k < kHid * kHid; k += blockDim.x) {
-    const __nv_bfloat16 v = __float2bfloat16_rn(M.params[kOffW2 + k]);
-    S.w2[(k / kHid) * kW2S + k % kHid] = v;
-    if (w2t) w2t[(k % kHid) * kW2S + k / kHid] = v;
+// Four consecutive parameters (16-byte loads where the caller's array allows them),
+// rounded to bf16.
+__device__ __forceinline__ void load4(const float* p, bool vec, __nv_bfloat16 (&o)[4]) {
+  float4 v;
+  if (vec) v = __ldg(reinterpret_cast<const float4*>(p));
+  else v = make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+  o[0] = __float2bfloat16_rn(v.x);
+  o[1] = __float2bfloat16_rn(v.y);
+  o[2] = __float2bfloat16_rn(v.z);
+  o[3] = __float2bfloat16_rn(v.w);
+}
+
+__device__ __forceinline__ void load_weights(const MlpArgs& M, SmemW& S, __nv_bfloat16* w2t) {
+  const bool vec = (reinterpret_cast<uintptr_t>(M.params) & 15u) == 0;
+#pragma unroll
+  for (int u = 0; u < kHid * kIn / 4 / kMlpThreads; ++u) {
+    const int k = 4 * (u * kMlpThreads + threadIdx.x);
+    __nv_bfloat16 v[4];
+    load4(M.params + kOffW1 + k, vec, v);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) S.w1[(k / kIn) * kW1S + k % kIn + c] = v[c];
+  }
+#pragma unroll
+  for (int u = 0; u < kHid * kHid / 4 / kMlpThreads; ++u) {
+    const int k = 4 * (u * kMlpThreads + threadIdx.x);
+    __nv_bfloat16 v[4];
+    load4(M.params + kOffW2 + k, vec, v);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      S.w2[(k / kHid) * kW2S + k % kHid + c] = v[c];
+      if (w2t) w2t[(k % kHid + c) * kW2S + k / kHid] = v[c];
+    }
   }
   for (int k = threadIdx.x; k < kHid; k += blockDim.x) {
     S.b1[k] = __bfloat162float(__float2bfloat16_rn(M.params[kOffB1 + k]));
@@ -430,94 +458,119 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_backward_kernel(MlpArgs M, co
   if (threadIdx.x == 0) out[kOffB3] = ((S.red3[0] + S.red3[1]) + S.red3[2]) + S.red3[3];
 }
 
-__global__ void reduce_parts_kernel(const float* __restrict__ part, int nparts, float* __restrict__ grad) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < kNParams; k += gridDim.x * blockDim.x) {
-    float s = 0.0f;
-    for (int c = 0; c < nparts; ++c) s += part[(size_t)c * kNParams + k];
-    grad[k] = s;
+// Sum of the per-CTA gradients: 32 parameters a CTA (a 128-byte line of each partial),
+// warp w adds partials w, w + kRedWarps, ... in order (its loads in flight together),
+// then the warps' sums in order.  (A thread a parameter through all partials waited
+// for ~320 loads in a row at a 64 x 64 grid: ~20 us.)
+constexpr int kRedWarps = 16;
+__global__ void __launch_bounds__(32 * kRedWarps) reduce_parts_kernel(const float* __restrict__ part, int nparts,
+                                                                      float* __restrict__ grad) {
+  __shared__ float s_sum[kRedWarps][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int k = blockIdx.x * 32 + lane;
+  float s = 0.0f;
+  if (k < kNParams) {
+#pragma unroll 8
+    for (int c = warp; c < nparts; c += kRedWarps) s += __ldg(part + (size_t)c * kNParams + k);
+  }
+  s_sum[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && k < kNParams) {
+    float t = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kRedWarps; ++w) t += s_sum[w][lane];
+    grad[k] = t;
   }
 }
 
 // ---------------------------------------------------------------- loss (fp64)
 
-constexpr int kRed = 256;  // threads of the reduction kernels
+constexpr int kRed = 256;         // threads of the loss kernels
+constexpr int kLossBlocks = 1024;  // most blocks of a loss kernel that forms sums (per residual vector)
 
-// Block sums of NV values into part[blockIdx.x * NV + k] (fixed order).
+// Sums of NV values over the grid (blockIdx.x), by the last block to finish: it adds
+// the blocks' sums, thread t those of blocks t, t + kRed, ..., then the threads' in a
+// fixed order, so that no launch and no serial chain over blocks follows.
 template <int NV>
-__device__ __forceinline__ void block_partials(double (&v)[NV], double* part) {
+__device__ __forceinline__ void grid_sums(double (&v)[NV], double* part, unsigned* ctr, double* out) {
+  __shared__ int s_last;
   block_sum<NV>(v);
-  if (threadIdx.x == 0)
+  if (threadIdx.x == 0) {
     for (int k = 0; k < NV; ++k) part[(size_t)blockIdx.x * NV + k] = v[k];
+    __threadfence();
+    s_last = atomicAdd(ctr, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double t[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) t[k] = 0.0;
+  for (unsigned b = threadIdx.x; b < gridDim.x; b += kRed) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) t[k] += __ldcg(part + (size_t)b * NV + k);
+  }
+  block_sum<NV>(t);
+  if (threadIdx.x == 0) {
+    for (int k = 0; k < NV; ++k) out[k] = t[k];
+    *ctr = 0u;
+  }
 }
 
-// Kaporin term, thread per row i: (A g_i)_a for a in P_i (merge of row a of A
-// with P_i), quad_i = g_i . (A g_i)_P, log G_ii; partial sums per block.
-__global__ void __launch_bounds__(kRed) kaporin_rows_kernel(int64_t n, const int32_t* __restrict__ rowptr,
-                                                            const int32_t* __restrict__ colind,
-                                                            const double* __restrict__ vals,
-                                                            const int32_t* __restrict__ trp,
-                                                            const int32_t* __restrict__ tci,
-                                                            const double* __restrict__ g, double* __restrict__ gag,
-                                                            double* part) {
+// y = G x, row i (tril CSR with the values g).
+__device__ __forceinline__ double g_row(const int32_t* __restrict__ trp, const int32_t* __restrict__ tci,
+                                        const double* __restrict__ g, const double* __restrict__ x, int64_t i) {
+  double s = 0.0;
+  for (int k = trp[i]; k < trp[i + 1]; ++k) s += g[k] * x[tci[k]];
+  return s;
+}
+
+// Kaporin term, thread per tril entry e = (i, a): (A g_i)_a by merging row a of A
+// with the pattern P_i; the sums of g_e (A g_i)_a (all rows' quadratic forms) and of
+// log G_ii.  (A thread per row walked its ~5 rows of A one after the other.)
+__global__ void __launch_bounds__(kRed) kaporin_kernel(int64_t ntril, const int32_t* __restrict__ rowptr,
+                                                       const int32_t* __restrict__ colind,
+                                                       const double* __restrict__ vals,
+                                                       const int32_t* __restrict__ trow,
+                                                       const int32_t* __restrict__ trp,
+                                                       const int32_t* __restrict__ tci, const double* __restrict__ g,
+                                                       double* __restrict__ gag, double* part, unsigned* ctr,
+                                                       double* sums) {
   double v[2] = {0.0, 0.0};
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int t0 = trp[i], m = trp[i + 1] - t0;
-    double quad = 0.0;
-    for (int a = 0; a < m; ++a) {
-      const int ra = tci[t0 + a];
-      double s = 0.0;
-      int c = 0;
-      for (int k = rowptr[ra]; k < rowptr[ra + 1] && c < m; ++k) {
-        const int col = colind[k];
-        while (c < m && tci[t0 + c] < col) ++c;
-        if (c < m && tci[t0 + c] == col) s += vals[k] * g[t0 + c];
-      }
-      gag[t0 + a] = s;
-      quad += g[t0 + a] * s;
-    }
-    v[0] += quad;
-    v[1] += log(g[t0 + m - 1]);
-  }
-  block_partials<2>(v, part);
-}
-
-// Sum of block partials (one thread per value, blocks in order).
-__global__ void sum_parts_kernel(const double* __restrict__ part, int nblocks, int nv, double* __restrict__ out) {
-  const int k = threadIdx.x;
-  if (k < nv) {
-    double s = 0.0;
-    for (int b = 0; b < nblocks; ++b) s += part[(size_t)b * nv + k];
-    out[k] = s;
-  }
-}
-
-// dL_K/dG_e = 2 (A g_i)_a / (n S) - [a == i] 2 / (n G_ii), S = quad / n.
-__global__ void kaporin_grad_kernel(int64_t n, const int32_t* __restrict__ trow, const int32_t* __restrict__ tci,
-                                    const int32_t* __restrict__ trp, const double* __restrict__ g,
-                                    const double* __restrict__ gag, const double* __restrict__ sums, int64_t ntril,
-                                    double* __restrict__ dg) {
-  const double S = sums[0] / (double)n;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ntril; e += (int64_t)gridDim.x * blockDim.x) {
-    const int i = trow[e];
-    double v = 2.0 * gag[e] / ((double)n * S);
-    if (tci[e] == i) v -= 2.0 / ((double)n * g[trp[i + 1] - 1]);
-    dg[e] = v;
+    const int i = trow[e], ra = tci[e];
+    const int t0 = trp[i], m = trp[i + 1] - t0;
+    double s = 0.0;
+    int c = 0;
+    for (int k = rowptr[ra]; k < rowptr[ra + 1] && c < m; ++k) {
+      const int col = colind[k];
+      while (c < m && tci[t0 + c] < col) ++c;
+      if (c < m && tci[t0 + c] == col) s += vals[k] * g[t0 + c];
+    }
+    gag[e] = s;
+    v[0] += g[e] * s;
+    if (ra == i) v[1] += log(g[e]);
   }
+  grid_sums<2>(v, part, ctr, sums);
 }
 
-// y = G x (tril CSR with the values g).
-__global__ void g_mul_kernel(int64_t n, const int32_t* __restrict__ trp, const int32_t* __restrict__ tci,
-                             const double* __restrict__ g, const double* __restrict__ x, double* __restrict__ y) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int k = trp[i]; k < trp[i + 1]; ++k) s += g[k] * x[tci[k]];
-    y[i] = s;
-  }
+// The residual term of the vectors r_k (blockIdx.y = k), a kernel a product, all
+// vectors in one launch: u = G r; v = G^T u; e = A v - r with e.e and r.r; A e; G A e.
+__global__ void __launch_bounds__(kRed) resid_g_kernel(int64_t n, const int32_t* __restrict__ trp,
+                                                       const int32_t* __restrict__ tci, const double* __restrict__ g,
+                                                       const double* __restrict__ x, double* __restrict__ y) {
+  x += (size_t)blockIdx.y * n;
+  y += (size_t)blockIdx.y * n;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    y[i] = g_row(trp, tci, g, x, i);
 }
 
 // y = G^T x through the ELL slot map of G^T (src: tril index or -1).
-__global__ void gt_mul_kernel(int64_t n, int w, const int32_t* __restrict__ src, const int32_t* __restrict__ col,
-                              const double* __restrict__ g, const double* __restrict__ x, double* __restrict__ y) {
+__global__ void __launch_bounds__(kRed) resid_gt_kernel(int64_t n, int w, const int32_t* __restrict__ src,
+                                                        const int32_t* __restrict__ col, const double* __restrict__ g,
+                                                        const double* __restrict__ x, double* __restrict__ y) {
+  x += (size_t)blockIdx.y * n;
+  y += (size_t)blockIdx.y * n;
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
     double s = 0.0;
     for (int m = 0; m < w; ++m) {
@@ -528,85 +581,128 @@ __global__ void gt_mul_kernel(int64_t n, int w, const int32_t* __restrict__ src,
   }
 }
 
-// y = A x - sub (sub may be null), with the partial sums of y.y and sub.sub.
-__global__ void __launch_bounds__(kRed) a_mul_kernel(int64_t n, const int32_t* __restrict__ rowptr,
-                                                     const int32_t* __restrict__ colind,
-                                                     const double* __restrict__ vals, const double* __restrict__ x,
-                                                     const double* __restrict__ sub, double* __restrict__ y,
-                                                     double* part) {
+// y = A x - sub with the sums of y.y and sub.sub (SUB), or y = A x.
+template <bool SUB>
+__global__ void __launch_bounds__(kRed) resid_a_kernel(int64_t n, const int32_t* __restrict__ rowptr,
+                                                       const int32_t* __restrict__ colind,
+                                                       const double* __restrict__ vals, const double* __restrict__ x,
+                                                       const double* __restrict__ sub, double* __restrict__ y,
+                                                       double* part, unsigned* ctr, double* sums) {
+  x += (size_t)blockIdx.y * n;
+  y += (size_t)blockIdx.y * n;
+  if (SUB) sub += (size_t)blockIdx.y * n;
   double v[2] = {0.0, 0.0};
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     double s = 0.0;
     for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) s += vals[k] * x[colind[k]];
-    if (sub) {
-      s -= sub[i];
-      v[1] += sub[i] * sub[i];
+    if (SUB) {
+      const double b = sub[i];
+      s -= b;
+      v[0] += s * s;
+      v[1] += b * b;
     }
     y[i] = s;
-    v[0] += s * s;
   }
-  block_partials<2>(v, part);
+  if (SUB) grid_sums<2>(v, part + (size_t)blockIdx.y * 2 * kLossBlocks, ctr + blockIdx.y, sums + 2 * blockIdx.y);
 }
 
-// dG_e += scale (u_i Ae_a + GAe_i r_a), scale = 2 lam / (K ||r||^2) from sums.
-__global__ void resid_grad_kernel(int64_t ntril, const int32_t* __restrict__ trow, const int32_t* __restrict__ tci,
-                                  const double* __restrict__ u, const double* __restrict__ ae,
-                                  const double* __restrict__ gae, const double* __restrict__ r,
-                                  const double* __restrict__ sums, double coef, double* __restrict__ dg) {
-  const double scale = coef / sums[1];  // sums[1] = r.r
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ntril; e += (int64_t)gridDim.x * blockDim.x) {
-    const int i = trow[e], a = tci[e];
-    dg[e] += scale * (u[i] * ae[a] + gae[i] * r[a]);
-  }
-}
-
-// dLoss/do = dLoss/dG dG/do.
-__global__ void dout_kernel(int64_t ntril, const int32_t* __restrict__ trow, const int32_t* __restrict__ tci,
-                            const double* __restrict__ rs64, const float* __restrict__ o,
-                            const double* __restrict__ dg, double c0, float* __restrict__ dout) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ntril; e += (int64_t)gridDim.x * blockDim.x) {
-    const int i = trow[e], j = tci[e];
-    const double d = i == j ? sigmoid_d((double)o[e] + c0) * rs64[i] : rs64[j];
-    dout[e] = (float)(dg[e] * d);
-  }
-}
-
-// fp32 copies of A's values and diagonal and 1 / sqrt(A_ii) in both
-// precisions, once per call (the MLP's feature inputs and G's scaling).
-__global__ void mlp_inputs_kernel(int64_t n, int64_t nnz, const double* __restrict__ vals,
-                                  const double* __restrict__ diag, float* __restrict__ a32, float* __restrict__ d32,
-                                  float* __restrict__ rs32, double* __restrict__ rs64) {
-  const int64_t m = nnz > n ? nnz : n;
-  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < m; k += (int64_t)gridDim.x * blockDim.x) {
-    if (k < nnz) a32[k] = (float)vals[k];
-    if (k < n) {
-      const float d = (float)diag[k];
-      d32[k] = d;
-      rs32[k] = 1.0f / sqrtf(d);
-      rs64[k] = 1.0 / sqrt(diag[k]);
+// dLoss/dG of every tril entry e = (i, a), then dLoss/do:
+//   dL_K/dG_e = 2 (A g_i)_a / (n S) - [a == i] 2 / (n G_ii), S = quad / n   (FIRST: from
+//   gag, in place), plus for the nk vectors of this launch coef / (r.r) (u_i Ae_a + GAe_i r_a);
+//   dLoss/do = dLoss/dG dG/do (LAST).
+__global__ void __launch_bounds__(kRed) entry_grad_kernel(
+    int64_t n, int64_t ntril, const int32_t* __restrict__ trow, const int32_t* __restrict__ tci,
+    const double* __restrict__ g, double* __restrict__ dg, const double* __restrict__ ksums, int first, int nk,
+    const double* __restrict__ u, const double* __restrict__ ae, const double* __restrict__ gae,
+    const double* __restrict__ r, const double* __restrict__ rsums, double coef, int last,
+    const double* __restrict__ rs64, const float* __restrict__ o, double c0, float* __restrict__ dout) {
+  __shared__ double s_scale;
+  const double S = ksums[0] / (double)n;
+  for (int64_t e0 = (int64_t)blockIdx.x * blockDim.x; e0 < ntril; e0 += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t e = e0 + threadIdx.x;
+    const bool live = e < ntril;
+    const int i = live ? trow[e] : 0, a = live ? tci[e] : 0;
+    double v = live ? dg[e] : 0.0;
+    if (first && live) {
+      v = 2.0 * v / ((double)n * S);
+      if (a == i) v -= 2.0 / ((double)n * g[e]);
+    }
+    for (int k = 0; k < nk; ++k) {
+      __syncthreads();
+      if (threadIdx.x == 0) s_scale = coef / rsums[2 * k + 1];  // rsums[2 k + 1] = r_k.r_k
+      __syncthreads();
+      const size_t b = (size_t)k * n;
+      if (live) v += s_scale * (u[b + i] * ae[b + a] + gae[b + i] * r[b + a]);
+    }
+    if (!live) continue;
+    if (last) {
+      const double d = i == a ? sigmoid_d((double)o[e] + c0) * rs64[i] : rs64[a];
+      dout[e] = (float)(v * d);
+    } else {
+      dg[e] = v;
     }
   }
 }
 
-// G from the outputs (F5), diagonal entries: thread per row (the diagonal is
-// the last tril entry of its row), G_ii = softplus(o + c0) / sqrt(A_ii) in
-// fp64, so a zero output gives Jacobi's D^-1/2 to rounding.
-__global__ void g_diag_kernel(int64_t n, const int32_t* __restrict__ trp, const double* __restrict__ rs64,
-                              const float* __restrict__ o, double c0, double* __restrict__ g) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int e = trp[i + 1] - 1;
-    g[e] = softplus_d((double)o[e] + c0) * rs64[i];
+// A_ii in fp32 and 1 / sqrt(A_ii) in both precisions (the features' and G's scaling),
+// once per call.
+__global__ void mlp_diag_kernel(int64_t n, const double* __restrict__ diag, float* __restrict__ d32,
+                                float* __restrict__ rs32, double* __restrict__ rs64) {
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += (int64_t)gridDim.x * blockDim.x) {
+    const float d = (float)diag[k];
+    d32[k] = d;
+    rs32[k] = 1.0f / sqrtf(d);
+    rs64[k] = 1.0 / sqrt(diag[k]);
   }
 }
 
-// Off-diagonal entries, thread per entry: G_ij = o / sqrt(A_jj) (the diagonal
-// ones are g_diag_kernel's; separate kernels keep warps from running both).
-__global__ void g_offdiag_kernel(int64_t ntril, const int32_t* __restrict__ trow, const int32_t* __restrict__ tci,
-                                 const double* __restrict__ rs64, const float* __restrict__ o,
-                                 double* __restrict__ g) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < ntril; e += (int64_t)gridDim.x * blockDim.x) {
-    const int i = trow[e], j = tci[e];
-    if (i != j) g[e] = (double)o[e] * rs64[j];
+// Every row's scaled entries s(i, i + o_m) in fp32, rounded to bf16 (thread per row).
+struct OffsetTable {
+  int offs[kMaxOffs];
+  int noffs;
+};
+__global__ void row_features_kernel(int64_t n, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colind,
+                                    const double* __restrict__ vals, const float* __restrict__ rs32, OffsetTable T,
+                                    RowFeatures* __restrict__ rf) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    union {
+      uint4 q[2];
+      __nv_bfloat16 s[16];
+    } r;
+    r.q[0] = r.q[1] = make_uint4(0u, 0u, 0u, 0u);
+    const float si = rs32[i];
+    for (int k = rowptr[i]; k < rowptr[i + 1]; ++k) {
+      const int c = colind[k];
+      const int m = offset_slot(T.offs, T.noffs, c - (int)i);
+      const __nv_bfloat16 v = __float2bfloat16_rn((float)vals[k] * si * rs32[c]);
+#pragma unroll
+      for (int u = 0; u < kMaxOffs; ++u)
+        if (u == m) r.s[u] = v;
+    }
+    uint4* dst = reinterpret_cast<uint4*>(rf + i);
+    dst[0] = r.q[0];
+    dst[1] = r.q[1];
+  }
+}
+
+// G from the outputs (F5): the first n threads the diagonal entries (the diagonal is
+// the last tril entry of its row), G_ii = softplus(o + c0) / sqrt(A_ii) in fp64, so a
+// zero output gives Jacobi's D^-1/2 to rounding; the others G_ij = o / sqrt(A_jj),
+// thread per entry (two ranges keep warps from running both).
+__global__ void g_kernel(int64_t n, int64_t ntril, const int32_t* __restrict__ trp, const int32_t* __restrict__ trow,
+                         const int32_t* __restrict__ tci, const double* __restrict__ rs64,
+                         const float* __restrict__ o, double c0, double* __restrict__ g) {
+  const int64_t base = (n + 31) / 32 * 32;
+  for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < base + ntril;
+       k += (int64_t)gridDim.x * blockDim.x) {
+    if (k < n) {
+      const int e = trp[k + 1] - 1;
+      g[e] = softplus_d((double)o[e] + c0) * rs64[k];
+    } else if (k >= base) {
+      const int64_t e = k - base;
+      const int i = trow[e], j = tci[e];
+      if (i != j) g[e] = (double)o[e] * rs64[j];
+    }
   }
 }
 
@@ -660,7 +756,7 @@ cg_status mlp_prepare(cg_handle* h) {
   if (nts > 8) return mfail(h, CG_ERR_INVALID, "learned FSAI: more than 8 offsets in tril(A)");
   CGM_CUDA(h, cudaMalloc(&f->offs, sizeof(int32_t) * kMaxOffs));
   const size_t nv = (size_t)std::max<int64_t>(h->n, 1);
-  CGM_CUDA(h, cudaMalloc(&f->a32, sizeof(float) * (size_t)std::max<int64_t>(h->nnz, 1)));
+  CGM_CUDA(h, cudaMalloc(&f->rowf, sizeof(RowFeatures) * nv));
   CGM_CUDA(h, cudaMalloc(&f->d32, sizeof(float) * nv));
   CGM_CUDA(h, cudaMalloc(&f->rs32, sizeof(float) * nv));
   CGM_CUDA(h, cudaMalloc(&f->rs64, sizeof(double) * nv));
@@ -677,22 +773,31 @@ MlpArgs make_args(const cg_handle* h, const float* params) {
   MlpArgs M{};
   M.n = h->n;
   M.ntril = f->ntril;
-  M.rowptr = h->rowptr;
-  M.colind = h->colind;
-  M.vals = h->vals;
-  M.diag = h->diag;
   M.trow = f->trow;
   M.tci = f->tci;
-  M.tsrc = f->tsrc;
   M.params = params;
-  M.a32 = f->a32;
+  M.rf = static_cast<const RowFeatures*>(f->rowf);
   M.d32 = f->d32;
-  M.rs32 = f->rs32;
   for (int k = 0; k < kMaxOffs; ++k) M.offs[k] = k < f->noffs ? f->host_offs[k] : 0;
   M.noffs = f->noffs;
   M.ntslots = f->ntslots;
   M.c0 = std::log(std::exp(1.0) - 1.0);
   return M;
+}
+
+// The network's inputs of the handle's matrix, the forward pass on `grid` CTAs and G
+// from its outputs.
+void enqueue_factor(const cg_handle* h, const MlpArgs& M, unsigned grid, double* g) {
+  const FsaiData* f = h->fsai;
+  const int64_t n = h->n, nt = f->ntril;
+  OffsetTable T{};
+  for (int k = 0; k < kMaxOffs; ++k) T.offs[k] = M.offs[k];
+  T.noffs = M.noffs;
+  mlp_diag_kernel<<<blocks_for(n), 256, 0, h->stream>>>(n, h->diag, f->d32, f->rs32, f->rs64);
+  row_features_kernel<<<blocks_for(n, 128), 128, 0, h->stream>>>(n, h->rowptr, h->colind, h->vals, f->rs32, T,
+                                                                 static_cast<RowFeatures*>(f->rowf));
+  mlp_forward_kernel<<<grid, kMlpThreads, 0, h->stream>>>(M, f->mlp_o);
+  g_kernel<<<blocks_for(n + 32 + nt), 256, 0, h->stream>>>(n, nt, f->trp, f->trow, f->tci, f->rs64, f->mlp_o, M.c0, g);
 }
 
 unsigned mlp_grid(const cg_handle* h, int64_t ntril) {
@@ -734,12 +839,7 @@ cg_status cg_fsai_load(cg_handle* h, const void* weights_bf16, int64_t bytes) {
   if (!f->params32) CGM_CUDA(h, cudaMalloc(&f->params32, sizeof(float) * kNParams));
   CGM_CUDA(h, cudaMemcpyAsync(f->params32, p32.data(), sizeof(float) * kNParams, cudaMemcpyHostToDevice, h->stream));
   const MlpArgs M = make_args(h, f->params32);
-  const int64_t n = h->n, nt = f->ntril;
-  mlp_inputs_kernel<<<blocks_for(std::max(n, h->nnz)), 256, 0, h->stream>>>(n, h->nnz, h->vals, h->diag, f->a32,
-                                                                            f->d32, f->rs32, f->rs64);
-  mlp_forward_kernel<<<mlp_forward_grid(h, nt), kMlpThreads, 0, h->stream>>>(M, f->mlp_o);
-  g_diag_kernel<<<blocks_for(n), 256, 0, h->stream>>>(n, f->trp, f->rs64, f->mlp_o, M.c0, f->g);
-  g_offdiag_kernel<<<blocks_for(nt), 256, 0, h->stream>>>(nt, f->trow, f->tci, f->rs64, f->mlp_o, f->g);
+  enqueue_factor(h, M, mlp_forward_grid(h, f->ntril), f->g);
   CGM_CUDA(h, cudaGetLastError());
   CGM_CUDA(h, cudaStreamSynchronize(h->stream));  // p32 is host memory of this call
   return cgi::fsai_commit(h, 2);
@@ -777,63 +877,75 @@ cg_status cg_fsai_loss_grad(cg_handle* h, const float* params, float* grad, cons
   if (s != CG_OK) return s;
   FsaiData* f = h->fsai;
   const int64_t n = h->n, nt = f->ntril;
-  const unsigned rb = blocks_for(n, kRed);
   const unsigned mg = mlp_grid(h, nt);
-  if (!f->work) {
-    CGM_CUDA(h, cudaMalloc(&f->work, sizeof(double) * (6 * (size_t)n + 2 * (size_t)nt)));
-    CGM_CUDA(h, cudaMalloc(&f->rpart, sizeof(double) * (8192 * 2 + 16)));
-    CGM_CUDA(h, cudaMalloc(&f->dout, sizeof(float) * (size_t)nt));
-    CGM_CUDA(h, cudaMalloc(&f->gpart, sizeof(float) * (size_t)(4 * h->sm_count) * kNParams));
+  // the residual vectors go through the products together, in chunks of up to kc that
+  // keep the three work vectors of each within kResidBytes (one vector at least)
+  constexpr int64_t kResidBytes = (int64_t)256 << 20;
+  const int kc = (int)std::max<int64_t>(1, std::min<int64_t>({nresid, kResidBytes / (24 * n), 1024}));
+  auto grow = [&](auto** p, size_t count) {  // a larger buffer in the old one's place
+    if (*p) cudaFree(*p);
+    *p = nullptr;
+    return cudaMalloc(p, sizeof(**p) * count);
+  };
+  if (f->work_k < kc) {
+    f->work_k = 0;
+    CGM_CUDA(h, grow(&f->work, 3 * (size_t)kc * (size_t)n + 2 * (size_t)nt));
+    CGM_CUDA(h, grow(&f->rpart, 2 * (size_t)kLossBlocks * (size_t)kc));
+    CGM_CUDA(h, grow(&f->rctr, (size_t)kc));
+    CGM_CUDA(h, cudaMemsetAsync(f->rctr, 0, sizeof(unsigned) * (size_t)kc, h->stream));
+    f->work_k = kc;
+  }
+  if (f->sums_k < nresid + 1) {
+    f->sums_k = 0;
+    CGM_CUDA(h, grow(&f->rsums, 2 * ((size_t)nresid + 1)));
+    f->sums_k = nresid + 1;
+  }
+  if (!f->dout) CGM_CUDA(h, cudaMalloc(&f->dout, sizeof(float) * (size_t)nt));
+  if (!f->gpart) {
     CGM_CUDA(h, cudaFuncSetAttribute(mlp_backward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)sizeof(SmemB)));
+    CGM_CUDA(h, cudaMalloc(&f->gpart, sizeof(float) * (size_t)(4 * h->sm_count) * kNParams));
   }
-  double* u = f->work;
-  double* v = u + n;
-  double* e = v + n;
-  double* ae = e + n;
-  double* gae = ae + n;
-  double* gl = gae + n;         // G of the current parameters (tril order)
-  double* gag = gl + nt;        // (A g_i)_a, then dLoss/dG
-  double* dgv = gag;            // reused: gag is consumed by kaporin_grad_kernel in place
-  double* sums = f->rpart + 8192 * 2;  // [0] quad, [1] log-diag, [2] r.r, [3..] residual losses
+  const size_t kn = (size_t)f->work_k * (size_t)n;
+  double* u = f->work;          // u = G r
+  double* v = u + kn;           // G^T u, then A e
+  double* e = v + kn;           // A G^T u - r, then G A e
+  double* gl = e + kn;          // G of the current parameters (tril order)
+  double* dgv = gl + nt;        // (A g_i)_a, then dLoss/dG
+  double* sums = f->rsums;      // [0] quad, [1] log-diag, [2 + 2 k] e.e, [3 + 2 k] r.r
   const MlpArgs M = make_args(h, params);
   const cudaStream_t st = h->stream;
-  mlp_inputs_kernel<<<blocks_for(std::max(n, h->nnz)), 256, 0, st>>>(n, h->nnz, h->vals, h->diag, f->a32, f->d32,
-                                                                     f->rs32, f->rs64);
-  mlp_forward_kernel<<<mg, kMlpThreads, 0, st>>>(M, f->mlp_o);
-  g_diag_kernel<<<blocks_for(n), 256, 0, st>>>(n, f->trp, f->rs64, f->mlp_o, M.c0, gl);
-  g_offdiag_kernel<<<blocks_for(nt), 256, 0, st>>>(nt, f->trow, f->tci, f->rs64, f->mlp_o, gl);
-  kaporin_rows_kernel<<<rb, kRed, 0, st>>>(n, h->rowptr, h->colind, h->vals, f->trp, f->tci, gl, gag, f->rpart);
-  sum_parts_kernel<<<1, 32, 0, st>>>(f->rpart, (int)rb, 2, sums);
-  kaporin_grad_kernel<<<blocks_for(nt), 256, 0, st>>>(n, f->trow, f->tci, f->trp, gl, gag, sums, nt, dgv);
-  std::vector<double> rloss((size_t)nresid, 0.0);
-  for (int k = 0; k < nresid; ++k) {
-    const double* r = resid + (size_t)k * n;
-    g_mul_kernel<<<blocks_for(n), 256, 0, st>>>(n, f->trp, f->tci, gl, r, u);             // u = G r
-    gt_mul_kernel<<<blocks_for(n), 256, 0, st>>>(n, f->gtw, f->gtsrc, f->gtcol, gl, u, v);  // v = G^T u
-    a_mul_kernel<<<rb, kRed, 0, st>>>(n, h->rowptr, h->colind, h->vals, v, r, e, f->rpart);  // e = A v - r
-    sum_parts_kernel<<<1, 32, 0, st>>>(f->rpart, (int)rb, 2, sums + 2);  // e.e, r.r
-    a_mul_kernel<<<rb, kRed, 0, st>>>(n, h->rowptr, h->colind, h->vals, e, nullptr, ae, f->rpart);  // Ae
-    g_mul_kernel<<<blocks_for(n), 256, 0, st>>>(n, f->trp, f->tci, gl, ae, gae);                 // G A e
-    // dG += 2 lam / (K r.r) (u_i Ae_a + GAe_i r_a)
-    resid_grad_kernel<<<blocks_for(nt), 256, 0, st>>>(nt, f->trow, f->tci, u, ae, gae, r, sums + 2,
-                                                     2.0 * lambda / nresid, dgv);
-    double er[2] = {0.0, 0.0};
-    CGM_CUDA(h, cudaMemcpyAsync(er, sums + 2, sizeof(er), cudaMemcpyDeviceToHost, st));
-    CGM_CUDA(h, cudaStreamSynchronize(st));  // sums[2..3] are reused by the next vector
-    rloss[(size_t)k] = er[0] / er[1];
+  enqueue_factor(h, M, mg, gl);
+  const unsigned lb = (unsigned)std::min<int64_t>(kLossBlocks, blocks_for(nt, kRed));
+  kaporin_kernel<<<lb, kRed, 0, st>>>(nt, h->rowptr, h->colind, h->vals, f->trow, f->trp, f->tci, gl, dgv, f->rpart,
+                                      f->rctr, sums);
+  for (int k0 = 0; k0 < nresid || k0 == 0; k0 += kc) {
+    const int nk = std::min(kc, nresid - k0);  // 0 without residual vectors
+    const double* r = resid + (size_t)k0 * n;
+    double* rs = sums + 2 + 2 * (size_t)k0;
+    if (nk > 0) {
+      const dim3 grid((unsigned)std::min<int64_t>(kLossBlocks, blocks_for(n, kRed)), (unsigned)nk);
+      resid_g_kernel<<<grid, kRed, 0, st>>>(n, f->trp, f->tci, gl, r, u);
+      resid_gt_kernel<<<grid, kRed, 0, st>>>(n, f->gtw, f->gtsrc, f->gtcol, gl, u, v);
+      resid_a_kernel<true><<<grid, kRed, 0, st>>>(n, h->rowptr, h->colind, h->vals, v, r, e, f->rpart, f->rctr, rs);
+      resid_a_kernel<false><<<grid, kRed, 0, st>>>(n, h->rowptr, h->colind, h->vals, e, nullptr, v, nullptr, nullptr,
+                                                   nullptr);
+      resid_g_kernel<<<grid, kRed, 0, st>>>(n, f->trp, f->tci, gl, v, e);
+    }
+    entry_grad_kernel<<<blocks_for(nt, kRed), kRed, 0, st>>>(
+        n, nt, f->trow, f->tci, gl, dgv, sums, k0 == 0, nk, u, v, e, r, rs, nresid > 0 ? 2.0 * lambda / nresid : 0.0,
+        k0 + kc >= nresid, f->rs64, f->mlp_o, M.c0, f->dout);
   }
-  dout_kernel<<<blocks_for(nt), 256, 0, st>>>(nt, f->trow, f->tci, f->rs64, f->mlp_o, dgv, M.c0, f->dout);
   mlp_backward_kernel<<<mg, kMlpThreads, sizeof(SmemB), st>>>(M, f->dout, f->gpart);
-  reduce_parts_kernel<<<blocks_for(kNParams), 256, 0, st>>>(f->gpart, (int)mg, grad);
+  reduce_parts_kernel<<<(kNParams + 31) / 32, 32 * kRedWarps, 0, st>>>(f->gpart, (int)mg, grad);
   CGM_CUDA(h, cudaGetLastError());
-  double hs[2] = {0.0, 0.0};
-  CGM_CUDA(h, cudaMemcpyAsync(hs, sums, sizeof(hs), cudaMemcpyDeviceToHost, st));
+  std::vector<double> hs(2 * ((size_t)nresid + 1), 0.0);
+  CGM_CUDA(h, cudaMemcpyAsync(hs.data(), sums, sizeof(double) * hs.size(), cudaMemcpyDeviceToHost, st));
   CGM_CUDA(h, cudaStreamSynchronize(st));
   double loss = std::log(hs[0] / (double)n) - 2.0 / (double)n * hs[1];
   if (nresid > 0) {
     double lr = 0.0;
-    for (double x : rloss) lr += x;
+    for (int k = 0; k < nresid; ++k) lr += hs[2 + 2 * (size_t)k] / hs[3 + 2 * (size_t)k];
     loss += lambda * lr / nresid;
   }
   if (loss_out) *loss_out = loss;
