@@ -68,6 +68,11 @@ struct ClusterParams {
   uint64_t timeout_ns;  // limit of every wait for an exchange
   unsigned skip_seq;    // fault injection: CTA 0 does not push exchange #skip_seq (1-based)
   DevState* st;
+  // a CSR whose row lengths the host does not know (null on handles): found malformed;
+  // the most entries of a CTA's rows, which say whether they fit in smem_bytes
+  const int* refused;
+  const int* slice_max;
+  size_t smem_bytes;
 };
 
 // ---- distributed shared memory and mbarrier primitives (PTX ISA 8.x, sm_90+)
@@ -293,8 +298,19 @@ __device__ __forceinline__ double row_dot(const Slice& A, int k0, int len, int n
   return s;
 }
 
+// Dynamic shared memory of a CTA: the vectors, and with the CSR held in shared
+// memory its row pointers (an even count) and, per entry, a value and an address.
+__host__ __device__ inline size_t cluster_smem(int rows, int64_t slice_nnz) {
+  size_t b = sizeof(double) * (size_t)kVec * (size_t)rows;
+  if (slice_nnz >= 0) b += sizeof(int) * (size_t)((rows + 2) & ~1) + 12 * (size_t)slice_nnz;
+  return b;
+}
+
 template <bool SMEM>
 __global__ void __launch_bounds__(kBlock, 1) pcg_cluster_kernel(ClusterParams P) {
+  if (P.refused) {  // every CTA alike: malformed, or the other form's system
+    if (*P.refused || (P.slice_max && (cluster_smem(P.R, *P.slice_max) <= P.smem_bytes) != SMEM)) return;
+  }
   cgx::cluster_group cl = cgx::this_cluster();
   const int rank = (int)cl.block_rank();
   const int C = (int)cl.num_blocks();
@@ -660,14 +676,6 @@ void cluster_shape(int64_t n, int cmax, int* rows, int* ctas) {
   *ctas = (int)((n + *rows - 1) / *rows);
 }
 
-// Dynamic shared memory of a CTA: the vectors, and with the CSR held in shared
-// memory its row pointers (an even count) and, per entry, a value and an address.
-size_t cluster_smem(int rows, int64_t slice_nnz) {
-  size_t b = sizeof(double) * (size_t)kVec * (size_t)rows;
-  if (slice_nnz >= 0) b += sizeof(int) * (size_t)((rows + 2) & ~1) + 12 * (size_t)slice_nnz;
-  return b;
-}
-
 }  // namespace
 
 int64_t cgi::cluster_max_rows() { return (int64_t)kClusterMax * kMaxRowsPerCta; }
@@ -792,4 +800,120 @@ cg_status cgi::cluster_solve(cg_handle* h, const double* b, double* x, double to
     h->err = std::string("cg_solve: ") + cg_status_string(status);
   }
   return status;
+}
+
+namespace {
+
+// Checks of a CSR nobody has looked at (thread per row): rowptr[0] = 0, rowptr[n] = nnz,
+// non-decreasing, colind in [0, n); with jac a positive diagonal in every row.  A row's
+// entries are read only when its own pointers lie in [0, nnz].  A_ii goes to diag, the
+// most entries of R rows from a multiple of R to *slice_max.
+__global__ void check_csr_kernel(int n, int nnz, int R, const int32_t* __restrict__ rowptr,
+                                 const int32_t* __restrict__ colind, const double* __restrict__ vals, int jac,
+                                 double* __restrict__ diag, int* refused, int* slice_max) {
+  const int i = (int)(blockIdx.x * blockDim.x + threadIdx.x);
+  if (i >= n) return;
+  const int a = rowptr[i], e = rowptr[i + 1];
+  bool bad = (i == 0 && a != 0) || (i == n - 1 && e != nnz) || a < 0 || e < a || e > nnz;
+  if (!bad) {
+    double d = 0.0;
+    bool found = false;
+    for (int k = a; k < e; ++k) {
+      const int c = colind[k];
+      bad = bad || c < 0 || c >= n;
+      if (c == i) {
+        d += vals[k];
+        found = true;
+      }
+    }
+    bad = bad || (jac && !(found && d > 0.0));
+    diag[i] = d;
+  }
+  if (bad) *refused = 1;
+  if (i % R == 0) atomicMax(slice_max, rowptr[i + R < n ? i + R : n] - a);
+}
+
+}  // namespace
+
+cudaError_t cgi::cluster_solve_checked(int n, int nnz, const int32_t* rowptr, const int32_t* colind,
+                                       const double* vals, const double* b, double* x, double tol, int maxit,
+                                       bool jac, int max_restarts, uint64_t timeout_ns, double* diag,
+                                       CheckedWords* words, cudaStream_t stream, bool* launched) {
+  *launched = false;
+  if (n > cluster_max_rows()) return cudaSuccess;
+  const void* fns[2] = {(const void*)pcg_cluster_kernel<true>, (const void*)pcg_cluster_kernel<false>};
+  int dev = 0, smem_optin = 0;
+  cudaFuncAttributes fa{};
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fns[0]);
+  if (e != cudaSuccess) return e;
+  const size_t smem = (size_t)smem_optin - fa.sharedSizeBytes;
+  int cmax = kClusterMax;
+  for (const void* fn : fns) {
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+      cudaGetLastError();
+      cmax = 8;
+    }
+  }
+  for (;;) {
+    ClusterParams P{};
+    int ctas = 0;
+    cluster_shape(n, cmax, &P.R, &ctas);
+    if (P.R > kMaxRowsPerCta) return cudaSuccess;  // too large for a portable cluster
+    // the CSR in shared memory when every CTA's rows fit: for sure when all entries fit
+    // one CTA, never when even an equal share does not; else the kernels look
+    const bool sure = cluster_smem(P.R, nnz) <= smem, never = cluster_smem(P.R, nnz / ctas) > smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)ctas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg[2] = {};
+    bool placed = true;
+    for (int f = 0; f < 2; ++f) {
+      cfg[f].gridDim = dim3((unsigned)ctas);
+      cfg[f].blockDim = dim3(kBlock);
+      cfg[f].dynamicSmemBytes = f == 0 ? (sure ? cluster_smem(P.R, nnz) : smem) : cluster_smem(P.R, -1);
+      cfg[f].stream = stream;
+      cfg[f].attrs = attr;
+      cfg[f].numAttrs = 1;
+      e = cudaFuncSetAttribute(fns[f], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg[f].dynamicSmemBytes);
+      if (e != cudaSuccess) return e;
+      int active = 0;
+      e = cudaOccupancyMaxActiveClusters(&active, fns[f], &cfg[f]);
+      placed = placed && e == cudaSuccess && active >= 1;
+    }
+    if (!placed) {
+      cudaGetLastError();
+      if (cmax == 8) return cudaSuccess;  // no cluster fits: the caller's one-CTA form
+      cmax = 8;
+      continue;
+    }
+    if ((e = cudaMemsetAsync(words, 0, sizeof(CheckedWords), stream)) != cudaSuccess) return e;
+    check_csr_kernel<<<(unsigned)((n + 127) / 128), 128, 0, stream>>>(n, nnz, P.R, rowptr, colind, vals, jac ? 1 : 0,
+                                                                      diag, &words->refused, &words->slice_max);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    P.n = n;
+    P.rmagic = (unsigned)((1ull << 32) / (unsigned long long)P.R + 1ull);
+    P.rowptr = rowptr;
+    P.colind = colind;
+    P.vals = vals;
+    P.diag = diag;
+    P.b = b;
+    P.x = x;
+    P.tol = tol;
+    P.maxit = maxit;
+    P.max_restarts = max_restarts;
+    P.jac = jac ? 1 : 0;
+    P.timeout_ns = timeout_ns;
+    P.st = &words->st;
+    P.refused = &words->refused;
+    P.slice_max = sure || never ? nullptr : &words->slice_max;
+    P.smem_bytes = smem;
+    if (!never) e = cudaLaunchKernelEx(&cfg[0], pcg_cluster_kernel<true>, P);
+    if (e == cudaSuccess && !sure) e = cudaLaunchKernelEx(&cfg[1], pcg_cluster_kernel<false>, P);
+    *launched = e == cudaSuccess;
+    return e;
+  }
 }

@@ -30,6 +30,18 @@ cg_status ensure_offsets(cg_handle* h);         // cg_handle::offs_all, once (cg
 int64_t cluster_max_rows();
 cg_status cluster_solve(cg_handle* h, const double* b, double* x, double tol, int32_t maxit, bool jac,
                         int32_t* iters_out, double* relres_out);
+// the cluster's loop on a CSR that is checked on the device first, without a handle or any
+// allocation (cg_noalloc.cu); *launched = false: no cluster holds the system, nothing
+// was enqueued.  diag: scratch of n doubles; words: the result, on the device
+struct CheckedWords {
+  DevState st;
+  int refused;    // malformed CSR
+  int slice_max;  // most entries of a CTA's rows
+};
+cudaError_t cluster_solve_checked(int n, int nnz, const int32_t* rowptr, const int32_t* colind, const double* vals,
+                                  const double* b, double* x, double tol, int maxit, bool jac, int max_restarts,
+                                  uint64_t timeout_ns, double* diag, CheckedWords* words, cudaStream_t stream,
+                                  bool* launched);
 }  // namespace cgi
 
 // Device memory owned by a handle.  The internal off-diagonal matrices and
