@@ -1084,7 +1084,7 @@ cg_status cg_create(int64_t n, const int32_t* rowptr, const int32_t* colind, con
   if (e == cudaSuccess) e = cudaMemcpy(h->rb, rb.data(), sizeof(int32_t) * rb.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&h->diag, sizeof(double) * nv);
   if (e == cudaSuccess) e = cudaMalloc(&h->ndiag, sizeof(int32_t) * nv);
-  if (e == cudaSuccess) e = cudaMalloc(&h->st, sizeof(DevState));
+  if (e == cudaSuccess) e = cudaMalloc(&h->st, kStBytes);
   if (e == cudaSuccess) e = cudaMallocHost(&h->host_st, sizeof(DevState));
   if (e == cudaSuccess) e = cudaEventCreate(&h->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&h->ev1);
@@ -1128,7 +1128,7 @@ cg_status cg_create(int64_t n, const int32_t* rowptr, const int32_t* colind, con
                           max_coresident(pcg_ir_kernel<true, true>, h->sm_count));
   const int g4 = std::min(max_coresident(pcg_ir_kernel<false, false>, h->sm_count),
                           max_coresident(pcg_ir_kernel<false, true>, h->sm_count));
-  h->grid_max = std::min(std::min(g1, g2), std::min(g3, g4));
+  h->grid_max = std::min(std::min(std::min(g1, g2), std::min(g3, g4)), kXCtas);
   const int g5 = std::min(std::min(max_coresident(g_upd_r<double, true>, h->sm_count),
                                    max_coresident(g_upd_r<double, false>, h->sm_count)),
                           max_coresident(g_upd_xp<float, true, true, true>, h->sm_count));
@@ -1235,6 +1235,7 @@ SolveParams make_solve_params(const cg_handle* h, bool jac, const double* b, dou
   P.part = h->part;
   P.pstride = h->grid_part;
   P.st = h->st;
+  P.xs = exchange_words(h->st);
   P.tol = tol;
   P.tol_in = h->tol_in_set ? h->tol_in : (carry ? kRuTolInner : kIrTolInner);
   P.maxit = maxit;
@@ -1292,25 +1293,34 @@ cg_status solve_impl(cg_handle* h, const double* b, double* x, double tol, int32
   cg_status s = prepare_impl(h, jac, fp64);
   if (s != CG_OK) return s;
 
-  const int G = auto_grid(h);
+  int G = auto_grid(h);
   SolveParams P = make_solve_params(h, jac, b, x, tol, maxit, fp64, carry);
   if (fsai) return cgi::fsai_solve(h, P, fp64, carry, G, iters_out, relres_out);
+  // stencil systems whose vectors the SMs' shared memory holds: one persistent launch
+  // that keeps them there (a grid size, the timers and the fault injection belong to
+  // the form below)
+  bool launched = false;
+  if (fp64 && h->loop_mode <= 1 && h->grid_opt == 0 && h->skip_seq == 0 && h->timers == 0)
+    CG_CUDA(h, cgi::resident_launch(h, P, jac, &G, &launched));
   // auto: fp64 takes the graph form from kGraphMinRows rows; the refinement's
   // fp32 vector passes are short, so it stays in the persistent form
-  const bool graph_mode = !carry && (h->loop_mode >= 2 || (h->loop_mode == 0 && fp64 && h->n >= kGraphMinRows));
+  const bool graph_mode = !launched && !carry &&
+                          (h->loop_mode >= 2 || (h->loop_mode == 0 && fp64 && h->n >= kGraphMinRows));
   if (graph_mode && fp64)
     return solve_graph64(h, P, jac, h->loop_mode == 3 ? kUnrollIters : 0, iters_out, relres_out);
   if (graph_mode) return solve_graph_ir(h, P, jac, iters_out, relres_out);
-  void* args[] = {&P};
-  const void* fn;
-  if (fp64)
-    fn = jac ? (const void*)pcg64_kernel<true> : (const void*)pcg64_kernel<false>;
-  else
-    fn = carry ? (jac ? (const void*)pcg_ir_kernel<true, true> : (const void*)pcg_ir_kernel<false, true>)
-               : (jac ? (const void*)pcg_ir_kernel<true, false> : (const void*)pcg_ir_kernel<false, false>);
-  CG_CUDA(h, cudaMemsetAsync(h->st, 0, sizeof(DevState), h->stream));
-  CG_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-  CG_CUDA(h, cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kBlock), args, 0, h->stream));
+  if (!launched) {
+    void* args[] = {&P};
+    const void* fn;
+    if (fp64)
+      fn = jac ? (const void*)pcg64_kernel<true> : (const void*)pcg64_kernel<false>;
+    else
+      fn = carry ? (jac ? (const void*)pcg_ir_kernel<true, true> : (const void*)pcg_ir_kernel<false, true>)
+                 : (jac ? (const void*)pcg_ir_kernel<true, false> : (const void*)pcg_ir_kernel<false, false>);
+    CG_CUDA(h, cudaMemsetAsync(h->st, 0, kStBytes, h->stream));
+    CG_CUDA(h, cudaEventRecord(h->ev0, h->stream));
+    CG_CUDA(h, cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kBlock), args, 0, h->stream));
+  }
   CG_CUDA(h, cudaEventRecord(h->ev1, h->stream));
   CG_CUDA(h, cudaMemcpyAsync(h->host_st, h->st, sizeof(DevState), cudaMemcpyDeviceToHost, h->stream));
   CG_CUDA(h, cudaStreamSynchronize(h->stream));

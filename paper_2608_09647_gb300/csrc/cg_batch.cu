@@ -85,6 +85,7 @@ struct BatchParams {
   double tol;
   int maxit, max_restarts;
   DevState* st;
+  XWord* xs;
   uint64_t timeout_ns;
   unsigned skip_seq;
   // fp32 inner solves with fp64 refinement (batch_ir_kernel only)
@@ -476,7 +477,8 @@ __global__ void __launch_bounds__(kBlock, MINB) batch_pcg_kernel(BatchParams P) 
   __shared__ int s_pref[kMaxBatch];
   __shared__ int s_scan[kWarps];
   __shared__ SegInfo s_seg;
-  Grid g(P.st, P.timeout_ns, P.skip_seq);
+  __shared__ XState s_x;
+  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
   double* __restrict__ r = P.r;
   double* __restrict__ p = P.p;
   double* __restrict__ q = P.q;
@@ -676,7 +678,8 @@ __global__ void __launch_bounds__(kBlock, MINB) batch_ir_kernel(BatchParams P) {
   __shared__ int s_pref[kMaxBatch];
   __shared__ int s_scan[kWarps];
   __shared__ SegInfo s_seg;
-  Grid g(P.st, P.timeout_ns, P.skip_seq);
+  __shared__ XState s_x;
+  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
   float* __restrict__ r = P.r32;
   float* __restrict__ p = P.p32;
   float* __restrict__ q = P.q32;
@@ -1270,6 +1273,7 @@ BatchParams make_params(cg_handle* h, bool jac, double tol, int maxit) {
   P.maxit = maxit;
   P.max_restarts = h->max_restarts;
   P.st = h->st;
+  P.xs = exchange_words(h->st);
   P.timeout_ns = (uint64_t)(h->timeout_ms * 1e6);
   P.skip_seq = h->skip_seq;
   P.val32 = B->val32[jac];
@@ -1295,7 +1299,7 @@ cudaError_t enqueue_solve(cg_handle* h, cudaStream_t s, bool jac, int var, int G
   P.carry = carry ? 1 : 0;
   P.tol_in = tol_in;
   const dim3 gg(64, (unsigned)B->nsys);
-  cudaError_t e = cudaMemsetAsync(h->st, 0, sizeof(DevState), s);
+  cudaError_t e = cudaMemsetAsync(h->st, 0, kStBytes, s);
   if (e != cudaSuccess) return e;
   batch_gather_kernel<<<gg, 256, 0, s>>>(B->d_b, B->d_x, B->d_n, B->d_r0, B->d_ntile, B->disq, B->dsq,
                                           jac ? 1 : 0, B->bh, B->xh);
@@ -1461,7 +1465,7 @@ cg_status cg_batch_create(int32_t nsys, const int64_t* n, const int32_t* const* 
   int dev = 0;
   CGB_CREATE(cudaGetDevice(&dev));
   CGB_CREATE(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev));
-  CGB_CREATE(cudaMalloc(&h->st, sizeof(DevState)));
+  CGB_CREATE(cudaMalloc(&h->st, kStBytes));
   CGB_CREATE(cudaMallocHost(&h->host_st, sizeof(DevState)));
   CGB_CREATE(cudaEventCreate(&h->ev0));
   CGB_CREATE(cudaEventCreate(&h->ev1));

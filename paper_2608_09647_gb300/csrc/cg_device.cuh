@@ -1,5 +1,5 @@
-// Device-side building blocks shared by the libcg kernels: bounded grid
-// barrier, fixed-order block and grid reductions, vector load helpers.
+// Device-side building blocks shared by the libcg kernels: exact sums, block and
+// grid reductions, the grid exchange (a bounded barrier that carries sums).
 #pragma once
 
 #include <cstdint>
@@ -93,6 +93,28 @@ __device__ __forceinline__ bool grid_barrier(DevState* st, unsigned nblocks, uin
   return s_ok != 0;
 }
 
+// One entry from shared memory (`own`) or from global memory through L2, by predicated
+// loads: as a branch per gather the loads of a row waited for one another.  The
+// address that is not taken is not touched.
+__device__ __forceinline__ double ld_own_or_l2(unsigned smem, const double* global, bool own) {
+  double v;
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %3, 0;\n @p ld.shared.f64 %0, [%1];\n @!p ld.global.cg.f64 %0, [%2];\n}"
+      : "=d"(v)
+      : "r"(smem), "l"(global), "r"((unsigned)own)
+      : "memory");
+  return v;
+}
+__device__ __forceinline__ float ld_own_or_l2(unsigned smem, const float* global, bool own) {
+  float v;
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %3, 0;\n @p ld.shared.f32 %0, [%1];\n @!p ld.global.cg.f32 %0, [%2];\n}"
+      : "=f"(v)
+      : "r"(smem), "l"(global), "r"((unsigned)own)
+      : "memory");
+  return v;
+}
+
 // ---- exact sums on the integer pipes (cg_exact.cuh).  GB300's fp64 unit issues
 // one warp instruction per ~64 clocks per SM sub-partition, so a tree of fp64
 // adds in one warp (5 levels for a warp, 8 for a CTA) sits on every reduction's
@@ -126,16 +148,24 @@ __device__ __forceinline__ cg_exact::i128 warp_sum64(long long X) {
   return (i128)s0 + (i128)s1 * ((i128)1 << 22) + (i128)s2 * ((i128)1 << 44);
 }
 
-// In every lane: the exact sum of the lanes' fp64 values at the warp's scale
-// (the largest exponent field among them), packed with that scale.
-__device__ __forceinline__ ulonglong2 warp_exact(double v) {
+// In every lane: the exact sum of the lanes' fp64 values at the warp's scale *E
+// (the largest exponent field among them).
+__device__ __forceinline__ cg_exact::i128 warp_exact_sum(double v, int* E, bool* bad) {
   const cg_exact::Parts p = cg_exact::parts(v);
   // one redux for the scale and the NaN flag (a bad sum is NaN; any scale >= every e will do)
   const unsigned eb = __reduce_max_sync(0xffffffffu, (unsigned)p.e | (p.bad ? 0x10000u : 0u));
-  const bool bad = eb > 0xFFFFu;
-  const int E = bad ? 2046 : (int)(eb & 0xFFFFu);
+  *bad = eb > 0xFFFFu;
+  *E = *bad ? 2046 : (int)(eb & 0xFFFFu);
+  return warp_sum64(cg_exact::to_fixed(p, *E));
+}
+
+// The same, packed with that scale.
+__device__ __forceinline__ ulonglong2 warp_exact(double v) {
+  int E;
+  bool bad;
+  const cg_exact::i128 S = warp_exact_sum(v, &E, &bad);
   unsigned long long lo, hi;
-  cg_exact::pack(warp_sum64(cg_exact::to_fixed(p, E)), E, bad, &lo, &hi);
+  cg_exact::pack(S, E, bad, &lo, &hi);
   return make_ulonglong2(lo, hi);
 }
 
@@ -165,7 +195,7 @@ __device__ __forceinline__ cg_exact::i128 sum_entries(const ulonglong2& w, bool 
 // then warp 0 adds the 8 warp sums exactly and rounds once to fp64.  The result
 // does not depend on which thread held which value.
 template <int NV>
-__device__ __forceinline__ void cta_sum0_exact(double (&v)[NV]) {
+__device__ __forceinline__ void cta_sum0(double (&v)[NV]) {
   __shared__ ulonglong2 s_w[NV][kWarps];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   ulonglong2 w[NV];
@@ -186,45 +216,6 @@ __device__ __forceinline__ void cta_sum0_exact(double (&v)[NV]) {
       v[j] = cg_exact::to_fp64(T, E, bad);
     }
   }
-}
-
-// Sum of v over the CTA in a fixed order, valid in thread 0 only.  A warp-wide
-// fp64 add occupies GB300's fp64 pipe (2 lanes per clock per SM, ~64 clocks of
-// one sub-partition's unit) whatever its active lanes, so the tree is kept to
-// one warp: every thread stores its values,
-// lane l of warp 0 sums threads l, l+32, ... in that order and the 32 lane
-// sums meet in an xor-tree: 416 fp64 lane operations per value, against
-// 3,328 for an xor-tree in every warp followed by every thread summing the
-// warp sums (block_sum).
-template <int NV>
-__device__ __forceinline__ void cta_sum0_fp64(double (&v)[NV]) {
-  __shared__ double s_v[NV][kBlock];
-  __syncthreads();  // s_v may still be read by warp 0 of a previous call
-#pragma unroll
-  for (int j = 0; j < NV; ++j) s_v[j][threadIdx.x] = v[j];
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      double t = s_v[j][lane];
-#pragma unroll
-      for (int w = 1; w < kWarps; ++w) t += s_v[j][w * 32 + lane];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-      v[j] = t;
-    }
-  }
-}
-
-
-// The CTA sum used by the loops: exact (cta_sum0_exact) or, in the fp64 persistent
-// kernels, whose 128-register budget has no room for the 128-bit integer steps,
-// the one-warp fp64 tree (cta_sum0_fp64).  Valid in warp 0.
-template <int NV, bool EXACT = true>
-__device__ __forceinline__ void cta_sum0(double (&v)[NV]) {
-  if constexpr (EXACT) cta_sum0_exact<NV>(v);
-  else cta_sum0_fp64<NV>(v);
 }
 
 // Sum of v over the CTA in a fixed order (warp xor-tree, then warp 0 over the
@@ -280,7 +271,7 @@ __device__ __forceinline__ bool below_stop(double rr, double stop, double stop2_
 // Every CTA computes the identical value (same loads, same order), so decisions
 // made from it agree across the grid without another barrier.
 template <int NV>
-__device__ __forceinline__ void grid_sum_exact_lanes(const double* part, unsigned G, double (&out)[NV]) {
+__device__ __forceinline__ void grid_sum_lanes(const double* part, unsigned G, double (&out)[NV]) {
   constexpr int kGridBatch = NV <= 2 ? 8 : 1;  // NV > 2: the once-per-solve residual sums
   __shared__ double s_out[NV];
   if (threadIdx.x < 32) {
@@ -338,61 +329,16 @@ __device__ __forceinline__ void grid_sum_exact_lanes(const double* part, unsigne
   __syncthreads();
 }
 
-// Sum of the G per-CTA partials part[j*G + c] in a fixed order (lane l of
-// warp 0 adds c = l, l + 32, ... in order, then an xor tree), given to every
-// thread.  Every CTA computes the identical value (same loads, same order), so
-// decisions made from it agree across the grid without another barrier.  Each
-// lane's loads go out kGridBatch at a time, so the sum waits for about
-// G / (32 kGridBatch) L2 round trips instead of G / 32.
-template <int NV>
-__device__ __forceinline__ void grid_sum_fp64(const double* part, unsigned G, double (&out)[NV]) {
-  constexpr int kGridBatch = NV <= 2 ? 8 : 1;  // NV > 2: the once-per-solve residual sums
-  __shared__ double s_out[NV];
-  if (threadIdx.x < 32) {
-    const unsigned lane = threadIdx.x;
-    double t[NV];
-#pragma unroll
-    for (int j = 0; j < NV; ++j) t[j] = 0.0;
-    for (unsigned c0 = lane; c0 < G; c0 += 32u * kGridBatch) {
-      double v[kGridBatch][NV];
-#pragma unroll
-      for (int u = 0; u < kGridBatch; ++u) {
-        const unsigned c = c0 + 32u * u;
-#pragma unroll
-        for (int j = 0; j < NV; ++j) v[u][j] = c < G ? __ldcg(part + (size_t)j * G + c) : 0.0;
-      }
-#pragma unroll
-      for (int u = 0; u < kGridBatch; ++u) {
-        if (c0 + 32u * u < G) {
-#pragma unroll
-          for (int j = 0; j < NV; ++j) t[j] += v[u][j];
-        }
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) t[j] += __shfl_xor_sync(0xffffffffu, t[j], o);
-      if (lane == 0) s_out[j] = t[j];
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < NV; ++j) out[j] = s_out[j];
-  __syncthreads();
-}
-
-
 // The same sum with every thread loading: thread t takes partials t, t + 256, ...
 // (at most kPer = 4 of them, all loads in flight: one L2 round trip), each warp
 // sums each of its kPer loads exactly (warp_exact), and warp 0 adds the warps'
 // entries, one a lane, exactly and rounds once.  For G > 1024, or in the
 // one-warp scalar kernels of the graph forms, the lane form.
 template <int NV>
-__device__ __forceinline__ void grid_sum_exact(const double* part, unsigned G, double (&out)[NV]) {
+__device__ __forceinline__ void grid_sum(const double* part, unsigned G, double (&out)[NV]) {
   constexpr int kPer = 4;
   if (G > (unsigned)(kPer * kBlock) || blockDim.x != (unsigned)kBlock) {
-    grid_sum_exact_lanes<NV>(part, G, out);
+    grid_sum_lanes<NV>(part, G, out);
     return;
   }
   __shared__ ulonglong2 s_w[NV][kPer * kWarps];
@@ -434,12 +380,258 @@ __device__ __forceinline__ void grid_sum_exact(const double* part, unsigned G, d
   __syncthreads();
 }
 
-// The sum of the G per-CTA partials used by the loops: exact, or the fp64 form in
-// the fp64 persistent kernels (see cta_sum0).
-template <int NV, bool EXACT = true>
-__device__ __forceinline__ void grid_sum(const double* part, unsigned G, double (&out)[NV]) {
-  if constexpr (EXACT) grid_sum_exact<NV>(part, G, out);
-  else grid_sum_fp64<NV>(part, G, out);
+// ---- exchanges of a co-resident (cooperatively launched) grid
+//
+// One exchange is a grid barrier that carries NV sums at no further cost: a CTA adds
+// its exact sum, as an integer at a scale every CTA knows, to accumulators in L2,
+// three words on lines of their own, and each word's top 9 bits count the CTAs that
+// have added.  A CTA has the grid's sum when every count
+// is complete: one reduction without a returned value and one poll, the round trip a
+// plain arrival counter takes.  (Partials read back after a counter's wait cost a
+// second round trip and a tree, ~4 us a sum of 304 CTAs; all CTAs polling all CTAs'
+// slots 6-9 us, and in two levels of ~18 slots 4 us, most of it fences.)
+//
+// The accumulators only grow: a CTA subtracts the words it read when their last use
+// was complete.  Exchanges alternate between two sets of words: nobody adds to a set
+// again before every CTA has arrived at the exchange in between, so has read it.
+//
+// The scale is that of the last sum of the same kind, with room both ways.  A CTA
+// whose sum does not fit (or is not finite) says so in the third word, and a total
+// far below the last one would lack bits: then, the same in every CTA, the largest
+// exponent is exchanged first and the sum is formed again at that scale.
+constexpr int kXCtas = cg_exact::kMaxAddends;  // most CTAs of a grid that exchanges sums
+constexpr int kXVals = 2;                      // most sums per exchange
+constexpr int kXKinds = 6;                     // kinds of sums whose scales are kept
+
+// One word a 128-byte line: per set a plain counter (barriers without a sum) and
+// three limbs a value, each in kXSplit words that every kXSplit-th CTA adds to and that
+// a poll reads together (atomics on one address go one after the other: 152 of them
+// took about as long as the round trip); then the largest-exponent word.
+struct XWord {
+  unsigned long long w;
+  unsigned long long pad[15];
+};
+constexpr int kXSplit = 4;
+constexpr int kXWords = kXSplit * (1 + 3 * kXVals);
+constexpr int kXAll = 2 * kXWords + 1;
+constexpr size_t kXBytes = sizeof(XWord) * kXAll;
+static_assert(kXSplit * 3 * kXVals <= 32, "a lane a word");
+
+// A CTA's exchanges, in shared memory: its grid (or group of a grid), the words at
+// their last use and the scales of the last sums.
+struct XState {
+  DevState* st;
+  XWord* words;
+  uint64_t timeout_ns;
+  unsigned G, rank;   // CTAs that exchange; this one's number among them
+  unsigned seq;       // exchanges so far
+  unsigned skip_seq;  // fault injection: do not add at this exchange (1-based; 0: never)
+  int scale[kXKinds];  // exponent field of the last sum; 0: none yet
+  unsigned long long prev[2][kXWords];
+};
+
+__device__ __forceinline__ void x_init(XState* x, DevState* st, XWord* words, unsigned G, unsigned rank,
+                                       unsigned skip_seq, uint64_t timeout_ns) {
+  for (int k = threadIdx.x; k < 2 * kXWords; k += blockDim.x) x->prev[k / kXWords][k % kXWords] = 0ull;
+  for (int k = threadIdx.x; k < kXKinds; k += blockDim.x) x->scale[k] = 0;
+  if (threadIdx.x == 0) {
+    x->st = st;
+    x->words = words;
+    x->timeout_ns = timeout_ns;
+    x->G = G;
+    x->rank = rank;
+    x->seq = 0;
+    x->skip_seq = skip_seq;
+  }
+  __syncthreads();
+}
+
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+__device__ __forceinline__ void red_add(XWord* p, unsigned long long v) {
+  asm volatile("red.relaxed.gpu.global.add.u64 [%0], %1;" ::"l"(&p->w), "l"(v) : "memory");
+}
+__device__ __forceinline__ void red_max(XWord* p, unsigned long long v) {
+  asm volatile("red.relaxed.gpu.global.max.u64 [%0], %1;" ::"l"(&p->w), "l"(v) : "memory");
+}
+template <bool ORDER>
+__device__ __forceinline__ unsigned long long ld_word(const XWord* p) {
+  unsigned long long v;
+  if (ORDER) asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&p->w) : "memory");
+  else asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(&p->w) : "memory");
+  return v;
+}
+
+// Warp 0 adds add[w] to the n words w0 + w of the exchange's set (lane kXSplit w + k
+// holds add[w] and word k of its split) and waits (bounded) until their counts, at bit
+// `at`, say that all G CTAs have; *diff: what the CTAs added to the lane's word.
+// False: a wait gave up.  ORDER: this CTA's global writes
+// (before the caller's last __syncthreads) come before its words, and the other CTAs'
+// writes before theirs are visible after the wait (acquiring polls: relaxed ones and a
+// fence after the wait took ~0.3 us more).
+template <bool ORDER>
+__device__ __forceinline__ bool x_round(XState* c, unsigned seq, int w0, int n, int at, unsigned long long add,
+                                        unsigned long long* diff) {
+  const int lane = threadIdx.x & 31;
+  bool ok = true;
+  unsigned long long d = 0;
+  if (ORDER) fence_gpu();
+  if (lane < kXSplit * n) {
+    const unsigned sub = (unsigned)lane % kXSplit;
+    const unsigned G = (c->G + kXSplit - 1 - sub) / kXSplit;  // CTAs that add to this word
+    XWord* w = c->words + (seq & 1u) * kXWords + kXSplit * w0 + lane;
+    unsigned long long* prev = &c->prev[seq & 1u][kXSplit * w0 + lane];
+    const unsigned long long was = *prev;
+    if (c->rank % kXSplit == sub && c->skip_seq != seq) red_add(w, add);
+    uint64_t t0 = 0;
+    for (unsigned spins = 0;; ++spins) {
+      const unsigned long long now = ld_word<ORDER>(w);
+      d = now - was;
+      if ((d >> at) == G) {
+        *prev = now;
+        break;
+      }
+      if (spins == 0) t0 = global_timer_ns();
+      if ((spins & 15u) == 15u) {
+        if (ld_relaxed_s32(&c->st->abort) != 0) { ok = false; break; }
+        if (global_timer_ns() - t0 > c->timeout_ns) {
+          if (atomicCAS(&c->st->abort, 0, 1) == 0) {
+            c->st->err_cta = (int)blockIdx.x;
+            c->st->err_barrier = (int)seq;
+          }
+          ok = false;
+          break;
+        }
+      }
+    }
+  }
+  *diff = d;
+  return __all_sync(0xffffffffu, ok);
+}
+
+// The sum of value j from the lanes that hold its words.
+__device__ __forceinline__ cg_exact::i128 x_join(unsigned long long d, int j, int* exceptions) {
+#pragma unroll
+  for (int o = 1; o < kXSplit; o <<= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+  return cg_exact::join_limbs(__shfl_sync(0xffffffffu, d, kXSplit * 3 * j), __shfl_sync(0xffffffffu, d, kXSplit * (3 * j + 1)),
+                              __shfl_sync(0xffffffffu, d, kXSplit * (3 * j + 2)), exceptions);
+}
+
+struct XSums {
+  double v0, v1;
+  bool ok;
+};
+
+// The next exchange of c, called by every thread.  Warp 0
+// gets the sums over the grid of the threads' v0 and v1 (NV of them, of kinds `kind`,
+// `kind` + 1; NV = 0 is a plain barrier, of any G), exact and rounded once, the same
+// bits in every CTA, and whether it succeeded; the other warps return at once and meet
+// warp 0 at the caller's next __syncthreads().  Global writes made by any CTA before
+// the exchange are visible to every CTA after that.  Every wait is bounded: a CTA that
+// waits longer than timeout_ns, or sees another's abort flag, records CG_ERR_TIMEOUT
+// and gets ok = false; the caller must then leave the kernel.
+// Not inlined: the 128-bit steps would cost the persistent kernels' loops registers.
+template <int NV, int WARPS = kWarps, bool ORDER = true>
+__device__ __noinline__ XSums grid_exchange(XState* c, int kind, double v0, double v1) {
+  constexpr int kN = NV > 0 ? NV : 1;
+  // the warps' sums at their own scales, and as limbs at the exchange's scale (all ones
+  // in the third limb: it does not fit there)
+  __shared__ ulonglong2 s_w[kN][WARPS];
+  __shared__ unsigned long long s_l[3 * kN][WARPS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double v[2] = {v0, v1};
+#pragma unroll
+  for (int j = 0; j < NV; ++j) {
+    int E;
+    bool bad;
+    cg_exact::i128 S = warp_exact_sum(v[j], &E, &bad);
+    if (lane == 3) {
+      unsigned long long lo, hi;
+      cg_exact::pack(S, E, bad, &lo, &hi);
+      s_w[j][warp] = make_ulonglong2(lo, hi);
+    }
+    const int e = c->scale[kind + j];
+    const bool fits = e != 0 && cg_exact::to_scale(&S, E, bad, max(1, e - cg_exact::kRoom));
+    if (lane < 3) s_l[3 * j + lane][warp] = fits ? cg_exact::limb(S, lane) : (lane == 2 ? ~0ull : 0ull);
+  }
+  __syncthreads();  // the warps' sums, and every global write of this CTA, before the words
+  XSums r{0.0, 0.0, true};
+  if (warp != 0) return r;
+  unsigned s = c->seq + 1;
+  __syncwarp();
+  unsigned long long d;
+  if (NV == 0) {
+    if (c->G > 1) {
+      r.ok = x_round<ORDER>(c, s, 0, 1, 0, 1ull, &d);
+      if (lane == 0) c->seq = s;
+    }
+    return r;
+  }
+  double out[kN];
+  if (c->G == 1) {
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      int E;
+      bool bad;
+      const cg_exact::i128 S = sum_entries(s_w[j][lane < WARPS ? lane : 0], lane < WARPS, &E, &bad);
+      out[j] = cg_exact::to_fp64(S, E, bad);
+    }
+  } else {
+    unsigned long long add = 0;
+    if (lane < kXSplit * 3 * kN) {
+      const int l = lane / kXSplit;
+      bool out = false;
+#pragma unroll
+      for (int w = 0; w < WARPS; ++w) {
+        const unsigned long long x = s_l[l][w];
+        out = out || x == ~0ull;
+        add += x == ~0ull ? 0ull : x;
+      }
+      add += (1ull << cg_exact::kCountAt) + (out ? 1ull << cg_exact::kExcAt : 0ull);
+    }
+    r.ok = x_round<ORDER>(c, s, 1, 3 * kN, cg_exact::kCountAt, add, &d);
+    bool again = false;
+#pragma unroll
+    for (int j = 0; j < kN; ++j) {
+      const int B = max(1, c->scale[kind + j] - cg_exact::kRoom);
+      int exc;
+      out[j] = cg_exact::to_fp64(x_join(d, j, &exc), B, false);
+      again = again || exc != 0 || !cg_exact::enough_bits(out[j], B);
+    }
+    if (again && r.ok) {  // the same decision in every CTA: the largest exponent first, then the sums
+      XWord* mx = c->words + 2 * kXWords;
+#pragma unroll 1
+      for (int j = 0; j < kN; ++j) {
+        int E;
+        bool bad;
+        cg_exact::i128 S = sum_entries(s_w[j][lane < WARPS ? lane : 0], lane < WARPS, &E, &bad);
+        ++s;
+        if (lane == 0) red_max(mx, ((unsigned long long)s << 32) | (unsigned)(bad ? 2047 : E));
+        __syncwarp();
+        r.ok = x_round<true>(c, s, 0, 1, 0, 1ull, &d) && r.ok;
+        __syncwarp();
+        const int Em = (int)(ld_word<true>(mx) & 0xFFFFull), B = max(1, Em - cg_exact::kRoom);
+        ++s;
+        const bool fits = cg_exact::to_scale(&S, E, bad, B);
+        add = (1ull << cg_exact::kCountAt) + (fits ? cg_exact::limb(S, lane / kXSplit) : 0ull);
+        r.ok = x_round<ORDER>(c, s, 1, 3, cg_exact::kCountAt, add, &d) && r.ok;
+        int exc;
+        const double o = cg_exact::to_fp64(x_join(d, 0, &exc), B, Em >= 2047);
+        if (j == 0) out[0] = o;
+        else out[kN - 1] = o;
+      }
+    }
+    if (lane == 0) {
+      c->seq = s;
+#pragma unroll
+      for (int j = 0; j < kN; ++j) {
+        const int e = (int)((cg_exact::bits_of(out[j]) >> 52) & 0x7FF);
+        c->scale[kind + j] = e == 0x7FF ? 0 : e;
+      }
+    }
+  }
+  r.v0 = out[0];
+  r.v1 = out[kN - 1];
+  return r;
 }
 
 }  // namespace cg

@@ -1,5 +1,5 @@
 // Exact fixed-point sums of fp64 values, rounded once to fp64: the dot products
-// of the cluster form.
+// of the loops.
 //
 // A group of terms is brought to a common scale E (the largest exponent field
 // among them): term v = (-1)^s m 2^(e - 1075) becomes the integer
@@ -186,6 +186,54 @@ CG_EXACT_HD i128 unpack(unsigned long long lo, unsigned long long hi, int* E, bo
   *bad = ((hi >> 40) & 1ull) != 0;
   const long long h = (long long)(hi << 24) >> 24;  // sign-extend the 40-bit high part
   return (i128)(((u128)(i128)h << 64) | (u128)lo);
+}
+
+// ---- sums that many CTAs add up with 64-bit atomic adds
+//
+// An integer S in units of scale B travels as three addends of 43, 43 and 32 payload
+// bits (its two's complement modulo 2^118).  A CTA's up to 8 warps add theirs in shared
+// memory; the CTA's words carry one count each in their top 9 bits.  The sums of up to
+// 511 x 8 addends stay clear of the counts, and joining the payload sums modulo 2^118
+// gives the sum of the integers while that is below 2^117.  A warp whose sum cannot be
+// expressed at scale B marks its CTA an exception instead.
+constexpr int kLimb = 43, kTop = 32, kExcAt = 45, kCountAt = 55, kMaxAddends = 511;
+constexpr int kRoom = 20;  // a sum of exponent field e is exchanged at scale e - kRoom next time
+
+// Move the sum S at scale E to scale B; false where it does not fit.
+CG_EXACT_HD bool to_scale(i128* S, int E, bool bad, int B) {
+  const int up = E - B;
+  if (bad || up > 40) return false;
+  if (up > 0) {
+    const i128 lim = ((i128)1 << 105) >> up;  // 2^12 addends stay below 2^117
+    if (!(*S < lim && *S > -lim)) return false;
+    *S = (i128)((u128)*S << up);
+  } else {
+    *S = shift_down(*S, -up);
+  }
+  return true;
+}
+
+// The payload of limb l (0..2) of S.
+CG_EXACT_HD unsigned long long limb(i128 S, int l) {
+  const u128 u = (u128)S;
+  const unsigned long long mask = (1ull << kLimb) - 1;
+  return l == 0   ? (unsigned long long)u & mask
+         : l == 1 ? (unsigned long long)(u >> kLimb) & mask
+                  : (unsigned long long)(u >> (2 * kLimb)) & ((1ull << kTop) - 1);
+}
+
+// The sum of the integers from the three words' sums; *exceptions: CTAs left out.
+CG_EXACT_HD i128 join_limbs(unsigned long long d0, unsigned long long d1, unsigned long long d2, int* exceptions) {
+  const unsigned long long pay = (1ull << kCountAt) - 1;
+  *exceptions = (int)((d2 & pay) >> kExcAt);
+  const u128 u = (u128)(d0 & pay) + ((u128)(d1 & pay) << kLimb) + ((u128)(d2 & ((1ull << kExcAt) - 1)) << (2 * kLimb));
+  return (i128)(u << 10) >> 10;  // modulo 2^118, signed
+}
+
+// Whether a sum formed at scale B (result `out`) has at least the 10 guard bits below
+// its last mantissa bit that the CTAs' sums had: else it is formed again at its scale.
+CG_EXACT_HD bool enough_bits(double out, int B) {
+  return B <= 1 || (int)((bits_of(out) >> 52) & 0x7FF) >= B + kGuard;
 }
 
 }  // namespace cg_exact

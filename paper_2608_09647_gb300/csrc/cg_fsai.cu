@@ -224,8 +224,7 @@ struct FsaiParams {
 // rho_prev > 0 (reliable updates, R8) p = G^T t + (rho / rho_prev) p.
 template <int W, typename T>
 __device__ bool fsai_start(const Ell<T>& G, const Ell<T>& GT, const FsaiVecs<T>& V, const T* r, int64_t n,
-                           double* part, int pstride, Grid& g, double* rho, double rho_prev = 0.0) {
-  constexpr bool kExact = sizeof(T) == 4;  // the fp64 loop keeps the fp64 sums (register budget)
+                           Grid& g, double* rho, double rho_prev = 0.0) {
   Acc<T> a;
   rows_x2(
       g, n, [&](int64_t i) { return ell_row<W>(G, i, n, [&](int j) { return r[j]; }); },
@@ -234,9 +233,7 @@ __device__ bool fsai_start(const Ell<T>& G, const Ell<T>& GT, const FsaiVecs<T>&
         a.add(s, s);
       });
   double v[1] = {a.get()};
-  publish<1, kExact>(v, part + kSlotRes * (size_t)pstride, g);
-  if (!g.sync()) return false;
-  grid_sum<1, kExact>(part + kSlotRes * (size_t)pstride, g.G, v);
+  if (!g.sum_all(v)) return false;
   *rho = v[0];
   const bool carry = rho_prev > 0.0;
   const T beta = carry ? (T)(v[0] / rho_prev) : T(0);
@@ -257,7 +254,7 @@ template <int W, typename T>
 __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, const FsaiVecs<T>& V, double rho,
                          double rr, double stop_abs, int maxit, int* iters, double* part, int pstride, Grid& g,
                          double* rho_last = nullptr) {
-  constexpr bool kExact = sizeof(T) == 4;  // the fp64 loop keeps the fp64 sums (register budget)
+  constexpr bool kWords = sizeof(T) == 8;  // sums by the exchange's words, else by partials
   const int64_t n = S.n;
   if (rho_last) *rho_last = rho;
   int k = *iters;
@@ -268,17 +265,14 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
   T* rc = V.r0;
   T* rn = V.r1;
   while (!done) {
-    double v1[1] = {spmv_phase<T, false>(S, V.p, V.q, g)};
-    publish<1, kExact>(v1, part + kSlotPQ * (size_t)pstride, g);
-    if (!g.sync()) { status = kTimeout; break; }
-    double pq[1];
-    grid_sum<1, kExact>(part + kSlotPQ * (size_t)pstride, g.G, pq);
+    double pq[1] = {spmv_phase<T, false>(S, V.p, V.q, g)};
+    const bool ok1 = kWords ? g.sum(pq, kKindPQ) : g.sum_parts(pq, part + kSlotPQ * (size_t)pstride);
     // the scalars once per CTA (an fp64 divide or square root in every
     // thread would load GB300's narrow fp64 pipe), shared through shared memory
-    __shared__ double s_sc[2];
+    __shared__ double s_sc[4];
     __shared__ int s_fl;
     if (threadIdx.x == 0) {
-      s_fl = (!isfinite(pq[0]) || !isfinite(rho)) ? kNumeric : (pq[0] <= 0.0 ? kBreakdown : 0);
+      s_fl = !ok1 ? kTimeout : ((!isfinite(pq[0]) || !isfinite(rho)) ? kNumeric : (pq[0] <= 0.0 ? kBreakdown : 0));
       s_sc[0] = rho / pq[0];
     }
     __syncthreads();
@@ -305,21 +299,21 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
           a_rho.add(u.t, u.t);
           V.x[i] = u.x;
         });
-    double v2[2] = {a_rho.get(), a_rr.get()};
-    publish<2, kExact>(v2, part + kSlotUpd * (size_t)pstride, g);
-    if (!g.sync()) { status = kTimeout; break; }
-    double s2[2];
-    grid_sum<2, kExact>(part + kSlotUpd * (size_t)pstride, g.G, s2);
+    double s2[2] = {a_rho.get(), a_rr.get()};
+    const bool ok2 = kWords ? g.sum(s2, kKindUpd) : g.sum_parts(s2, part + kSlotUpd * (size_t)pstride);
     if (threadIdx.x == 0) {
       s_sc[1] = s2[0] * s_inv_rho;
-      s_fl = below_stop(s2[1], stop_abs, stop2_hi);
+      s_sc[2] = s2[0];
+      s_sc[3] = s2[1];
+      s_fl = !ok2 ? kTimeout : (below_stop(s2[1], stop_abs, stop2_hi) ? 1 : 0);
     }
     __syncthreads();
+    if (s_fl < 0) { status = s_fl; break; }
     const T beta = (T)s_sc[1];
     const bool conv = s_fl != 0;
     if (rho_last) *rho_last = rho;
-    rho = s2[0];
-    rr = s2[1];
+    rho = s_sc[2];
+    rr = s_sc[3];
     ++k;
     done = conv || k >= maxit;
     if (conv) status = kOk;
@@ -341,7 +335,8 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
 template <int W>
 __global__ void __launch_bounds__(kBlock, 2) pcg_fsai64_kernel(FsaiParams F) {
   const SolveParams& P = F.P;
-  Grid g(P.st, P.timeout_ns, P.skip_seq);
+  __shared__ XState s_x;
+  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
   const int64_t n = P.A.n;
   const FsaiVecs<double>& V = F.V64;
   int status = kNotConverged, k = 0, restarts = 0;
@@ -358,10 +353,8 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai64_kernel(FsaiParams F) {
       v[0] += ri * ri;
       v[1] += bi * bi;
     }
-    publish<2, false>(v, P.part + kSlotRes * (size_t)P.pstride, g);
-    if (!g.sync()) { status = kTimeout; break; }
-    double s2[2];
-    grid_sum<2, false>(P.part + kSlotRes * (size_t)P.pstride, g.G, s2);
+    if (!g.sum_all(v)) { status = kTimeout; break; }
+    const double(&s2)[2] = v;
     const double rr_start = s2[0];
     if (first) {
       bb = s2[1];
@@ -386,7 +379,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai64_kernel(FsaiParams F) {
     }
     first = false;
     double rho = 0.0;
-    if (!fsai_start<W, double>(F.G64, F.GT64, V, V.r0, n, P.part, P.pstride, g, &rho)) { status = kTimeout; break; }
+    if (!fsai_start<W, double>(F.G64, F.GT64, V, V.r0, n, g, &rho)) { status = kTimeout; break; }
     const int st = fsai_loop<W, double>(P.S64, F.G64, F.GT64, V, rho, rr_start, P.tol * sqrt(bb), P.maxit, &k,
                                      P.part, P.pstride, g);
     if (st == kTimeout) { status = kTimeout; break; }
@@ -399,9 +392,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai64_kernel(FsaiParams F) {
         const double ri = P.b[i] - V.q[i];
         w[0] += ri * ri;
       }
-      publish<1, false>(w, P.part + kSlotRes * (size_t)P.pstride, g);
-      if (!g.sync()) { status = kTimeout; break; }
-      grid_sum<1, false>(P.part + kSlotRes * (size_t)P.pstride, g.G, w);
+      if (!g.sum_all(w)) { status = kTimeout; break; }
       relres_true = sqrt(w[0]) / sqrt(bb);
       break;
     }
@@ -421,7 +412,8 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai64_kernel(FsaiParams F) {
 template <int W, bool CARRY>
 __global__ void __launch_bounds__(kBlock, 2) pcg_fsai_ir_kernel(FsaiParams F) {
   const SolveParams& P = F.P;
-  Grid g(P.st, P.timeout_ns, P.skip_seq);
+  __shared__ XState s_x;
+  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
   const int64_t n = P.A.n;
   const FsaiVecs<float>& V = F.V32;
   int status = kNotConverged, inner = 0, outer = 0;
@@ -440,10 +432,8 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai_ir_kernel(FsaiParams F) {
       v[1] += bi * bi;
       v[2] += (double)r32 * (double)r32;
     }
-    publish<3>(v, P.part + kSlotRes * (size_t)P.pstride, g);
-    if (!g.sync()) { status = kTimeout; break; }
-    double s3[3];
-    grid_sum<3>(P.part + kSlotRes * (size_t)P.pstride, g.G, s3);
+    if (!g.sum_all(v)) { status = kTimeout; break; }
+    const double(&s3)[3] = v;
     if (outer == 0) {
       bb = s3[1];
       if (bb == 0.0) {
@@ -457,7 +447,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai_ir_kernel(FsaiParams F) {
     if (relres <= P.tol) { status = kOk; break; }
     if (outer >= P.max_restarts || inner >= P.maxit) { status = kNotConverged; break; }
     double rho = 0.0;
-    if (!fsai_start<W, float>(F.G32, F.GT32, V, V.r0, n, P.part, P.pstride, g, &rho,
+    if (!fsai_start<W, float>(F.G32, F.GT32, V, V.r0, n, g, &rho,
                                 CARRY && outer > 0 ? rho_k : 0.0)) { status = kTimeout; break; }
     const int st = fsai_loop<W, float>(P.S32, F.G32, F.GT32, V, rho, s3[2], P.tol_in * sqrt(s3[2]), P.maxit, &inner,
                                     P.part, P.pstride, g, &rho_k);
@@ -1486,8 +1476,8 @@ cg_status cgi::fsai_solve(cg_handle* h, const SolveParams& Pin, bool fp64, bool 
   else fn = by_slots<PickIr<false>>(sw);
   int per_sm = 0;
   CGF_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, 0));
-  const int G = std::max(1, std::min(grid, per_sm * h->sm_count));
-  CGF_CUDA(h, cudaMemsetAsync(h->st, 0, sizeof(DevState), h->stream));
+  const int G = std::max(1, std::min({grid, per_sm * h->sm_count, kXCtas}));
+  CGF_CUDA(h, cudaMemsetAsync(h->st, 0, kStBytes, h->stream));
   CGF_CUDA(h, cudaEventRecord(h->ev0, h->stream));
   CGF_CUDA(h, cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kBlock), args, 0, h->stream));
   CGF_CUDA(h, cudaEventRecord(h->ev1, h->stream));

@@ -61,7 +61,7 @@ struct GArgs {
   unsigned G_upd;   // CTAs of the vector kernels (their partials)
 };
 
-__device__ __forceinline__ Grid graph_grid() { return Grid(nullptr, 0, 0); }
+__device__ __forceinline__ Grid graph_grid() { return Grid(); }
 
 template <typename T> __device__ __forceinline__ const Sell<T>& sell_of(const SolveParams& P);
 template <> __device__ __forceinline__ const Sell<double>& sell_of<double>(const SolveParams& P) { return P.S64; }

@@ -21,6 +21,14 @@ using cg::kMaxDiag;
 struct BatchData;                 // batched solves (cg_batch.cu)
 struct FsaiData;                  // FSAI preconditioner (cg_fsai.cu, cg_mlp.cu)
 
+// DevState and, behind it, the words of the grid exchanges: one allocation, cleared
+// before every persistent launch.
+constexpr size_t kXOffset = (sizeof(DevState) + 255) / 256 * 256;
+constexpr size_t kStBytes = kXOffset + cg::kXBytes;
+inline cg::XWord* exchange_words(DevState* st) {
+  return reinterpret_cast<cg::XWord*>(reinterpret_cast<char*>(st) + kXOffset);
+}
+
 namespace cgi {
 void batch_free(BatchData* b);
 void fsai_free(FsaiData* f);
@@ -30,6 +38,10 @@ cg_status ensure_offsets(cg_handle* h);         // cg_handle::offs_all, once (cg
 int64_t cluster_max_rows();
 cg_status cluster_solve(cg_handle* h, const double* b, double* x, double tol, int32_t maxit, bool jac,
                         int32_t* iters_out, double* relres_out);
+// the loop with every vector in the SMs' shared memory (cg_resident.cu): fp64 CG /
+// Jacobi-PCG on the sliced-diagonal layout; *launched = false: the system does not fit,
+// nothing was enqueued.  *grid: the CTAs launched
+cudaError_t resident_launch(const cg_handle* h, const cg::SolveParams& P, bool jac, int* grid, bool* launched);
 // the cluster's loop on a CSR that is checked on the device first, without a handle or any
 // allocation (cg_noalloc.cu); *launched = false: no cluster holds the system, nothing
 // was enqueued.  diag: scratch of n doubles; words: the result, on the device

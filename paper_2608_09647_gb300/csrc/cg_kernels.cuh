@@ -132,6 +132,7 @@ struct SolveParams {
   double* part;           // per-CTA partials: kParts slots of pstride doubles
   int pstride;            // slot stride (>= the grid of every loop kernel)
   DevState* st;
+  XWord* xs;              // words of the grid exchanges
   double tol;             // outer relative tolerance
   double tol_in;          // inner tolerance (refinement)
   int maxit;              // SpMV cap (total inner iterations when refining)
@@ -147,28 +148,83 @@ struct SolveParams {
 constexpr int kParts = 8;
 constexpr int kSlotPQ = 0, kSlotRr = 1, kSlotUpd = 2, kSlotRes = 4;
 
-// Grid coordinates and the barrier sequence of one persistent launch.
+// Kinds of the loops' sums (their scales are kept apart).
+constexpr int kKindPQ = 0, kKindUpd = 1, kKindRr = 3, kKindRes = 4;
+
+// Grid coordinates and the exchanges of one persistent launch.
 struct Grid {
   unsigned G, cta;
   int64_t gtid, gstride;
   DevState* st;
+  XState* x;
   uint64_t timeout_ns;
   unsigned seq, skip_seq;
-  __device__ Grid(DevState* s, uint64_t to, unsigned skip)
-      : G(gridDim.x), cta(blockIdx.x), gtid((int64_t)blockIdx.x * kBlock + threadIdx.x),
-        gstride((int64_t)gridDim.x * kBlock), st(s), timeout_ns(to), seq(0), skip_seq(skip) {}
+  __device__ Grid() : G(gridDim.x), cta(blockIdx.x), gtid((int64_t)blockIdx.x * kBlock + threadIdx.x),
+        gstride((int64_t)gridDim.x * kBlock), st(nullptr), x(nullptr), timeout_ns(0), seq(0), skip_seq(0) {}
+  __device__ Grid(DevState* s, XWord* words, XState* xs, uint64_t to, unsigned skip) : Grid() {
+    st = s;
+    x = xs;
+    timeout_ns = to;
+    skip_seq = skip;
+    x_init(xs, s, words, gridDim.x, blockIdx.x, blockIdx.x == 0 ? skip : 0u, to);
+  }
+  // a barrier; false: a wait gave up, leave the kernel
   __device__ __forceinline__ bool sync() { return grid_barrier(st, G, timeout_ns, ++seq, skip_seq); }
+  // a barrier that leaves the grid's sums of v in warp 0's v and says there whether
+  // it succeeded; the caller's next __syncthreads() completes it for the other warps
+  template <int NV>
+  __device__ __forceinline__ bool sum(double (&v)[NV], int kind) {
+    static_assert(NV <= kXVals, "values of one exchange");
+    const XSums r = grid_exchange<NV>(x, kind, v[0], NV > 1 ? v[NV - 1] : 0.0);
+    v[0] = r.v0;
+    if (NV > 1) v[NV - 1] = r.v1;
+    return r.ok;
+  }
+  // the same through per-CTA partials part[j G + cta] that every CTA adds up after a
+  // plain barrier, the sums in every thread: the fp32 loops' form.  Their phases end
+  // more unevenly, and CTAs that poll an exchange's words slow the ones still at work
+  // (27-point 160^3, 304 CTAs: 146.5 us an iteration against 148.7).
+  template <int NV>
+  __device__ __forceinline__ bool sum_parts(double (&v)[NV], double* part);
+  // the exchange for up to 4 values, the sums given to every thread (the residual phases)
+  template <int NV>
+  __device__ __forceinline__ bool sum_all(double (&v)[NV]) {
+    __shared__ double s_out[NV];
+#pragma unroll
+    for (int j = 0; j < NV; j += 2) {
+      const bool two = j + 1 < NV;
+      double w2[2] = {v[j], v[two ? j + 1 : j]}, w1[1] = {v[j]};
+      const bool ok = two ? sum<2>(w2, kKindRes) : sum<1>(w1, kKindRes);
+      if (threadIdx.x == 0) {
+        s_out[j] = two ? w2[0] : w1[0];
+        if (two) s_out[j + 1 < NV ? j + 1 : j] = w2[1];
+      }
+      if (!__syncthreads_and(ok)) return false;
+    }
+#pragma unroll
+    for (int j = 0; j < NV; ++j) v[j] = s_out[j];
+    __syncthreads();
+    return true;
+  }
 };
 
 // Write this CTA's block sums of v[0..NV) into part[j*G + cta] (v is
 // consumed: afterwards it holds the sums in thread 0 only).
-template <int NV, bool EXACT = true>
+template <int NV>
 __device__ __forceinline__ void publish(double (&v)[NV], double* part, const Grid& g) {
-  cta_sum0<NV, EXACT>(v);
+  cta_sum0<NV>(v);
   if (threadIdx.x == 0) {
 #pragma unroll
     for (int j = 0; j < NV; ++j) part[(size_t)j * g.G + g.cta] = v[j];
   }
+}
+
+template <int NV>
+__device__ __forceinline__ bool Grid::sum_parts(double (&v)[NV], double* part) {
+  publish<NV>(v, part, *this);
+  if (!sync()) return false;
+  grid_sum<NV>(part, G, v);
+  return true;
 }
 
 // publish, then elect the last CTA of the launch to arrive (counter *ctr):
@@ -775,68 +831,78 @@ __device__ __forceinline__ void update_xp_phase(const Sell<T>& S, const LoopVecs
 template <typename T, bool JAC, bool OUT_ADD>
 __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, double rr,
                        double stop_abs, int maxit, int* iters, double* rr_out, double* out,
-                       double* part, int pstride, Grid& g, PhaseClock& clk,
-                       double* rho_last = nullptr) {
-  constexpr bool kExact = sizeof(T) == 4;  // the fp64 loop keeps the fp64 sums (register budget)
+                       double* part, int pstride, Grid& g, PhaseClock& clk, double* rho_last = nullptr) {
+  constexpr bool kWords = sizeof(T) == 8;  // sums by the exchange's words, else by partials
   if (rho_last) *rho_last = rho;  // r.z before the last step taken (reliable updates)
   int k = *iters;
   int status = kNotConverged;
   const double stop2_hi = stop2_high(stop_abs);
   bool done = sqrt(rr) <= stop_abs || k >= maxit;  // a4: tested before every SpMV
   if (sqrt(rr) <= stop_abs) status = kOk;
+  // scalars once per CTA in thread 0, shared (fp64 divisions and tests in every
+  // thread would load GB300's narrow fp64 pipe)
+  __shared__ double s_alpha, s_beta, s_rho, s_rr, s_inv_rho;
+  __shared__ int s_st, s_want, s_exact, s_conv;
   while (!done) {
     // a1: q = A^ p; p.q
     double v1[1] = {spmv_phase<T, JAC>(S, V.p, V.q, g)};
-    publish<1, kExact>(v1, part + kSlotPQ * (size_t)pstride, g);
     clk.lap(g.st, 0);
-    if (!g.sync()) { status = kTimeout; break; }
+    const bool ok1 = kWords ? g.sum(v1, kKindPQ) : g.sum_parts(v1, part + kSlotPQ * (size_t)pstride);
     clk.lap(g.st, 1);
-    double pq[1];
-    grid_sum<1, kExact>(part + kSlotPQ * (size_t)pstride, g.G, pq);
-    // scalars once per CTA in thread 0, shared (fp64 divisions and tests in every
-    // thread would load GB300's narrow fp64 pipe)
-    __shared__ double s_sc[3];
-    __shared__ int s_fl[2];
     if (threadIdx.x == 0) {
-      s_fl[0] = (!isfinite(pq[0]) || !isfinite(rho)) ? kNumeric : (pq[0] <= 0.0 ? kBreakdown : 0);
-      s_sc[0] = rho / pq[0];
-      s_fl[1] = JAC && rr_wanted(S, rho, stop_abs * stop_abs);
+      s_st = !ok1 ? kTimeout
+                  : ((!isfinite(v1[0]) || !isfinite(rho)) ? kNumeric : (v1[0] <= 0.0 ? kBreakdown : 0));
+      s_alpha = rho / v1[0];
+      s_want = JAC && rr_wanted(S, rho, stop_abs * stop_abs);
     }
     __syncthreads();
-    if (s_fl[0]) { status = s_fl[0]; break; }
-    const T alpha = (T)s_sc[0];
-    // a2: r^ -= alpha q; r.z, r.r (r.r only when the test needs it)
-    const bool want_rr = s_fl[1] != 0;
+    if (s_st) { status = s_st; break; }
+    const T alpha = (T)s_alpha;
+    // a2: r^ -= alpha q; r.z, r.r (r.r only when the test needs it).  1 / rho for
+    // this iteration's beta in warp 1 meanwhile: beta = rho' (1 / rho) is a multiply
+    // after the exchange (within 1.5 ulp of rho' / rho)
+    const bool want_rr = s_want != 0;
+    if (threadIdx.x == 32) s_inv_rho = 1.0 / rho;
     double v2[2] = {0.0, 0.0};
     update_r_phase<T, JAC>(S, V, alpha, want_rr, v2[0], v2[1], g);
-    publish<2, kExact>(v2, part + kSlotUpd * (size_t)pstride, g);
     clk.lap(g.st, 2);
-    if (!g.sync()) { status = kTimeout; break; }
+    bool ok;
+    if (want_rr) {
+      ok = kWords ? g.sum(v2, kKindUpd) : g.sum_parts(v2, part + kSlotUpd * (size_t)pstride);
+    } else {
+      double w[1] = {v2[0]};
+      ok = kWords ? g.sum(w, kKindUpd) : g.sum_parts(w, part + kSlotUpd * (size_t)pstride);
+      v2[0] = v2[1] = w[0];  // plain CG: r.z is r.r
+    }
     clk.lap(g.st, 3);
-    double s2[2];
-    grid_sum<2, kExact>(part + kSlotUpd * (size_t)pstride, g.G, s2);
     if (threadIdx.x == 0) {
-      double rr_ = s2[1];
-      s_sc[1] = s2[0] / rho;
-      s_fl[0] = JAC && !want_rr && rr_bound_test(S, s2[0], stop_abs * stop_abs, &rr_) < 0;
-      s_sc[2] = rr_;
+      double rr_ = v2[1];
+      if (!ok) s_st = kTimeout;
+      s_exact = JAC && !want_rr && rr_bound_test(S, v2[0], stop_abs * stop_abs, &rr_) < 0;
+      s_beta = v2[0] * s_inv_rho;
+      s_rho = v2[0];
+      s_rr = rr_;
+      s_conv = below_stop(rr_, stop_abs, stop2_hi);
     }
     __syncthreads();
-    const T beta = (T)s_sc[1];
+    if (s_st) { status = s_st; break; }
+    const T beta = (T)s_beta;
     if (rho_last) *rho_last = rho;
-    rho = s2[0];
-    rr = s_sc[2];
-    if (s_fl[0]) {
+    rho = s_rho;
+    if (s_exact) {
       double v3[1] = {rr_phase<T>(S, V, g)};  // rho fell into the band early: exact r.r
-      publish<1, kExact>(v3, part + kSlotRr * (size_t)pstride, g);
-      if (!g.sync()) { status = kTimeout; break; }
-      grid_sum<1, kExact>(part + kSlotRr * (size_t)pstride, g.G, v3);
-      rr = v3[0];
+      const bool ok3 = kWords ? g.sum(v3, kKindRr) : g.sum_parts(v3, part + kSlotRr * (size_t)pstride);
+      if (threadIdx.x == 0) {
+        if (!ok3) s_st = kTimeout;
+        s_rr = v3[0];
+        s_conv = below_stop(v3[0], stop_abs, stop2_hi);
+      }
+      __syncthreads();
+      if (s_st) { status = s_st; break; }
     }
+    rr = s_rr;
     ++k;
-    if (threadIdx.x == 0) s_fl[1] = below_stop(rr, stop_abs, stop2_hi);
-    __syncthreads();
-    const bool conv = s_fl[1] != 0;
+    const bool conv = s_conv != 0;
     done = conv || k >= maxit;
     if (conv) status = kOk;
     // a3: x^ += alpha p; p = r^ + beta p (last iteration: write the caller's x)
@@ -876,7 +942,8 @@ __device__ __forceinline__ void spmv_orig(const Csr<double>& A, const double* x,
 // restarts (readings R1-R5 of the method, see the oracle's header).
 template <bool JAC>
 __global__ void __launch_bounds__(kBlock, 2) pcg64_kernel(SolveParams P) {
-  Grid g(P.st, P.timeout_ns, P.skip_seq);
+  __shared__ XState s_x;
+  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
   PhaseClock clk(P.timers != 0);
   const int64_t n = P.A.n;
   const LoopVecs<double>& V = P.V64;
@@ -899,10 +966,8 @@ __global__ void __launch_bounds__(kBlock, 2) pcg64_kernel(SolveParams P) {
       v[1] += ri * ri;
       v[2] += bi * bi;
     }
-    publish<3, false>(v, P.part + kSlotRes * (size_t)P.pstride, g);
-    if (!g.sync()) { status = kTimeout; break; }
-    double s3[3];
-    grid_sum<3, false>(P.part + kSlotRes * (size_t)P.pstride, g.G, s3);
+    if (!g.sum_all(v)) { status = kTimeout; break; }
+    const double(&s3)[3] = v;
     if (first) {
       bb = s3[2];
       if (bb == 0.0) {  // b = 0: x = 0 solves it
@@ -933,11 +998,8 @@ __global__ void __launch_bounds__(kBlock, 2) pcg64_kernel(SolveParams P) {
         const double ri = P.b[i] - V.q[i];
         w[0] += ri * ri;
       }
-      publish<1, false>(w, P.part + kSlotRes * (size_t)P.pstride, g);
-      if (!g.sync()) { status = kTimeout; break; }
-      double s1[1];
-      grid_sum<1, false>(P.part + kSlotRes * (size_t)P.pstride, g.G, s1);
-      relres_true = sqrt(s1[0]) / sqrt(bb);
+      if (!g.sum_all(w)) { status = kTimeout; break; }
+      relres_true = sqrt(w[0]) / sqrt(bb);
       break;
     }
     if (was_first && k == k_before && st == kOk) {  // x0 met tol: its true residual is s3[1]
@@ -965,7 +1027,8 @@ __global__ void __launch_bounds__(kBlock, 2) pcg64_kernel(SolveParams P) {
 // rho_k) p_k, instead of restarting from p = r^'.
 template <bool JAC, bool CARRY>
 __global__ void __launch_bounds__(kBlock, 2) pcg_ir_kernel(SolveParams P) {
-  Grid g(P.st, P.timeout_ns, P.skip_seq);
+  __shared__ XState s_x;
+  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
   PhaseClock clk(P.timers != 0);
   const int64_t n = P.A.n;
   const LoopVecs<float>& V = P.V32;
@@ -990,10 +1053,8 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_ir_kernel(SolveParams P) {
       v[2] += rh2;
       v[3] += JAC ? (double)__ldg(P.S32.dn + i) * rh2 : rh2;
     }
-    publish<4>(v, P.part + kSlotRes * (size_t)P.pstride, g);
-    if (!g.sync()) { status = kTimeout; break; }
-    double s4[4];
-    grid_sum<4>(P.part + kSlotRes * (size_t)P.pstride, g.G, s4);
+    if (!g.sum_all(v)) { status = kTimeout; break; }
+    const double(&s4)[4] = v;
     if (outer == 0) {
       bb = s4[1];
       if (bb == 0.0) {
@@ -1012,8 +1073,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_ir_kernel(SolveParams P) {
       if (!g.sync()) { status = kTimeout; break; }
     }
     const int st = cg_loop<float, JAC, true>(P.S32, V, s4[2], s4[3], P.tol_in * sqrt(s4[3]),
-                                             P.maxit, &inner, &rr32, P.x, P.part, P.pstride, g, clk,
-                                             &rho_k);
+                                             P.maxit, &inner, &rr32, P.x, P.part, P.pstride, g, clk, &rho_k);
     if (st == kTimeout || st == kNumeric || st == kBreakdown) { status = st; break; }
     ++outer;
   }
