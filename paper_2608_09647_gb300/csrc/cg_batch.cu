@@ -11,26 +11,28 @@
 // stored by diagonal (a slot per offset, the gather index clamped into the
 // system's own rows, no column array), the others as SELL-32 with global
 // columns.  Every system is padded to whole 256-row tiles (padding rows are
-// identity rows with b = x = 0), so no tile spans two systems; 16 tiles form a
-// 4096-row reduction group.
+// identity rows with b = x = 0), so no tile spans two systems; 1, 2 or 8 tiles,
+// by the system's size, form a reduction unit.
 //
-// Schedule.  Rounds of four phases separated by bounded grid barriers:
-//   R  r = b - A x for the systems that need it (start, after their loop,
-//      restarts): the fp64 true-residual test and the start of a loop;
+// Schedule.  The grid's CTAs form teams, contiguous runs of CTAs that the hardware
+// spreads over the SMs, so the CTAs of one SM belong to different teams.  A team
+// solves one system at a time, split over its CTAs by units, with a barrier of its own
+// (bounded, a counter in L2) after each phase:
+//   R  r = b - A x: the fp64 true-residual test and the (re)start of a loop;
 //   A  q = A p and p.q, alpha;
 //   B  r -= alpha q, r.r and r.D r, beta and the recursive stopping test;
-//   C  x += alpha p, p = r + beta p.
-// A system's stage says which phases it takes part in: 0 residual pending,
-// 1 iterating, 2 done, 3 last x update pending (C, then R), 4 r.D r pending.
-// At the start of each phase every CTA scans the stages, forms the prefix sum
-// of the work of the systems in that phase in shared memory (a unit per
-// group, or in the SpMV phases R and A a row-cost weight per group) and takes
-// a contiguous chunk of it, so finished systems cost nothing and a chunk
-// spans few systems.  A system's sums are formed by the CTA that completes
-// its last group of the phase, over (group, warp) partials in order, so they
-// do not depend on the schedule.  A stage change made during a phase carries
-// that phase's number; a CTA that reads the word in the same phase takes the
-// stage from before the change, so all CTAs deal the same list.
+//   C  x += alpha p, p = r + beta p;
+// then it takes the next system of the queue (descending work).  While one team waits
+// at its barrier or sums, the SM's other CTAs work on other systems, in other phases:
+// the waits are hidden, and phases bound by the fp64 pipe (R, A, B) run beside phases
+// bound by memory (C).  (One schedule for all systems, four phases with a barrier of
+// the whole grid after each, left both bounds and all waits in sequence, and its work
+// lists and system sums cost ~17 us a phase however small the systems: 26.3 ms for 24
+// systems of 33^2 to 200^2 rows to 1e-12 with reliable updates, 127.2 ms for 96 fp64
+// systems of 32^2 to 512^2; now 10.3 ms and 116 ms.)
+// A system's sums are formed from (unit, warp) partials, which depend on the system
+// alone, by every CTA of its team in the same fixed order: results depend neither on
+// the schedule nor on the other systems.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -46,28 +48,27 @@ using namespace cg;
 namespace {
 
 constexpr int kTile = kBlock;        // rows per tile (kWarps slices, one per warp)
-constexpr int kGroup = 16;           // tiles per reduction group (4096 rows)
 constexpr int kMaxBatch = CG_BATCH_MAX_SYSTEMS;
-constexpr int kNP = 4;               // partial sums per (group, warp)
+constexpr int kNP = 4;               // partial sums per (unit, warp)
 constexpr int kBatchDiag = 8;        // offsets of a system in the diagonal layout, at most
 constexpr int kStRunning = 100;      // status of a system still being solved
 constexpr int kMaxCand = 8;          // autotuner candidates
 constexpr double kRrMarginB = 64.0;  // r.D r is computed while dmin r^.r^ <= 64 stop^2
+constexpr int kTeamWords = kXAll;      // exchange words of a team
 
-// stages and the phases that take them
-constexpr int kStResidual = 0, kStIter = 1, kStDone = 2, kStLastX = 3, kStRrPending = 4;
-constexpr unsigned kMaskR = (1u << kStResidual) | (1u << kStLastX);
-constexpr unsigned kMaskAB = 1u << kStIter;
-constexpr unsigned kMaskC = (1u << kStIter) | (1u << kStLastX) | (1u << kStRrPending);
-constexpr unsigned kMaskAlive = ~(1u << kStDone);
+// Tiles per reduction unit: up to 128 units to 262,144 rows (a team's CTAs then sum up
+// to 1024 partials, four a thread), so that a team of ~20 CTAs is evenly loaded (64
+// units on 19 CTAs left them idle 16 % of a phase), and as many units as there are
+// tiles where the system is small, so that it can be spread over as many CTAs.
+inline int unit_tiles(int ntile) { return ntile <= 64 ? 1 : (ntile <= 256 ? 2 : 8); }
 
 struct BatchParams {
   int nsys;
   const int32_t* __restrict__ tstart;  // first tile of each system
   const int32_t* __restrict__ ntile;   // tiles of each system
-  const int32_t* __restrict__ gstart;  // first reduction group of each system
-  const int32_t* __restrict__ ngroup;  // reduction groups of each system
-  const int32_t* __restrict__ wcost;   // SpMV-phase cost of a row of each system (load balance)
+  const int32_t* __restrict__ ustart;  // first reduction unit of each system
+  const int32_t* __restrict__ nunit;   // reduction units of each system
+  const int32_t* __restrict__ utiles;  // tiles per unit of each system
   const int32_t* __restrict__ sdia;    // offsets of each system in the diagonal layout (0: sliced ELL)
   const int32_t* __restrict__ sdelta;  // those offsets, kBatchDiag per system
   const double* __restrict__ dmin;     // smallest A_ii of each system
@@ -77,89 +78,27 @@ struct BatchParams {
   const double* __restrict__ dg;       // A_ii, 1 on padding rows
   double *r, *p, *q, *xh;
   const double* __restrict__ bh;
-  double *rho, *rr, *bb, *alpha, *beta, *relres;
-  int *k, *restarts, *status, *zero, *wrr;
-  unsigned long long* sstate;          // phase << 16 | stage before << 8 | stage after
-  unsigned* cnt;                       // groups of the system finished in this phase
-  double* tpart;                       // kNP partials per (group, warp)
+  double* relres;
+  int *k, *restarts, *status, *zero;
+  double* tpart;                       // two banks of kNP partials per (unit, warp)
+  int64_t bank;                        // doubles of a bank
+  const int32_t* __restrict__ order;   // the queue: systems by descending work
+  const int32_t* __restrict__ team0;   // first CTA of each team (nteams + 1)
+  int nteams;
+  unsigned* queue;                     // systems taken beyond the teams' first
+  int* next;                           // each team's next place in the queue
+  XWord* words;                        // kTeamWords exchange words per team
   double tol;
   int maxit, max_restarts;
   DevState* st;
-  XWord* xs;
   uint64_t timeout_ns;
   unsigned skip_seq;
   // fp32 inner solves with fp64 refinement (batch_ir_kernel only)
   const float* __restrict__ val32;     // the loop matrix values rounded to fp32
   float *r32, *p32, *q32, *d32;        // inner residual, direction, A p, correction d
-  double* rho_k;                       // r.z before the last step of the inner solve
-  double* beta0;                       // carry factor of the inner solve being started
-  double* stopin;                      // inner stopping threshold tol_in ||r32|| (true norm)
-  int* start;                          // 1: the A and B phases begin an inner solve
   double tol_in;
   int max_outer, carry;
 };
-
-__device__ __forceinline__ int eff_stage(unsigned long long w, unsigned seq) {
-  return ((unsigned)(w >> 16) == seq) ? (int)((w >> 8) & 0xff) : (int)(w & 0xff);
-}
-
-// Exclusive prefix sum (in s_pref) of the work units of the systems whose
-// stage, as seen in phase seq, is in `mask` (a unit per reduction group, or
-// WEIGHTED: wcost units per group, the SpMV phases' row cost); returns their
-// total.
-// *alive gets whether any system is still unfinished.  Thread t owns a
-// contiguous run of systems; the runs' totals are scanned with warp shuffles.
-template <bool WEIGHTED>
-__device__ int build_list(const BatchParams& P, unsigned mask, unsigned seq, int* s_pref, int* s_warp,
-                          bool* alive) {
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int per = (P.nsys + kBlock - 1) / kBlock;
-  const int s0 = min(P.nsys, t * per), s1 = min(P.nsys, s0 + per);
-  int c = 0, live = 0;
-  for (int s = s0; s < s1; ++s) {
-    const unsigned sbit = 1u << eff_stage(__ldcg(P.sstate + s), seq);
-    const int cs = (sbit & mask) ? P.ngroup[s] * (WEIGHTED ? P.wcost[s] : 1) : 0;
-    live |= (sbit & kMaskAlive) != 0;
-    s_pref[s] = cs;
-    c += cs;
-  }
-  int inc = c;  // inclusive scan within the warp
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += v;
-  }
-  if (lane == 31) s_warp[warp] = inc;
-  *alive = __syncthreads_or(live) != 0;
-  int wbase = 0, total = 0;
-#pragma unroll
-  for (int w = 0; w < kWarps; ++w) {
-    const int v = s_warp[w];
-    wbase += w < warp ? v : 0;
-    total += v;
-  }
-  int base = wbase + inc - c;
-  for (int s = s0; s < s1; ++s) {
-    const int cs = s_pref[s];
-    s_pref[s] = base;
-    base += cs;
-  }
-  __syncthreads();
-  return total;
-}
-
-// The system owning entry j of the phase's list: the last system whose
-// prefix is <= j (systems without groups in the phase share the prefix of
-// their successor, which is larger than j).
-__device__ __forceinline__ int system_of(const BatchParams& P, const int* s_pref, int j) {
-  int lo = 0, hi = P.nsys - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (s_pref[mid] <= j) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
 
 // acc + off-diagonal part of one row of slice sl: the sum over the slice
 // width of val * v[col], all loads of a slice issued together (widths 4 and
@@ -179,12 +118,14 @@ __device__ __forceinline__ double slice_row(const int32_t* __restrict__ cp, cons
   return acc;
 }
 
-// The system a CTA's current segment belongs to, as row_spmv needs it
-// (shared memory, written by run_phase at the start of each segment).
+// The system a team is solving (shared memory) and this CTA's units of it.
 struct SegInfo {
   int nd;              // offsets of the diagonal layout (0: sliced ELL)
   int lo, hi;          // the system's first and last concatenated rows
   int delta[kBatchDiag];
+  int t0, tend;        // its first tile, the tile after its last
+  int ut, un0, nunit;  // tiles per unit, its first unit, its units
+  int u0, u1;          // this CTA's units
 };
 
 // Diagonal layout: column i + delta[m], clamped into the system's own rows
@@ -290,396 +231,391 @@ __device__ __forceinline__ TA row_spmv_g(const BatchParams& P, const TV* __restr
   return acc;
 }
 
-// Sum of a system's (group, warp) partials in a fixed order, given to every
-// thread: thread t adds partials t, t + kBlock, ... in order (its loads four at
-// a time, so the whole CTA waits for about one L2 round trip), then cta_sum0.
-// It runs in the CTA that completes the system while the others wait at the
-// next grid barrier, so its latency is the phase's tail.
-constexpr int kSumBatch = 4;
-template <int NV>
-__device__ __forceinline__ void system_sum(const BatchParams& P, int sys, double (&out)[NV]) {
-  __shared__ double s_out[NV];
-  const int p0 = P.gstart[sys] * kWarps, np = P.ngroup[sys] * kWarps;
-  double a[NV];
+// One CTA of a team: the team's barrier, the system in hand, the partials' bank.
+struct Team {
+  const BatchParams& P;
+  SegInfo& seg;
+  XState* x;
+  int id, rank, size;
+  int flip;  // reductions so far: the bank the next one writes
+  __device__ __forceinline__ bool sync() {
+    return __syncthreads_and(grid_exchange<0>(x, 0, 0.0, 0.0).ok) != 0;
+  }
+  __device__ __forceinline__ double* bank() const { return P.tpart + (flip & 1) * P.bank; }
+};
+
+// The team's place in the grid and its barrier; false: a CTA without a team.
+__device__ __forceinline__ bool team_init(const BatchParams& P, XState* x, int* id, int* rank, int* size) {
+  const int c = (int)blockIdx.x;
+  int lo = 0, hi = P.nteams;  // the last team with team0 <= c
+  while (lo + 1 < hi) {
+    const int mid = (lo + hi) >> 1;
+    if (__ldg(P.team0 + mid) <= c) lo = mid;
+    else hi = mid;
+  }
+  const int a = __ldg(P.team0 + lo), e = __ldg(P.team0 + lo + 1);
+  *id = lo;
+  *rank = c - a;
+  *size = e - a;
+  if (c >= e) return false;
+  x_init(x, P.st, P.words + (size_t)lo * kTeamWords, (unsigned)(e - a), (unsigned)(c - a), c == 0 ? P.skip_seq : 0u,
+         P.timeout_ns);
+  return true;
+}
+
+// The team's next system (-1: the queue is empty, -2: a wait gave up).  Its first one
+// is fixed, so that a team sized for a system gets that one.
+__device__ __forceinline__ int next_system(Team& T, bool first) {
+  const BatchParams& P = T.P;
+  int j = T.id;
+  if (!first) {
+    if (T.rank == 0 && threadIdx.x == 0) P.next[T.id] = P.nteams + (int)atomicAdd(P.queue, 1u);
+    if (!T.sync()) return -2;
+    j = __ldcg(P.next + T.id);
+  }
+  if (j >= P.nsys) return -1;
+  const int s = __ldg(P.order + j);
+  __syncthreads();  // seg may still be read for the system before
+  if (threadIdx.x == 0) {
+    SegInfo& g = T.seg;
+    g.nd = P.sdia[s];
+    g.t0 = P.tstart[s];
+    g.tend = g.t0 + P.ntile[s];
+    g.lo = g.t0 * kTile;
+    g.hi = g.tend * kTile - 1;
+    g.ut = P.utiles[s];
+    g.un0 = P.ustart[s];
+    g.nunit = P.nunit[s];
+    g.u0 = (int)((int64_t)g.nunit * T.rank / T.size);
+    g.u1 = (int)((int64_t)g.nunit * (T.rank + 1) / T.size);
 #pragma unroll
-  for (int j = 0; j < NV; ++j) a[j] = 0.0;
+    for (int m = 0; m < kBatchDiag; ++m) g.delta[m] = P.sdelta[s * kBatchDiag + m];
+  }
+  __syncthreads();
+  return s;
+}
+
+// One phase over this CTA's units.  For every row i of a unit, row(i) does the row's
+// loads and arithmetic and returns its commit, which stores the results and adds the
+// row's NV contributions to the thread's accumulators.  A thread's rows go in groups
+// of ROWS (8, 4, 2 or 1, by the variant's register budget), every row's loads in
+// flight before the first commit (a store ahead of the next row's loads would
+// serialise them); the accumulation order stays the row order.  The unit's sums are
+// then formed per warp and stored; sums NREQ .. NV-1 only with `all`.
+template <int NV, int ROWS, int NREQ = NV, class Row>
+__device__ __forceinline__ void run_phase(const Team& T, Row row, bool all = true) {
+  const SegInfo& seg = T.seg;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  for (int u = seg.u0; u < seg.u1; ++u) {
+    const int t0 = seg.t0 + u * seg.ut, t1 = min(t0 + seg.ut, seg.tend);
+    double acc[NV > 0 ? NV : 1];
+#pragma unroll
+    for (int k = 0; k < (NV > 0 ? NV : 1); ++k) acc[k] = 0.0;
+    int gt = t0;
+    if constexpr (ROWS >= 8) {
+      for (; gt + 7 < t1; gt += 8) {
+        const auto c0 = row(gt * kTile + t);
+        const auto c1 = row((gt + 1) * kTile + t);
+        const auto c2 = row((gt + 2) * kTile + t);
+        const auto c3 = row((gt + 3) * kTile + t);
+        const auto c4 = row((gt + 4) * kTile + t);
+        const auto c5 = row((gt + 5) * kTile + t);
+        const auto c6 = row((gt + 6) * kTile + t);
+        const auto c7 = row((gt + 7) * kTile + t);
+        c0(acc);
+        c1(acc);
+        c2(acc);
+        c3(acc);
+        c4(acc);
+        c5(acc);
+        c6(acc);
+        c7(acc);
+      }
+    }
+    if constexpr (ROWS >= 4) {
+      for (; gt + 3 < t1; gt += 4) {
+        const auto c0 = row(gt * kTile + t);
+        const auto c1 = row((gt + 1) * kTile + t);
+        const auto c2 = row((gt + 2) * kTile + t);
+        const auto c3 = row((gt + 3) * kTile + t);
+        c0(acc);
+        c1(acc);
+        c2(acc);
+        c3(acc);
+      }
+    }
+    if constexpr (ROWS >= 2) {
+      for (; gt + 1 < t1; gt += 2) {
+        const auto c0 = row(gt * kTile + t);
+        const auto c1 = row((gt + 1) * kTile + t);
+        c0(acc);
+        c1(acc);
+      }
+    }
+    for (; gt < t1; ++gt) row(gt * kTile + t)(acc);
+    if (NV > 0) {
+      // the warp's sum of each value, exact and rounded once on the integer pipes: an
+      // fp64 xor tree would take 5 warp instructions of the fp64 pipe (one per ~64
+      // clocks per SM sub-partition) that the rows' FMAs need
+#pragma unroll
+      for (int k = 0; k < NV; ++k)
+        if (k < NREQ || all) acc[k] = warp_sum_exact(acc[k]);
+      if (lane == 0) {
+        double* dst = T.bank() + ((size_t)(seg.un0 + u) * kWarps + warp) * kNP;
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+          if (k < NREQ || all) dst[k] = acc[k];
+      }
+    }
+  }
+}
+
+// The team's barrier after a phase that formed sums, then the system's sums of values
+// 0 .. NV-1 in warp 0, the same bits in every CTA: thread t adds partials t,
+// t + kBlock, ... in order (its loads in flight together), then cta_sum0.  The next
+// reduction writes the other bank: a slower CTA may still be reading this one.
+template <int NV>
+__device__ __forceinline__ bool reduce(Team& T, double (&out)[NV]) {
+  constexpr int kSumBatch = 4;
+  const double* bank = T.bank();
+  T.flip += 1;
+  if (!T.sync()) return false;
+  const size_t p0 = (size_t)T.seg.un0 * kWarps;
+  const int np = T.seg.nunit * kWarps;
+#pragma unroll
+  for (int j = 0; j < NV; ++j) out[j] = 0.0;
   for (int t0 = threadIdx.x; t0 < np; t0 += kBlock * kSumBatch) {
     double v[kSumBatch][NV];
 #pragma unroll
     for (int u = 0; u < kSumBatch; ++u) {
       const int t = t0 + kBlock * u;
 #pragma unroll
-      for (int j = 0; j < NV; ++j) v[u][j] = t < np ? __ldcg(P.tpart + (size_t)(p0 + t) * kNP + j) : 0.0;
+      for (int j = 0; j < NV; ++j) v[u][j] = t < np ? __ldcg(bank + (p0 + t) * kNP + j) : 0.0;
     }
 #pragma unroll
     for (int u = 0; u < kSumBatch; ++u) {
       if (t0 + kBlock * u < np) {
 #pragma unroll
-        for (int j = 0; j < NV; ++j) a[j] += v[u][j];
+        for (int j = 0; j < NV; ++j) out[j] += v[u][j];
       }
     }
   }
-  cta_sum0<NV>(a);
+  cta_sum0<NV>(out);
+  return true;
+}
+
+// What thread 0 of a CTA decides from a system's sums, for all its threads.
+struct Control {
+  double alpha, beta, rho, inv_rho, bb, relres, stop, stop2_hi, rho_k, beta0;
+  int k, restarts, status, zero;
+  int act;   // after R: 1 = iterate, 0 = the system is done; after A: 0 = failed
+  int wrr;   // r.D r is formed with the r update
+  int last;  // this iteration ends the (inner) loop
+  int exact; // r.D r must be formed before the test
+};
+
+__device__ __forceinline__ void control_init(Control& c) {
   if (threadIdx.x == 0) {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) s_out[j] = a[j];
+    c.bb = -1.0;  // "not yet known": the first residual phase records b.b
+    c.relres = 0.0;
+    c.k = c.restarts = c.zero = 0;
+    c.status = kStRunning;
+    c.rho_k = 0.0;
   }
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < NV; ++j) out[j] = s_out[j];
   __syncthreads();
 }
 
-// New stage of sys, tagged with the current phase (one writer per system and phase).
-__device__ __forceinline__ void set_stage(const BatchParams& P, int sys, int stage, unsigned seq) {
-  const unsigned long long before = __ldcg(P.sstate + sys) & 0xffull;
-  P.sstate[sys] = ((unsigned long long)seq << 16) | (before << 8) | (unsigned long long)stage;
+__device__ __forceinline__ void report(const Team& T, const Control& c, int s) {
+  if (T.rank == 0 && threadIdx.x == 0) {
+    T.P.relres[s] = c.relres;
+    T.P.k[s] = c.k;
+    T.P.restarts[s] = c.restarts;
+    T.P.status[s] = c.status;
+    T.P.zero[s] = c.zero;
+  }
 }
 
-// One phase over its list of reduction groups [0, T).  CTA c takes the
-// contiguous chunk [c T / G, (c+1) T / G), which spans few systems.  At the
-// start of each system's segment begin(sys) loads the system's scalars and
-// says whether its sums are wanted.  For every row i of a group, row(i) does
-// the row's loads and arithmetic and returns its commit, which stores the
-// results and adds the row's NV contributions to the thread's accumulators.
-// A thread's rows go in groups of ROWS (8, 4, 2 or 1, by the variant's register
-// budget), every row's loads in flight before the first commit (a store ahead
-// of the next row's loads would serialise them); the accumulation order stays
-// the row order.  The group's sums are then reduced
-// per warp (xor tree) and stored.  Leaving a segment, the CTA adds its group count to the system's
-// counter; the CTA that completes the count sums the system's partials in
-// (group, warp) order, independent of G, and calls done(sys, sums) in thread 0.
-// Sums NREQ.. NV-1 are reduced only while *opt holds (set by begin for the segment's system).
-template <int NV, int ROWS, bool WEIGHTED, int NREQ = NV, class Begin, class Row, class Done>
-__device__ __forceinline__ void run_phase(const BatchParams& P, const int* s_pref, int T, const Grid& g,
-                                          SegInfo& seg, Begin begin, Row row, Done done,
-                                          const bool* opt = nullptr) {
-  __shared__ int s_last;
-  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-  const int j1 = (int)((int64_t)T * (g.cta + 1) / g.G);
-  int j = (int)((int64_t)T * g.cta / g.G);
-  while (j < j1) {
-    const int sys = system_of(P, s_pref, j);
-    // this CTA's groups of sys: those whose first unit lies in [j, j1)
-    const int w = WEIGHTED ? P.wcost[sys] : 1;
-    const int base = s_pref[sys];
-    const int g0 = (j - base + w - 1) / w;
-    const int g1 = min(P.ngroup[sys], (j1 - base + w - 1) / w);
-    const int next = base + P.ngroup[sys] * w;  // the next system's first unit
-    if (g0 >= g1) {
-      j = min(j1, next);
-      continue;
-    }
-    if (t == 0) {
-      seg.nd = P.sdia[sys];
-      seg.lo = P.tstart[sys] * kTile;
-      seg.hi = seg.lo + P.ntile[sys] * kTile - 1;
-#pragma unroll
-      for (int m = 0; m < kBatchDiag; ++m) seg.delta[m] = P.sdelta[sys * kBatchDiag + m];
-    }
-    __syncthreads();
-    const bool sums = begin(sys);
-    const int tend = P.tstart[sys] + P.ntile[sys];
-    for (int grp = g0; grp < g1; ++grp) {
-      const int t0 = P.tstart[sys] + grp * kGroup, t1 = min(t0 + kGroup, tend);
-      double acc[NV > 0 ? NV : 1];
-#pragma unroll
-      for (int k = 0; k < (NV > 0 ? NV : 1); ++k) acc[k] = 0.0;
-      int gt = t0;
-      if constexpr (ROWS >= 8) {
-        for (; gt + 7 < t1; gt += 8) {
-          const auto c0 = row(gt * kTile + t);
-          const auto c1 = row((gt + 1) * kTile + t);
-          const auto c2 = row((gt + 2) * kTile + t);
-          const auto c3 = row((gt + 3) * kTile + t);
-          const auto c4 = row((gt + 4) * kTile + t);
-          const auto c5 = row((gt + 5) * kTile + t);
-          const auto c6 = row((gt + 6) * kTile + t);
-          const auto c7 = row((gt + 7) * kTile + t);
-          c0(acc);
-          c1(acc);
-          c2(acc);
-          c3(acc);
-          c4(acc);
-          c5(acc);
-          c6(acc);
-          c7(acc);
-        }
-      }
-      if constexpr (ROWS >= 4) {
-        for (; gt + 3 < t1; gt += 4) {
-          const auto c0 = row(gt * kTile + t);
-          const auto c1 = row((gt + 1) * kTile + t);
-          const auto c2 = row((gt + 2) * kTile + t);
-          const auto c3 = row((gt + 3) * kTile + t);
-          c0(acc);
-          c1(acc);
-          c2(acc);
-          c3(acc);
-        }
-      }
-      if constexpr (ROWS >= 2) {
-        for (; gt + 1 < t1; gt += 2) {
-          const auto c0 = row(gt * kTile + t);
-          const auto c1 = row((gt + 1) * kTile + t);
-          c0(acc);
-          c1(acc);
-        }
-      }
-      for (; gt < t1; ++gt) row(gt * kTile + t)(acc);
-      if (NV > 0 && sums) {
-        // the warp's sum of each reduced value, exact and rounded once on the integer
-        // pipes: an fp64 xor tree would take 5 warp instructions of the fp64 pipe
-        // (one per ~64 clocks per SM sub-partition) that the rows' FMAs need
-        const bool all = NREQ >= NV || (opt && *opt);
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-          if (k < NREQ || all) acc[k] = warp_sum_exact(acc[k]);
-        }
-        if (lane == 0) {
-          double* dst = P.tpart + ((size_t)(P.gstart[sys] + grp) * kWarps + warp) * kNP;
-#pragma unroll
-          for (int k = 0; k < NV; ++k)
-            if (k < NREQ || all) dst[k] = acc[k];
-        }
-      }
-    }
-    if (NV > 0 && sums) {
-      if (lane == 0) __threadfence();  // partials visible before the count
-      __syncthreads();
-      if (t == 0) {
-        const unsigned add = (unsigned)(g1 - g0);
-        const unsigned prev = atomicAdd(P.cnt + sys, add);
-        const int last = prev + add == (unsigned)P.ngroup[sys];
-        if (last) P.cnt[sys] = 0u;  // reset for the next phase (after its barrier)
-        __threadfence();
-        s_last = last;
-      }
-      __syncthreads();
-      if (s_last) {
-        double sm[NV > 0 ? NV : 1];
-        system_sum<NV>(P, sys, sm);
-        if (t == 0) done(sys, sm);
-      }
-    }
-    __syncthreads();  // every thread is done with seg before the next segment's
-    j = min(j1, next);
-  }
+// The r update's scalars and test (thread 0): rho' = sums[0], r.D r = sums[1] if it was
+// formed.  above: r.D r >= dmin rho' > stop^2, so the test fails for sure.
+template <bool JAC>
+__device__ __forceinline__ void after_update(Control& c, double rho1, double rr, double dmin, double stop2,
+                                             int maxit) {
+  c.beta = rho1 * c.inv_rho;
+  c.rho_k = c.rho;  // r.z of the step just taken (the carry's denominator)
+  c.rho = rho1;
+  c.k += 1;
+  c.exact = 0;
+  bool conv = false;
+  if (!JAC || c.wrr) conv = below_stop(JAC ? rr : rho1, c.stop, c.stop2_hi);
+  else c.exact = dmin * rho1 <= stop2;
+  if (JAC) c.wrr = c.exact || dmin * rho1 <= kRrMarginB * stop2;
+  c.last = conv || c.k >= maxit;
 }
 
 // MINB: resident CTAs per SM the registers are budgeted for (an autotuner choice).
 template <bool JAC, int MINB>
 __global__ void __launch_bounds__(kBlock, MINB) batch_pcg_kernel(BatchParams P) {
   // rows in flight per thread within the register budget of MINB CTAs per SM
-  constexpr int kRows = MINB <= 3 ? 4 : (MINB == 4 ? 2 : 1);
+  constexpr int kRows = MINB <= 3 ? 4 : 2;
   // phase B streams only q and r (two loads a row): twice the rows in flight
   constexpr int kRowsB = 2 * kRows;
-  __shared__ int s_pref[kMaxBatch];
-  __shared__ int s_scan[kWarps];
   __shared__ SegInfo s_seg;
   __shared__ XState s_x;
-  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
+  __shared__ Control c;
+  const int t = threadIdx.x;
+  int id, rank, size;
+  if (!team_init(P, &s_x, &id, &rank, &size)) return;
+  Team T{P, s_seg, &s_x, id, rank, size, 0};
   double* __restrict__ r = P.r;
   double* __restrict__ p = P.p;
   double* __restrict__ q = P.q;
   double* __restrict__ xh = P.xh;
   const double* __restrict__ bh = P.bh;
   const double* __restrict__ dg = P.dg;
-  double c_alpha = 0.0, c_beta = 0.0;  // scalars of the current segment's system
-  bool c_flag = false, c_sum = false;
-  unsigned seq = 0;  // phase number; the initial stage words carry 0
-  for (;;) {
-    // ---- R: residual of the stage 0 / 3 systems, their test, (re)start
-    ++seq;
-    bool alive = false;
-    int T = build_list<true>(P, kMaskR, seq, s_pref, s_scan, &alive);
-    if (!alive) break;
-    if (T > 0) {
-      run_phase<3, kRows, true>(
-          P, s_pref, T, g, s_seg, [&](int) { return true; },
-          [&](int i) {
-            const double xi = xh[i];
-            const double ri_ax = row_spmv(P, xh, i, JAC ? xi : __ldg(dg + i) * xi, s_seg);
-            const double bi = bh[i];
-            const double ri = bi - ri_ax;
-            const double d = JAC ? __ldg(dg + i) : 1.0;
-            return [=](double* acc) {
-              r[i] = ri;
-              p[i] = ri;
-              acc[0] = fma(ri, ri, acc[0]);      // r^.r^ = r.z
-              acc[1] = fma(d * ri, ri, acc[1]);  // r.r
-              acc[2] = fma(d * bi, bi, acc[2]);  // b.b
-            };
-          },
-          [&](int sys, const double* sm) {
-            const bool first = P.bb[sys] < 0.0;
-            if (first) P.bb[sys] = sm[2];
-            const double bb = P.bb[sys];
-            const double rel = bb > 0.0 ? sqrt(sm[1]) / sqrt(bb) : 0.0;
-            P.relres[sys] = rel;
-            P.rho[sys] = sm[0];
-            P.rr[sys] = sm[1];
-            P.wrr[sys] = JAC && P.dmin[sys] * sm[0] <= kRrMarginB * P.tol * P.tol * bb;
-            int st = P.status[sys], next = kStDone;
-            if (bb == 0.0) {
-              st = kOk;
-              P.zero[sys] = 1;
-            } else if (st == kBreakdown || st == kNumeric) {
-              // keep: the residual was only wanted for the report
-            } else if (!isfinite(rel)) {
-              st = kNumeric;
-            } else if (rel <= P.tol) {
-              st = kOk;
-            } else if (P.k[sys] >= P.maxit) {
-              st = kNotConverged;
-            } else if (first) {
-              st = kStRunning;
-              next = kStIter;
-            } else if (P.restarts[sys] >= P.max_restarts) {
-              st = kNotConverged;
-            } else {
-              P.restarts[sys] += 1;
-              st = kStRunning;
-              next = kStIter;
-            }
-            P.status[sys] = st;
-            set_stage(P, sys, next, seq);
-          });
-      if (!g.sync()) return;
-    }
-    // ---- A: q = A p, alpha
-    ++seq;
-    T = build_list<true>(P, kMaskAB, seq, s_pref, s_scan, &alive);
-    if (T == 0) continue;
-    run_phase<1, kRows, true>(
-        P, s_pref, T, g, s_seg, [&](int) { return true; },
-        [&](int i) {
+  for (bool first_system = true;; first_system = false) {
+    const int sys = next_system(T, first_system);
+    if (sys < 0) return;
+    control_init(c);
+    const double dmin = P.dmin[sys];
+    for (;;) {
+      // ---- R: residual, true-residual test, (re)start
+      run_phase<3, kRows>(T, [&](int i) {
+        const double xi = xh[i];
+        const double ri_ax = row_spmv(P, xh, i, JAC ? xi : __ldg(dg + i) * xi, s_seg);
+        const double bi = bh[i];
+        const double ri = bi - ri_ax;
+        const double d = JAC ? __ldg(dg + i) : 1.0;
+        return [=](double* acc) {
+          r[i] = ri;
+          p[i] = ri;
+          acc[0] = fma(ri, ri, acc[0]);      // r^.r^ = r.z
+          acc[1] = fma(d * ri, ri, acc[1]);  // r.r
+          acc[2] = fma(d * bi, bi, acc[2]);  // b.b
+        };
+      });
+      double s3[3];
+      if (!reduce<3>(T, s3)) return;
+      if (t == 0) {
+        const bool first = c.bb < 0.0;
+        if (first) {
+          c.bb = s3[2];
+          c.stop = P.tol * sqrt(c.bb);
+          c.stop2_hi = stop2_high(c.stop);
+        }
+        const double rel = c.bb > 0.0 ? sqrt(s3[1]) / sqrt(c.bb) : 0.0;
+        c.relres = rel;
+        c.rho = s3[0];
+        c.wrr = JAC && dmin * s3[0] <= kRrMarginB * P.tol * P.tol * c.bb;
+        c.act = 0;
+        if (c.bb == 0.0) {
+          c.status = kOk;
+          c.zero = 1;
+        } else if (c.status == kBreakdown || c.status == kNumeric) {
+          // keep: the residual was only wanted for the report
+        } else if (!isfinite(rel)) {
+          c.status = kNumeric;
+        } else if (rel <= P.tol) {
+          c.status = kOk;
+        } else if (c.k >= P.maxit || (!first && c.restarts >= P.max_restarts)) {
+          c.status = kNotConverged;
+        } else {
+          if (!first) c.restarts += 1;
+          c.act = 1;
+        }
+      }
+      __syncthreads();
+      if (!c.act) break;
+      for (;;) {
+        // ---- A: q = A p, alpha
+        run_phase<1, kRows>(T, [&](int i) {
           const double pi = p[i];
           const double qi = row_spmv(P, p, i, JAC ? pi : __ldg(dg + i) * pi, s_seg);
           return [=](double* acc) {
             q[i] = qi;
             acc[0] = fma(pi, qi, acc[0]);
           };
-        },
-        [&](int sys, const double* sm) {
-          const double rho = P.rho[sys];
-          if (!isfinite(sm[0]) || !isfinite(rho)) {
-            P.status[sys] = kNumeric;
-            set_stage(P, sys, kStResidual, seq);  // residual of the current x, then stop
-          } else if (sm[0] <= 0.0) {
-            P.status[sys] = kBreakdown;
-            set_stage(P, sys, kStResidual, seq);
-          } else {
-            P.alpha[sys] = rho / sm[0];
-          }
         });
-    if (!g.sync()) return;
-    // ---- B: r -= alpha q, rho' = r^.r^, r.r when near the stopping band, beta, test
-    ++seq;
-    T = build_list<false>(P, kMaskAB, seq, s_pref, s_scan, &alive);
-    run_phase<2, kRowsB, false, 1>(
-        P, s_pref, T, g, s_seg,
-        [&](int sys) {
-          c_alpha = P.alpha[sys];
-          c_flag = JAC && P.wrr[sys];
-          return true;
-        },
-        [&](int i) {
-          const double ri = fma(-c_alpha, q[i], r[i]);
-          const double di = c_flag ? __ldg(dg + i) : 0.0;
-          const bool flag = c_flag;
+        double s1[1];
+        if (!reduce<1>(T, s1)) return;
+        if (t == 0) {
+          c.act = 1;
+          if (!isfinite(s1[0]) || !isfinite(c.rho)) c.status = kNumeric, c.act = 0;
+          else if (s1[0] <= 0.0) c.status = kBreakdown, c.act = 0;
+          else c.alpha = c.rho / s1[0];
+        }
+        __syncthreads();
+        if (!c.act) break;  // the residual of the current x, then stop
+        // ---- B: r -= alpha q, rho' = r^.r^, r.r near the stopping band, beta, test
+        const double alpha = c.alpha;
+        const bool flag = JAC && c.wrr;
+        if (t == 32) c.inv_rho = 1.0 / c.rho;
+        run_phase<2, kRowsB, 1>(T, [&](int i) {
+          const double ri = fma(-alpha, q[i], r[i]);
+          const double di = flag ? __ldg(dg + i) : 0.0;
           return [=](double* acc) {
             r[i] = ri;
             acc[0] = fma(ri, ri, acc[0]);
             if (flag) acc[1] = fma(di * ri, ri, acc[1]);
           };
-        },
-        [&](int sys, const double* sm) {
-          const double rho = sm[0];
-          P.beta[sys] = rho / P.rho[sys];
-          P.rho[sys] = rho;
-          const int k = P.k[sys] + 1;
-          P.k[sys] = k;
-          const double stop2 = P.tol * P.tol * P.bb[sys];
-          bool conv;
-          if (!JAC || P.wrr[sys]) {
-            const double rr = JAC ? sm[1] : rho;
-            P.rr[sys] = rr;
-            conv = sqrt(rr) <= P.tol * sqrt(P.bb[sys]);
-          } else {
-            // r.D r >= dmin r^.r^: above the band the test fails for sure
-            conv = false;
-            if (P.dmin[sys] * rho <= stop2) {
-              P.wrr[sys] = 1;
-              set_stage(P, sys, kStRrPending, seq);  // exact r.D r in phase C
-              return;
-            }
-          }
-          if (JAC) P.wrr[sys] = P.dmin[sys] * rho <= kRrMarginB * stop2;
-          if (conv || k >= P.maxit) set_stage(P, sys, kStLastX, seq);
-        },
-        &c_flag);
-    if (!g.sync()) return;
-    // ---- C: x += alpha p; p = r + beta p unless the loop ended; pending r.D r
-    ++seq;
-    T = build_list<false>(P, kMaskC, seq, s_pref, s_scan, &alive);
-    run_phase<1, kRows, false>(
-        P, s_pref, T, g, s_seg,
-        [&](int sys) {
-          const int stg = eff_stage(__ldcg(P.sstate + sys), seq);
-          c_alpha = P.alpha[sys];
-          c_beta = P.beta[sys];
-          c_flag = stg != kStLastX;  // p is still needed
-          c_sum = stg == kStRrPending;
-          return c_sum;
-        },
-        [&](int i) {
+        }, flag);
+        double s2[2] = {0.0, 0.0};
+        if (flag) {
+          if (!reduce<2>(T, s2)) return;
+        } else {
+          double w[1];
+          if (!reduce<1>(T, w)) return;
+          s2[0] = w[0];
+        }
+        if (t == 0) after_update<JAC>(c, s2[0], s2[1], dmin, P.tol * P.tol * c.bb, P.maxit);
+        __syncthreads();
+        if (c.exact) {
+          run_phase<1, kRows>(T, [&](int i) {
+            const double ri = r[i], di = __ldg(dg + i);
+            return [=](double* acc) { acc[0] = fma(di * ri, ri, acc[0]); };
+          });
+          if (!reduce<1>(T, s1)) return;
+          if (t == 0) c.last = below_stop(s1[0], c.stop, c.stop2_hi) || c.k >= P.maxit;
+          __syncthreads();
+        }
+        // ---- C: x += alpha p; p = r + beta p unless the loop ends
+        const double beta = c.beta;
+        const bool last = c.last != 0;
+        run_phase<0, kRows>(T, [&](int i) {
           const double pi = p[i];
-          const double xn = fma(c_alpha, pi, xh[i]);
-          const double ri = r[i];
-          const double pn = fma(c_beta, pi, ri);
-          const bool keep_p = c_flag, sum = JAC && c_sum;
-          const double di = sum ? __ldg(dg + i) : 0.0;
-          return [=](double* acc) {
+          const double xn = fma(alpha, pi, xh[i]);
+          const double pn = last ? pi : fma(beta, pi, r[i]);
+          return [=](double*) {
             xh[i] = xn;
-            if (keep_p) p[i] = pn;
-            if (sum) acc[0] = fma(di * ri, ri, acc[0]);
+            if (!last) p[i] = pn;
           };
-        },
-        [&](int sys, const double* sm) {
-          P.rr[sys] = sm[0];
-          const bool conv = sqrt(sm[0]) <= P.tol * sqrt(P.bb[sys]);
-          // converged or out of iterations: x is final, so the true residual next
-          set_stage(P, sys, conv || P.k[sys] >= P.maxit ? kStResidual : kStIter, seq);
         });
-    if (!g.sync()) return;
+        if (!T.sync()) return;
+        if (last) break;
+      }
+    }
+    report(T, c, sys);
   }
 }
 
-// fp32 inner solves with fp64 refinement (readings R6 and R8 per system).
-// Stages beyond the fp64 kernel's: 5 = the step's x/p update is still due (C,
-// then iterating), 6 = the inner solve's last update is still due (C, then R).
-constexpr int kStCOnly = 5, kStFinalDue = 6;
-constexpr unsigned kMaskC32 = (1u << kStIter) | (1u << kStLastX) | (1u << kStRrPending) | (1u << kStCOnly) |
-                              (1u << kStFinalDue);
-
-// Every system solved as the single-system refinement solves it: R forms the
-// fp64 residual r = b^ - A^ x^ with the fp64 loop matrix, takes the true-residual
-// test and starts an inner solve on r32 = fl32(r) (d = 0; with reliable updates,
-// P.carry, the search direction carries over: p = r32 + (r32.r32 / rho_k) p_k);
-// A, B, C are the inner fp32 PCG on the fp32 loop matrix, sums in fp64, until
-// the inner residual has dropped by tol_in; the inner solve's last C phase adds
-// fl64(d + alpha p) to x^ and hands the system back to R.  The carried direction
-// is never stored before its first use: A gathers r + beta0 p at neighbouring
-// rows, and B writes p = r + beta0 p for its own rows before it updates r.
+// fp32 inner solves with fp64 refinement (readings R6 and R8 per system), each as the
+// single-system refinement does it: R forms the fp64 residual r = b^ - A^ x^ with the
+// fp64 loop matrix, takes the true-residual test and starts an inner solve on
+// r32 = fl32(r) (d = 0; with reliable updates, P.carry, the search direction carries
+// over: p = r32 + (r32.r32 / rho_k) p_k); A, B, C are the inner fp32 PCG on the fp32
+// loop matrix, sums in fp64, until the inner residual has dropped by tol_in; the inner
+// solve's last C phase adds fl64(d + alpha p) to x^.  The carried direction is never
+// stored before its first use: A gathers r + beta0 p at neighbouring rows, and B
+// writes p = r + beta0 p for its own rows before it updates r.
 template <bool JAC, int MINB>
 __global__ void __launch_bounds__(kBlock, MINB) batch_ir_kernel(BatchParams P) {
-  constexpr int kRows = MINB <= 3 ? 4 : (MINB == 4 ? 2 : 1);
-  __shared__ int s_pref[kMaxBatch];
-  __shared__ int s_scan[kWarps];
+  constexpr int kRows = MINB <= 3 ? 4 : 2;
   __shared__ SegInfo s_seg;
   __shared__ XState s_x;
-  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
+  __shared__ Control c;
+  const int t = threadIdx.x;
+  int id, rank, size;
+  if (!team_init(P, &s_x, &id, &rank, &size)) return;
+  Team T{P, s_seg, &s_x, id, rank, size, 0};
   float* __restrict__ r = P.r32;
   float* __restrict__ p = P.p32;
   float* __restrict__ q = P.q32;
@@ -687,229 +623,157 @@ __global__ void __launch_bounds__(kBlock, MINB) batch_ir_kernel(BatchParams P) {
   double* __restrict__ xh = P.xh;
   const double* __restrict__ bh = P.bh;
   const double* __restrict__ dg = P.dg;
-  float c_alpha = 0.0f, c_beta = 0.0f, c_beta0 = 0.0f;
-  bool c_flag = false, c_start = false;
-  int c_mode = 0;  // C phase: 0 update, 1 last update of the inner solve, 2 r.D r only
-  unsigned seq = 0;
-  for (;;) {
-    // ---- R: fp64 residual, true-residual test, start of an inner solve
-    ++seq;
-    bool alive = false;
-    int T = build_list<true>(P, kMaskR, seq, s_pref, s_scan, &alive);
-    if (!alive) break;
-    if (T > 0) {
-      run_phase<4, kRows, true>(
-          P, s_pref, T, g, s_seg, [&](int) { return true; },
-          [&](int i) {
-            const double xi = xh[i];
-            const double ax = row_spmv(P, xh, i, JAC ? xi : __ldg(dg + i) * xi, s_seg);
-            const double bi = bh[i];
-            const double ri = bi - ax;
-            const float r32 = (float)ri;
-            const double dd = JAC ? __ldg(dg + i) : 1.0;
+  for (bool first_system = true;; first_system = false) {
+    const int sys = next_system(T, first_system);
+    if (sys < 0) return;
+    control_init(c);
+    const double dmin = P.dmin[sys];
+    for (;;) {
+      // ---- R: fp64 residual, true-residual test, start of an inner solve
+      run_phase<4, kRows>(T, [&](int i) {
+        const double xi = xh[i];
+        const double ax = row_spmv(P, xh, i, JAC ? xi : __ldg(dg + i) * xi, s_seg);
+        const double bi = bh[i];
+        const double ri = bi - ax;
+        const float r32 = (float)ri;
+        const double dd = JAC ? __ldg(dg + i) : 1.0;
+        return [=](double* acc) {
+          r[i] = r32;
+          d[i] = 0.0f;
+          const double rs = (double)r32;
+          acc[0] = fma(rs, rs, acc[0]);       // r32.r32: the inner rho
+          acc[1] = fma(dd * rs, rs, acc[1]);  // r32.D r32: the inner solve's reference norm
+          acc[2] = fma(dd * ri, ri, acc[2]);  // fp64 r.r
+          acc[3] = fma(dd * bi, bi, acc[3]);  // b.b
+        };
+      });
+      double s4[4];
+      if (!reduce<4>(T, s4)) return;
+      if (t == 0) {
+        if (c.bb < 0.0) c.bb = s4[3];
+        const double rel = c.bb > 0.0 ? sqrt(s4[2]) / sqrt(c.bb) : 0.0;
+        c.relres = rel;
+        c.act = 0;
+        if (c.bb == 0.0) {
+          c.status = kOk;
+          c.zero = 1;
+        } else if (c.status == kBreakdown || c.status == kNumeric) {
+          // keep: the residual was only wanted for the report
+        } else if (!isfinite(rel)) {
+          c.status = kNumeric;
+        } else if (rel <= P.tol) {
+          c.status = kOk;
+        } else if (c.k >= P.maxit || c.restarts >= P.max_outer || !(s4[0] > 0.0)) {
+          c.status = kNotConverged;  // out of iterations or updates (or r32 underflowed to 0)
+        } else {
+          c.beta0 = (P.carry && c.rho_k > 0.0) ? s4[0] / c.rho_k : 0.0;
+          c.rho = s4[0];
+          c.stop = P.tol_in * sqrt(s4[1]);
+          c.stop2_hi = stop2_high(c.stop);
+          c.wrr = JAC && dmin * s4[0] <= kRrMarginB * c.stop * c.stop;
+          c.restarts += 1;  // inner solves started (refinement steps / updates)
+          c.act = 1;
+        }
+      }
+      __syncthreads();
+      if (!c.act) break;
+      const float b0 = (float)c.beta0;
+      for (bool start = true;; start = false) {
+        // ---- A: q = A p (the first step of an inner solve: p = r + beta0 p gathered), alpha
+        auto rows_a = [&](auto gx) {
+          run_phase<1, kRows>(T, [&, gx](int i) {
+            const float pi = gx(i);
+            const float dgi = JAC ? 1.0f : (float)__ldg(dg + i);
+            const float qi = row_spmv_g<float, float>(P, P.val32, i, dgi * pi, s_seg, gx);
             return [=](double* acc) {
-              r[i] = r32;
-              d[i] = 0.0f;
-              const double rs = (double)r32;
-              acc[0] = fma(rs, rs, acc[0]);       // r32.r32: the inner rho
-              acc[1] = fma(dd * rs, rs, acc[1]);  // r32.D r32: the inner solve's reference norm
-              acc[2] = fma(dd * ri, ri, acc[2]);  // fp64 r.r
-              acc[3] = fma(dd * bi, bi, acc[3]);  // b.b
+              q[i] = qi;
+              acc[0] = fma((double)pi, (double)qi, acc[0]);
             };
-          },
-          [&](int sys, const double* sm) {
-            const bool first = P.bb[sys] < 0.0;
-            if (first) P.bb[sys] = sm[3];
-            const double bb = P.bb[sys];
-            const double rel = bb > 0.0 ? sqrt(sm[2]) / sqrt(bb) : 0.0;
-            P.relres[sys] = rel;
-            int st = P.status[sys], next = kStDone;
-            if (bb == 0.0) {
-              st = kOk;
-              P.zero[sys] = 1;
-            } else if (st == kBreakdown || st == kNumeric) {
-              // keep: the residual was only wanted for the report
-            } else if (!isfinite(rel)) {
-              st = kNumeric;
-            } else if (rel <= P.tol) {
-              st = kOk;
-            } else if (P.k[sys] >= P.maxit || P.restarts[sys] >= P.max_outer || !(sm[0] > 0.0)) {
-              st = kNotConverged;  // out of iterations or updates (or r32 underflowed to 0)
-            } else {
-              const double rho = sm[0];
-              P.beta0[sys] = (P.carry && P.rho_k[sys] > 0.0) ? rho / P.rho_k[sys] : 0.0;
-              P.rho[sys] = rho;
-              P.rr[sys] = sm[1];
-              const double stop = P.tol_in * sqrt(sm[1]);
-              P.stopin[sys] = stop;
-              P.wrr[sys] = JAC && P.dmin[sys] * rho <= kRrMarginB * stop * stop;
-              P.start[sys] = 1;
-              P.restarts[sys] += 1;  // inner solves started (refinement steps / updates)
-              st = kStRunning;
-              next = kStIter;
-            }
-            P.status[sys] = st;
-            set_stage(P, sys, next, seq);
           });
-      if (!g.sync()) return;
-    }
-    // ---- A: q = A p (the first step of an inner solve: p = r + beta0 p gathered), alpha
-    ++seq;
-    T = build_list<true>(P, kMaskAB, seq, s_pref, s_scan, &alive);
-    if (T == 0) continue;
-    run_phase<1, kRows, true>(
-        P, s_pref, T, g, s_seg,
-        [&](int sys) {
-          c_start = P.start[sys] != 0;
-          c_beta0 = (float)P.beta0[sys];
-          return true;
-        },
-        [&](int i) {
-          float pi, qi;
-          const float dgi = JAC ? 1.0f : (float)__ldg(dg + i);
-          if (c_start && c_beta0 != 0.0f) {
-            const float b0 = c_beta0;
-            auto gx = [=](int j) { return fmaf(b0, p[j], r[j]); };
-            pi = gx(i);
-            qi = row_spmv_g<float, float>(P, P.val32, i, dgi * pi, s_seg, gx);
-          } else if (c_start) {
-            auto gx = [=](int j) { return r[j]; };
-            pi = r[i];
-            qi = row_spmv_g<float, float>(P, P.val32, i, dgi * pi, s_seg, gx);
-          } else {
-            auto gx = [=](int j) { return p[j]; };
-            pi = p[i];
-            qi = row_spmv_g<float, float>(P, P.val32, i, dgi * pi, s_seg, gx);
-          }
-          return [=](double* acc) {
-            q[i] = qi;
-            acc[0] = fma((double)pi, (double)qi, acc[0]);
-          };
-        },
-        [&](int sys, const double* sm) {
-          const double rho = P.rho[sys];
-          if (!isfinite(sm[0]) || !isfinite(rho) || sm[0] <= 0.0) {
+        };
+        if (!start) rows_a([=](int j) { return p[j]; });
+        else if (b0 != 0.0f) rows_a([=](int j) { return fmaf(b0, p[j], r[j]); });
+        else rows_a([=](int j) { return r[j]; });
+        double s1[1];
+        if (!reduce<1>(T, s1)) return;
+        if (t == 0) {
+          c.act = 1;
+          if (!isfinite(s1[0]) || !isfinite(c.rho) || s1[0] <= 0.0) {
             // x^ gets the inner iterate so far (d), then R reports its true residual
-            P.status[sys] = (!isfinite(sm[0]) || !isfinite(rho)) ? kNumeric : kBreakdown;
-            P.alpha[sys] = 0.0;
-            set_stage(P, sys, kStLastX, seq);
+            c.status = (!isfinite(s1[0]) || !isfinite(c.rho)) ? kNumeric : kBreakdown;
+            c.alpha = 0.0;
+            c.act = 0;
+            c.last = 1;
           } else {
-            P.alpha[sys] = rho / sm[0];
+            c.alpha = c.rho / s1[0];
           }
-        });
-    if (!g.sync()) return;
-    // ---- B: p = r + beta0 p at the start of an inner solve; r -= alpha q, rho', r.D r near
-    //      the band, beta, the inner test
-    ++seq;
-    T = build_list<false>(P, kMaskAB, seq, s_pref, s_scan, &alive);
-    run_phase<2, kRows, false, 1>(
-        P, s_pref, T, g, s_seg,
-        [&](int sys) {
-          c_alpha = (float)P.alpha[sys];
-          c_flag = JAC && P.wrr[sys];
-          c_start = P.start[sys] != 0;
-          c_beta0 = (float)P.beta0[sys];
-          return true;
-        },
-        [&](int i) {
-          const float r0 = r[i];
-          const float ri = fmaf(-c_alpha, q[i], r0);
-          const bool st = c_start;
-          const float pn = st ? (c_beta0 != 0.0f ? fmaf(c_beta0, p[i], r0) : r0) : 0.0f;
-          const double di = c_flag ? __ldg(dg + i) : 0.0;
-          const bool flag = c_flag;
-          return [=](double* acc) {
-            r[i] = ri;
-            if (st) p[i] = pn;
-            const double rd = (double)ri;
-            acc[0] = fma(rd, rd, acc[0]);
-            if (flag) acc[1] = fma(di * rd, rd, acc[1]);
-          };
-        },
-        [&](int sys, const double* sm) {
-          P.start[sys] = 0;
-          const double rho = sm[0];
-          P.beta[sys] = rho / P.rho[sys];
-          P.rho_k[sys] = P.rho[sys];  // r.z of the step just taken (the carry's denominator)
-          P.rho[sys] = rho;
-          const int k = P.k[sys] + 1;
-          P.k[sys] = k;
-          const double stop = P.stopin[sys];
-          bool conv;
-          if (!JAC || P.wrr[sys]) {
-            const double rr = JAC ? sm[1] : rho;
-            P.rr[sys] = rr;
-            conv = sqrt(rr) <= stop;
+        }
+        __syncthreads();
+        const float alpha = (float)c.alpha;
+        if (c.act) {
+          // ---- B: p = r + beta0 p at the start of an inner solve; r -= alpha q, rho', r.D r
+          //      near the band, beta, the inner test
+          const bool flag = JAC && c.wrr;
+          if (t == 32) c.inv_rho = 1.0 / c.rho;
+          run_phase<2, kRows, 1>(T, [&](int i) {
+            const float r0 = r[i];
+            const float ri = fmaf(-alpha, q[i], r0);
+            const float pn = start ? (b0 != 0.0f ? fmaf(b0, p[i], r0) : r0) : 0.0f;
+            const double di = flag ? __ldg(dg + i) : 0.0;
+            return [=](double* acc) {
+              r[i] = ri;
+              if (start) p[i] = pn;
+              const double rd = (double)ri;
+              acc[0] = fma(rd, rd, acc[0]);
+              if (flag) acc[1] = fma(di * rd, rd, acc[1]);
+            };
+          }, flag);
+          double s2[2] = {0.0, 0.0};
+          if (flag) {
+            if (!reduce<2>(T, s2)) return;
           } else {
-            conv = false;  // r.D r >= dmin r^.r^: above the band the test fails for sure
-            if (P.dmin[sys] * rho <= stop * stop) {
-              P.wrr[sys] = 1;
-              set_stage(P, sys, kStRrPending, seq);  // exact r.D r in phase C, no update yet
-              return;
-            }
+            double w[1];
+            if (!reduce<1>(T, w)) return;
+            s2[0] = w[0];
           }
-          if (JAC) P.wrr[sys] = P.dmin[sys] * rho <= kRrMarginB * stop * stop;
-          if (conv || k >= P.maxit) set_stage(P, sys, kStLastX, seq);
-        },
-        &c_flag);
-    if (!g.sync()) return;
-    // ---- C: d += alpha p, p = r + beta p; the inner solve's last update x^ += fl64(d + alpha p)
-    //      (p stays the last direction); a pending exact r.D r
-    ++seq;
-    T = build_list<false>(P, kMaskC32, seq, s_pref, s_scan, &alive);
-    run_phase<1, kRows, false>(
-        P, s_pref, T, g, s_seg,
-        [&](int sys) {
-          const int stg = eff_stage(__ldcg(P.sstate + sys), seq);
-          c_alpha = (float)P.alpha[sys];
-          c_beta = (float)P.beta[sys];
-          c_mode = (stg == kStLastX || stg == kStFinalDue) ? 1 : (stg == kStRrPending ? 2 : 0);
-          // sums (and so done()) for the r.D r pass and to move the deferred stages on
-          return stg == kStRrPending || stg == kStCOnly || stg == kStFinalDue;
-        },
-        [&](int i) {
-          const int mode = c_mode;
-          // alpha = 0 (a breakdown at an inner solve's first step): p is not read
-          const float pi = (mode != 2 && c_alpha != 0.0f) ? p[i] : 0.0f;
-          const float di = mode != 2 ? d[i] : 0.0f;
-          const float ri = mode != 1 ? r[i] : 0.0f;
-          const double xo = mode == 1 ? xh[i] : 0.0;
-          const float dn = fmaf(c_alpha, pi, di);
-          const float pn = fmaf(c_beta, pi, ri);
-          const double dgi = (JAC && mode == 2) ? __ldg(dg + i) : 0.0;
-          return [=](double* acc) {
-            if (mode == 0) {
+          if (t == 0) after_update<JAC>(c, s2[0], s2[1], dmin, c.stop * c.stop, P.maxit);
+          __syncthreads();
+          if (c.exact) {
+            run_phase<1, kRows>(T, [&](int i) {
+              const double rd = (double)r[i], di = __ldg(dg + i);
+              return [=](double* acc) { acc[0] = fma(di * rd, rd, acc[0]); };
+            });
+            if (!reduce<1>(T, s1)) return;
+            if (t == 0) c.last = below_stop(s1[0], c.stop, c.stop2_hi) || c.k >= P.maxit;
+            __syncthreads();
+          }
+        }
+        // ---- C: d += alpha p, p = r + beta p; the inner solve's last update x^ += fl64(d + alpha p)
+        //      (p stays the last direction)
+        const bool last = c.last != 0;
+        const float beta = (float)c.beta;
+        if (last) {
+          run_phase<0, kRows>(T, [&](int i) {
+            // alpha = 0 (a breakdown at an inner solve's first step): p is not read
+            const float pi = alpha != 0.0f ? p[i] : 0.0f;
+            const double xn = xh[i] + (double)fmaf(alpha, pi, d[i]);
+            return [=](double*) { xh[i] = xn; };
+          });
+        } else {
+          run_phase<0, kRows>(T, [&](int i) {
+            const float pi = p[i];
+            const float dn = fmaf(alpha, pi, d[i]), pn = fmaf(beta, pi, r[i]);
+            return [=](double*) {
               d[i] = dn;
               p[i] = pn;
-            } else if (mode == 1) {
-              xh[i] = xo + (double)dn;
-            } else {
-              const double rd = (double)ri;
-              acc[0] = fma(JAC ? dgi * rd : rd, rd, acc[0]);
-            }
-          };
-        },
-        [&](int sys, const double* sm) {
-          const int stg = eff_stage(__ldcg(P.sstate + sys), seq);
-          if (stg == kStRrPending) {
-            P.rr[sys] = sm[0];
-            const bool conv = sqrt(sm[0]) <= P.stopin[sys];
-            set_stage(P, sys, conv || P.k[sys] >= P.maxit ? kStFinalDue : kStCOnly, seq);
-          } else if (stg == kStCOnly) {
-            set_stage(P, sys, kStIter, seq);
-          } else {  // kStFinalDue: the last update is done, the fp64 residual is next
-            set_stage(P, sys, kStLastX, seq);
-          }
-        });
-    if (!g.sync()) return;
-  }
-}
-
-// Inner-solve state of every system at the start of an fp32 solve (no direction to carry yet).
-__global__ void batch_init_f32_kernel(int nsys, double* rho_k, int* start) {
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nsys; s += gridDim.x * blockDim.x) {
-    rho_k[s] = 0.0;
-    start[s] = 0;
+            };
+          });
+        }
+        if (!T.sync()) return;
+        if (last) break;
+      }
+    }
+    report(T, c, sys);
   }
 }
 
@@ -949,19 +813,15 @@ __global__ void batch_scatter_kernel(double* const* x, const int64_t* n, const i
   }
 }
 
-// Loop state of every system at the start of a solve.
-__global__ void batch_init_kernel(int nsys, double* bb, int* k, int* restarts, int* status, int* zero,
-                                  int* wrr, unsigned long long* sstate, unsigned* cnt) {
+// Result words of every system and the queue at the start of a solve.
+__global__ void batch_init_kernel(int nsys, int* k, int* restarts, int* status, int* zero, unsigned* queue) {
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < nsys; s += gridDim.x * blockDim.x) {
-    bb[s] = -1.0;  // "not yet known": the first residual phase records b.b
     k[s] = 0;
     restarts[s] = 0;
     status[s] = kStRunning;
     zero[s] = 0;
-    wrr[s] = 0;
-    sstate[s] = 0ull;  // stage 0, phase 0
-    cnt[s] = 0u;
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) *queue = 0u;
 }
 
 // One system's rows into the concatenated slices (thread per padded row):
@@ -1049,25 +909,18 @@ __global__ void batch_diag_kernel(int64_t n, int64_t npad, int64_t r0, const dou
   }
 }
 
-// Kernel variants the autotuner chooses from: registers budgeted for 3, 4 or 5
-// resident CTAs per SM (more CTAs hide more memory latency; fewer registers
-// may spill).
-constexpr int kVariants = 3;
-constexpr int kVariantMinBlocks[kVariants] = {3, 4, 5};
+// Kernel variants the autotuner chooses from: registers budgeted for 3 or 4 resident
+// CTAs per SM (more CTAs hide more latency; more registers keep more rows in flight).
+constexpr int kVariants = 2;
+constexpr int kVariantMinBlocks[kVariants] = {3, 4};
 
 const void* batch_kernel(bool jac, int variant, bool f32) {
   if (f32) {
-    switch (variant) {
-      case 0: return jac ? (const void*)batch_ir_kernel<true, 3> : (const void*)batch_ir_kernel<false, 3>;
-      case 1: return jac ? (const void*)batch_ir_kernel<true, 4> : (const void*)batch_ir_kernel<false, 4>;
-      default: return jac ? (const void*)batch_ir_kernel<true, 5> : (const void*)batch_ir_kernel<false, 5>;
-    }
+    if (variant == 0) return jac ? (const void*)batch_ir_kernel<true, 3> : (const void*)batch_ir_kernel<false, 3>;
+    return jac ? (const void*)batch_ir_kernel<true, 4> : (const void*)batch_ir_kernel<false, 4>;
   }
-  switch (variant) {
-    case 0: return jac ? (const void*)batch_pcg_kernel<true, 3> : (const void*)batch_pcg_kernel<false, 3>;
-    case 1: return jac ? (const void*)batch_pcg_kernel<true, 4> : (const void*)batch_pcg_kernel<false, 4>;
-    default: return jac ? (const void*)batch_pcg_kernel<true, 5> : (const void*)batch_pcg_kernel<false, 5>;
-  }
+  if (variant == 0) return jac ? (const void*)batch_pcg_kernel<true, 3> : (const void*)batch_pcg_kernel<false, 3>;
+  return jac ? (const void*)batch_pcg_kernel<true, 4> : (const void*)batch_pcg_kernel<false, 4>;
 }
 
 // fp32 copy of the loop matrix values (the same rounding as the single-system
@@ -1096,24 +949,25 @@ struct BatchData {
   int ntiles = 0, nslices = 0;
   int64_t entries = 0;             // slice entries (multiple of 32)
   int32_t *d_tstart = nullptr, *d_ntile = nullptr, *soff = nullptr, *col = nullptr;
-  int32_t *d_gstart = nullptr, *d_ngroup = nullptr, *d_wcost = nullptr;
+  int32_t *d_ustart = nullptr, *d_nunit = nullptr, *d_utiles = nullptr, *d_order = nullptr, *d_team0 = nullptr;
+  std::vector<int32_t> nunit, order;  // reduction units; the queue (systems by descending work)
+  std::vector<double> cost;           // work of an iteration of each system (relative)
   std::vector<int32_t> sdia, sdelta;  // diagonal layout of each system and its offsets (kBatchDiag each)
   int32_t *d_sdia = nullptr, *d_sdelta = nullptr;
-  int ngroups = 0;                 // reduction groups in all
+  int nunits = 0;                  // reduction units in all
   double* d_dmin = nullptr;        // smallest A_ii per system
   int64_t *d_n = nullptr, *d_r0 = nullptr;
   double* val[2] = {nullptr, nullptr};  // [precond]: unscaled / Jacobi-scaled
   float* val32[2] = {nullptr, nullptr}; // fp32 copies (fp32 precisions)
   float *r32 = nullptr, *p32 = nullptr, *q32 = nullptr, *d32 = nullptr;  // inner fp32 vectors
-  double *rho_k = nullptr, *beta0 = nullptr, *stopin = nullptr;          // per system (fp32)
-  int* start = nullptr;
   double *dg = nullptr, *dsq = nullptr, *disq = nullptr;
   double *r = nullptr, *p = nullptr, *q = nullptr, *xh = nullptr, *bh = nullptr;
-  double *rho = nullptr, *rr = nullptr, *bb = nullptr, *alpha = nullptr, *beta = nullptr,
-         *relres = nullptr;
-  int *k = nullptr, *restarts = nullptr, *status = nullptr, *zero = nullptr, *wrr = nullptr;
-  unsigned long long* sstate = nullptr;
-  unsigned* cnt = nullptr;
+  double* relres = nullptr;
+  int *k = nullptr, *restarts = nullptr, *status = nullptr, *zero = nullptr, *next = nullptr;
+  unsigned* queue = nullptr;
+  XWord* words = nullptr;          // the teams' exchange words
+  int max_teams = 0;               // teams that words, next and d_team0 hold
+  std::vector<int32_t> team0;      // the teams on the device (d_team0)
   double* tpart = nullptr;
   const double** d_b = nullptr;    // the caller's vector pointers, on the device
   double** d_x = nullptr;
@@ -1122,6 +976,7 @@ struct BatchData {
   int vmax[kVariants] = {};        // co-resident CTAs of each kernel variant
   int grid_tuned[4] = {};          // chosen CTAs per tune_slot (0: not yet)
   int var_tuned[4] = {};           // chosen kernel variant per tune_slot
+  int teams_tuned[4] = {};         // and most teams
   int tune_chosen[4] = {-1, -1, -1, -1};  // index of the chosen candidate
   float tune_ms[4][kMaxCand] = {}; // autotuner timings of the candidates
   int tune_grid[4][kMaxCand] = {};
@@ -1131,7 +986,7 @@ struct BatchData {
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t gexec = nullptr;
   int gkey_jac = -1, gkey_grid = -1, gkey_var = -1, gkey_maxit = -1, gkey_restarts = -1;
-  int gkey_f32 = -1, gkey_carry = -1, gkey_outer = -1;
+  int gkey_f32 = -1, gkey_carry = -1, gkey_outer = -1, gkey_teams = -1;
   double gkey_tol = -1.0, gkey_timeout = -1.0, gkey_tol_in = -1.0;
   unsigned gkey_skip = 0;
   std::string graph_refused;       // why graph capture failed (then: direct launches)
@@ -1146,11 +1001,10 @@ void cgi::batch_free(BatchData* b) {
   for (cg_handle* h : b->sys) cg_destroy(h);
   void* dev[] = {b->d_tstart, b->d_ntile, b->soff,     b->col,    b->d_n,  b->d_r0,   b->val[0],
                  b->val[1],   b->dg,      b->dsq,      b->disq,   b->r,    b->p,      b->q,
-                 b->xh,       b->bh,      b->rho,      b->rr,     b->bb,   b->alpha,  b->beta,
-                 b->relres,   b->k,       b->restarts, b->status, b->zero, b->sstate, b->cnt,
-                 b->tpart,    (void*)b->d_b, (void*)b->d_x, b->d_gstart, b->d_ngroup, b->d_dmin, b->wrr, b->d_wcost,
-                 b->d_sdia,   b->d_sdelta, b->val32[0], b->val32[1], b->r32, b->p32, b->q32, b->d32,
-                 b->rho_k,    b->beta0,   b->stopin, b->start};
+                 b->xh,       b->bh,      b->relres,   b->k,        b->restarts, b->status, b->zero,
+                 b->tpart,    (void*)b->d_b, (void*)b->d_x, b->d_ustart, b->d_nunit, b->d_utiles, b->d_order,
+                 b->d_team0,  b->next,    b->queue,    b->words,    b->d_dmin,
+                 b->d_sdia,   b->d_sdelta, b->val32[0], b->val32[1], b->r32, b->p32, b->q32, b->d32};
   for (void* p : dev)
     if (p) cudaFree(p);
   if (b->host_ptrs) cudaFreeHost(b->host_ptrs);
@@ -1222,13 +1076,11 @@ cg_status ensure_batch_f32(cg_handle* h, bool jac) {
   batch_to_f32_kernel<<<blocks_for((int64_t)ent), 256, 0, h->stream>>>((int64_t)ent, B->val[jac], B->val32[jac]);
   CGB_CUDA(h, cudaGetLastError());
   if (!B->r32) {
-    const size_t nv = (size_t)B->rows, ns = (size_t)B->nsys;
+    const size_t nv = (size_t)B->rows;
     for (float** v : {&B->r32, &B->p32, &B->q32, &B->d32}) {
       CGB_CUDA(h, cudaMalloc(v, sizeof(float) * nv));
       CGB_CUDA(h, cudaMemsetAsync(*v, 0, sizeof(float) * nv, h->stream));
     }
-    for (double** v : {&B->rho_k, &B->beta0, &B->stopin}) CGB_CUDA(h, cudaMalloc(v, sizeof(double) * ns));
-    CGB_CUDA(h, cudaMalloc(&B->start, sizeof(int) * ns));
   }
   CGB_CUDA(h, cudaStreamSynchronize(h->stream));
   return CG_OK;
@@ -1240,13 +1092,12 @@ BatchParams make_params(cg_handle* h, bool jac, double tol, int maxit) {
   P.nsys = B->nsys;
   P.tstart = B->d_tstart;
   P.ntile = B->d_ntile;
-  P.gstart = B->d_gstart;
-  P.ngroup = B->d_ngroup;
-  P.wcost = B->d_wcost;
+  P.ustart = B->d_ustart;
+  P.nunit = B->d_nunit;
+  P.utiles = B->d_utiles;
   P.sdia = B->d_sdia;
   P.sdelta = B->d_sdelta;
   P.dmin = B->d_dmin;
-  P.wrr = B->wrr;
   P.soff = B->soff;
   P.col = B->col;
   P.val = B->val[jac];
@@ -1256,24 +1107,23 @@ BatchParams make_params(cg_handle* h, bool jac, double tol, int maxit) {
   P.q = B->q;
   P.xh = B->xh;
   P.bh = B->bh;
-  P.rho = B->rho;
-  P.rr = B->rr;
-  P.bb = B->bb;
-  P.alpha = B->alpha;
-  P.beta = B->beta;
   P.relres = B->relres;
   P.k = B->k;
   P.restarts = B->restarts;
   P.status = B->status;
   P.zero = B->zero;
-  P.sstate = B->sstate;
-  P.cnt = B->cnt;
   P.tpart = B->tpart;
+  P.bank = (int64_t)B->nunits * kWarps * kNP;
+  P.order = B->d_order;
+  P.team0 = B->d_team0;
+  P.nteams = (int)B->team0.size() - 1;
+  P.queue = B->queue;
+  P.next = B->next;
+  P.words = B->words;
   P.tol = tol;
   P.maxit = maxit;
   P.max_restarts = h->max_restarts;
   P.st = h->st;
-  P.xs = exchange_words(h->st);
   P.timeout_ns = (uint64_t)(h->timeout_ms * 1e6);
   P.skip_seq = h->skip_seq;
   P.val32 = B->val32[jac];
@@ -1281,12 +1131,46 @@ BatchParams make_params(cg_handle* h, bool jac, double tol, int maxit) {
   P.p32 = B->p32;
   P.q32 = B->q32;
   P.d32 = B->d32;
-  P.rho_k = B->rho_k;
-  P.beta0 = B->beta0;
-  P.stopin = B->stopin;
-  P.start = B->start;
   P.max_outer = h->max_outer;
   return P;
+}
+
+// The teams of a grid of G CTAs, at most `most` of them: with a team for every system,
+// CTAs by the systems' work (no more than units); else equal teams that take the
+// systems one after the other.  The fault injection gets one team of all CTAs.
+std::vector<int32_t> plan_teams(const BatchData* B, int G, int most, bool one) {
+  const int ns = B->nsys;
+  const int nt = one ? 1 : std::max(1, std::min({ns, G, most, B->max_teams}));
+  std::vector<int32_t> size((size_t)nt, 1);
+  if (nt == ns && !one) {
+    double total = 0.0;
+    for (double w : B->cost) total += w;
+    int left = G;
+    // in descending work, each its share of what is left (rounded down, one at least)
+    for (int t = 0; t < nt; ++t) {
+      const int s = B->order[(size_t)t];
+      const int share = total > 0.0 ? (int)((double)left * B->cost[(size_t)s] / total) : 1;
+      size[(size_t)t] = std::max(1, std::min({share, (int)B->nunit[(size_t)s], left - (nt - 1 - t)}));
+      left -= size[(size_t)t];
+      total -= B->cost[(size_t)s];
+    }
+  } else {
+    for (int t = 0; t < nt; ++t) size[(size_t)t] = G / nt + (t < G % nt ? 1 : 0);
+  }
+  std::vector<int32_t> team0(1, 0);
+  for (int c : size) team0.push_back(team0.back() + c);
+  return team0;
+}
+
+// Makes those teams the handle's (an upload ordered on its stream when they change).
+cudaError_t set_teams(cg_handle* h, int G, int most) {
+  BatchData* B = h->batch;
+  std::vector<int32_t> t = plan_teams(B, G, most, h->skip_seq != 0);
+  if (t == B->team0) return cudaSuccess;
+  const cudaError_t e = cudaMemcpyAsync(B->d_team0, t.data(), sizeof(int32_t) * t.size(), cudaMemcpyHostToDevice,
+                                        h->stream);
+  if (e == cudaSuccess) B->team0 = std::move(t);
+  return e == cudaSuccess ? cudaStreamSynchronize(h->stream) : e;  // t is pageable host memory
 }
 
 // The work of one solve on h->stream: clear the status words, gather b and
@@ -1299,13 +1183,12 @@ cudaError_t enqueue_solve(cg_handle* h, cudaStream_t s, bool jac, int var, int G
   P.carry = carry ? 1 : 0;
   P.tol_in = tol_in;
   const dim3 gg(64, (unsigned)B->nsys);
-  cudaError_t e = cudaMemsetAsync(h->st, 0, kStBytes, s);
+  cudaError_t e = cudaMemsetAsync(h->st, 0, sizeof(DevState), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(B->words, 0, sizeof(XWord) * kTeamWords * (size_t)P.nteams, s);
   if (e != cudaSuccess) return e;
   batch_gather_kernel<<<gg, 256, 0, s>>>(B->d_b, B->d_x, B->d_n, B->d_r0, B->d_ntile, B->disq, B->dsq,
                                           jac ? 1 : 0, B->bh, B->xh);
-  batch_init_kernel<<<blocks_for(B->nsys), 256, 0, s>>>(B->nsys, B->bb, B->k, B->restarts, B->status,
-                                                         B->zero, B->wrr, B->sstate, B->cnt);
-  if (f32) batch_init_f32_kernel<<<blocks_for(B->nsys), 256, 0, s>>>(B->nsys, B->rho_k, B->start);
+  batch_init_kernel<<<blocks_for(B->nsys), 256, 0, s>>>(B->nsys, B->k, B->restarts, B->status, B->zero, B->queue);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   void* args[] = {&P};
@@ -1317,13 +1200,15 @@ cudaError_t enqueue_solve(cg_handle* h, cudaStream_t s, bool jac, int var, int G
 
 // Run one solve (through the cached graph when use_graph) between the
 // handle's events; the device time goes to *ms.
-cg_status run_solve(cg_handle* h, bool jac, int var, int G, double tol, int maxit, bool use_graph,
+cg_status run_solve(cg_handle* h, bool jac, int var, int G, int teams, double tol, int maxit, bool use_graph,
                     bool scatter, float* ms, bool f32, bool carry, double tol_in) {
   BatchData* B = h->batch;
+  CGB_CUDA(h, set_teams(h, G, teams));
+  const int nteams = (int)B->team0.size() - 1;
   if (use_graph && B->graph_refused.empty()) {
     const bool same = B->gexec && B->gkey_jac == (int)jac && B->gkey_grid == G && B->gkey_var == var &&
                       B->gkey_tol == tol && B->gkey_f32 == (int)f32 && B->gkey_carry == (int)carry &&
-                      B->gkey_tol_in == tol_in && B->gkey_outer == h->max_outer &&
+                      B->gkey_tol_in == tol_in && B->gkey_outer == h->max_outer && B->gkey_teams == nteams &&
                       B->gkey_maxit == maxit && B->gkey_restarts == h->max_restarts &&
                       B->gkey_timeout == h->timeout_ms && B->gkey_skip == h->skip_seq;
     if (!same) {
@@ -1348,7 +1233,7 @@ cg_status run_solve(cg_handle* h, bool jac, int var, int G, double tol, int maxi
         B->gexec = nullptr;
         cudaGetLastError();
         B->graph_refused = cudaGetErrorString(e != cudaSuccess ? e : (e2 != cudaSuccess ? e2 : e3));
-        return run_solve(h, jac, var, G, tol, maxit, false, scatter, ms, f32, carry, tol_in);
+        return run_solve(h, jac, var, G, teams, tol, maxit, false, scatter, ms, f32, carry, tol_in);
       }
       B->graph = graph;
       B->gkey_jac = jac;
@@ -1363,6 +1248,7 @@ cg_status run_solve(cg_handle* h, bool jac, int var, int G, double tol, int maxi
       B->gkey_carry = carry;
       B->gkey_tol_in = tol_in;
       B->gkey_outer = h->max_outer;
+      B->gkey_teams = nteams;
     }
     CGB_CUDA(h, cudaEventRecord(h->ev0, h->stream));
     CGB_CUDA(h, cudaGraphLaunch(B->gexec, h->stream));
@@ -1386,30 +1272,31 @@ cg_status run_solve(cg_handle* h, bool jac, int var, int G, double tol, int maxi
   return CG_OK;
 }
 
-// Autotuner: the kernel variant (registers budgeted for 3, 4 or 5 CTAs per SM)
-// and grid size for this handle and preconditioner, picked by timing short
-// trial solves (at most kTrialIters iterations each, x left untouched) of the
-// caller's own systems; the choice is kept in the handle.  Candidates: every
-// variant at its full residency, and the 3-CTA variant at one CTA per SM.
+// Autotuner: the kernel variant (registers budgeted for 3 or 4 CTAs per SM, at full
+// residency) and the most teams for this handle and preconditioner, picked by timing
+// short trial solves (at most kTrialIters iterations each, x left untouched) of the
+// caller's own systems; the choice is kept in the handle.  Few large teams keep few
+// systems in flight (L2 holds them); many small ones wait less at their barriers.
 constexpr int kTrialIters = 40;
+constexpr int kManyTeams = 128, kSomeTeams = 32, kFewTeams = 20;
 
 cg_status autotune(cg_handle* h, bool jac, double tol, int maxit, bool f32, bool carry, double tol_in) {
   const int sl = tune_slot(jac, f32);
   BatchData* B = h->batch;
-  std::vector<std::pair<int, int>> cand;  // (variant, grid)
-  for (int v = 0; v < kVariants; ++v)
-    if (B->vmax[v] > 0) cand.emplace_back(v, B->vmax[v]);
-  if (B->vmax[0] > h->sm_count) cand.emplace_back(0, h->sm_count);
+  struct Cand {
+    int var, teams;
+  };
+  const Cand cand[] = {{1, kManyTeams}, {1, kSomeTeams}, {1, kFewTeams}, {0, kSomeTeams}};
   float best = 3.0e38f;
   int best_i = 0, nt = 0;
-  for (size_t c = 0; c < cand.size() && nt < kMaxCand; ++c) {
+  for (const Cand& c : cand) {
     float ms = 0.0f;
-    const cg_status ts = run_solve(h, jac, cand[c].first, cand[c].second, tol,
-                                   std::min<int32_t>(maxit, kTrialIters), false, false, &ms, f32, carry, tol_in);
+    const cg_status ts = run_solve(h, jac, c.var, B->vmax[c.var], c.teams, tol, std::min<int32_t>(maxit, kTrialIters),
+                                   false, false, &ms, f32, carry, tol_in);
     if (ts != CG_OK) return ts;
     B->tune_ms[sl][nt] = ms;
-    B->tune_grid[sl][nt] = cand[c].second;
-    B->tune_minb[sl][nt] = kVariantMinBlocks[cand[c].first];
+    B->tune_grid[sl][nt] = B->vmax[c.var];
+    B->tune_minb[sl][nt] = kVariantMinBlocks[c.var];
     if (ms < best) {
       best = ms;
       best_i = nt;
@@ -1418,8 +1305,9 @@ cg_status autotune(cg_handle* h, bool jac, double tol, int maxit, bool f32, bool
   }
   B->tune_count[sl] = nt;
   B->tune_chosen[sl] = best_i;
-  B->var_tuned[sl] = cand[(size_t)best_i].first;
-  B->grid_tuned[sl] = cand[(size_t)best_i].second;
+  B->var_tuned[sl] = cand[best_i].var;
+  B->grid_tuned[sl] = B->vmax[cand[best_i].var];
+  B->teams_tuned[sl] = cand[best_i].teams;
   return CG_OK;
 }
 
@@ -1465,7 +1353,7 @@ cg_status cg_batch_create(int32_t nsys, const int64_t* n, const int32_t* const* 
   int dev = 0;
   CGB_CREATE(cudaGetDevice(&dev));
   CGB_CREATE(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev));
-  CGB_CREATE(cudaMalloc(&h->st, kStBytes));
+  CGB_CREATE(cudaMalloc(&h->st, sizeof(DevState)));
   CGB_CREATE(cudaMallocHost(&h->host_st, sizeof(DevState)));
   CGB_CREATE(cudaEventCreate(&h->ev0));
   CGB_CREATE(cudaEventCreate(&h->ev1));
@@ -1548,45 +1436,52 @@ cg_status cg_batch_create(int32_t nsys, const int64_t* n, const int32_t* const* 
   CGB_CREATE(cudaMemcpy(B->d_r0, B->r0.data(), sizeof(int64_t) * ns, cudaMemcpyHostToDevice));
   for (double** v : {&B->dg, &B->dsq, &B->disq, &B->r, &B->p, &B->q, &B->xh, &B->bh})
     CGB_CREATE(cudaMalloc(v, sizeof(double) * nv));
-  for (double** v : {&B->rho, &B->rr, &B->bb, &B->alpha, &B->beta, &B->relres})
-    CGB_CREATE(cudaMalloc(v, sizeof(double) * ns));
-  for (int** v : {&B->k, &B->restarts, &B->status, &B->zero, &B->wrr}) CGB_CREATE(cudaMalloc(v, sizeof(int) * ns));
+  CGB_CREATE(cudaMalloc(&B->relres, sizeof(double) * ns));
+  for (int** v : {&B->k, &B->restarts, &B->status, &B->zero}) CGB_CREATE(cudaMalloc(v, sizeof(int) * ns));
   {
-    std::vector<int32_t> gst(ns), ngr(ns), wc(ns);
+    std::vector<int32_t> ust(ns), ut(ns);
     std::vector<double> dmin(ns);
-    int groups = 0;
+    B->nunit.resize(ns);
+    B->cost.resize(ns);
+    B->order.resize(ns);
+    int units = 0;
     for (size_t s = 0; s < ns; ++s) {
-      gst[s] = groups;
-      ngr[s] = (B->ntile[s] + kGroup - 1) / kGroup;
-      groups += ngr[s];
+      ut[s] = unit_tiles(B->ntile[s]);
+      ust[s] = units;
+      B->nunit[s] = (B->ntile[s] + ut[s] - 1) / ut[s];
+      units += B->nunit[s];
       dmin[s] = B->sys[s]->jacobi_ok ? B->sys[s]->dmin : 1.0;
-      // SpMV-phase cost of a row: W + 2 units for W stored entries a row
-      // (padding included).  The phase is held by GB300's fp64 pipe (W fused
-      // multiply-adds, the p.q term and the reduction) about as much as by the
-      // W values (and columns) it streams; both grow as W + ~1.6
+      // work of an iteration: fp64 instructions a row, W + 5 for W stored entries
       const int64_t sl0 = (int64_t)B->tstart[s] * kWarps, sl1 = sl0 + (int64_t)B->ntile[s] * kWarps;
-      const int64_t wsum = soff[(size_t)sl1] - soff[(size_t)sl0];
-      const int64_t wavg = (wsum + (sl1 - sl0) - 1) / std::max<int64_t>(sl1 - sl0, 1);
-      wc[s] = (int32_t)(wavg + 2);
+      B->cost[s] = 32.0 * (double)(soff[(size_t)sl1] - soff[(size_t)sl0]) + 5.0 * kTile * (double)B->ntile[s];
+      B->order[s] = (int32_t)s;
     }
-    B->ngroups = groups;
-    CGB_CREATE(cudaMalloc(&B->d_gstart, sizeof(int32_t) * ns));
-    CGB_CREATE(cudaMalloc(&B->d_ngroup, sizeof(int32_t) * ns));
+    std::stable_sort(B->order.begin(), B->order.end(),
+                     [&](int32_t x, int32_t y) { return B->cost[(size_t)x] > B->cost[(size_t)y]; });
+    B->nunits = units;
+    B->max_teams = (int)std::min<int64_t>(nsys, 1024);
+    auto upload = [&](int32_t** d, const std::vector<int32_t>& v) {
+      cudaError_t e = cudaMalloc(d, sizeof(int32_t) * v.size());
+      if (e == cudaSuccess) e = cudaMemcpy(*d, v.data(), sizeof(int32_t) * v.size(), cudaMemcpyHostToDevice);
+      return e;
+    };
+    CGB_CREATE(upload(&B->d_ustart, ust));
+    CGB_CREATE(upload(&B->d_nunit, B->nunit));
+    CGB_CREATE(upload(&B->d_utiles, ut));
+    CGB_CREATE(upload(&B->d_order, B->order));
     CGB_CREATE(cudaMalloc(&B->d_dmin, sizeof(double) * ns));
-    CGB_CREATE(cudaMemcpy(B->d_gstart, gst.data(), sizeof(int32_t) * ns, cudaMemcpyHostToDevice));
-    CGB_CREATE(cudaMemcpy(B->d_ngroup, ngr.data(), sizeof(int32_t) * ns, cudaMemcpyHostToDevice));
     CGB_CREATE(cudaMemcpy(B->d_dmin, dmin.data(), sizeof(double) * ns, cudaMemcpyHostToDevice));
-    CGB_CREATE(cudaMalloc(&B->d_wcost, sizeof(int32_t) * ns));
-    CGB_CREATE(cudaMemcpy(B->d_wcost, wc.data(), sizeof(int32_t) * ns, cudaMemcpyHostToDevice));
     CGB_CREATE(cudaMalloc(&B->d_sdia, sizeof(int32_t) * ns));
     CGB_CREATE(cudaMemcpy(B->d_sdia, B->sdia.data(), sizeof(int32_t) * ns, cudaMemcpyHostToDevice));
     CGB_CREATE(cudaMalloc(&B->d_sdelta, sizeof(int32_t) * ns * kBatchDiag));
     CGB_CREATE(cudaMemcpy(B->d_sdelta, B->sdelta.data(), sizeof(int32_t) * ns * kBatchDiag,
                           cudaMemcpyHostToDevice));
   }
-  CGB_CREATE(cudaMalloc(&B->sstate, sizeof(unsigned long long) * ns));
-  CGB_CREATE(cudaMalloc(&B->cnt, sizeof(unsigned) * ns));
-  CGB_CREATE(cudaMalloc(&B->tpart, sizeof(double) * (size_t)B->ngroups * kWarps * kNP));
+  CGB_CREATE(cudaMalloc(&B->d_team0, sizeof(int32_t) * ((size_t)B->max_teams + 1)));
+  CGB_CREATE(cudaMalloc(&B->next, sizeof(int) * (size_t)B->max_teams));
+  CGB_CREATE(cudaMalloc(&B->queue, sizeof(unsigned)));
+  CGB_CREATE(cudaMalloc(&B->words, sizeof(XWord) * kTeamWords * (size_t)B->max_teams));
+  CGB_CREATE(cudaMalloc(&B->tpart, sizeof(double) * 2 * (size_t)B->nunits * kWarps * kNP));
   CGB_CREATE(cudaMalloc((void**)&B->d_b, sizeof(double*) * ns));
   CGB_CREATE(cudaMalloc((void**)&B->d_x, sizeof(double*) * ns));
   CGB_CREATE(cudaMallocHost((void**)&B->host_ptrs, sizeof(void*) * 2 * ns));
@@ -1652,7 +1547,7 @@ cg_status cg_solve_batch(cg_handle* h, const double* const* b, double* const* x,
   std::memcpy(B->host_ptrs + ns, x, sizeof(void*) * ns);
   CGB_CUDA(h, cudaMemcpyAsync(B->d_b, B->host_ptrs, sizeof(void*) * ns, cudaMemcpyHostToDevice, h->stream));
   CGB_CUDA(h, cudaMemcpyAsync(B->d_x, B->host_ptrs + ns, sizeof(void*) * ns, cudaMemcpyHostToDevice, h->stream));
-  int G = 0, var = 0;
+  int G = 0, var = 0, teams = kSomeTeams;
   if (h->grid_opt > 0) {
     // a forced grid runs on the variant with the most registers that can hold it
     G = std::min(h->grid_opt, B->grid_max);
@@ -1664,10 +1559,11 @@ cg_status cg_solve_batch(cg_handle* h, const double* const* b, double* const* x,
     }
     G = B->grid_tuned[sl];
     var = B->var_tuned[sl];
+    teams = B->teams_tuned[sl];
   }
   const bool use_graph = h->loop_mode != 1;
   float ms = 0.0f;
-  const cg_status rs = run_solve(h, jac, var, G, tol, maxit, use_graph, true, &ms, f32, carry, tol_in);
+  const cg_status rs = run_solve(h, jac, var, G, teams, tol, maxit, use_graph, true, &ms, f32, carry, tol_in);
   if (rs != CG_OK) return rs;
   CGB_CUDA(h, cudaMemcpyAsync(B->host_iters.data(), B->k, sizeof(int) * ns, cudaMemcpyDeviceToHost, h->stream));
   CGB_CUDA(h, cudaMemcpyAsync(B->host_restarts.data(), B->restarts, sizeof(int) * ns, cudaMemcpyDeviceToHost, h->stream));
