@@ -58,6 +58,47 @@ __device__ __forceinline__ int thread_row_limit(int len) {
   return __popc(wide) > kWideRows ? kThreadRowWide : kThreadRow;
 }
 
+// The bounds of a row block: its positions [r0, r1) and entries [k0, k1).
+struct BlockSpan {
+  int r0, r1, k0, k1;
+};
+__device__ __forceinline__ BlockSpan block_span(const int32_t* __restrict__ rb, const int32_t* __restrict__ rptr, int b) {
+  BlockSpan s;
+  s.r0 = __ldg(rb + b);
+  s.r1 = __ldg(rb + b + 1);
+  s.k0 = __ldg(rptr + s.r0);
+  s.k1 = __ldg(rptr + s.r1);
+  return s;
+}
+
+// The sum of a row's len staged entries from a, in storage order, by one thread; every
+// lane of the warp takes wlen steps, keeping its sum past its own row's end.
+__device__ __forceinline__ double row_chain(const double* __restrict__ x, const int* s_col, const double* s_val, int a,
+                                            int len, int wlen) {
+  double s = 0.0;
+  int k = 0;
+  for (; k + kRowUnroll <= wlen; k += kRowUnroll) {  // kRowUnroll gathers in flight together
+    double xv[kRowUnroll], vv[kRowUnroll];
+#pragma unroll
+    for (int u = 0; u < kRowUnroll; ++u) {
+      const bool in = k + u < len;
+      vv[u] = in ? s_val[a + k + u] : 0.0;
+      xv[u] = in ? __ldg(x + s_col[a + k + u]) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < kRowUnroll; ++u) {
+      const double nx = fma(vv[u], xv[u], s);
+      s = k + u < len ? nx : s;
+    }
+  }
+  for (; k < wlen; ++k) {
+    const bool in = k < len;
+    const double nx = fma(in ? s_val[a + k] : 0.0, in ? __ldg(x + s_col[a + k]) : 0.0, s);
+    s = in ? nx : s;
+  }
+  return s;
+}
+
 // One row block of y = A x with one fused multiply-add per nonzero (header
 // comment).  The block's column indices and values are copied with 16-byte
 // loads into s_col / s_val at their offset from the window start a0.  Rows of
@@ -67,10 +108,10 @@ __device__ __forceinline__ int thread_row_limit(int len) {
 // (lanes stride over the row, a fixed xor tree joins them), so one long row
 // does not hold a warp of short ones.
 __device__ __forceinline__ void spmv_rowblock_fma(const Csr<double>& A, const double* __restrict__ x,
-                                                  double* __restrict__ y, int b, int* s_col, double* s_val,
-                                                  int* s_med, int* s_nmed) {
-  const int r0 = __ldg(A.rb + b), r1 = __ldg(A.rb + b + 1);
-  const int k0 = __ldg(A.rowptr + r0), k1 = __ldg(A.rowptr + r1);
+                                                  double* __restrict__ y, const BlockSpan& B, int bn,
+                                                  BlockSpan& next, int* s_col, double* s_val, int* s_med,
+                                                  int* s_sort) {
+  const int r0 = B.r0, r1 = B.r1, k0 = B.k0, k1 = B.k1;
   const int t = threadIdx.x;
   if (k1 - k0 > kCapV) {  // long row (r1 == r0 + 1 by construction): strided FMA, fixed tree
     double acc = 0.0;
@@ -78,11 +119,11 @@ __device__ __forceinline__ void spmv_rowblock_fma(const Csr<double>& A, const do
     double v[1] = {acc};
     block_sum<1>(v);
     if (t == 0) y[r0] = v[0];
+    if (bn < A.nrb) next = block_span(A.rb, A.rowptr, bn);
     return;
   }
   const int a0 = A.vec ? (k0 & ~3) : k0;
   const int nq = (k1 - a0 + 3) >> 2;
-  if (t == 0) *s_nmed = 0;
   int4 c4[kQuadPasses];
   double2 va[kQuadPasses], vb[kQuadPasses];
 #pragma unroll
@@ -119,58 +160,100 @@ __device__ __forceinline__ void spmv_rowblock_fma(const Csr<double>& A, const do
       *reinterpret_cast<double2*>(s_val + 4 * qd + 2) = vb[j];
     }
   }
-  __syncthreads();
-  const int i = r0 + t;
+  const int i = r0 + t, nrows = r1 - r0;
   int a = 0, len = 0;
   if (i < r1) {
     a = __ldg(A.rowptr + i) - a0;
     len = __ldg(A.rowptr + i + 1) - a0 - a;
   }
-  if (len > thread_row_limit(len)) {
-    s_med[atomicAdd(s_nmed, 1)] = i;  // a warp sums it below (the order of the list does not matter)
-    len = -1;
+  const bool med = len > thread_row_limit(len);
+  // few rows of many entries (27-point stencils: 75 a block): two threads a row below
+  const bool halves = 2 * nrows <= kBlock && k1 - k0 > kThreadRow * nrows;
+  if (halves && i < r1) s_med[t] = (a << 12) | len;
+  // the steps this warp's FMA chain would take beyond what its rows hold
+  const int mine = med ? 0 : len;
+  const int steps = __reduce_max_sync(0xffffffffu, mine), held = __reduce_add_sync(0xffffffffu, mine);
+  const int live = __popc(__ballot_sync(0xffffffffu, i < r1 && !med));
+  const bool uneven = __syncthreads_or(med || 4 * held < 3 * live * steps) != 0;
+  if (bn < A.nrb) next = block_span(A.rb, A.rowptr, bn);
+  if (uneven) {
+    // Rows of mixed lengths: a warp of 32 consecutive ones runs to its longest (GB300
+    // issues an fp64 warp instruction in full whatever its active lanes: ~14 steps a
+    // warp where the rows of a power-law graph average 6, two thirds of the kernel's
+    // time on the fp64 pipe), so the block's rows are sorted by length first (counting
+    // sort, 32 keys).  Which thread sums a row does not change its sum.
+    const int lane = t & 31;
+    const int key = i < r1 ? (med ? 0 : 31 - min(len, 30)) : 31;
+    const unsigned same = __match_any_sync(0xffffffffu, i < r1 ? key : 32);  // one atomic a key and warp
+    const int lead = __ffs(same) - 1;
+    int rank = 0;
+    if (lane == lead && i < r1) rank = atomicAdd(s_sort + key, __popc(same));
+    rank = __shfl_sync(0xffffffffu, rank, lead) + __popc(same & ((1u << lane) - 1u));
+    __syncthreads();  // the counts, and the staged entries
+    const int cnt = s_sort[lane];
+    int before = cnt;  // rows of smaller keys
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, before, o);
+      if (lane >= o) before += v;
+    }
+    before -= cnt;
+    const int nmed = __shfl_sync(0xffffffffu, cnt, 0);
+    const int pos = __shfl_sync(0xffffffffu, before, key) + rank;
+    if (i < r1) s_med[pos] = (a << 20) | (len << 8) | t;  // a < 2^12, len < 2^12, t < 2^8
+    __syncthreads();
+    if (t < 32) s_sort[t] = 0;  // for the next block
+    // the long rows by eight lanes each (strided, fixed tree), 32 at a time
+    for (int m = t >> 3; m < (nmed + 3) / 4 * 4; m += kBlock / 8) {
+      const int e = m < nmed ? s_med[m] : 0;
+      const int am = (unsigned)e >> 20, lm = (e >> 8) & 0xFFF;
+      double acc = 0.0;
+      for (int k = t & 7; k < lm; k += 8) acc = fma(s_val[am + k], __ldg(x + s_col[am + k]), acc);
+#pragma unroll
+      for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if ((t & 7) == 0 && m < nmed) y[r0 + (e & 0xFF)] = acc;
+    }
+    const int at = nmed + t;
+    const int e = at < nrows ? s_med[at] : 0;
+    a = (unsigned)e >> 20;
+    len = (e >> 8) & 0xFFF;
+    const int wlen = __reduce_max_sync(0xffffffffu, len);
+    const double s = row_chain(x, s_col, s_val, a, len, wlen);
+    if (at < nrows) y[r0 + (e & 0xFF)] = s;
+    __syncthreads();  // s_col / s_val / s_med are reused by the next row block
+    return;
   }
-  // one row a thread; the warp's FMA chain runs to its longest row (GB300 issues
-  // an fp64 warp instruction in full whatever its active lanes), each lane keeping
+  if (halves) {
+    // two threads a row, each the chain of half its entries: with one, 75 of 256 threads
+    // worked, each through 27 dependent steps
+    const int r = t >> 1;
+    const int e = r < nrows ? s_med[r] : 0;
+    const int el = e & 0xFFF, h = (el + 1) >> 1;
+    const int ea = ((unsigned)e >> 12) + ((t & 1) ? h : 0), en = (t & 1) ? el - h : h;
+    double s = row_chain(x, s_col, s_val, ea, en, __reduce_max_sync(0xffffffffu, en));
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    if (!(t & 1) && r < nrows) y[r0 + r] = s;
+    __syncthreads();  // s_col / s_val / s_med are reused by the next row block
+    return;
+  }
+  // one row a thread; the warp's FMA chain runs to its longest row, each lane keeping
   // its sum past its own row's end
-  const int wlen = __reduce_max_sync(0xffffffffu, len);
-  if (i < r1 && len >= 0) {
-    double s = 0.0;
-    int k = 0;
-    for (; k + kRowUnroll <= wlen; k += kRowUnroll) {  // kRowUnroll gathers in flight together
-      double xv[kRowUnroll], vv[kRowUnroll];
-#pragma unroll
-      for (int u = 0; u < kRowUnroll; ++u) {
-        const bool in = k + u < len;
-        vv[u] = in ? s_val[a + k + u] : 0.0;
-        xv[u] = in ? __ldg(x + s_col[a + k + u]) : 0.0;
-      }
-#pragma unroll
-      for (int u = 0; u < kRowUnroll; ++u) {
-        const double nx = fma(vv[u], xv[u], s);
-        s = k + u < len ? nx : s;
-      }
-    }
-    for (; k < wlen; ++k) {
-      const bool in = k < len;
-      const double nx = fma(in ? s_val[a + k] : 0.0, in ? __ldg(x + s_col[a + k]) : 0.0, s);
-      s = in ? nx : s;
-    }
-    y[i] = s;
-  }
+  const double s = row_chain(x, s_col, s_val, a, len, steps);
+  if (i < r1) y[i] = s;
+  __syncthreads();  // s_col / s_val are reused by the next row block
+}
+
+// Row blocks cta, cta + stride, ... of y = A x by one CTA (static shared memory of the caller).
+__device__ __forceinline__ void spmv_rowblocks(const Csr<double>& A, const double* x, double* y, int cta, int stride,
+                                               int* s_col, double* s_val, int* s_med, int* s_sort) {
+  if (threadIdx.x < 32) s_sort[threadIdx.x] = 0;
   __syncthreads();
-  const int nmed = *s_nmed;
-  const int lane = t & 31;
-  for (int m = t >> 5; m < nmed; m += kWarps) {
-    const int row = s_med[m];
-    const int a = __ldg(A.rowptr + row) - a0, e = __ldg(A.rowptr + row + 1) - a0;
-    double acc = 0.0;
-    for (int k = a + lane; k < e; k += 32) acc = fma(s_val[k], __ldg(x + s_col[k]), acc);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) y[row] = acc;
+  BlockSpan B{0, 0, 0, 0}, next{0, 0, 0, 0};
+  if (cta < A.nrb) B = block_span(A.rb, A.rowptr, cta);
+  for (int b = cta; b < A.nrb; b += stride) {
+    spmv_rowblock_fma(A, x, y, B, b + stride, next, s_col, s_val, s_med, s_sort);
+    B = next;
   }
-  __syncthreads();  // s_col / s_val / s_med are reused by the next row block
 }
 
 // Stand-alone y = A x over all row blocks (cg_spmv, the graph form's residuals);
@@ -182,8 +265,8 @@ __global__ void __launch_bounds__(kBlock, 6) spmv_kernel(Csr<T> A, const T* x, T
   __shared__ __align__(16) int s_col[kCap];
   __shared__ __align__(16) double s_val[kCap];
   __shared__ int s_med[kBlock];
-  __shared__ int s_nmed;
-  for (int b = blockIdx.x; b < A.nrb; b += gridDim.x) spmv_rowblock_fma(A, x, y, b, s_col, s_val, s_med, &s_nmed);
+  __shared__ int s_sort[32];
+  spmv_rowblocks(A, x, y, (int)blockIdx.x, (int)gridDim.x, s_col, s_val, s_med, s_sort);
 }
 
 }  // namespace cg

@@ -472,7 +472,7 @@ __device__ __forceinline__ double spmv_phase_dia(const Sell<T>& S, const T* __re
 // The CSR loop layout (matrices whose rows are too uneven for slices): one row
 // block of q = A^ p, staged as the caller-CSR SpMV stages it (16-byte loads of
 // columns and values into shared memory), rows of at most kThreadRow entries by
-// a thread, longer ones by a warp, a row beyond the block cap by the CTA; the
+// a thread, longer ones by eight lanes, a row beyond the block cap by the CTA; the
 // diagonal term starts each row's sum; the row's p_i q_i goes to dot.
 template <typename T> struct Quad;
 template <> struct Quad<double> {
@@ -498,13 +498,14 @@ template <> struct Quad<float> {
 
 constexpr int kRowStep = 4;  // a row's gathers in flight together in the CSR loop layout
 
+// `next` gets the bounds of block bn (if below S.nrb), read while this block is summed.
 template <typename T, bool JAC>
-__device__ __forceinline__ void loop_rowblock(const Sell<T>& S, const T* __restrict__ p, T* __restrict__ q, int b,
-                                              int* s_col, T* s_val, int* s_med, int* s_nmed, Acc<T>& dot) {
-  // positions [r0, r1) of block b; position ps holds row S.perm[ps] (the rows of a
+__device__ __forceinline__ void loop_rowblock(const Sell<T>& S, const T* __restrict__ p, T* __restrict__ q,
+                                              const BlockSpan& B, int bn, BlockSpan& next, int* s_col, T* s_val,
+                                              int2* s_row, Acc<T>& dot) {
+  // positions [r0, r1) of the block; position ps holds row S.perm[ps] (the rows of a
   // block sorted by descending length) with entries at [rptr[ps], rptr[ps+1])
-  const int r0 = __ldg(S.rb + b), r1 = __ldg(S.rb + b + 1);
-  const int k0 = __ldg(S.rptr + r0), k1 = __ldg(S.rptr + r1);
+  const int r0 = B.r0, r1 = B.r1, k0 = B.k0, k1 = B.k1;
   const int t = threadIdx.x;
   if (k1 - k0 > kCapV) {  // one long row: strided FMA, fixed tree
     double acc = 0.0;
@@ -518,11 +519,18 @@ __device__ __forceinline__ void loop_rowblock(const Sell<T>& S, const T* __restr
       q[i] = qi;
       dot.add(pi, qi);
     }
+    if (bn < S.nrb) next = block_span(S.rb, S.rptr, bn);
     return;
   }
   const int a0 = k0 & ~3;  // the loop arrays start on 256-byte boundaries
   const int nq = (k1 - a0 + 3) >> 2;
-  if (t == 0) *s_nmed = 0;
+  const int ps = r0 + t;
+  int len = 0;
+  if (ps < r1) {
+    const int a = __ldg(S.rptr + ps) - a0;
+    len = __ldg(S.rptr + ps + 1) - a0 - a;
+    s_row[t] = make_int2((a << 12) | len, __ldg(S.perm + ps));  // a, len < 2^12
+  }
 #pragma unroll
   for (int j = 0; j < kQuadPasses; ++j) {
     const int qd = t + j * kBlock;
@@ -545,25 +553,34 @@ __device__ __forceinline__ void loop_rowblock(const Sell<T>& S, const T* __restr
     *reinterpret_cast<int4*>(s_col + 4 * qd) = make_int4(c[0], c[1], c[2], c[3]);
     Quad<T>::store(s_val + 4 * qd, v);
   }
-  __syncthreads();
-  const int ps = r0 + t;
-  int a = 0, len = 0, i = 0;
-  if (ps < r1) {
-    a = __ldg(S.rptr + ps) - a0;
-    len = __ldg(S.rptr + ps + 1) - a0 - a;
-    i = __ldg(S.perm + ps);
+  // (the barrier after the staging also counts the long rows, the block's first)
+  const int nmed = __syncthreads_count(len > kThreadRow);
+  if (bn < S.nrb) next = block_span(S.rb, S.rptr, bn);
+  // long rows by eight lanes each (strided, fixed tree), 32 rows at a time: a warp per
+  // row held the block for a chain of loads and a 5-level fp64 tree per row
+  for (int m = t >> 3; m < (nmed + 3) / 4 * 4; m += kBlock / 8) {
+    const int2 e = m < nmed ? s_row[m] : make_int2(0, 0);
+    const int am = (unsigned)e.x >> 12, lm = e.x & 0xFFF;
+    T acc = T(0);
+    for (int k = t & 7; k < lm; k += 8) acc = fma(s_val[am + k], p[s_col[am + k]], acc);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((t & 7) == 0 && m < nmed) {
+      const T pi = p[e.y];
+      const T qi = (JAC ? pi : __ldg(S.dg + e.y) * pi) + acc;
+      q[e.y] = qi;
+      dot.add(pi, qi);
+    }
   }
-  // (the rows of a block are sorted by length, so the first warps hold the long
-  // ones: those are shared out among all warps instead of kept by one)
-  if (len > kThreadRow) {
-    s_med[atomicAdd(s_nmed, 1)] = ps;
-    len = -1;
-  }
-  // a warp's rows, one a thread: the FMA chain runs to the warp's longest row
-  // (one fp64 warp instruction per step), each lane keeping its sum past its
-  // own row's end
+  // a warp's other rows, one a thread: the FMA chain runs to the warp's longest row
+  // (one fp64 warp instruction per step), each lane keeping its sum past its own
+  // row's end
+  const bool mine = nmed + t < r1 - r0;
+  const int2 e = mine ? s_row[nmed + t] : make_int2(0, 0);
+  const int a = (unsigned)e.x >> 12, i = e.y;
+  len = e.x & 0xFFF;
   const int wlen = __reduce_max_sync(0xffffffffu, len);
-  if (len >= 0 && ps < r1) {
+  if (mine) {
     const T pi = p[i];
     T acc = JAC ? pi : __ldg(S.dg + i) * pi;
     int k = 0;
@@ -589,24 +606,6 @@ __device__ __forceinline__ void loop_rowblock(const Sell<T>& S, const T* __restr
     q[i] = acc;
     dot.add(pi, acc);
   }
-  __syncthreads();
-  const int nmed = *s_nmed;
-  const int lane = t & 31;
-  for (int m = t >> 5; m < nmed; m += kWarps) {
-    const int pm = s_med[m];
-    const int row = __ldg(S.perm + pm);
-    const int am = __ldg(S.rptr + pm) - a0, em = __ldg(S.rptr + pm + 1) - a0;
-    T acc = T(0);
-    for (int k = am + lane; k < em; k += 32) acc = fma(s_val[k], p[s_col[k]], acc);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) {
-      const T pi = p[row];
-      const T qi = (JAC ? pi : __ldg(S.dg + row) * pi) + acc;
-      q[row] = qi;
-      dot.add(pi, qi);
-    }
-  }
   __syncthreads();  // the staging buffers are reused by the next row block
 }
 
@@ -615,10 +614,14 @@ __device__ __forceinline__ double spmv_phase_csr(const Sell<T>& S, const T* __re
                                                  const Grid& g) {
   __shared__ __align__(16) int s_col[kCap];
   __shared__ __align__(16) T s_val[kCap];
-  __shared__ int s_med[kBlock];
-  __shared__ int s_nmed;
+  __shared__ int2 s_row[kBlock];
   Acc<T> dot;
-  for (int b = (int)g.cta; b < S.nrb; b += (int)g.G) loop_rowblock<T, JAC>(S, p, q, b, s_col, s_val, s_med, &s_nmed, dot);
+  BlockSpan B{0, 0, 0, 0}, next{0, 0, 0, 0};
+  if ((int)g.cta < S.nrb) B = block_span(S.rb, S.rptr, (int)g.cta);
+  for (int b = (int)g.cta; b < S.nrb; b += (int)g.G) {
+    loop_rowblock<T, JAC>(S, p, q, B, b + (int)g.G, next, s_col, s_val, s_row, dot);
+    B = next;
+  }
   return dot.get();
 }
 
@@ -934,8 +937,8 @@ __device__ __forceinline__ void spmv_orig(const Csr<double>& A, const double* x,
   __shared__ __align__(16) int s_col[kCap];
   __shared__ __align__(16) double s_val[kCap];
   __shared__ int s_med[kBlock];
-  __shared__ int s_nmed;
-  for (int b = (int)g.cta; b < A.nrb; b += (int)g.G) spmv_rowblock_fma(A, x, q, b, s_col, s_val, s_med, &s_nmed);
+  __shared__ int s_sort[32];
+  spmv_rowblocks(A, x, q, (int)g.cta, (int)g.G, s_col, s_val, s_med, s_sort);
 }
 
 // fp64 (Jacobi-)PCG with true-residual check and residual-replacement
