@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -27,27 +28,164 @@ void cgi::set_create_error(const std::string& msg) { g_create_error = msg; }
 
 namespace {
 
-// Device checks of a CSR whose rowptr the host has already validated:
-// colind in [0, n); per row the diagonal sum A_ii and the number of stored
-// diagonal entries; counters[1] counts rows without a positive diagonal.
-__global__ void validate_kernel(int64_t n, const int32_t* __restrict__ rowptr,
-                                const int32_t* __restrict__ colind, const double* __restrict__ vals,
-                                double* diag, int32_t* ndiag, unsigned long long* counters) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
+// ---- creation: the caller's CSR is checked and cut into row blocks on the device
+// (copying the row pointers to the host and walking them there, with a synchronisation
+// and an allocation per step, took most of a 912,673-row handle's 1.7 ms)
+
+struct SetupWords {
+  unsigned long long bad_row;        // smallest row whose pointers decrease (all ones: none)
+  unsigned long long bad_col;        // entries with a column outside [0, n)
+  unsigned long long bad_diag;       // rows without a positive diagonal
+  unsigned long long ndiag;          // stored diagonal entries
+  unsigned long long dmin, dmax;     // range of a positive diagonal: its IEEE bits order like its values
+  unsigned long long nlong;          // rows of more than kCapV entries
+  int first, nnz;                    // rowptr[0], rowptr[n]
+  int nrb;                           // row blocks
+  int pad;
+};
+
+__global__ void rowptr_check_kernel(int64_t n, const int32_t* __restrict__ rowptr, SetupWords* w) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    if (rowptr[i + 1] < rowptr[i]) atomicMin(&w->bad_row, (unsigned long long)i);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    w->first = rowptr[0];
+    w->nnz = rowptr[n];
+  }
+}
+
+__device__ __forceinline__ unsigned long long warp_min(unsigned long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long u = __shfl_xor_sync(0xffffffffu, v, o);
+    v = u < v ? u : v;
+  }
+  return v;
+}
+
+// Checks of a CSR whose rowptr has been checked: colind in [0, n); per row the
+// diagonal sum A_ii and the number of stored diagonal entries; the counts and the
+// diagonal's range, one set of atomics a block (an atomic a thread for the range
+// alone had taken 340 us).
+__global__ void __launch_bounds__(256) validate_kernel(int64_t n, const int32_t* __restrict__ rowptr,
+                                                       const int32_t* __restrict__ colind,
+                                                       const double* __restrict__ vals, double* diag, int32_t* ndiag,
+                                                       SetupWords* w) {
+  __shared__ unsigned long long s_lo[8], s_hi[8];
+  __shared__ unsigned s_n[3];
+  const int t = threadIdx.x;
+  if (t < 3) s_n[t] = 0u;
+  __syncthreads();
+  unsigned bad = 0, nopos = 0, nd = 0;
+  unsigned long long lo = ~0ull, hi = 0ull;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + t; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int a = rowptr[i], e = rowptr[i + 1];
     double d = 0.0;
     int found = 0;
-    unsigned long long bad = 0;
     for (int k = a; k < e; ++k) {
       const int c = colind[k];
       if (c < 0 || (int64_t)c >= n) { ++bad; continue; }
       if ((int64_t)c == i) { d += vals[k]; ++found; }
     }
-    if (bad) atomicAdd(&counters[0], bad);
     diag[i] = d;
     ndiag[i] = found;
-    if (!(found && d > 0.0)) atomicAdd(&counters[1], 1ull);
+    nd += (unsigned)found;
+    if (found && d > 0.0) {
+      const unsigned long long b = (unsigned long long)__double_as_longlong(d);
+      lo = b < lo ? b : lo;
+      hi = b > hi ? b : hi;
+    } else {
+      ++nopos;
+    }
+  }
+  if (bad) atomicAdd(&s_n[0], bad);
+  if (nopos) atomicAdd(&s_n[1], nopos);
+  const unsigned wnd = __reduce_add_sync(0xffffffffu, nd);
+  lo = warp_min(lo);
+  hi = ~warp_min(~hi);
+  if ((t & 31) == 0) {
+    if (wnd) atomicAdd(&s_n[2], wnd);
+    s_lo[t >> 5] = lo;
+    s_hi[t >> 5] = hi;
+  }
+  __syncthreads();
+  if (t == 0) {
+    for (int k = 1; k < 8; ++k) {
+      lo = s_lo[k] < lo ? s_lo[k] : lo;
+      hi = s_hi[k] > hi ? s_hi[k] : hi;
+    }
+    if (s_n[0]) atomicAdd(&w->bad_col, (unsigned long long)s_n[0]);
+    if (s_n[1]) atomicAdd(&w->bad_diag, (unsigned long long)s_n[1]);
+    atomicAdd(&w->ndiag, (unsigned long long)s_n[2]);
+    atomicMin(&w->dmin, lo);
+    atomicMax(&w->dmax, hi);
+  }
+}
+
+// Row blocks: greedily as many rows as stay within kCapV entries and kBlock rows, a row
+// of more than kCapV entries alone; the cut starts anew every kCutRows rows, so that a
+// thread cuts each stretch (a few per cent more blocks than one cut of all rows).
+constexpr int kCutRows = 1024;
+
+// The end of the block that starts at row r of a stretch that ends at row e.
+__device__ __forceinline__ int64_t block_end(const int32_t* __restrict__ rowptr, int64_t r, int64_t e) {
+  const int base = rowptr[r];
+  if (rowptr[r + 1] - base > kCapV) return r + 1;
+  int64_t hi = r + kBlock < e ? r + kBlock : e;
+  if (rowptr[hi] - base <= kCapV) return hi;
+  int64_t lo = r + 1;  // rowptr[lo] - base <= kCapV < rowptr[hi] - base
+  while (lo + 1 < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (rowptr[mid] - base <= kCapV) lo = mid;
+    else hi = mid;
+  }
+  return lo;
+}
+
+// WRITE = false: counts[c] = blocks of stretch c; true: their first rows from offset counts[c].
+template <bool WRITE>
+__global__ void cut_kernel(int64_t n, const int32_t* __restrict__ rowptr, int* counts, int32_t* rb, SetupWords* w) {
+  const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (c * kCutRows >= n) return;
+  const int64_t e = (c + 1) * kCutRows < n ? (c + 1) * kCutRows : n;
+  int m = 0;
+  unsigned long long longs = 0;
+  const int off = WRITE ? counts[c] : 0;
+  for (int64_t r = c * kCutRows; r < e; ++m) {
+    if (WRITE) rb[off + m] = (int32_t)r;
+    else if (rowptr[r + 1] - rowptr[r] > kCapV) ++longs;
+    r = block_end(rowptr, r, e);
+  }
+  if (!WRITE) {
+    counts[c] = m;
+    if (longs) atomicAdd(&w->nlong, longs);
+  }
+}
+
+// counts to offsets (one block); the total to w->nrb and rb's end.
+__global__ void __launch_bounds__(1024) cut_scan_kernel(int64_t nc, int64_t n, int* counts, int32_t* rb, SetupWords* w) {
+  __shared__ int s_warp[32];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int64_t per = (nc + 1023) / 1024, c0 = min((int64_t)t * per, nc), c1 = min(c0 + per, nc);
+  int sum = 0;
+  for (int64_t c = c0; c < c1; ++c) sum += counts[c];
+  int inc = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
+  }
+  if (lane == 31) s_warp[warp] = inc;
+  __syncthreads();
+  int base = inc - sum;
+  for (int k = 0; k < warp; ++k) base += s_warp[k];
+  for (int64_t c = c0; c < c1; ++c) {
+    const int v = counts[c];
+    counts[c] = base;
+    base += v;
+  }
+  if (t == 1023) {
+    w->nrb = base;
+    rb[base] = (int32_t)n;
   }
 }
 
@@ -128,20 +266,6 @@ __global__ void fill_csr_kernel(int64_t n, const int32_t* __restrict__ rowptr, c
   }
 }
 
-// Range of a positive diagonal: min / max of the IEEE bit patterns, which
-// order like the values for positive doubles.
-__global__ void diag_range_kernel(int64_t n, const double* __restrict__ d, unsigned long long* mm) {
-  unsigned long long lo = ~0ull, hi = 0ull;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(d[i]);
-    lo = b < lo ? b : lo;
-    hi = b > hi ? b : hi;
-  }
-  atomicMin(&mm[0], lo);
-  atomicMax(&mm[1], hi);
-}
-
 // Distinct off-diagonal offsets j - i into a 64-slot open-addressing table
 // (kOffEmpty marks a free slot); *overflow is set when they do not fit.
 constexpr int kOffSlots = 64;
@@ -172,23 +296,46 @@ __global__ void offsets_kernel(int64_t n, const int32_t* __restrict__ rowptr,
 // Sliced-diagonal values (thread per row): slot m of row i holds the sum of
 // the row's entries in column i + delta[m] (0 where there is none); with
 // SCALE the Jacobi scaling A_ij / sqrt(A_ii A_jj).  The array is zeroed
-// before, so lanes past n stay 0.
-template <typename T, bool SCALE>
+// before, so lanes past n stay 0.  ND > 0: at most ND diagonals, the row's entries
+// read once and its slots kept in registers.
+struct DiaOffsets {
+  int32_t d[kMaxDiag];
+};
+template <typename T, bool SCALE, int ND>
 __global__ void fill_dia_kernel(int64_t n, const int32_t* __restrict__ rowptr,
                                 const int32_t* __restrict__ colind,
                                 const double* __restrict__ vals,
                                 const double* __restrict__ disq, int ndiag,
-                                const int32_t* __restrict__ delta, T* val) {
+                                DiaOffsets delta, T* val) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t base = (i >> 5) * ndiag * 32 + (i & 31);
     const double si = SCALE ? disq[i] : 1.0;
-    for (int m = 0; m < ndiag; ++m) {
-      const int64_t target = i + delta[m];
-      double v = 0.0;
-      for (int k = rowptr[i]; k < rowptr[i + 1]; ++k)
-        if ((int64_t)colind[k] == target) v += SCALE ? vals[k] * (si * disq[target]) : vals[k];
-      val[base + (int64_t)m * 32] = (T)v;
+    const int a = rowptr[i], e = rowptr[i + 1];
+    if constexpr (ND > 0) {
+      double v[ND];
+#pragma unroll
+      for (int m = 0; m < ND; ++m) v[m] = 0.0;
+      for (int k = a; k < e; ++k) {
+        const int c = colind[k];
+        const int o = c - (int)i;
+        if (o == 0) continue;
+        const double x = SCALE ? vals[k] * (si * disq[c]) : vals[k];
+#pragma unroll
+        for (int m = 0; m < ND; ++m)
+          if (m < ndiag && delta.d[m] == o) v[m] += x;
+      }
+#pragma unroll
+      for (int m = 0; m < ND; ++m)
+        if (m < ndiag) val[base + (int64_t)m * 32] = (T)v[m];
+    } else {
+      for (int m = 0; m < ndiag; ++m) {
+        const int64_t target = i + delta.d[m];
+        double v = 0.0;
+        for (int k = a; k < e; ++k)
+          if ((int64_t)colind[k] == target) v += SCALE ? vals[k] * (si * disq[target]) : vals[k];
+        val[base + (int64_t)m * 32] = (T)v;
+      }
     }
   }
 }
@@ -280,6 +427,33 @@ int max_coresident(K kernel, int sm_count) {
   return per_sm * sm_count;
 }
 
+// Co-resident CTAs of the persistent kernels (the smallest over the kernels we may
+// launch) and CTAs of the graph form's vector kernels: facts of the device, asked once.
+void residency(int dev, int sm_count, int* persistent, int* vectors) {
+  constexpr int kMaxDevices = 64;
+  static std::mutex mu;
+  static int known[kMaxDevices][2];
+  std::lock_guard<std::mutex> lock(mu);
+  int* k = known[dev < 0 || dev >= kMaxDevices ? 0 : dev];
+  if (k[0] <= 0 || k[1] <= 0 || dev < 0 || dev >= kMaxDevices) {
+    int g = kXCtas;
+    for (int r : {max_coresident(pcg64_kernel<true>, sm_count), max_coresident(pcg64_kernel<false>, sm_count),
+                  max_coresident(pcg_ir_kernel<true, false>, sm_count), max_coresident(pcg_ir_kernel<true, true>, sm_count),
+                  max_coresident(pcg_ir_kernel<false, false>, sm_count),
+                  max_coresident(pcg_ir_kernel<false, true>, sm_count)})
+      g = std::min(g, r);
+    int v = max_coresident(g_res64<true>, sm_count);
+    for (int r : {max_coresident(g_upd_r<double, true>, sm_count), max_coresident(g_upd_r<double, false>, sm_count),
+                  max_coresident(g_upd_xp<float, true, true, true>, sm_count),
+                  max_coresident(g_upd_xp<double, true, false, true>, sm_count)})
+      v = std::min(v, r);
+    k[0] = g;
+    k[1] = v;
+  }
+  *persistent = k[0];
+  *vectors = k[1];
+}
+
 // Loop-matrix bytes beyond the entries read once per SpMV: the row of each
 // slice position (SELL-C-sigma) or the row pointers (CSR layout).
 int64_t loop_index_bytes(const cg_handle* h) {
@@ -312,6 +486,15 @@ int auto_grid(const cg_handle* h) {
 
 }  // namespace
 
+// The row pointers on the host, for the layouts and splits made there.
+cg_status cgi::ensure_host_rowptr(cg_handle* h) {
+  if (!h->host_rowptr.empty()) return CG_OK;
+  std::vector<int32_t> rp((size_t)h->n + 1);
+  CG_CUDA(h, cudaMemcpy(rp.data(), h->rowptr, sizeof(int32_t) * rp.size(), cudaMemcpyDeviceToHost));
+  h->host_rowptr = std::move(rp);
+  return CG_OK;
+}
+
 // Every distinct off-diagonal offset j - i of the caller's CSR, once per
 // handle (device table of kOffSlots slots; noffs_all = -1 when they do not fit).
 cg_status cgi::ensure_offsets(cg_handle* h) {
@@ -343,56 +526,57 @@ cg_status cgi::ensure_offsets(cg_handle* h) {
 
 namespace {
 
+// Elements of an n-vector's place in a shared allocation (whole 256 bytes of fp32).
+size_t padded(int64_t n) { return ((size_t)std::max<int64_t>(n, 1) + 63) / 64 * 64; }
+
+// sqrt(A_ii), 1/sqrt(A_ii) and the fp32 copies: one allocation, last step of the layout.
+cg_status ensure_diag_vectors(cg_handle* h) {
+  const size_t nv = padded(h->n);
+  double* base = nullptr;
+  CG_CUDA(h, cudaMalloc(&base, (2 * sizeof(double) + 2 * sizeof(float)) * nv));
+  h->dsq = base;
+  h->disq = base + nv;
+  h->diag32 = reinterpret_cast<float*>(base + 2 * nv);
+  h->disq32 = h->diag32 + nv;
+  if (h->n > 0) {
+    diag_kernel<<<grid_for(h->n), 256>>>(h->n, h->diag, h->dsq, h->disq, h->diag32, h->disq32);
+    CG_CUDA(h, cudaGetLastError());
+    CG_CUDA(h, cudaDeviceSynchronize());
+  }
+  return CG_OK;
+}
+
 // SELL-32 structure of the off-diagonal part (shared by every value
 // variant) and the diagonal vectors.
 cg_status ensure_offdiag(cg_handle* h) {
-  if (h->soff) return CG_OK;
+  if (h->disq) return CG_OK;
   const int64_t n = h->n;
-  std::vector<int32_t> nd((size_t)n);
-  if (n > 0) CG_CUDA(h, cudaMemcpy(nd.data(), h->ndiag, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost));
-  const std::vector<int32_t>& rp = h->host_rowptr;
   const int64_t ns = (n + 31) / 32;
   // sliced-diagonal layout when the off-diagonal part lies on <= kMaxDiag
   // diagonals that are at least 90 % full
-  int64_t nnz_od_all = 0;
-  for (int64_t i = 0; i < n; ++i) nnz_od_all += rp[(size_t)i + 1] - rp[(size_t)i] - nd[(size_t)i];
+  const int64_t nnz_od_all = h->nnz - h->ndiag_all;
   if (n > 0 && nnz_od_all > 0) {
     const cg_status so = cgi::ensure_offsets(h);
     if (so != CG_OK) return so;
     const int nd_ = std::max(h->noffs_all, 0);
-    const bool fits = h->noffs_all >= 0;
-    std::vector<int32_t> offs(h->offs_all, h->offs_all + nd_);
-    if (fits && nd_ > 0 && nd_ <= kMaxDiag && nnz_od_all * 10 >= (int64_t)nd_ * n * 9) {
+    if (h->noffs_all >= 0 && nd_ > 0 && nd_ <= kMaxDiag && nnz_od_all * 10 >= (int64_t)nd_ * n * 9) {
       h->dia = 1;
       h->uniform_w = nd_;
-      for (int m = 0; m < nd_; ++m) h->delta[m] = offs[(size_t)m];
+      for (int m = 0; m < nd_; ++m) h->delta[m] = h->offs_all[m];
       h->nslices = (int32_t)ns;
       h->sell_entries = ns * 32 * nd_;
       h->nnz_od = nnz_od_all;
       h->nlong = 0;
       h->nnz_long = 0;
-      std::vector<int32_t> soff((size_t)ns + 1);
-      for (int64_t s2 = 0; s2 <= ns; ++s2) soff[(size_t)s2] = (int32_t)(s2 * nd_);
-      std::vector<uint32_t> lmask((size_t)std::max<int64_t>(ns, 1), 0u);
-      CG_CUDA(h, cudaMalloc(&h->soff, sizeof(int32_t) * soff.size()));
-      CG_CUDA(h, cudaMemcpy(h->soff, soff.data(), sizeof(int32_t) * soff.size(), cudaMemcpyHostToDevice));
-      CG_CUDA(h, cudaMalloc(&h->lmask, sizeof(uint32_t) * lmask.size()));
-      CG_CUDA(h, cudaMemcpy(h->lmask, lmask.data(), sizeof(uint32_t) * lmask.size(), cudaMemcpyHostToDevice));
-      CG_CUDA(h, cudaMalloc(&h->delta_dev, sizeof(int32_t) * kMaxDiag));
-      CG_CUDA(h, cudaMemcpy(h->delta_dev, h->delta, sizeof(int32_t) * kMaxDiag, cudaMemcpyHostToDevice));
-      CG_CUDA(h, cudaMalloc(&h->lptr, sizeof(int32_t)));
-      CG_CUDA(h, cudaMemset(h->lptr, 0, sizeof(int32_t)));
-      const size_t nv = (size_t)std::max<int64_t>(n, 1);
-      CG_CUDA(h, cudaMalloc(&h->dsq, sizeof(double) * nv));
-      CG_CUDA(h, cudaMalloc(&h->disq, sizeof(double) * nv));
-      CG_CUDA(h, cudaMalloc(&h->diag32, sizeof(float) * nv));
-      CG_CUDA(h, cudaMalloc(&h->disq32, sizeof(float) * nv));
-      diag_kernel<<<grid_for(n), 256>>>(n, h->diag, h->dsq, h->disq, h->diag32, h->disq32);
-      CG_CUDA(h, cudaGetLastError());
-      CG_CUDA(h, cudaDeviceSynchronize());
-      return CG_OK;
+      return ensure_diag_vectors(h);
     }
   }
+  // the other layouts are laid out on the host
+  const cg_status hr = cgi::ensure_host_rowptr(h);
+  if (hr != CG_OK) return hr;
+  std::vector<int32_t> nd((size_t)n);
+  if (n > 0) CG_CUDA(h, cudaMemcpy(nd.data(), h->ndiag, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToHost));
+  const std::vector<int32_t>& rp = h->host_rowptr;
   std::vector<int32_t> soff((size_t)ns + 1, 0);
   std::vector<uint32_t> lmask((size_t)std::max<int64_t>(ns, 1), 0u);
   std::vector<int32_t> lrow, lptr(1, 0);
@@ -507,7 +691,6 @@ cg_status ensure_offdiag(cg_handle* h) {
     h->nlong = 0;
     h->nnz_long = 0;
     h->lnrb = (int32_t)(lrb.size() - 1);
-    const size_t nv = (size_t)std::max<int64_t>(n, 1);
     CG_CUDA(h, cudaMalloc(&h->lrp, sizeof(int32_t) * lrp.size()));
     CG_CUDA(h, cudaMemcpy(h->lrp, lrp.data(), sizeof(int32_t) * lrp.size(), cudaMemcpyHostToDevice));
     CG_CUDA(h, cudaMalloc(&h->lrb, sizeof(int32_t) * lrb.size()));
@@ -519,14 +702,7 @@ cg_status ensure_offdiag(cg_handle* h) {
     CG_CUDA(h, cudaMalloc(&h->lptr, sizeof(int32_t)));
     CG_CUDA(h, cudaMemset(h->lptr, 0, sizeof(int32_t)));
     CG_CUDA(h, cudaMalloc(&h->lcol, sizeof(int32_t)));
-    CG_CUDA(h, cudaMalloc(&h->dsq, sizeof(double) * nv));
-    CG_CUDA(h, cudaMalloc(&h->disq, sizeof(double) * nv));
-    CG_CUDA(h, cudaMalloc(&h->diag32, sizeof(float) * nv));
-    CG_CUDA(h, cudaMalloc(&h->disq32, sizeof(float) * nv));
-    diag_kernel<<<grid_for(n), 256>>>(n, h->diag, h->dsq, h->disq, h->diag32, h->disq32);
-    CG_CUDA(h, cudaGetLastError());
-    CG_CUDA(h, cudaDeviceSynchronize());
-    return CG_OK;
+    return ensure_diag_vectors(h);
   }
   int64_t off = 0;
   for (int64_t s = 0; s < ns; ++s) {
@@ -545,7 +721,6 @@ cg_status ensure_offdiag(cg_handle* h) {
   h->nnz_od = nnz_od;
   h->nlong = (int32_t)lrow.size();
   h->nnz_long = lptr.back();
-  const size_t nv = (size_t)std::max<int64_t>(n, 1);
   CG_CUDA(h, cudaMalloc(&h->soff, sizeof(int32_t) * soff.size()));
   CG_CUDA(h, cudaMemcpy(h->soff, soff.data(), sizeof(int32_t) * soff.size(), cudaMemcpyHostToDevice));
   CG_CUDA(h, cudaMalloc(&h->lmask, sizeof(uint32_t) * lmask.size()));
@@ -560,16 +735,7 @@ cg_status ensure_offdiag(cg_handle* h) {
   if (!lrow.empty())
     CG_CUDA(h, cudaMemcpy(h->lrow, lrow.data(), sizeof(int32_t) * lrow.size(), cudaMemcpyHostToDevice));
   CG_CUDA(h, cudaMemcpy(h->lptr, lptr.data(), sizeof(int32_t) * lptr.size(), cudaMemcpyHostToDevice));
-  CG_CUDA(h, cudaMalloc(&h->dsq, sizeof(double) * nv));
-  CG_CUDA(h, cudaMalloc(&h->disq, sizeof(double) * nv));
-  CG_CUDA(h, cudaMalloc(&h->diag32, sizeof(float) * nv));
-  CG_CUDA(h, cudaMalloc(&h->disq32, sizeof(float) * nv));
-  if (n > 0) {
-    diag_kernel<<<grid_for(n), 256>>>(n, h->diag, h->dsq, h->disq, h->diag32, h->disq32);
-    CG_CUDA(h, cudaGetLastError());
-    CG_CUDA(h, cudaDeviceSynchronize());
-  }
-  return CG_OK;
+  return ensure_diag_vectors(h);
 }
 
 // Loop-matrix values for (precision, precond), built on first use; the first
@@ -598,12 +764,12 @@ cg_status ensure_vals(cg_handle* h, T** sval, T** lval, bool scale) {
   }
   if (h->dia) {
     CG_CUDA(h, cudaMemset(*sval, 0, sizeof(T) * (size_t)std::max<int64_t>(h->sell_entries, 1)));
-    if (scale)
-      fill_dia_kernel<T, true><<<grid_for(h->n), 256>>>(h->n, h->rowptr, h->colind, h->vals, h->disq,
-                                                        h->uniform_w, h->delta_dev, *sval);
-    else
-      fill_dia_kernel<T, false><<<grid_for(h->n), 256>>>(h->n, h->rowptr, h->colind, h->vals, h->disq,
-                                                         h->uniform_w, h->delta_dev, *sval);
+    DiaOffsets d{};
+    for (int m = 0; m < h->uniform_w; ++m) d.d[m] = h->delta[m];
+    const bool few = h->uniform_w <= 8;
+    auto fill = scale ? (few ? fill_dia_kernel<T, true, 8> : fill_dia_kernel<T, true, 0>)
+                      : (few ? fill_dia_kernel<T, false, 8> : fill_dia_kernel<T, false, 0>);
+    fill<<<grid_for(h->n), 256>>>(h->n, h->rowptr, h->colind, h->vals, h->disq, h->uniform_w, d, *sval);
     CG_CUDA(h, cudaGetLastError());
     CG_CUDA(h, cudaDeviceSynchronize());
     return CG_OK;
@@ -667,11 +833,11 @@ Sell<T> make_sell(const cg_handle* h, const T* val, const T* lval, const T* diag
 template <typename T>
 cg_status ensure_vectors(cg_handle* h, T** r, T** p, T** q, T** xh) {
   if (*r) return CG_OK;
-  const size_t nv = (size_t)std::max<int64_t>(h->n, 1);
-  CG_CUDA(h, cudaMalloc(r, sizeof(T) * nv));
-  CG_CUDA(h, cudaMalloc(p, sizeof(T) * nv));
-  CG_CUDA(h, cudaMalloc(q, sizeof(T) * nv));
-  CG_CUDA(h, cudaMalloc(xh, sizeof(T) * nv));
+  const size_t nv = padded(h->n);
+  CG_CUDA(h, cudaMalloc(r, 4 * sizeof(T) * nv));  // one allocation, at *r
+  *p = *r + nv;
+  *q = *p + nv;
+  *xh = *q + nv;
   return CG_OK;
 }
 
@@ -683,19 +849,15 @@ void destroy_graph(cudaGraphExec_t* e, cudaGraph_t* g) {
 void free_all(cg_handle* h) {
   if (h->batch) cgi::batch_free(h->batch);
   if (h->fsai) cgi::fsai_free(h->fsai);
-  void* dev[] = {h->rb,        h->diag,      h->ndiag,     h->dsq,       h->disq,       h->delta_dev,
-                 h->diag32,    h->disq32,    h->soff,      h->lmask,     h->scol,
-                 h->lrow,      h->lptr,      h->lcol,      h->sval64[0], h->sval64[1],
-                 h->sval32[0], h->sval32[1], h->lval64[0], h->lval64[1], h->lval32[0],
-                 h->lval32[1], h->r,         h->p,         h->q,         h->xh,
-                 h->r32,       h->p32,       h->q32,       h->xh32,      h->part,
-                 h->st,        h->stage_b,   h->stage_x,   h->sperm,     h->spos,
-                 h->lrp,       h->lrb};
+  // (dsq, r, r32 and st head shared allocations; diag32, p, gs and so on lie in them)
+  void* dev[] = {h->rb,        h->diag,      h->ndiag,     h->dsq,       h->soff,      h->lmask,
+                 h->scol,      h->lrow,      h->lptr,      h->lcol,      h->sval64[0], h->sval64[1],
+                 h->sval32[0], h->sval32[1], h->lval64[0], h->lval64[1], h->lval32[0], h->lval32[1],
+                 h->r,         h->r32,       h->part,      h->st,        h->stage_b,   h->stage_x,
+                 h->sperm,     h->spos,      h->lrp,       h->lrb};
   for (void* p : dev)
     if (p) cudaFree(p);
   if (h->host_st) cudaFreeHost(h->host_st);
-  if (h->host_gs) cudaFreeHost(h->host_gs);
-  if (h->gs) cudaFree(h->gs);
   destroy_graph(&h->gexec, &h->graph);
   destroy_graph(&h->gexec_it, &h->graph_it);
   destroy_graph(&h->gexec_ep, &h->graph_ep);
@@ -1064,83 +1226,78 @@ cg_status cg_create(int64_t n, const int32_t* rowptr, const int32_t* colind, con
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return bail(cuda_fail(h, e, "cg_create: device query"));
 
-  // rowptr checks on the host (the row-block cut needs it there anyway)
-  h->host_rowptr.resize((size_t)n + 1);
-  std::vector<int32_t>& hrp = h->host_rowptr;
-  e = cudaMemcpy(hrp.data(), rowptr, sizeof(int32_t) * ((size_t)n + 1), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return bail(cuda_fail(h, e, "cg_create: rowptr copy"));
-  if (hrp[0] != 0) return bail(fail(h, CG_ERR_INVALID, "cg_create: rowptr[0] != 0"));
-  for (int64_t i = 0; i < n; ++i)
-    if (hrp[(size_t)i + 1] < hrp[(size_t)i])
-      return bail(fail(h, CG_ERR_INVALID, "cg_create: rowptr decreases at row " + std::to_string(i)));
-  h->nnz = hrp[(size_t)n];
-  if (h->nnz > 0 && (!colind || !vals))
-    return bail(fail(h, CG_ERR_INVALID, "cg_create: colind/vals NULL with nnz > 0"));
-
-  std::vector<int32_t> rb = build_row_blocks(hrp.data(), n, &h->long_rows);
-  h->nrb = (int32_t)(rb.size() - 1);
-  const size_t nv = (size_t)std::max<int64_t>(n, 1);
-  e = cudaMalloc(&h->rb, sizeof(int32_t) * rb.size());
-  if (e == cudaSuccess) e = cudaMemcpy(h->rb, rb.data(), sizeof(int32_t) * rb.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess) e = cudaMalloc(&h->diag, sizeof(double) * nv);
-  if (e == cudaSuccess) e = cudaMalloc(&h->ndiag, sizeof(int32_t) * nv);
-  if (e == cudaSuccess) e = cudaMalloc(&h->st, kStBytes);
-  if (e == cudaSuccess) e = cudaMallocHost(&h->host_st, sizeof(DevState));
+  // device words (DevState, exchange words, graph state, setup counters) and their
+  // pinned copies: one allocation each
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  const size_t gs_at = up(kStBytes), sw_at = gs_at + up(sizeof(GState));
+  const size_t hgs_at = up(sizeof(DevState)), hsw_at = hgs_at + up(sizeof(GState));
+  e = cudaMalloc((void**)&h->st, sw_at + sizeof(SetupWords));
+  if (e == cudaSuccess) e = cudaMallocHost((void**)&h->host_st, hsw_at + sizeof(SetupWords));
   if (e == cudaSuccess) e = cudaEventCreate(&h->ev0);
   if (e == cudaSuccess) e = cudaEventCreate(&h->ev1);
   if (e != cudaSuccess) return bail(cuda_fail(h, e, "cg_create: allocation"));
+  h->gs = reinterpret_cast<GState*>(reinterpret_cast<char*>(h->st) + gs_at);
+  h->host_gs = reinterpret_cast<GState*>(reinterpret_cast<char*>(h->host_st) + hgs_at);
+  SetupWords* sw = reinterpret_cast<SetupWords*>(reinterpret_cast<char*>(h->st) + sw_at);
+  SetupWords* hw = reinterpret_cast<SetupWords*>(reinterpret_cast<char*>(h->host_st) + hsw_at);
 
-  // colind range and diagonal (device pass)
-  unsigned long long* cnt = nullptr;
-  e = cudaMalloc(&cnt, 2 * sizeof(unsigned long long));
-  if (e == cudaSuccess) e = cudaMemset(cnt, 0, 2 * sizeof(unsigned long long));
-  if (e == cudaSuccess && n > 0) {
-    validate_kernel<<<grid_for(n), 256>>>(n, rowptr, colind, vals, h->diag, h->ndiag, cnt);
+  // the row pointers first: nothing is read through them before they are checked
+  *hw = SetupWords{};
+  hw->bad_row = hw->dmin = ~0ull;
+  e = cudaMemcpyAsync(sw, hw, sizeof(SetupWords), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) {
+    rowptr_check_kernel<<<grid_for(n), 256>>>(n, rowptr, sw);
     e = cudaGetLastError();
   }
-  unsigned long long hc[2] = {0, 0};
-  if (e == cudaSuccess) e = cudaMemcpy(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost);
-  if (cnt) cudaFree(cnt);
+  if (e == cudaSuccess) e = cudaMemcpy(hw, sw, sizeof(SetupWords), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess) return bail(cuda_fail(h, e, "cg_create: row pointers"));
+  if (hw->first != 0) return bail(fail(h, CG_ERR_INVALID, "cg_create: rowptr[0] != 0"));
+  if (hw->bad_row != ~0ull)
+    return bail(fail(h, CG_ERR_INVALID, "cg_create: rowptr decreases at row " + std::to_string(hw->bad_row)));
+  h->nnz = hw->nnz;
+  if (h->nnz > 0 && (!colind || !vals))
+    return bail(fail(h, CG_ERR_INVALID, "cg_create: colind/vals NULL with nnz > 0"));
+
+  // colind range, diagonal and row blocks.  Two neighbouring blocks of a stretch hold
+  // more than kCapV entries or one of them kBlock rows, which bounds their number.
+  const size_t nv = (size_t)std::max<int64_t>(n, 1);
+  const int64_t ncut = (n + kCutRows - 1) / kCutRows;
+  const int64_t most = 2 * (h->nnz / kCapV) + 2 * (n / kBlock) + 2 * ncut + 2;
+  e = cudaMalloc(&h->rb, sizeof(int32_t) * (size_t)(most + ncut + 1));
+  if (e == cudaSuccess) e = cudaMalloc(&h->diag, sizeof(double) * nv);
+  if (e == cudaSuccess) e = cudaMalloc(&h->ndiag, sizeof(int32_t) * nv);
+  if (e != cudaSuccess) return bail(cuda_fail(h, e, "cg_create: allocation"));
+  int* counts = h->rb + most;
+  if (n > 0) {
+    validate_kernel<<<std::min<unsigned>(grid_for(n), 8u * (unsigned)h->sm_count), 256>>>(n, rowptr, colind, vals,
+                                                                                          h->diag, h->ndiag, sw);
+    cut_kernel<false><<<(unsigned)((ncut + 63) / 64), 64>>>(n, rowptr, counts, h->rb, sw);
+  }
+  cut_scan_kernel<<<1, 1024>>>(ncut, n, counts, h->rb, sw);
+  if (n > 0) cut_kernel<true><<<(unsigned)((ncut + 63) / 64), 64>>>(n, rowptr, counts, h->rb, sw);
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpy(hw, sw, sizeof(SetupWords), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return bail(cuda_fail(h, e, "cg_create: validation"));
-  if (hc[0] != 0)
-    return bail(fail(h, CG_ERR_INVALID, "cg_create: " + std::to_string(hc[0]) + " column indices outside [0, n)"));
-  h->jacobi_ok = (hc[1] == 0);
+  if (hw->bad_col != 0)
+    return bail(fail(h, CG_ERR_INVALID, "cg_create: " + std::to_string(hw->bad_col) + " column indices outside [0, n)"));
+  h->nrb = hw->nrb;
+  h->long_rows = (int64_t)hw->nlong;
+  h->ndiag_all = (int64_t)hw->ndiag;
+  h->jacobi_ok = hw->bad_diag == 0;
   if (h->jacobi_ok && n > 0) {
-    unsigned long long* mm = nullptr;
-    unsigned long long hmm[2] = {~0ull, 0ull};
-    e = cudaMalloc(&mm, sizeof(hmm));
-    if (e == cudaSuccess) e = cudaMemcpy(mm, hmm, sizeof(hmm), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) {
-      diag_range_kernel<<<std::min<unsigned>(grid_for(n), 1024u), 256>>>(n, h->diag, mm);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpy(hmm, mm, sizeof(hmm), cudaMemcpyDeviceToHost);
-    if (mm) cudaFree(mm);
-    if (e != cudaSuccess) return bail(cuda_fail(h, e, "cg_create: diagonal range"));
-    std::memcpy(&h->dmin, &hmm[0], sizeof(double));
-    std::memcpy(&h->dmax, &hmm[1], sizeof(double));
+    std::memcpy(&h->dmin, &hw->dmin, sizeof(double));
+    std::memcpy(&h->dmax, &hw->dmax, sizeof(double));
+  }
+  if (n <= cgi::cluster_max_rows()) {  // the cluster form splits small systems on the host
+    const cg_status hs = cgi::ensure_host_rowptr(h);
+    if (hs != CG_OK) return bail(hs);
   }
 
-  // persistent-kernel residency (the smallest over the kernels we may launch)
-  const int g1 = max_coresident(pcg64_kernel<true>, h->sm_count);
-  const int g2 = max_coresident(pcg64_kernel<false>, h->sm_count);
-  const int g3 = std::min(max_coresident(pcg_ir_kernel<true, false>, h->sm_count),
-                          max_coresident(pcg_ir_kernel<true, true>, h->sm_count));
-  const int g4 = std::min(max_coresident(pcg_ir_kernel<false, false>, h->sm_count),
-                          max_coresident(pcg_ir_kernel<false, true>, h->sm_count));
-  h->grid_max = std::min(std::min(std::min(g1, g2), std::min(g3, g4)), kXCtas);
-  const int g5 = std::min(std::min(max_coresident(g_upd_r<double, true>, h->sm_count),
-                                   max_coresident(g_upd_r<double, false>, h->sm_count)),
-                          max_coresident(g_upd_xp<float, true, true, true>, h->sm_count));
-  const int g6 = std::min(max_coresident(g_upd_xp<double, true, false, true>, h->sm_count),
-                          max_coresident(g_res64<true>, h->sm_count));
-  h->grid_graph = std::min(g5, g6);
+  residency(dev, h->sm_count, &h->grid_max, &h->grid_graph);
   h->grid_part = 64 * h->sm_count;  // bounds every loop kernel's grid
   if (h->grid_max <= 0 || h->grid_graph <= 0 || h->grid_max > h->grid_part || h->grid_graph > h->grid_part)
     return bail(fail(h, CG_ERR_CUDA, "cg_create: occupancy query failed"));
   e = cudaMalloc(&h->part, sizeof(double) * (size_t)kParts * (size_t)h->grid_part);
-  if (e == cudaSuccess) e = cudaMalloc(&h->gs, sizeof(GState));
-  if (e == cudaSuccess) e = cudaMallocHost(&h->host_gs, sizeof(GState));
   if (e != cudaSuccess) return bail(cuda_fail(h, e, "cg_create: partials"));
   *out = h;
   return CG_OK;

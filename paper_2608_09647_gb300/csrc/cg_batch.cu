@@ -1408,6 +1408,8 @@ cg_status cg_batch_create(int32_t nsys, const int64_t* n, const int32_t* const* 
     }
     std::vector<int32_t> nd((size_t)hs->n);
     CGB_CREATE(cudaMemcpy(nd.data(), hs->ndiag, sizeof(int32_t) * (size_t)hs->n, cudaMemcpyDeviceToHost));
+    const cg_status hr = cgi::ensure_host_rowptr(hs);
+    if (hr != CG_OK) return bail(bfail(h, hr, "cg_batch_create: system " + std::to_string(s) + ": " + hs->err));
     const std::vector<int32_t>& rp = hs->host_rowptr;
     const int nsl = B->ntile[(size_t)s] * kWarps;
     for (int j = 0; j < nsl; ++j) {

@@ -709,6 +709,8 @@ cg_status cgi::cluster_solve(cg_handle* h, const double* b, double* x, double to
     if (rows > kMaxRowsPerCta) return (h->err = "cg_solve: system too large for the cluster form", CG_ERR_INVALID);
     // the CSR goes to shared memory when the largest CTA slice fits beside the vectors
     int64_t slice = 0;
+    const cg_status hr = cgi::ensure_host_rowptr(h);
+    if (hr != CG_OK) return hr;
     const std::vector<int32_t>& rp = h->host_rowptr;
     for (int c = 0; c < ctas; ++c) {
       const int64_t a = (int64_t)c * rows, z = std::min<int64_t>(h->n, a + rows);

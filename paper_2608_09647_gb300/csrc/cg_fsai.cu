@@ -1255,6 +1255,8 @@ cg_status pattern_host(cg_handle* h, FsaiData* f) {
   std::vector<int32_t> ci((size_t)nnz);
   if (nnz > 0)
     CGF_CUDA(h, cudaMemcpy(ci.data(), h->colind, sizeof(int32_t) * (size_t)nnz, cudaMemcpyDeviceToHost));
+  const cg_status hr = cgi::ensure_host_rowptr(h);
+  if (hr != CG_OK) return hr;
   const std::vector<int32_t>& rp = h->host_rowptr;
   std::vector<int32_t> trp((size_t)n + 1, 0), tci, tsrc;
   tci.reserve((size_t)(nnz / 2 + n));

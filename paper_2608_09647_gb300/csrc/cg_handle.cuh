@@ -34,6 +34,7 @@ void batch_free(BatchData* b);
 void fsai_free(FsaiData* f);
 void set_create_error(const std::string& msg);  // message of cg_last_error(NULL)
 cg_status ensure_offsets(cg_handle* h);         // cg_handle::offs_all, once (cg_api.cu)
+cg_status ensure_host_rowptr(cg_handle* h);     // cg_handle::host_rowptr, once (cg_api.cu)
 // the loop in one thread-block cluster (cg_cluster.cu): fp64 CG / Jacobi-PCG of small systems
 int64_t cluster_max_rows();
 cg_status cluster_solve(cg_handle* h, const double* b, double* x, double tol, int32_t maxit, bool jac,
@@ -66,7 +67,8 @@ struct cg_handle {
   int32_t* rb = nullptr;            // row blocks of the caller CSR
   int32_t nrb = 0;
   int64_t long_rows = 0;
-  std::vector<int32_t> host_rowptr;
+  std::vector<int32_t> host_rowptr;  // empty until cgi::ensure_host_rowptr
+  int64_t ndiag_all = 0;            // stored diagonal entries
   // diagonal data
   double* diag = nullptr;           // A_ii (sum of stored diagonal entries)
   int32_t* ndiag = nullptr;         // diagonal entries per row
@@ -86,7 +88,6 @@ struct cg_handle {
   static constexpr int32_t kOffsUnknown = -2;
   int32_t noffs_all = kOffsUnknown;
   int32_t offs_all[kOffsAll] = {};
-  int32_t* delta_dev = nullptr;
   int32_t* soff = nullptr;
   uint32_t* lmask = nullptr;
   int32_t csr = 0;                  // 1: the loop matrix is an off-diagonal CSR in row blocks
