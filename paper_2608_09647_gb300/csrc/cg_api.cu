@@ -738,6 +738,49 @@ cg_status ensure_offdiag(cg_handle* h) {
   return ensure_diag_vectors(h);
 }
 
+// *sym = whether slot m of row i and slot nd-1-m of row i + delta[m] are the same number,
+// bit for bit, everywhere (Sell::sym).  Only asked where the persistent SpMV gains by
+// reading half of the slices: while that half and the loop's four vectors stay in the
+// near half of the 126 MB L2.  Refinement, us an iteration, all slots read and half:
+// 7 points 128^3 rows (59 MB) 30.3 and 27.1, 160^3 (115 MB) 47.6 and 54.6; Q1 1000^2
+// (32 MB) 20.8 and 19.4, 2000^2 (128 MB) 48.0 and 62.9; 5 points 1000^2 (24 MB) 17.7 and
+// 16.7, 2000^2 (96 MB) 38.9 and 42.8.  Larger systems stream either way, and the mirrored
+// reads are the less regular ones.
+constexpr int64_t kSymMinBytes = (int64_t)1 << 20, kSymMaxBytes = (int64_t)63 << 20;
+
+template <typename T>
+__global__ void symmetry_kernel(int64_t n, int nd, DiaOffsets delta, const T* __restrict__ val, int* __restrict__ bad) {
+  int differ = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    for (int m = 0; m < nd / 2; ++m) {
+      const int64_t j = i + delta.d[m];
+      const T a = val[((i >> 5) * nd + m) * 32 + (i & 31)];
+      const T b = j >= 0 ? val[((j >> 5) * nd + nd - 1 - m) * 32 + (j & 31)] : T(0);
+      differ |= !(a == b);
+    }
+  }
+  if (__syncthreads_or(differ) && threadIdx.x == 0) *bad = 1;
+}
+
+template <typename T>
+cg_status check_symmetry(cg_handle* h, const T* val, const DiaOffsets& d, int32_t* sym) {
+  const int nd = h->uniform_w;
+  *sym = 0;
+  const int64_t resident = (int64_t)sizeof(T) * (h->sell_entries / 2 + 4 * h->n);
+  if (sizeof(T) != 4 || (nd != 4 && nd != 6 && nd != 8) || resident < kSymMinBytes || resident > kSymMaxBytes)
+    return CG_OK;
+  for (int m = 0; m < nd / 2; ++m)
+    if (d.d[m] >= 0 || d.d[m] != -d.d[nd - 1 - m]) return CG_OK;
+  int* bad = &h->st->status;  // free between solves
+  int host = 0;
+  CG_CUDA(h, cudaMemset(bad, 0, sizeof(int)));
+  symmetry_kernel<T><<<grid_for(h->n), 256>>>(h->n, nd, d, val, bad);
+  CG_CUDA(h, cudaGetLastError());
+  CG_CUDA(h, cudaMemcpy(&host, bad, sizeof(int), cudaMemcpyDeviceToHost));
+  *sym = host == 0;
+  return CG_OK;
+}
+
 // Loop-matrix values for (precision, precond), built on first use; the first
 // variant built also writes the shared column indices.
 template <typename T>
@@ -771,6 +814,8 @@ cg_status ensure_vals(cg_handle* h, T** sval, T** lval, bool scale) {
                       : (few ? fill_dia_kernel<T, false, 8> : fill_dia_kernel<T, false, 0>);
     fill<<<grid_for(h->n), 256>>>(h->n, h->rowptr, h->colind, h->vals, h->disq, h->uniform_w, d, *sval);
     CG_CUDA(h, cudaGetLastError());
+    const cg_status ss = check_symmetry(h, *sval, d, &h->sym32[scale]);
+    if (ss != CG_OK) return ss;
     CG_CUDA(h, cudaDeviceSynchronize());
     return CG_OK;
   }
@@ -801,12 +846,13 @@ cg_status ensure_vals(cg_handle* h, T** sval, T** lval, bool scale) {
 }
 
 template <typename T>
-Sell<T> make_sell(const cg_handle* h, const T* val, const T* lval, const T* diag, const T* disq) {
+Sell<T> make_sell(const cg_handle* h, const T* val, const T* lval, const T* diag, const T* disq, int32_t sym) {
   Sell<T> S{};
   S.n = h->n;
   S.nslices = h->nslices;
   S.uw = h->uniform_w;
   S.dia = h->dia;
+  S.sym = sym;
   for (int m = 0; m < kMaxDiag; ++m) S.delta[m] = h->delta[m];
   S.soff = h->soff;
   S.perm = h->sperm;
@@ -1381,8 +1427,8 @@ SolveParams make_solve_params(const cg_handle* h, bool jac, const double* b, dou
                               int32_t maxit, bool fp64, bool carry) {
   SolveParams P{};
   P.A = make_csr(h);
-  P.S64 = make_sell<double>(h, h->sval64[jac], h->lval64[jac], h->diag, h->disq);
-  P.S32 = make_sell<float>(h, h->sval32[jac], h->lval32[jac], h->diag32, h->disq32);
+  P.S64 = make_sell<double>(h, h->sval64[jac], h->lval64[jac], h->diag, h->disq, 0);
+  P.S32 = make_sell<float>(h, h->sval32[jac], h->lval32[jac], h->diag32, h->disq32, h->sym32[jac]);
   P.V64 = LoopVecs<double>{h->r, h->p, h->q, h->xh};
   P.V32 = LoopVecs<float>{h->r32, h->p32, h->q32, h->xh32};
   P.b = b;

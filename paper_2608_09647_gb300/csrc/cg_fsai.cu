@@ -117,19 +117,13 @@ __global__ void fill_ell_kernel(int64_t n, int w, const int32_t* __restrict__ sr
   }
 }
 
-// Diagonal layouts of G and G^T: entry e = (i, j) of tril(A) in slot s_e of
-// row i of G and in slot nd - 1 - s_e of row j of G^T (the offsets of G^T are
-// those of G negated, in reverse order).  Every position is written at most
-// once; the rest stays 0 from the memset.
+// Diagonal layout of G: entry e = (i, j) of tril(A) in its slot of row i.  Every
+// position is written at most once; the rest stays 0 from the memset.
 template <typename T>
-__global__ void fill_dia_kernel(int64_t nt, int64_t n, int nd, const int32_t* __restrict__ trow,
-                                const int32_t* __restrict__ tci, const int8_t* __restrict__ slot,
-                                const double* __restrict__ g, T* __restrict__ gv, T* __restrict__ gtv) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nt; e += (int64_t)gridDim.x * blockDim.x) {
-    const int s = slot[e];
-    gv[(int64_t)s * n + trow[e]] = (T)g[e];
-    gtv[(int64_t)(nd - 1 - s) * n + tci[e]] = (T)g[e];
-  }
+__global__ void fill_dia_kernel(int64_t nt, int64_t n, const int32_t* __restrict__ trow,
+                                const int8_t* __restrict__ slot, const double* __restrict__ g, T* __restrict__ gv) {
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nt; e += (int64_t)gridDim.x * blockDim.x)
+    gv[(int64_t)slot[e] * n + trow[e]] = (T)g[e];
 }
 
 __global__ void g_positive_kernel(int64_t n, const int32_t* __restrict__ trp, const double* __restrict__ g,
@@ -145,7 +139,9 @@ __global__ void g_positive_kernel(int64_t n, const int32_t* __restrict__ trp, co
 
 // G or G^T for the loop: slot m of row i at [m n + i]; the column is col[m n + i]
 // (ELL) or, in the diagonal layout (DIA), i + delta[m] clamped into [0, n) (the
-// value is 0 wherever the diagonal leaves the pattern).
+// value is 0 wherever the diagonal leaves the pattern).  In the diagonal layout both
+// read the values of G: a second copy for G^T (20 MB at 1000^2 rows, fp32) took a
+// refinement of that size, which L2 otherwise holds, from 29.4 to 31.0 us an iteration.
 template <typename T>
 struct Ell {
   const int32_t* col;
@@ -164,10 +160,33 @@ constexpr int kEll = 0, kDiaAny = -1;
 // sum_m E(i, m) * f(column of slot m) in slot order.  With W slots known at
 // compile time every load of the row is issued before the first product (a
 // loop over a run-time count waits a full memory latency per slot).
-template <int W, typename T, typename Fn>
+template <int W, bool GT = false, typename T, typename Fn>
 __device__ __forceinline__ T ell_row(const Ell<T>& E, int64_t i, int64_t n, Fn&& f) {
   T s = T(0);
-  if constexpr (W > 0) {
+  if constexpr (GT && W != kEll) {
+    // G^T(i, c) = G(c, i): slot m of row i is slot w-1-m of row c = i + delta[m] >= i
+    const auto value = [&](int w, int m, int c) {
+      return c < (int)n ? __ldg(E.val + (int64_t)(w - 1 - m) * n + c) : T(0);
+    };
+    if constexpr (W > 0) {
+      T e[W], v[W];
+#pragma unroll
+      for (int m = 0; m < W; ++m) {
+        const int c = (int)i + E.delta[m];
+        e[m] = value(W, m, c);
+        v[m] = f(min(c, (int)n - 1));
+      }
+#pragma unroll
+      for (int m = 0; m < W; ++m) s = fma(e[m], v[m], s);
+    } else {
+#pragma unroll
+      for (int m = 0; m < kFsaiMaxDiag; ++m) {
+        if (m >= E.w) continue;
+        const int c = (int)i + E.delta[m];
+        s = fma(value(E.w, m, c), f(min(c, (int)n - 1)), s);
+      }
+    }
+  } else if constexpr (W > 0) {
     T e[W], v[W];
 #pragma unroll
     for (int m = 0; m < W; ++m) {
@@ -240,7 +259,7 @@ __device__ bool fsai_start(const Ell<T>& G, const Ell<T>& GT, const FsaiVecs<T>&
   rows_x2(
       g, n,
       [&](int64_t i) {
-        const T s = ell_row<W>(GT, i, n, [&](int j) { return V.t[j]; });
+        const T s = ell_row<W, true>(GT, i, n, [&](int j) { return V.t[j]; });
         return carry ? fma(beta, V.p[i], s) : s;
       },
       [&](int64_t i, T pi) { V.p[i] = pi; });
@@ -322,7 +341,7 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
     rn = tmp;
     if (!done) {
       rows_x2(
-          g, n, [&](int64_t i) { return fma(beta, V.p[i], ell_row<W>(GT, i, n, [&](int j) { return V.t[j]; })); },
+          g, n, [&](int64_t i) { return fma(beta, V.p[i], ell_row<W, true>(GT, i, n, [&](int j) { return V.t[j]; })); },
           [&](int64_t i, T pi) { V.p[i] = pi; });
       if (!g.sync()) { status = kTimeout; break; }
     }
@@ -593,7 +612,7 @@ __global__ void __launch_bounds__(kBlock, kFsaiPhaseCtas) gf_p0(FArgs F) {
   const float beta0 = (float)F.a.gs->beta0;
   float* p = P.V32.p;
   for (int64_t i = g.gtid; i < n; i += g.gstride) {
-    const float s = ell_row<W>(F.GT, i, n, [&](int j) { return F.t[j]; });
+    const float s = ell_row<W, true>(F.GT, i, n, [&](int j) { return F.t[j]; });
     p[i] = beta0 != 0.0f ? fmaf(beta0, p[i], s) : s;
   }
 }
@@ -694,7 +713,7 @@ __global__ void __launch_bounds__(kBlock, kFsaiPhaseCtas) gf_upd_p(FArgs F) {
   const float beta = (float)gs->beta;
   float* p = P.V32.p;
   rows_x2(
-      g, n, [&](int64_t i) { return fmaf(beta, p[i], ell_row<W>(F.GT, i, n, [&](int j) { return F.t[j]; })); },
+      g, n, [&](int64_t i) { return fmaf(beta, p[i], ell_row<W, true>(F.GT, i, n, [&](int j) { return F.t[j]; })); },
       [&](int64_t i, float pi) { p[i] = pi; });
 }
 
@@ -1418,13 +1437,9 @@ cg_status cgi::fsai_commit(cg_handle* h, int kind) {
   if (f->dia) {
     const size_t w = (size_t)f->nd * (size_t)n;
     CGF_CUDA(h, cudaMemsetAsync(f->gval64, 0, sizeof(double) * w, h->stream));
-    CGF_CUDA(h, cudaMemsetAsync(f->gtval64, 0, sizeof(double) * w, h->stream));
     CGF_CUDA(h, cudaMemsetAsync(f->gval32, 0, sizeof(float) * w, h->stream));
-    CGF_CUDA(h, cudaMemsetAsync(f->gtval32, 0, sizeof(float) * w, h->stream));
-    fill_dia_kernel<double><<<blocks_for(f->ntril), 256, 0, h->stream>>>(f->ntril, n, f->nd, f->trow, f->tci,
-                                                                         f->tslot, f->g, f->gval64, f->gtval64);
-    fill_dia_kernel<float><<<blocks_for(f->ntril), 256, 0, h->stream>>>(f->ntril, n, f->nd, f->trow, f->tci,
-                                                                        f->tslot, f->g, f->gval32, f->gtval32);
+    fill_dia_kernel<double><<<blocks_for(f->ntril), 256, 0, h->stream>>>(f->ntril, n, f->trow, f->tslot, f->g, f->gval64);
+    fill_dia_kernel<float><<<blocks_for(f->ntril), 256, 0, h->stream>>>(f->ntril, n, f->trow, f->tslot, f->g, f->gval32);
   } else {
     fill_ell_kernel<double><<<blocks_for((int64_t)f->gw * n), 256, 0, h->stream>>>(n, f->gw, f->gsrc, f->g, f->gval64);
     fill_ell_kernel<float><<<blocks_for((int64_t)f->gw * n), 256, 0, h->stream>>>(n, f->gw, f->gsrc, f->g, f->gval32);
@@ -1448,9 +1463,9 @@ cg_status cgi::fsai_solve(cg_handle* h, const SolveParams& Pin, bool fp64, bool 
   F.P = Pin;
   const int w = f->dia ? f->nd : f->gw, wt = f->dia ? f->nd : f->gtw;
   F.G64 = Ell<double>{f->gcol, f->gval64, w, {}};
-  F.GT64 = Ell<double>{f->gtcol, f->gtval64, wt, {}};
+  F.GT64 = Ell<double>{f->gtcol, f->dia ? f->gval64 : f->gtval64, wt, {}};
   F.G32 = Ell<float>{f->gcol, f->gval32, w, {}};
-  F.GT32 = Ell<float>{f->gtcol, f->gtval32, wt, {}};
+  F.GT32 = Ell<float>{f->gtcol, f->dia ? f->gval32 : f->gtval32, wt, {}};
   for (int m = 0; m < (f->dia ? f->nd : 0); ++m) {
     F.G64.delta[m] = F.G32.delta[m] = f->doff[m];
     F.GT64.delta[m] = F.GT32.delta[m] = -f->doff[f->nd - 1 - m];

@@ -103,6 +103,7 @@ struct cg_handle {
   int64_t nnz_long = 0;
   double* sval64[2] = {nullptr, nullptr};  // [precond]: unscaled / Jacobi-scaled
   float* sval32[2] = {nullptr, nullptr};
+  int32_t sym32[2] = {};            // Sell::sym of sval32
   double* lval64[2] = {nullptr, nullptr};
   float* lval32[2] = {nullptr, nullptr};
   bool scol_written = false;

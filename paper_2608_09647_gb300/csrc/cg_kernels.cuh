@@ -67,6 +67,7 @@ struct Sell {
   int32_t uw;  // >= 0: every slice has width uw and no row is long (soff, lmask unread)
   int32_t dia;                // 1: sliced-diagonal layout, width uw = number of diagonals
   int32_t delta[kMaxDiag];    // diagonal offsets (dia only)
+  int32_t sym;                // 1: dia, and slot m of row i is slot uw-1-m of row i + delta[m], bit for bit
   const int32_t* __restrict__ soff;
   const uint32_t* __restrict__ lmask;
   const int32_t* __restrict__ col;
@@ -315,6 +316,24 @@ __device__ __forceinline__ int ld_stream(const int* p) { return __ldcs(p); }
 __device__ __forceinline__ double ld_stream(const double* p) { return __ldcs(p); }
 __device__ __forceinline__ float ld_stream(const float* p) { return __ldcs(p); }
 
+// How spmv_phase_w finds a slot's column and value: in the slice; the column from
+// delta[]; or (kSym, matrices equal to their transpose bit for bit) the value of a slot
+// left of the diagonal from the row it mirrors, so that only the right half of the
+// slices comes from memory and the left half is found in cache a band of rows later.
+constexpr int kCols = 0, kDia = 1, kSym = 2;
+
+template <typename T, int W, int DIA>
+__device__ __forceinline__ T dia_val(const Sell<T>& S, const T* __restrict__ vp, int i, int m) {
+  if constexpr (DIA == kSym) {
+    if (m >= W / 2) return __ldg(vp + m * 32);
+    const int j = i + S.delta[m];
+    const T* u = S.val + (W - 1 - m) * 32;
+    return j >= 0 ? __ldg(u + ((int64_t)(j >> 5) * ((W - 1) * 32) + j)) : T(0);
+  } else {
+    return ld_stream(vp + m * 32);
+  }
+}
+
 // a1 over the grid for uniform slices of compile-time width W (no long rows):
 // every load of a slice is issued at once and the register footprint is
 // exactly what W needs, which keeps occupancy high.  DIA: the column of slot m
@@ -324,7 +343,7 @@ __device__ __forceinline__ float ld_stream(const float* p) { return __ldcs(p); }
 // columns are issued together, then the multiply-adds.  DIA: the column of
 // slot m is i + delta[m], clamped into [0, n) with two 32-bit min/max (only
 // zero-valued slots of the first and last slices ever need the clamp).
-template <typename T, int W, bool DIA>
+template <typename T, int W, int DIA>
 __device__ __forceinline__ T slice_sum(const Sell<T>& S, const T* __restrict__ p, int64_t s,
                                        int i32, int lane, T acc) {
   constexpr int CH = W > 16 ? (W + 1) / 2 : W;
@@ -337,7 +356,7 @@ __device__ __forceinline__ T slice_sum(const Sell<T>& S, const T* __restrict__ p
     for (int u = 0; u < CH; ++u) {
       const int m = m0 + u;
       if (m < W) {
-        v[u] = ld_stream(vp + m * 32);
+        v[u] = dia_val<T, W, DIA>(S, vp, i32, m);
         const int c = DIA ? min(max(i32 + S.delta[m], 0), nm1)
                           : ld_stream(S.col + s * (W * 32) + lane + m * 32);
         pc[u] = p[c];
@@ -355,7 +374,7 @@ __device__ __forceinline__ T slice_sum(const Sell<T>& S, const T* __restrict__ p
 // contiguous band of rows and the neighbours' lines are shared through L2.
 // The diagonal term starts the fused multiply-add chain: W + 1 FMAs per row
 // with the p.q term.
-template <typename T, bool JAC, int W, bool DIA>
+template <typename T, bool JAC, int W, int DIA>
 __device__ __forceinline__ double spmv_phase_w(const Sell<T>& S, const T* __restrict__ p,
                                                T* __restrict__ q, const Grid& g) {
   const int lane = threadIdx.x & 31;
@@ -385,7 +404,7 @@ __device__ __forceinline__ double spmv_phase_w(const Sell<T>& S, const T* __rest
         const T* vp = S.val + (int64_t)sh * (W * 32) + lane;
 #pragma unroll
         for (int m = 0; m < W; ++m) {
-          v[h][m] = ld_stream(vp + m * 32);
+          v[h][m] = dia_val<T, W, DIA>(S, vp, i, m);
           const int c = DIA ? min(max(i + S.delta[m], 0), nm1) : ld_stream(S.col + (int64_t)sh * (W * 32) + lane + m * 32);
           pc[h][m] = p[c];
         }
@@ -633,15 +652,20 @@ __device__ __forceinline__ double spmv_phase(const Sell<T>& S, const T* __restri
                                              T* __restrict__ q, const Grid& g) {
   if (S.csr) return spmv_phase_csr<T, JAC>(S, p, q, g);
   if (S.dia) {
-    if (S.uw == 4) return spmv_phase_w<T, JAC, 4, true>(S, p, q, g);
-    if (S.uw == 6) return spmv_phase_w<T, JAC, 6, true>(S, p, q, g);
-    if (S.uw == 8) return spmv_phase_w<T, JAC, 8, true>(S, p, q, g);
-    if (S.uw == 26) return spmv_phase_w<T, JAC, 26, true>(S, p, q, g);
+    if constexpr (sizeof(T) == 4) {
+      if (S.sym && S.uw == 4) return spmv_phase_w<T, JAC, 4, kSym>(S, p, q, g);
+      if (S.sym && S.uw == 6) return spmv_phase_w<T, JAC, 6, kSym>(S, p, q, g);
+      if (S.sym && S.uw == 8) return spmv_phase_w<T, JAC, 8, kSym>(S, p, q, g);
+    }
+    if (S.uw == 4) return spmv_phase_w<T, JAC, 4, kDia>(S, p, q, g);
+    if (S.uw == 6) return spmv_phase_w<T, JAC, 6, kDia>(S, p, q, g);
+    if (S.uw == 8) return spmv_phase_w<T, JAC, 8, kDia>(S, p, q, g);
+    if (S.uw == 26) return spmv_phase_w<T, JAC, 26, kDia>(S, p, q, g);
     return spmv_phase_dia<T, JAC>(S, p, q, g);
   }
-  if (S.uw == 4) return spmv_phase_w<T, JAC, 4, false>(S, p, q, g);
-  if (S.uw == 6) return spmv_phase_w<T, JAC, 6, false>(S, p, q, g);
-  if (S.uw == 8) return spmv_phase_w<T, JAC, 8, false>(S, p, q, g);
+  if (S.uw == 4) return spmv_phase_w<T, JAC, 4, kCols>(S, p, q, g);
+  if (S.uw == 6) return spmv_phase_w<T, JAC, 6, kCols>(S, p, q, g);
+  if (S.uw == 8) return spmv_phase_w<T, JAC, 8, kCols>(S, p, q, g);
   const int lane = threadIdx.x & 31;
   const int gw = (int)g.cta * kWarps + (int)(threadIdx.x >> 5);
   const int W = (int)g.G * kWarps;
