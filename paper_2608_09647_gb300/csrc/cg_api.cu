@@ -419,6 +419,8 @@ std::vector<int32_t> build_row_blocks(const int32_t* rowptr, int64_t n, int64_t*
   return rb;
 }
 
+size_t padded(int64_t n) { return ((size_t)std::max<int64_t>(n, 1) + 63) / 64 * 64; }
+
 template <typename K>
 int max_coresident(K kernel, int sm_count) {
   int per_sm = 0;
@@ -476,6 +478,18 @@ unsigned spmv_grid(const cg_handle* h) {
   return (unsigned)std::max<int64_t>(1, std::min<int64_t>(h->nrb, (int64_t)per_sm * h->sm_count));
 }
 
+// Whether the fp32 loop's SpMV takes its ring (spmv_phase_ring): 26 off-diagonal offsets
+// in runs of three neighbours, the middle one around the diagonal, and slices enough for
+// every warp to run ahead (two chunks a slice, a ring of three).
+bool ring_applies(const cg_handle* h, int G) {
+  constexpr int64_t kMinSlices = 4;  // of a warp
+  if (!h->dia || h->uniform_w != kRingW || h->nslices < kMinSlices * G * kWarps) return false;
+  const auto at = [&](int k) { return k < 13 ? h->delta[k] : k == 13 ? 0 : h->delta[k - 1]; };
+  for (int k = 0; k < 27; k += 3)
+    if (at(k + 1) != at(k) + 1 || at(k + 2) != at(k) + 2) return false;
+  return h->n <= INT32_MAX - 256;
+}
+
 int auto_grid(const cg_handle* h) {
   if (h->grid_opt > 0) return std::min(h->grid_opt, h->grid_max);
   // enough CTAs for the larger of the row-block and vector work, capped by residency
@@ -527,7 +541,6 @@ cg_status cgi::ensure_offsets(cg_handle* h) {
 namespace {
 
 // Elements of an n-vector's place in a shared allocation (whole 256 bytes of fp32).
-size_t padded(int64_t n) { return ((size_t)std::max<int64_t>(n, 1) + 63) / 64 * 64; }
 
 // sqrt(A_ii), 1/sqrt(A_ii) and the fp32 copies: one allocation, last step of the layout.
 cg_status ensure_diag_vectors(cg_handle* h) {
@@ -881,6 +894,8 @@ cg_status ensure_vectors(cg_handle* h, T** r, T** p, T** q, T** xh) {
   if (*r) return CG_OK;
   const size_t nv = padded(h->n);
   CG_CUDA(h, cudaMalloc(r, 4 * sizeof(T) * nv));  // one allocation, at *r
+  if (sizeof(T) == 4)  // p's entries past n are read (times 0) by spmv_phase_ring
+    CG_CUDA(h, cudaMemset(*r + nv, 0, sizeof(T) * nv));
   *p = *r + nv;
   *q = *p + nv;
   *xh = *q + nv;
@@ -1520,9 +1535,19 @@ cg_status solve_impl(cg_handle* h, const double* b, double* x, double tol, int32
     else
       fn = carry ? (jac ? (const void*)pcg_ir_kernel<true, true> : (const void*)pcg_ir_kernel<false, true>)
                  : (jac ? (const void*)pcg_ir_kernel<true, false> : (const void*)pcg_ir_kernel<false, false>);
+    size_t smem = 0;
+    if (!fp64 && ring_applies(h, G)) {
+      int per_sm = 0;
+      CG_CUDA(h, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes));
+      CG_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, kRingBytes));
+      if (per_sm * h->sm_count >= G) {
+        P.S32.ring = (int32_t)padded(h->n);
+        smem = kRingBytes;
+      }
+    }
     CG_CUDA(h, cudaMemsetAsync(h->st, 0, kStBytes, h->stream));
     CG_CUDA(h, cudaEventRecord(h->ev0, h->stream));
-    CG_CUDA(h, cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kBlock), args, 0, h->stream));
+    CG_CUDA(h, cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kBlock), args, smem, h->stream));
   }
   CG_CUDA(h, cudaEventRecord(h->ev1, h->stream));
   CG_CUDA(h, cudaMemcpyAsync(h->host_st, h->st, sizeof(DevState), cudaMemcpyDeviceToHost, h->stream));

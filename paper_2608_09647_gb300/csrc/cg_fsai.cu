@@ -1382,12 +1382,14 @@ cg_status alloc_loop_arrays(cg_handle* h, FsaiData* f) {
   const int64_t n = h->n, nt = f->ntril;
   const size_t nv = (size_t)std::max<int64_t>(n, 1);
   const int gw = std::max(f->gw, f->nd);  // value arrays serve either layout
-  const int gtw = std::max(f->gtw, f->nd);
+  const int gtw = f->gtw;
   CGF_CUDA(h, cudaMalloc(&f->g, sizeof(double) * (size_t)std::max<int64_t>(nt, 1)));
   CGF_CUDA(h, cudaMalloc(&f->gval64, sizeof(double) * (size_t)gw * nv));
   CGF_CUDA(h, cudaMalloc(&f->gval32, sizeof(float) * (size_t)gw * nv));
-  CGF_CUDA(h, cudaMalloc(&f->gtval64, sizeof(double) * (size_t)gtw * nv));
-  CGF_CUDA(h, cudaMalloc(&f->gtval32, sizeof(float) * (size_t)gtw * nv));
+  if (!f->dia) {
+    CGF_CUDA(h, cudaMalloc(&f->gtval64, sizeof(double) * (size_t)gtw * nv));
+    CGF_CUDA(h, cudaMalloc(&f->gtval32, sizeof(float) * (size_t)gtw * nv));
+  }
   for (double** v : {&f->r0, &f->r1, &f->t}) CGF_CUDA(h, cudaMalloc(v, sizeof(double) * nv));
   for (float** v : {&f->r0_32, &f->r1_32, &f->t_32, &f->x_32}) CGF_CUDA(h, cudaMalloc(v, sizeof(float) * nv));
   return CG_OK;

@@ -67,6 +67,8 @@ struct Sell {
   int32_t uw;  // >= 0: every slice has width uw and no row is long (soff, lmask unread)
   int32_t dia;                // 1: sliced-diagonal layout, width uw = number of diagonals
   int32_t delta[kMaxDiag];    // diagonal offsets (dia only)
+  int32_t ring;               // > 0: spmv_phase_ring, on kRingBytes of dynamic shared memory;
+                              //      the allocated length of the vectors
   int32_t sym;                // 1: dia, and slot m of row i is slot uw-1-m of row i + delta[m], bit for bit
   const int32_t* __restrict__ soff;
   const uint32_t* __restrict__ lmask;
@@ -160,8 +162,9 @@ struct Grid {
   XState* x;
   uint64_t timeout_ns;
   unsigned seq, skip_seq;
+  unsigned fills;  // this warp's ring chunks so far (spmv_phase_ring)
   __device__ Grid() : G(gridDim.x), cta(blockIdx.x), gtid((int64_t)blockIdx.x * kBlock + threadIdx.x),
-        gstride((int64_t)gridDim.x * kBlock), st(nullptr), x(nullptr), timeout_ns(0), seq(0), skip_seq(0) {}
+        gstride((int64_t)gridDim.x * kBlock), st(nullptr), x(nullptr), timeout_ns(0), seq(0), skip_seq(0), fills(0) {}
   __device__ Grid(DevState* s, XWord* words, XState* xs, uint64_t to, unsigned skip) : Grid() {
     st = s;
     x = xs;
@@ -439,6 +442,155 @@ __device__ __forceinline__ double spmv_phase_w(const Sell<T>& S, const T* __rest
   return dot.get();
 }
 
+// Refinement on 27-point stencils (any grid at least four points wide): the SpMV of the
+// persistent loop with its operands brought into shared memory ahead of the products.
+// With two CTAs per SM the loop holds only 16 warps, and 27 + 26 loads into registers
+// per slice left memory waiting: half of the warps' time was a wait for a load.  Here a
+// warp has a ring of half slices of values (13 columns, one bulk copy each by one lane,
+// an mbarrier per stage) and two windows of p, filled a slice ahead: the columns of a
+// slice are 9 runs of 34 neighbouring entries of p, 90 16-byte copies, three a lane,
+// where the gathers took 26 loads and their clamps.  160^3 rows, 304 CTAs: the SpMV in the
+// loop 111 -> 95 us (426 MB of values: 63 us at the memory's rate), a solve to 1e-12
+// 44.9 -> 43.5 ms.
+constexpr int kRingW = 26, kRingChunk = kRingW / 2, kRingDepth = 3;
+constexpr int kRingChunkBytes = kRingChunk * 32 * (int)sizeof(float);
+constexpr int kRingBars = 128 * ((kWarps * kRingDepth * 8 + 127) / 128);
+constexpr int kRuns = 9, kRunPieces = 10;         // 16-byte pieces of a run: 3 + 34 entries at most
+constexpr int kWinDepth = 2, kWinBytes = kRuns * kRunPieces * 16;
+constexpr int kRingBytes = kRingBars + kWarps * (kRingDepth * kRingChunkBytes + kWinDepth * kWinBytes);
+
+struct Ring {
+  unsigned bar, buf;  // shared addresses of this warp's mbarriers and chunks
+  const float* mem;   // the same chunks
+  unsigned win;       // and of its windows of p
+  const float* wmem;
+  __device__ __forceinline__ Ring() {
+    extern __shared__ __align__(128) unsigned char ring_smem[];
+    const int warp = threadIdx.x >> 5;
+    mem = reinterpret_cast<const float*>(ring_smem + kRingBars + warp * kRingDepth * kRingChunkBytes);
+    bar = (unsigned)__cvta_generic_to_shared(ring_smem) + warp * kRingDepth * 8;
+    buf = (unsigned)__cvta_generic_to_shared(mem);
+    wmem = reinterpret_cast<const float*>(ring_smem + kRingBars + kWarps * kRingDepth * kRingChunkBytes +
+                                          warp * kWinDepth * kWinBytes);
+    win = (unsigned)__cvta_generic_to_shared(wmem);
+  }
+  // once per launch, by every warp
+  __device__ __forceinline__ void init() const {
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+      for (int d = 0; d < kRingDepth; ++d) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8 * d) : "memory");
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+  }
+  // one lane: chunk number f of this warp's stream comes from src
+  __device__ __forceinline__ void fill(unsigned f, const float* src) const {
+    const unsigned d = f % kRingDepth, b = bar + 8 * d;
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(kRingChunkBytes) : "memory");
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(
+            buf + d * kRingChunkBytes),
+        "l"(src), "r"(kRingChunkBytes), "r"(b), "l"(policy)
+        : "memory");
+  }
+  // all lanes: chunk f has arrived (bounded; on giving up the launch is marked aborted)
+  __device__ __forceinline__ void wait(unsigned f, const Grid& g) const {
+    const unsigned b = bar + 8 * (f % kRingDepth), parity = (f / kRingDepth) & 1u;
+    uint64_t t0 = 0;
+    for (unsigned spins = 0;; ++spins) {
+      unsigned ok;
+      asm volatile(
+          "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+          : "=r"(ok)
+          : "r"(b), "r"(parity)
+          : "memory");
+      if (ok) return;
+      if (spins == 0) t0 = global_timer_ns();
+      else if ((spins & 15u) == 0u && global_timer_ns() - t0 > g.timeout_ns) {
+        atomicExch(&g.st->abort, 1);
+        return;
+      }
+    }
+  }
+  __device__ __forceinline__ const float* chunk(unsigned f) const { return mem + (f % kRingDepth) * (kRingChunkBytes / 4); }
+};
+
+// a1 over the grid by the ring, one slice a warp at a time.  Slot m reads position m' = m
+// (m < 13) or m + 1 of the 27 ordered offsets, the diagonal's among them: run m' / 3, its
+// entry m' % 3 + lane.
+// (S.ring is the allocated length of p, whose entries past n are 0.)
+template <bool JAC>
+__device__ __forceinline__ double spmv_phase_ring(const Sell<float>& S, const float* __restrict__ p,
+                                                  float* __restrict__ q, Grid& g) {
+  const Ring R;
+  const int lane = threadIdx.x & 31;
+  const int s0 = (int)g.cta * kWarps + (int)(threadIdx.x >> 5);
+  const int Wt = (int)g.G * kWarps;
+  const int n = (int)S.n, last = S.ring - 4;  // start of p's last piece
+  const int slices = s0 < S.nslices ? (S.nslices - s0 + Wt - 1) / Wt : 0;  // of this warp
+  const unsigned f0 = g.fills;
+  const auto source = [&](int c) {  // chunk c of this warp's slices
+    return S.val + (int64_t)(s0 + (c >> 1) * Wt) * (kRingW * 32) + (c & 1) * (kRingChunk * 32);
+  };
+  if (lane == 0)
+    for (int c = 0; c < kRingDepth && c < 2 * slices; ++c) R.fill(f0 + c, source(c));
+  constexpr int kPer = (kRuns * kRunPieces + 31) / 32;
+  int off[kPer];  // this lane's pieces: their place in p from the slice's first row
+#pragma unroll
+  for (int u = 0; u < kPer; ++u) {
+    const int e = min(lane + 32 * u, kRuns * kRunPieces - 1), r = e / kRunPieces;
+    off[u] = (S.delta[r <= 4 ? 3 * r : 3 * r - 1] & ~3) + 4 * (e - r * kRunPieces);
+  }
+  const auto windows = [&](int k) {  // of this warp's slice k
+    const int i0 = (s0 + k * Wt) * 32;
+    const unsigned dst = R.win + (k & 1) * kWinBytes + lane * 16;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u)
+      if (lane + 32 * u < kRuns * kRunPieces)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + u * 512),
+                     "l"(p + min(max(i0 + off[u], 0), last))
+                     : "memory");
+  };
+  const auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
+  if (slices > 0) windows(0);
+  commit();
+  Acc<float> dot;
+  for (int k = 0; k < slices; ++k) {
+    const int i = (s0 + k * Wt) * 32 + lane;
+    if (k + 1 < slices) windows(k + 1);
+    commit();
+    const float di = JAC ? 1.0f : __ldg(S.dg + min(i, n - 1));
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    __syncwarp();  // slice k's windows have arrived
+    const float* w = R.wmem + (k & 1) * (kWinBytes / 4) + lane;
+    const float pi = w[4 * kRunPieces * 4 + (S.delta[12] & 3) + 1];  // run 4 starts left of the diagonal
+    float acc = JAC ? pi : di * pi;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const unsigned f = f0 + 2 * k + h;
+      R.wait(f, g);
+      const float* v = R.chunk(f) + lane;
+#pragma unroll
+      for (int u = 0; u < kRingChunk; ++u) {
+        const int m = h * kRingChunk + u, mm = m < 13 ? m : m + 1, r = mm / 3, d0 = r <= 4 ? 3 * r : 3 * r - 1;
+        acc = fmaf(v[u * 32], w[r * kRunPieces * 4 + (S.delta[d0] & 3) + mm % 3], acc);
+      }
+      __syncwarp();  // the chunk (and with h = 1 the windows) have been read
+      const int c = 2 * k + h + kRingDepth;
+      if (lane == 0 && c < 2 * slices) R.fill(f0 + c, source(c));
+    }
+    if (i < n) {
+      q[i] = acc;
+      dot.add(pi, acc);
+    }
+  }
+  g.fills = f0 + 2 * slices;
+  return dot.get();
+}
+
 // Sliced-diagonal layout of any width up to kMaxDiag (loads in groups of kUnroll).
 template <typename T, bool JAC>
 __device__ __forceinline__ double spmv_phase_dia(const Sell<T>& S, const T* __restrict__ p,
@@ -647,11 +799,13 @@ __device__ __forceinline__ double spmv_phase_csr(const Sell<T>& S, const T* __re
 // a1 over the grid: q = A^ p and this thread's share of p.q.  Warps take
 // slices round-robin; long rows are summed by a warp each.  Uniform slices of
 // width 4, 6 or 8 go to the specialised loop.
-template <typename T, bool JAC>
+template <typename T, bool JAC, bool RING = false>
 __device__ __forceinline__ double spmv_phase(const Sell<T>& S, const T* __restrict__ p,
-                                             T* __restrict__ q, const Grid& g) {
+                                             T* __restrict__ q, Grid& g) {
   if (S.csr) return spmv_phase_csr<T, JAC>(S, p, q, g);
   if (S.dia) {
+    if constexpr (sizeof(T) == 4 && RING)
+      if (S.ring) return spmv_phase_ring<JAC>(S, p, q, g);
     if constexpr (sizeof(T) == 4) {
       if (S.sym && S.uw == 4) return spmv_phase_w<T, JAC, 4, kSym>(S, p, q, g);
       if (S.sym && S.uw == 6) return spmv_phase_w<T, JAC, 6, kSym>(S, p, q, g);
@@ -872,7 +1026,7 @@ __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, doubl
   __shared__ int s_st, s_want, s_exact, s_conv;
   while (!done) {
     // a1: q = A^ p; p.q
-    double v1[1] = {spmv_phase<T, JAC>(S, V.p, V.q, g)};
+    double v1[1] = {spmv_phase<T, JAC, true>(S, V.p, V.q, g)};
     clk.lap(g.st, 0);
     const bool ok1 = kWords ? g.sum(v1, kKindPQ) : g.sum_parts(v1, part + kSlotPQ * (size_t)pstride);
     clk.lap(g.st, 1);
@@ -1057,6 +1211,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_ir_kernel(SolveParams P) {
   __shared__ XState s_x;
   Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
   PhaseClock clk(P.timers != 0);
+  if (P.S32.ring) Ring().init();
   const int64_t n = P.A.n;
   const LoopVecs<float>& V = P.V32;
   int status = kNotConverged, inner = 0, outer = 0;
