@@ -77,7 +77,9 @@ typedef enum {
   CG_OPT_PHASE_TIMERS = 6,        /* 1: record CTA 0's time per loop phase in cg_solve_info */
   CG_OPT_LOOP_MODE = 7            /* loop form: 0 auto (fp64 Jacobi / plain CG: cluster form up to
                                      16384 rows unless CG_OPT_GRID_CTAS, CG_OPT_DEBUG_SKIP_ARRIVAL
-                                     or CG_OPT_PHASE_TIMERS is set, graph from 2^18 rows; fp32
+                                     or CG_OPT_PHASE_TIMERS is set; with the same exceptions form 1
+                                     for stencil matrices whose vectors fit the SMs' shared memory
+                                     (about 10^6 rows); else graph from 2^18 rows; fp32
                                      FSAI refinement: graph from 2^21 rows; else persistent),
                                      1 one persistent cooperative launch, 2 CUDA graph with a
                                      device-side WHILE node (nested WHILE nodes for fp32
@@ -236,9 +238,9 @@ cg_status cg_batch_create(int32_t nsys, const int64_t* n, const int32_t* const* 
  * x[s] (host arrays of DEVICE pointers, length n[s]) are system s's rhs and
  * initial guess / solution.  One persistent cooperative kernel, captured with
  * its gather and scatter kernels in a CUDA graph (CG_OPT_LOOP_MODE 1: direct
- * launch), iterates all systems; a converged system drops out of the tile
- * schedule.  The kernel variant (registers budgeted for 3, 4 or 5 resident
- * CTAs per SM) and grid size come from an autotuner that times short trial
+ * launch), iterates all systems: teams of CTAs take one system at a time
+ * from a queue.  The kernel variant (registers budgeted for 3 or 4 resident
+ * CTAs per SM) and the number of teams come from an autotuner that times short trial
  * solves of these systems at the first solve of each (preconditioner,
  * precision kind) (x is not touched by the trials; the choice is kept in the
  * handle); CG_OPT_GRID_CTAS > 0 forces the grid instead.  iters[s] and
@@ -360,8 +362,9 @@ cg_status cg_adam_step(float* params, const float* grad, float* m, float* v, int
  * solution out); cuda_stream is a cudaStream_t (NULL = legacy default);
  * iters_out / relres_out are host pointers and may be NULL.  The solve follows
  * cg_solve's rules (relative test before each SpMV, fp64 true residual, up to
- * 3 residual-replacement restarts) but runs in a single CTA, so it suits small
- * systems only.  It blocks until the result is on the host.
+ * 3 residual-replacement restarts).  Systems of up to 32,768 rows run in one
+ * thread-block cluster, larger ones in a single CTA, so it suits small systems
+ * only.  It blocks until the result is on the host.
  *
  * Errors: CG_ERR_INVALID when n exceeds CG_NOALLOC_MAX_ROWS, a size or
  * pointer is bad, the CSR is malformed (checked on the device: rowptr[0] = 0,

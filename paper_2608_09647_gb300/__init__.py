@@ -246,7 +246,8 @@ def cg_solve_host(h: Handle, b_host, x_host, tol: float = 1e-8, maxit: int = 100
 def cg_solve_noalloc(rowptr, colind, vals, b, x, tol: float = 1e-8, maxit: int = 1000,
                      precond: int = CG_PRECOND_JACOBI):
     """Handle-free solve that allocates no device memory (for callers that cannot call
-    cudaMalloc); n <= CG_NOALLOC_MAX_ROWS, single CTA, so small systems only.  Runs on
+    cudaMalloc); n <= CG_NOALLOC_MAX_ROWS; up to 32,768 rows in one thread-block
+    cluster, above that in a single CTA (small systems only).  Runs on
     the current stream; x holds x0 on entry.  Returns (status, iters, relres_true)."""
     import torch
     n = rowptr.numel() - 1

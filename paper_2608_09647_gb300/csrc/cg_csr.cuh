@@ -3,7 +3,7 @@
 // form, and the true residuals and refinement residuals of the persistent
 // kernels.
 //
-// The rows are cut on the host into row blocks of at most kCapV nonzeros and
+// The rows are cut (on the device, at creation) into row blocks of at most kCapV nonzeros and
 // kBlock rows; a row with more than kCapV nonzeros is a block of its own (a
 // "long" block, which the CTA strides over and reduces).  spmv_rowblock_fma:
 // the block's column indices and values are copied to shared memory with
