@@ -1048,7 +1048,7 @@ __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, doubl
     update_r_phase<T, JAC>(S, V, alpha, want_rr, v2[0], v2[1], g);
     clk.lap(g.st, 2);
     bool ok;
-    if (want_rr) {
+    if (JAC && (!kWords || want_rr)) {  // by partials one form for both: a second costs more than it saves
       ok = kWords ? g.sum(v2, kKindUpd) : g.sum_parts(v2, part + kSlotUpd * (size_t)pstride);
     } else {
       double w[1] = {v2[0]};
