@@ -8,6 +8,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -507,6 +508,28 @@ cg_status cgi::ensure_host_rowptr(cg_handle* h) {
   CG_CUDA(h, cudaMemcpy(rp.data(), h->rowptr, sizeof(int32_t) * rp.size(), cudaMemcpyDeviceToHost));
   h->host_rowptr = std::move(rp);
   return CG_OK;
+}
+
+cudaError_t cgi::allow_dynamic_smem(const void* fn, size_t* limit) {
+  static std::mutex mu;
+  static std::map<std::pair<const void*, int>, size_t> known;
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto at = known.find({fn, dev});
+  if (at != known.end()) {
+    *limit = at->second;
+    return cudaSuccess;
+  }
+  cudaFuncAttributes fa{};
+  e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fn);
+  if (e != cudaSuccess) return e;
+  const size_t most = (size_t)optin > fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
+  e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  if (e == cudaSuccess) known[{fn, dev}] = *limit = most;
+  return e;
 }
 
 // Every distinct off-diagonal offset j - i of the caller's CSR, once per
@@ -1538,8 +1561,10 @@ cg_status solve_impl(cg_handle* h, const double* b, double* x, double tol, int32
     size_t smem = 0;
     if (!fp64 && ring_applies(h, G)) {
       int per_sm = 0;
-      CG_CUDA(h, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kRingBytes));
-      CG_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, kRingBytes));
+      size_t limit = 0;
+      CG_CUDA(h, cgi::allow_dynamic_smem(fn, &limit));
+      if ((size_t)kRingBytes <= limit)
+        CG_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, kRingBytes));
       if (per_sm * h->sm_count >= G) {
         P.S32.ring = (int32_t)padded(h->n);
         smem = kRingBytes;

@@ -690,10 +690,10 @@ cg_status cgi::cluster_solve(cg_handle* h, const double* b, double* x, double to
     h->err = std::string("cg_solve (cluster form): ") + where + ": " + cudaGetErrorString(e);
     return e == cudaErrorMemoryAllocation ? CG_ERR_OOM : CG_ERR_CUDA;
   };
-  int dev = 0, smem_optin = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e != cudaSuccess) return cuda_err(e, "device attributes");
+  size_t limit[2] = {};
+  cudaError_t e = cgi::allow_dynamic_smem((const void*)pcg_cluster_kernel<true>, &limit[0]);
+  if (e == cudaSuccess) e = cgi::allow_dynamic_smem((const void*)pcg_cluster_kernel<false>, &limit[1]);
+  if (e != cudaSuccess) return cuda_err(e, "shared memory size");
   // the largest cluster the device can place: 16 CTAs (non-portable), else 8
   int cmax = kClusterMax;
   for (const void* fn : {(const void*)pcg_cluster_kernel<true>, (const void*)pcg_cluster_kernel<false>}) {
@@ -716,14 +716,10 @@ cg_status cgi::cluster_solve(cg_handle* h, const double* b, double* x, double to
       const int64_t a = (int64_t)c * rows, z = std::min<int64_t>(h->n, a + rows);
       slice = std::max<int64_t>(slice, (int64_t)rp[(size_t)z] - rp[(size_t)a]);
     }
-    cudaFuncAttributes fa{};
-    if ((e = cudaFuncGetAttributes(&fa, (const void*)pcg_cluster_kernel<true>)) != cudaSuccess)
-      return cuda_err(e, "kernel attributes");
-    const bool in_smem = cluster_smem(rows, slice) + fa.sharedSizeBytes <= (size_t)smem_optin;
+    const bool in_smem = cluster_smem(rows, slice) <= limit[0];
     const void* fn = in_smem ? (const void*)pcg_cluster_kernel<true> : (const void*)pcg_cluster_kernel<false>;
     const size_t smem = cluster_smem(rows, in_smem ? slice : -1);
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return cuda_err(e, "shared memory size");
+    if (smem > limit[in_smem ? 0 : 1]) return cuda_err(cudaErrorInvalidValue, "shared memory size");
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -844,13 +840,10 @@ cudaError_t cgi::cluster_solve_checked(int n, int nnz, const int32_t* rowptr, co
   *launched = false;
   if (n > cluster_max_rows()) return cudaSuccess;
   const void* fns[2] = {(const void*)pcg_cluster_kernel<true>, (const void*)pcg_cluster_kernel<false>};
-  int dev = 0, smem_optin = 0;
-  cudaFuncAttributes fa{};
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fns[0]);
+  size_t smem = 0, limit = 0;
+  cudaError_t e = allow_dynamic_smem(fns[0], &smem);
+  if (e == cudaSuccess) e = allow_dynamic_smem(fns[1], &limit);
   if (e != cudaSuccess) return e;
-  const size_t smem = (size_t)smem_optin - fa.sharedSizeBytes;
   int cmax = kClusterMax;
   for (const void* fn : fns) {
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
@@ -880,8 +873,7 @@ cudaError_t cgi::cluster_solve_checked(int n, int nnz, const int32_t* rowptr, co
       cfg[f].stream = stream;
       cfg[f].attrs = attr;
       cfg[f].numAttrs = 1;
-      e = cudaFuncSetAttribute(fns[f], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cfg[f].dynamicSmemBytes);
-      if (e != cudaSuccess) return e;
+      if (cfg[f].dynamicSmemBytes > (f == 0 ? smem : limit)) return cudaErrorInvalidValue;
       int active = 0;
       e = cudaOccupancyMaxActiveClusters(&active, fns[f], &cfg[f]);
       placed = placed && e == cudaSuccess && active >= 1;

@@ -35,6 +35,11 @@ void fsai_free(FsaiData* f);
 void set_create_error(const std::string& msg);  // message of cg_last_error(NULL)
 cg_status ensure_offsets(cg_handle* h);         // cg_handle::offs_all, once (cg_api.cu)
 cg_status ensure_host_rowptr(cg_handle* h);     // cg_handle::host_rowptr, once (cg_api.cu)
+// *limit: the most dynamic shared memory a launch of fn on the current device may ask for
+// (the opt-in maximum less fn's static memory).  The function attribute is raised to it at
+// the first call on a device and never lowered: it belongs to the function, not to a
+// launch, and a size set for each system let another thread's launch of a larger one fail.
+cudaError_t allow_dynamic_smem(const void* fn, size_t* limit);
 // the loop in one thread-block cluster (cg_cluster.cu): fp64 CG / Jacobi-PCG of small systems
 int64_t cluster_max_rows();
 cg_status cluster_solve(cg_handle* h, const double* b, double* x, double tol, int32_t maxit, bool jac,

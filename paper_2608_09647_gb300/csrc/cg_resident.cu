@@ -313,29 +313,26 @@ const void* kernel_for(int uw, bool jac) {
 cudaError_t cgi::resident_launch(const cg_handle* h, const SolveParams& P, bool jac, int* grid, bool* launched) {
   *launched = false;
   if (!h->dia || h->n < 1) return cudaSuccess;
-  int dev = 0, optin = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   const int ctas = std::min(h->sm_count, 255);
   const int spc = (int)((h->nslices + ctas - 1) / ctas);
   for (int ms = 1; ms >= 0; --ms) {
     const void* fn = ms ? kernel_for<true>(h->uniform_w, jac) : kernel_for<false>(h->uniform_w, jac);
-    cudaFuncAttributes fa{};
-    if ((e = cudaFuncGetAttributes(&fa, fn)) != cudaSuccess) return e;
+    size_t limit = 0;
+    if ((e = allow_dynamic_smem(fn, &limit)) != cudaSuccess) return e;
     const size_t smem = sizeof(double) * 32 * (size_t)spc * (size_t)(kVecs + (ms ? h->uniform_w : 0));
-    if (smem + fa.sharedSizeBytes > (size_t)optin) continue;
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    if (smem > limit) continue;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kThreads, smem)) != cudaSuccess) return e;
-    *grid = (int)((h->nslices + spc - 1) / spc);
-    if (per_sm < 1 || *grid > per_sm * h->sm_count) continue;
+    const int G = (int)((h->nslices + spc - 1) / spc);
+    if (per_sm < 1 || G > per_sm * h->sm_count) continue;
+    *grid = G;
     if ((e = cudaMemsetAsync(h->st, 0, kStBytes, h->stream)) != cudaSuccess) return e;
     if ((e = cudaEventRecord(h->ev0, h->stream)) != cudaSuccess) return e;
     ResidentParams RP{P, spc};
     void* args[] = {&RP};
     *launched = true;
-    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)*grid), dim3(kThreads), args, smem, h->stream);
+    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)G), dim3(kThreads), args, smem, h->stream);
   }
   return cudaSuccess;
 }
