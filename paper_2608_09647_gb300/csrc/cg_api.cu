@@ -916,12 +916,22 @@ template <typename T>
 cg_status ensure_vectors(cg_handle* h, T** r, T** p, T** q, T** xh) {
   if (*r) return CG_OK;
   const size_t nv = padded(h->n);
-  CG_CUDA(h, cudaMalloc(r, 4 * sizeof(T) * nv));  // one allocation, at *r
-  if (sizeof(T) == 4)  // p's entries past n are read (times 0) by spmv_phase_ring
-    CG_CUDA(h, cudaMemset(*r + nv, 0, sizeof(T) * nv));
-  *p = *r + nv;
-  *q = *p + nv;
-  *xh = *q + nv;
+  T* base = nullptr;
+  CG_CUDA(h, cudaMalloc(&base, 4 * sizeof(T) * nv));  // one allocation, at *r
+  if (sizeof(T) == 4) {  // p's entries past n are read (times 0) by spmv_phase_ring
+    // waited for: the solve's stream need not be ordered after the legacy stream's work,
+    // and a late clear would hit the p of a solve under way
+    cudaError_t e = cudaMemset(base + nv, 0, sizeof(T) * nv);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+    if (e != cudaSuccess) {
+      cudaFree(base);
+      return cuda_fail(h, e, "work vectors");
+    }
+  }
+  *r = base;
+  *p = base + nv;
+  *q = base + 2 * nv;
+  *xh = base + 3 * nv;
   return CG_OK;
 }
 
