@@ -106,8 +106,9 @@ typedef struct {
                              (Jacobi; 88 n without; fp32 refinement 8 nnz + 4(n+1) + 52/44 n) */
   int64_t kernel_bytes_per_iter; /* bytes one iteration of this library's loop must move:
                              its off-diagonal slices (fp64: 8 B/entry in the diagonal layout,
-                             12 B with a column array; fp32: 4 / 8 B) plus 88 n (Jacobi) /
-                             80 n bytes of vectors (fp64; half that in fp32) */
+                             12 B with a column array; fp32: 4 / 8 B, of half the slots where
+                             the persistent loop reads a symmetric matrix's mirrored values)
+                             plus 88 n (Jacobi) / 80 n bytes of vectors (fp64; half that in fp32) */
   double phase_ms[6];     /* with CG_OPT_PHASE_TIMERS: CTA 0 time in the SpMV, r-update and
                              x/p-update phases, each followed by its grid-barrier wait */
   int32_t loop_form;      /* CG_OPT_LOOP_MODE form that ran: 1 persistent, 2 graph WHILE, 3 unrolled,

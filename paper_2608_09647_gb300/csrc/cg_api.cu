@@ -784,33 +784,32 @@ cg_status ensure_offdiag(cg_handle* h) {
 // reads are the less regular ones.
 constexpr int64_t kSymMinBytes = (int64_t)1 << 20, kSymMaxBytes = (int64_t)63 << 20;
 
-template <typename T>
-__global__ void symmetry_kernel(int64_t n, int nd, DiaOffsets delta, const T* __restrict__ val, int* __restrict__ bad) {
+__global__ void symmetry_kernel(int64_t n, int nd, DiaOffsets delta, const float* __restrict__ val,
+                                int* __restrict__ bad) {
   int differ = 0;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     for (int m = 0; m < nd / 2; ++m) {
       const int64_t j = i + delta.d[m];
-      const T a = val[((i >> 5) * nd + m) * 32 + (i & 31)];
-      const T b = j >= 0 ? val[((j >> 5) * nd + nd - 1 - m) * 32 + (j & 31)] : T(0);
+      const float a = val[((i >> 5) * nd + m) * 32 + (i & 31)];
+      const float b = j >= 0 ? val[((j >> 5) * nd + nd - 1 - m) * 32 + (j & 31)] : 0.0f;
       differ |= !(a == b);
     }
   }
   if (__syncthreads_or(differ) && threadIdx.x == 0) *bad = 1;
 }
 
-template <typename T>
-cg_status check_symmetry(cg_handle* h, const T* val, const DiaOffsets& d, int32_t* sym) {
+cg_status check_symmetry(cg_handle* h, const float* val, const DiaOffsets& d, int32_t* sym) {
   const int nd = h->uniform_w;
   *sym = 0;
-  const int64_t resident = (int64_t)sizeof(T) * (h->sell_entries / 2 + 4 * h->n);
-  if (sizeof(T) != 4 || (nd != 4 && nd != 6 && nd != 8) || resident < kSymMinBytes || resident > kSymMaxBytes)
+  const int64_t resident = (int64_t)sizeof(float) * (h->sell_entries / 2 + 4 * h->n);
+  if ((nd != 4 && nd != 6 && nd != 8) || resident < kSymMinBytes || resident > kSymMaxBytes)
     return CG_OK;
   for (int m = 0; m < nd / 2; ++m)
     if (d.d[m] >= 0 || d.d[m] != -d.d[nd - 1 - m]) return CG_OK;
   int* bad = &h->st->status;  // free between solves
   int host = 0;
   CG_CUDA(h, cudaMemset(bad, 0, sizeof(int)));
-  symmetry_kernel<T><<<grid_for(h->n), 256>>>(h->n, nd, d, val, bad);
+  symmetry_kernel<<<grid_for(h->n), 256>>>(h->n, nd, d, val, bad);
   CG_CUDA(h, cudaGetLastError());
   CG_CUDA(h, cudaMemcpy(&host, bad, sizeof(int), cudaMemcpyDeviceToHost));
   *sym = host == 0;
@@ -850,8 +849,10 @@ cg_status ensure_vals(cg_handle* h, T** sval, T** lval, bool scale) {
                       : (few ? fill_dia_kernel<T, false, 8> : fill_dia_kernel<T, false, 0>);
     fill<<<grid_for(h->n), 256>>>(h->n, h->rowptr, h->colind, h->vals, h->disq, h->uniform_w, d, *sval);
     CG_CUDA(h, cudaGetLastError());
-    const cg_status ss = check_symmetry(h, *sval, d, &h->sym32[scale]);
-    if (ss != CG_OK) return ss;
+    if constexpr (sizeof(T) == 4) {  // (sym32 is the fp32 values': the fp64 ones, built later, leave it)
+      const cg_status ss = check_symmetry(h, *sval, d, &h->sym32[scale]);
+      if (ss != CG_OK) return ss;
+    }
     CG_CUDA(h, cudaDeviceSynchronize());
     return CG_OK;
   }
@@ -1607,7 +1608,7 @@ cg_status solve_impl(cg_handle* h, const double* b, double* x, double tol, int32
   h->last.bytes_moved = per_iter * (int64_t)ds.iters;
   // bytes this kernel's loop must move per iteration: the SELL-32 slices
   // (padding included), the long-row CSR and the vector streams
-  const int64_t ent = h->sell_entries + h->nnz_long;
+  const int64_t ent = (h->sell_entries >> (!fp64 && P.S32.sym ? 1 : 0)) + h->nnz_long;  // (half of mirrored slices)
   const int64_t cb = h->dia ? 0 : 4;  // column bytes per entry
   const int64_t vb = 80 + (jac && h->dmin != h->dmax ? 8 : 0);  // vector bytes per row (fp64)
   h->last.kernel_bytes_per_iter = fp64 ? (8 + cb) * ent + 4 * (int64_t)h->nlong + vb * n
