@@ -440,7 +440,7 @@ __device__ __forceinline__ void report(const Team& T, const Control& c, int s) {
 template <bool JAC>
 __device__ __forceinline__ void after_update(Control& c, double rho1, double rr, double dmin, double stop2,
                                              int maxit) {
-  c.beta = rho1 * c.inv_rho;
+  c.beta = beta_of(rho1, c.rho, c.inv_rho);
   c.rho_k = c.rho;  // r.z of the step just taken (the carry's denominator)
   c.rho = rho1;
   c.k += 1;

@@ -555,8 +555,7 @@ __global__ void __launch_bounds__(kBlock, 1) pcg_cluster_kernel(ClusterParams P)
       }
       push_sums<1>(v1, X, rank, C, (int)(e & 1u), P.skip_seq == e + 1u && rank == 0);
       // 1 / rho for this iteration's beta, on another SM sub-partition while warp 0
-      // waits for p.q and forms alpha: beta = rho' (1 / rho) costs a multiply on
-      // the path where rho' / rho cost a division (within 1.5 ulp of it)
+      // waits for p.q and forms alpha (beta_of)
       if (t == 32) s_inv_rho = 1.0 / s_rho;
       if (t < 32) {
         const bool ok = wait_sums(X, e, tmo);
@@ -623,7 +622,7 @@ __global__ void __launch_bounds__(kBlock, 1) pcg_cluster_kernel(ClusterParams P)
             record_timeout();
             st_in = kTimeout;
           } else {
-            s_beta = s2[0] * s_inv_rho;
+            s_beta = beta_of(s2[0], rho, s_inv_rho);
             rho = s2[0];
             s_rho = rho;
             rr = s2[1];

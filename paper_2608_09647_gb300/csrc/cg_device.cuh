@@ -218,6 +218,14 @@ __device__ __forceinline__ void cta_sum0(double (&v)[NV]) {
   }
 }
 
+// beta = rho' / rho as rho' (1 / rho), a multiply on the critical path where a division
+// would be (within 1.5 ulp of it); the division itself where 1 / rho is not a normal
+// number (rho below about 2^-1024 would make it infinite, above 2^1022 lose bits).
+__device__ __forceinline__ double beta_of(double rho1, double rho, double inv_rho) {
+  const unsigned e = ((unsigned)__double2hiint(inv_rho) >> 20) & 0x7FFu;
+  return e - 1u < 0x7FEu ? rho1 * inv_rho : rho1 / rho;
+}
+
 // Sum of v over the CTA in a fixed order (warp xor-tree, then warp 0 over the
 // per-warp sums); the result is returned to every thread.
 template <int NV>

@@ -297,8 +297,7 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
     __syncthreads();
     if (s_fl) { status = s_fl; break; }
     const T alpha = (T)s_sc[0];
-    // 1 / rho for this iteration's beta, in warp 1 during the r update: beta =
-    // rho' (1 / rho) is a multiply after the next grid sum (within 1.5 ulp of rho' / rho)
+    // 1 / rho for this iteration's beta (beta_of), in warp 1 during the r update
     __shared__ double s_inv_rho;
     if (threadIdx.x == 32) s_inv_rho = 1.0 / rho;
     Acc<T> a_rho, a_rr;
@@ -321,7 +320,7 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
     double s2[2] = {a_rho.get(), a_rr.get()};
     const bool ok2 = kWords ? g.sum(s2, kKindUpd) : g.sum_parts(s2, part + kSlotUpd * (size_t)pstride);
     if (threadIdx.x == 0) {
-      s_sc[1] = s2[0] * s_inv_rho;
+      s_sc[1] = beta_of(s2[0], rho, s_inv_rho);
       s_sc[2] = s2[0];
       s_sc[3] = s2[1];
       s_fl = !ok2 ? kTimeout : (below_stop(s2[1], stop_abs, stop2_hi) ? 1 : 0);

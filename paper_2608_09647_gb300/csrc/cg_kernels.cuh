@@ -1040,8 +1040,7 @@ __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, doubl
     if (s_st) { status = s_st; break; }
     const T alpha = (T)s_alpha;
     // a2: r^ -= alpha q; r.z, r.r (r.r only when the test needs it).  1 / rho for
-    // this iteration's beta in warp 1 meanwhile: beta = rho' (1 / rho) is a multiply
-    // after the exchange (within 1.5 ulp of rho' / rho)
+    // this iteration's beta (beta_of) in warp 1 meanwhile
     const bool want_rr = s_want != 0;
     if (threadIdx.x == 32) s_inv_rho = 1.0 / rho;
     double v2[2] = {0.0, 0.0};
@@ -1060,7 +1059,7 @@ __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, doubl
       double rr_ = v2[1];
       if (!ok) s_st = kTimeout;
       s_exact = JAC && !want_rr && rr_bound_test(S, v2[0], stop_abs * stop_abs, &rr_) < 0;
-      s_beta = v2[0] * s_inv_rho;
+      s_beta = beta_of(v2[0], rho, s_inv_rho);
       s_rho = v2[0];
       s_rr = rr_;
       s_conv = below_stop(rr_, stop_abs, stop2_hi);

@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kThreads, 1) pcg64_resident_kernel(ResidentPar
       __syncthreads();
       if (s_st) { st = s_st; break; }
       // a2: r^ -= alpha q; r.z, r.r (r.r only when the test needs it); 1 / rho for
-      // this iteration's beta in warp 1 meanwhile (beta = rho' (1 / rho))
+      // this iteration's beta (beta_of) in warp 1 meanwhile
       const double alpha = s_alpha;
       const bool want_rr = s_want != 0;
       if (t == 32) s_inv_rho = 1.0 / rho;
@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kThreads, 1) pcg64_resident_kernel(ResidentPar
         double rr_ = x2.v1;
         if (!x2.ok) s_st = kTimeout;
         s_exact = JAC && !want_rr && rr_bound_test(S, x2.v0, stop * stop, &rr_) < 0;
-        s_beta = x2.v0 * s_inv_rho;
+        s_beta = beta_of(x2.v0, rho, s_inv_rho);
         s_rho = x2.v0;
         s_rr = rr_;
         s_conv = below_stop(rr_, stop, stop2_hi);
