@@ -73,7 +73,9 @@ typedef enum {
   CG_OPT_IR_MAX_OUTER = 4,        /* refinement steps / reliable updates cap (default 30) */
   CG_OPT_DEBUG_SKIP_ARRIVAL = 5,  /* fault injection: CTA 0 skips arrival at grid barrier #value
                                      (cluster form: does not push exchange #value; 1-based; 0 = off),
-                                     so every wait runs into its limit */
+                                     so every wait runs into its limit; 2^30 + k: in the fp32
+                                     refinement of a 27-point matrix, a warp of CTA 0 does not start
+                                     its k-th copy of values to shared memory */
   CG_OPT_PHASE_TIMERS = 6,        /* 1: record CTA 0's time per loop phase in cg_solve_info */
   CG_OPT_LOOP_MODE = 7            /* loop form: 0 auto (fp64 Jacobi / plain CG: cluster form up to
                                      16384 rows unless CG_OPT_GRID_CTAS, CG_OPT_DEBUG_SKIP_ARRIVAL

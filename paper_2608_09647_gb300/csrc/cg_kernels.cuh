@@ -457,6 +457,7 @@ constexpr int kRingChunkBytes = kRingChunk * 32 * (int)sizeof(float);
 constexpr int kRingBars = 128 * ((kWarps * kRingDepth * 8 + 127) / 128);
 constexpr int kRuns = 9, kRunPieces = 10;         // 16-byte pieces of a run: 3 + 34 entries at most
 constexpr int kWinDepth = 2, kWinBytes = kRuns * kRunPieces * 16;
+constexpr unsigned kSkipCopy = 1u << 30;          // skip_seq beyond every barrier's number: a ring's copy
 constexpr int kRingBytes = kRingBars + kWarps * (kRingDepth * kRingChunkBytes + kWinDepth * kWinBytes);
 
 struct Ring {
@@ -496,24 +497,36 @@ struct Ring {
         "l"(src), "r"(kRingChunkBytes), "r"(b), "l"(policy)
         : "memory");
   }
-  // all lanes: chunk f has arrived (bounded; on giving up the launch is marked aborted)
-  __device__ __forceinline__ void wait(unsigned f, const Grid& g) const {
+  // all lanes: whether chunk f has arrived (false: not within timeout_ns)
+  __device__ __forceinline__ bool wait(unsigned f, uint64_t timeout_ns) const {
     const unsigned b = bar + 8 * (f % kRingDepth), parity = (f / kRingDepth) & 1u;
     uint64_t t0 = 0;
+    unsigned ok;
     for (unsigned spins = 0;; ++spins) {
-      unsigned ok;
       asm volatile(
           "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
           : "=r"(ok)
           : "r"(b), "r"(parity)
           : "memory");
-      if (ok) return;
+      if (ok) break;
       if (spins == 0) t0 = global_timer_ns();
-      else if ((spins & 15u) == 0u && global_timer_ns() - t0 > g.timeout_ns) {
-        atomicExch(&g.st->abort, 1);
-        return;
-      }
+      else if ((spins & 15u) == 0u && global_timer_ns() - t0 > timeout_ns) break;
     }
+    return __all_sync(0xffffffffu, ok != 0u);
+  }
+  // the warp's wait for chunk f gave up: the launch is marked aborted and the copies still
+  // under way (chunks f to end - 1, the windows) are waited for, with the same limit each,
+  // since the CTA must not leave while they write its shared memory.  The NaN makes the
+  // phase's sum NaN, which ends the loop in every CTA.
+  __device__ __noinline__ double gave_up(DevState* st, unsigned barrier, uint64_t timeout_ns, unsigned f,
+                                         unsigned end) const {
+    if ((threadIdx.x & 31) == 0 && atomicCAS(&st->abort, 0, 1) == 0) {
+      st->err_cta = (int)blockIdx.x;
+      st->err_barrier = (int)barrier;
+    }
+    for (; f != end; ++f) wait(f, timeout_ns);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    return __longlong_as_double(0x7FF8000000000000ll);
   }
   __device__ __forceinline__ const float* chunk(unsigned f) const { return mem + (f % kRingDepth) * (kRingChunkBytes / 4); }
 };
@@ -521,7 +534,8 @@ struct Ring {
 // a1 over the grid by the ring, one slice a warp at a time.  Slot m reads position m' = m
 // (m < 13) or m + 1 of the 27 ordered offsets, the diagonal's among them: run m' / 3, its
 // entry m' % 3 + lane.
-// (S.ring is the allocated length of p, whose entries past n are 0.)
+// (S.ring is the allocated length of p, whose entries past n are 0.)  Fault injection:
+// with skip_seq = kSkipCopy + k, CTA 0's first warp does not start its k-th chunk.
 template <bool JAC>
 __device__ __forceinline__ double spmv_phase_ring(const Sell<float>& S, const float* __restrict__ p,
                                                   float* __restrict__ q, Grid& g) {
@@ -535,8 +549,11 @@ __device__ __forceinline__ double spmv_phase_ring(const Sell<float>& S, const fl
   const auto source = [&](int c) {  // chunk c of this warp's slices
     return S.val + (int64_t)(s0 + (c >> 1) * Wt) * (kRingW * 32) + (c & 1) * (kRingChunk * 32);
   };
+  const auto fill = [&](int c) {
+    if (threadIdx.x != 0 || g.cta != 0 || g.skip_seq != kSkipCopy + 1u + f0 + c) R.fill(f0 + c, source(c));
+  };
   if (lane == 0)
-    for (int c = 0; c < kRingDepth && c < 2 * slices; ++c) R.fill(f0 + c, source(c));
+    for (int c = 0; c < kRingDepth && c < 2 * slices; ++c) fill(c);
   constexpr int kPer = (kRuns * kRunPieces + 31) / 32;
   int off[kPer];  // this lane's pieces: their place in p from the slice's first row
 #pragma unroll
@@ -571,7 +588,8 @@ __device__ __forceinline__ double spmv_phase_ring(const Sell<float>& S, const fl
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const unsigned f = f0 + 2 * k + h;
-      R.wait(f, g);
+      if (!R.wait(f, g.timeout_ns))
+        return R.gave_up(g.st, g.seq + 1, g.timeout_ns, f, f0 + min(2 * slices, 2 * k + h + kRingDepth));
       const float* v = R.chunk(f) + lane;
 #pragma unroll
       for (int u = 0; u < kRingChunk; ++u) {
@@ -580,7 +598,7 @@ __device__ __forceinline__ double spmv_phase_ring(const Sell<float>& S, const fl
       }
       __syncwarp();  // the chunk (and with h = 1 the windows) have been read
       const int c = 2 * k + h + kRingDepth;
-      if (lane == 0 && c < 2 * slices) R.fill(f0 + c, source(c));
+      if (lane == 0 && c < 2 * slices) fill(c);
     }
     if (i < n) {
       q[i] = acc;
