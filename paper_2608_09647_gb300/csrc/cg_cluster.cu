@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(kBlock, 1) pcg_cluster_kernel(ClusterParams P)
       // ---- B: r -= alpha q, z = D^-1 r; r.z, r.r; then x += alpha p while they are in
       // flight (plain CG: z is r and r.z is r.r, one sum)
       arm(P.jac ? 2 : 1);
-      const double alpha = s_alpha;
+      const double alpha = s_alpha, inv_rho = s_inv_rho;  // (read before the wait, off the path after it)
       const double* pcur = par ? pb1 : pb0;
       if (P.jac) {
         double v2[2] = {0.0, 0.0};
@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(kBlock, 1) pcg_cluster_kernel(ClusterParams P)
             record_timeout();
             st_in = kTimeout;
           } else {
-            s_beta = beta_of(s2[0], rho, s_inv_rho);
+            s_beta = beta_of(s2[0], rho, inv_rho);
             rho = s2[0];
             s_rho = rho;
             rr = s2[1];
