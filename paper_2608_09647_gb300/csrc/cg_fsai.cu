@@ -243,7 +243,7 @@ struct FsaiParams {
 // rho_prev > 0 (reliable updates, R8) p = G^T t + (rho / rho_prev) p.
 template <int W, typename T>
 __device__ bool fsai_start(const Ell<T>& G, const Ell<T>& GT, const FsaiVecs<T>& V, const T* r, int64_t n,
-                           Grid& g, double* rho, double rho_prev = 0.0) {
+                           double* part, int pstride, Grid& g, double* rho, double rho_prev = 0.0) {
   Acc<T> a;
   rows_x2(
       g, n, [&](int64_t i) { return ell_row<W>(G, i, n, [&](int j) { return r[j]; }); },
@@ -252,7 +252,8 @@ __device__ bool fsai_start(const Ell<T>& G, const Ell<T>& GT, const FsaiVecs<T>&
         a.add(s, s);
       });
   double v[1] = {a.get()};
-  if (!g.sum_all(v)) return false;
+  const bool ok = sizeof(T) == 8 ? g.sum_all(v, kKindStart) : g.sum_parts(v, part + kSlotStart * (size_t)pstride);
+  if (!ok) return false;
   *rho = v[0];
   const bool carry = rho_prev > 0.0;
   const T beta = carry ? (T)(v[0] / rho_prev) : T(0);
@@ -397,7 +398,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai64_kernel(FsaiParams F) {
     }
     first = false;
     double rho = 0.0;
-    if (!fsai_start<W, double>(F.G64, F.GT64, V, V.r0, n, g, &rho)) { status = kTimeout; break; }
+    if (!fsai_start<W, double>(F.G64, F.GT64, V, V.r0, n, P.part, P.pstride, g, &rho)) { status = kTimeout; break; }
     const int st = fsai_loop<W, double>(P.S64, F.G64, F.GT64, V, rho, rr_start, P.tol * sqrt(bb), P.maxit, &k,
                                      P.part, P.pstride, g);
     if (st == kTimeout) { status = kTimeout; break; }
@@ -430,8 +431,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai64_kernel(FsaiParams F) {
 template <int W, bool CARRY>
 __global__ void __launch_bounds__(kBlock, 2) pcg_fsai_ir_kernel(FsaiParams F) {
   const SolveParams& P = F.P;
-  __shared__ XState s_x;
-  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
+  Grid g(P.st, P.timeout_ns, P.skip_seq);
   const int64_t n = P.A.n;
   const FsaiVecs<float>& V = F.V32;
   int status = kNotConverged, inner = 0, outer = 0;
@@ -450,7 +450,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai_ir_kernel(FsaiParams F) {
       v[1] += bi * bi;
       v[2] += (double)r32 * (double)r32;
     }
-    if (!g.sum_all(v)) { status = kTimeout; break; }
+    if (!g.sum_parts(v, P.part + kSlotRes * (size_t)P.pstride)) { status = kTimeout; break; }
     const double(&s3)[3] = v;
     if (outer == 0) {
       bb = s3[1];
@@ -465,8 +465,8 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai_ir_kernel(FsaiParams F) {
     if (relres <= P.tol) { status = kOk; break; }
     if (outer >= P.max_restarts || inner >= P.maxit) { status = kNotConverged; break; }
     double rho = 0.0;
-    if (!fsai_start<W, float>(F.G32, F.GT32, V, V.r0, n, g, &rho,
-                                CARRY && outer > 0 ? rho_k : 0.0)) { status = kTimeout; break; }
+    if (!fsai_start<W, float>(F.G32, F.GT32, V, V.r0, n, P.part, P.pstride, g, &rho,
+                              CARRY && outer > 0 ? rho_k : 0.0)) { status = kTimeout; break; }
     const int st = fsai_loop<W, float>(P.S32, F.G32, F.GT32, V, rho, s3[2], P.tol_in * sqrt(s3[2]), P.maxit, &inner,
                                     P.part, P.pstride, g, &rho_k);
     if (st == kTimeout || st == kNumeric || st == kBreakdown) { status = st; break; }
@@ -493,7 +493,6 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai_ir_kernel(FsaiParams F) {
 // Every phase is its own kernel (the kernel boundaries are the barriers).  The
 // last CTA of a reducing kernel sums its fixed-order partials once and stores
 // the scalars for the next kernel, so no CTA waits on a reduction at its start.
-constexpr int kSlotT = kSlotRes + 3;  // t.t of the start pass
 constexpr int64_t kFsaiGraphMinRows = 1 << 21;  // auto loop form: graph from here (fp32 inner)
 constexpr int kFsaiUnroll = 8;                   // inner iterations per graph of the unrolled form
 constexpr int kFsaiOuterKernels = 6;             // kernels of one outer step
@@ -542,7 +541,7 @@ __global__ void __launch_bounds__(kBlock, kFsaiPhaseCtas) gf_t(FArgs F) {
     a.add(s, s);
   }
   double v[1] = {a.get()};
-  publish<1>(v, P.part + kSlotT * (size_t)P.pstride, g);
+  publish<1>(v, P.part + kSlotStart * (size_t)P.pstride, g);
 }
 
 // One CTA: the fp64 residual test and limits; the next inner solve's state.
@@ -551,7 +550,7 @@ __global__ void gf_start(FArgs F) {
   const SolveParams& P = F.a.P;
   double s[3], tt[1];
   grid_sum<3>(P.part + kSlotRes * (size_t)P.pstride, F.a.G_upd, s);
-  grid_sum<1>(P.part + kSlotT * (size_t)P.pstride, F.a.G_upd, tt);
+  grid_sum<1>(P.part + kSlotStart * (size_t)P.pstride, F.a.G_upd, tt);
   if (threadIdx.x != 0) return;
   GState* gs = F.a.gs;
   if (!gs->started) {

@@ -149,10 +149,12 @@ struct SolveParams {
 // update phase, 4..7 = the residual phase.  Disjoint slots mean a CTA never overwrites a
 // partial that a slower CTA still has to read.
 constexpr int kParts = 8;
-constexpr int kSlotPQ = 0, kSlotRr = 1, kSlotUpd = 2, kSlotRes = 4;
+constexpr int kSlotPQ = 0, kSlotRr = 1, kSlotUpd = 2, kSlotRes = 4, kSlotStart = kSlotRes + 3;
 
-// Kinds of the loops' sums (their scales are kept apart).
-constexpr int kKindPQ = 0, kKindUpd = 1, kKindRr = 3, kKindRes = 4;
+// Kinds of the loops' sums (their scales are kept apart: two quantities of one kind would
+// find the other's scale, and a sum that does not suit the scale is formed anew, in two
+// more rounds).  The residual phase's up to three, and the start's r.z with FSAI.
+constexpr int kKindPQ = 0, kKindUpd = 1, kKindRr = 3, kKindRes = 4, kKindStart = 7;
 
 // Grid coordinates and the exchanges of one persistent launch.
 struct Grid {
@@ -165,11 +167,13 @@ struct Grid {
   unsigned fills;  // this warp's ring chunks so far (spmv_phase_ring)
   __device__ Grid() : G(gridDim.x), cta(blockIdx.x), gtid((int64_t)blockIdx.x * kBlock + threadIdx.x),
         gstride((int64_t)gridDim.x * kBlock), st(nullptr), x(nullptr), timeout_ns(0), seq(0), skip_seq(0), fills(0) {}
-  __device__ Grid(DevState* s, XWord* words, XState* xs, uint64_t to, unsigned skip) : Grid() {
+  __device__ Grid(DevState* s, uint64_t to, unsigned skip) : Grid() {
     st = s;
-    x = xs;
     timeout_ns = to;
     skip_seq = skip;
+  }
+  __device__ Grid(DevState* s, XWord* words, XState* xs, uint64_t to, unsigned skip) : Grid(s, to, skip) {
+    x = xs;
     x_init(xs, s, words, gridDim.x, blockIdx.x, blockIdx.x == 0 ? skip : 0u, to);
   }
   // a barrier; false: a wait gave up, leave the kernel
@@ -185,20 +189,23 @@ struct Grid {
     return r.ok;
   }
   // the same through per-CTA partials part[j G + cta] that every CTA adds up after a
-  // plain barrier, the sums in every thread: the fp32 loops' form.  Their phases end
+  // plain barrier, the sums in every thread: the fp32 kernels' form.  Their phases end
   // more unevenly, and CTAs that poll an exchange's words slow the ones still at work
-  // (27-point 160^3, 304 CTAs: 146.5 us an iteration against 148.7).
+  // (27-point 160^3, 304 CTAs: 146.5 us an iteration against 148.7); a residual's sums,
+  // up to four, cost one barrier.  A slot of part is written again only after another
+  // barrier: a slower CTA may still be reading it until then.
   template <int NV>
   __device__ __forceinline__ bool sum_parts(double (&v)[NV], double* part);
-  // the exchange for up to 4 values, the sums given to every thread (the residual phases)
+  // exchanges for up to 3 values of kinds `kind`, ..., the sums given to every thread
+  // (the residual phases)
   template <int NV>
-  __device__ __forceinline__ bool sum_all(double (&v)[NV]) {
+  __device__ __forceinline__ bool sum_all(double (&v)[NV], int kind = kKindRes) {
     __shared__ double s_out[NV];
 #pragma unroll
     for (int j = 0; j < NV; j += 2) {
       const bool two = j + 1 < NV;
       double w2[2] = {v[j], v[two ? j + 1 : j]}, w1[1] = {v[j]};
-      const bool ok = two ? sum<2>(w2, kKindRes) : sum<1>(w1, kKindRes);
+      const bool ok = two ? sum<2>(w2, kind + j) : sum<1>(w1, kind + j);
       if (threadIdx.x == 0) {
         s_out[j] = two ? w2[0] : w1[0];
         if (two) s_out[j + 1 < NV ? j + 1 : j] = w2[1];
@@ -1225,8 +1232,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg64_kernel(SolveParams P) {
 // rho_k) p_k, instead of restarting from p = r^'.
 template <bool JAC, bool CARRY>
 __global__ void __launch_bounds__(kBlock, 2) pcg_ir_kernel(SolveParams P) {
-  __shared__ XState s_x;
-  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
+  Grid g(P.st, P.timeout_ns, P.skip_seq);
   PhaseClock clk(P.timers != 0);
   if (P.S32.ring) Ring().init();
   const int64_t n = P.A.n;
@@ -1252,7 +1258,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_ir_kernel(SolveParams P) {
       v[2] += rh2;
       v[3] += JAC ? (double)__ldg(P.S32.dn + i) * rh2 : rh2;
     }
-    if (!g.sum_all(v)) { status = kTimeout; break; }
+    if (!g.sum_parts(v, P.part + kSlotRes * (size_t)P.pstride)) { status = kTimeout; break; }
     const double(&s4)[4] = v;
     if (outer == 0) {
       bb = s4[1];

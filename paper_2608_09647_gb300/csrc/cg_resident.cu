@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kThreads, 1) pcg64_resident_kernel(ResidentPar
       s_sum[1] = a.v1;
     }
     if (!__syncthreads_and(a.ok)) { status = kTimeout; break; }
-    const XSums c = grid_exchange<1, kRWarps, true>(&s_x, kKindRes, v[2], 0.0);
+    const XSums c = grid_exchange<1, kRWarps, true>(&s_x, kKindRes + 2, v[2], 0.0);
     if (t == 0) s_sum[2] = c.v0;
     if (!__syncthreads_and(c.ok)) { status = kTimeout; break; }
     const double rho0 = s_sum[0], rr0 = s_sum[1];
