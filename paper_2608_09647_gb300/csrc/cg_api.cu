@@ -422,6 +422,18 @@ std::vector<int32_t> build_row_blocks(const int32_t* rowptr, int64_t n, int64_t*
 
 size_t padded(int64_t n) { return ((size_t)std::max<int64_t>(n, 1) + 63) / 64 * 64; }
 
+const void* refinement_kernel(bool jac, bool carry, int product) {
+  if (product == kStaged)
+    return carry ? (jac ? (const void*)pcg_ir_kernel<true, true, kStaged> : (const void*)pcg_ir_kernel<false, true, kStaged>)
+                 : (jac ? (const void*)pcg_ir_kernel<true, false, kStaged> : (const void*)pcg_ir_kernel<false, false, kStaged>);
+  if (product == kMirrored)
+    return carry
+               ? (jac ? (const void*)pcg_ir_kernel<true, true, kMirrored> : (const void*)pcg_ir_kernel<false, true, kMirrored>)
+               : (jac ? (const void*)pcg_ir_kernel<true, false, kMirrored> : (const void*)pcg_ir_kernel<false, false, kMirrored>);
+  return carry ? (jac ? (const void*)pcg_ir_kernel<true, true, kAsStored> : (const void*)pcg_ir_kernel<false, true, kAsStored>)
+               : (jac ? (const void*)pcg_ir_kernel<true, false, kAsStored> : (const void*)pcg_ir_kernel<false, false, kAsStored>);
+}
+
 template <typename K>
 int max_coresident(K kernel, int sm_count) {
   int per_sm = 0;
@@ -440,11 +452,11 @@ void residency(int dev, int sm_count, int* persistent, int* vectors) {
   int* k = known[dev < 0 || dev >= kMaxDevices ? 0 : dev];
   if (k[0] <= 0 || k[1] <= 0 || dev < 0 || dev >= kMaxDevices) {
     int g = kXCtas;
-    for (int r : {max_coresident(pcg64_kernel<true>, sm_count), max_coresident(pcg64_kernel<false>, sm_count),
-                  max_coresident(pcg_ir_kernel<true, false>, sm_count), max_coresident(pcg_ir_kernel<true, true>, sm_count),
-                  max_coresident(pcg_ir_kernel<false, false>, sm_count),
-                  max_coresident(pcg_ir_kernel<false, true>, sm_count)})
+    for (int r : {max_coresident(pcg64_kernel<true>, sm_count), max_coresident(pcg64_kernel<false>, sm_count)})
       g = std::min(g, r);
+    for (int product : {kAsStored, kStaged, kMirrored})
+      for (int f = 0; f < 4; ++f)
+        g = std::min(g, max_coresident(refinement_kernel((f & 1) != 0, (f & 2) != 0, product), sm_count));
     int v = max_coresident(g_res64<true>, sm_count);
     for (int r : {max_coresident(g_upd_r<double, true>, sm_count), max_coresident(g_upd_r<double, false>, sm_count),
                   max_coresident(g_upd_xp<float, true, true, true>, sm_count),
@@ -480,10 +492,15 @@ unsigned spmv_grid(const cg_handle* h) {
 }
 
 // Whether the fp32 loop's SpMV takes its ring (spmv_phase_ring): 26 off-diagonal offsets
-// in runs of three neighbours, the middle one around the diagonal, and slices enough for
-// every warp to run ahead (two chunks a slice, a ring of three).
+// in runs of three neighbours, the middle one around the diagonal, and 16 slices a warp.
+// On the whole chip that is 1.25 million rows, whose 130 MB of values are as large as the
+// L2: where they stay in it, the loads into registers find them there, and the ring's
+// copies, which ask L2 not to keep them, do not.  Refinement to 1e-12, ms, loads and ring,
+// ir: 68^3 rows 3.42 and 3.67, 104^3 7.01 and 7.33, 108^3 7.67 and 7.80, 124^3 10.4 and
+// 9.94, 150^3 17.6 and 16.9; ru: 74^3 5.21 and 5.36, 104^3 9.49 and 9.34, 124^3 14.6 and
+// 13.5, 150^3 24.7 and 23.2.
 bool ring_applies(const cg_handle* h, int G) {
-  constexpr int64_t kMinSlices = 4;  // of a warp
+  constexpr int64_t kMinSlices = 16;  // of a warp
   if (!h->dia || h->uniform_w != kRingW || h->nslices < kMinSlices * G * kWarps) return false;
   const auto at = [&](int k) { return k < 13 ? h->delta[k] : k == 13 ? 0 : h->delta[k - 1]; };
   for (int k = 0; k < 27; k += 3)
@@ -777,12 +794,15 @@ cg_status ensure_offdiag(cg_handle* h) {
 // *sym = whether slot m of row i and slot nd-1-m of row i + delta[m] are the same number,
 // bit for bit, everywhere (Sell::sym).  Only asked where the persistent SpMV gains by
 // reading half of the slices: while that half and the loop's four vectors stay in the
-// near half of the 126 MB L2.  Refinement, us an iteration, all slots read and half:
-// 7 points 128^3 rows (59 MB) 30.3 and 27.1, 160^3 (115 MB) 47.6 and 54.6; Q1 1000^2
-// (32 MB) 20.8 and 19.4, 2000^2 (128 MB) 48.0 and 62.9; 5 points 1000^2 (24 MB) 17.7 and
-// 16.7, 2000^2 (96 MB) 38.9 and 42.8.  Larger systems stream either way, and the mirrored
-// reads are the less regular ones.
-constexpr int64_t kSymMinBytes = (int64_t)1 << 20, kSymMaxBytes = (int64_t)63 << 20;
+// near half of the 126 MB L2, and are enough for bandwidth to count.  Refinement, us an
+// iteration, all slots read and half: 7 points 70^3 rows (10 MB) 17.1 and 17.4, 80^3
+// (14 MB) 19.7 and 19.2, 100^3 (28 MB) 26.4 and 24.9, 126^3 (56 MB) 37.2 and 34.8, 160^3
+// (115 MB) 47.6 and 54.6; 9 points 600^2 (12 MB) 17.1 and 17.5, 800^2 (20 MB) 22.3 and
+// 21.3, 1400^2 (63 MB) 39.7 and 35.7; Q1 2000^2 (128 MB) 48.0 and 62.9; 5 points 600^2
+// (9 MB) 16.1 and 16.3, 800^2 (15 MB) 18.5 and 18.5, 1400^2 (47 MB) 33.4 and 30.6, 2000^2
+// (96 MB) 38.9 and 42.8.  Larger systems stream either way, and the mirrored reads are
+// the less regular ones.
+constexpr int64_t kSymMinBytes = (int64_t)16 << 20, kSymMaxBytes = (int64_t)63 << 20;
 
 __global__ void symmetry_kernel(int64_t n, int nd, DiaOffsets delta, const float* __restrict__ val,
                                 int* __restrict__ bad) {
@@ -1567,17 +1587,18 @@ cg_status solve_impl(cg_handle* h, const double* b, double* x, double tol, int32
     if (fp64)
       fn = jac ? (const void*)pcg64_kernel<true> : (const void*)pcg64_kernel<false>;
     else
-      fn = carry ? (jac ? (const void*)pcg_ir_kernel<true, true> : (const void*)pcg_ir_kernel<false, true>)
-                 : (jac ? (const void*)pcg_ir_kernel<true, false> : (const void*)pcg_ir_kernel<false, false>);
+      fn = refinement_kernel(jac, carry, P.S32.sym ? kMirrored : kAsStored);
     size_t smem = 0;
     if (!fp64 && ring_applies(h, G)) {
       int per_sm = 0;
       size_t limit = 0;
-      CG_CUDA(h, cgi::allow_dynamic_smem(fn, &limit));
+      const void* staged = refinement_kernel(jac, carry, kStaged);
+      CG_CUDA(h, cgi::allow_dynamic_smem(staged, &limit));
       if ((size_t)kRingBytes <= limit)
-        CG_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, kRingBytes));
+        CG_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, staged, kBlock, kRingBytes));
       if (per_sm * h->sm_count >= G) {
         P.S32.ring = (int32_t)padded(h->n);
+        fn = staged;
         smem = kRingBytes;
       }
     }

@@ -55,11 +55,17 @@ __device__ __forceinline__ int ld_relaxed_s32(const int* p) {
 // must then leave the kernel.  `seq` numbers the barriers of the launch
 // (1-based) for the fault-injection hook: when skip_seq == seq, CTA 0 does not
 // arrive, so the barrier can never complete and every CTA's wait runs out.
-// With a single CTA this is a plain __syncthreads().
+// With a single CTA this is a plain __syncthreads().  Thread 32 runs `meanwhile` while
+// thread 0 waits; what it writes to shared memory is visible to every thread afterwards.
+struct Nothing {
+  __device__ __forceinline__ void operator()() const {}
+};
+template <class F = Nothing>
 __device__ __forceinline__ bool grid_barrier(DevState* st, unsigned nblocks, uint64_t timeout_ns,
-                                             unsigned seq, unsigned skip_seq) {
+                                             unsigned seq, unsigned skip_seq, F meanwhile = F()) {
   __shared__ int s_ok;
   if (nblocks == 1) {
+    if (threadIdx.x == 32) meanwhile();
     __syncthreads();
     return true;
   }
@@ -89,6 +95,7 @@ __device__ __forceinline__ bool grid_barrier(DevState* st, unsigned nblocks, uin
     }
     s_ok = ok;
   }
+  if (threadIdx.x == 32) meanwhile();
   __syncthreads();
   return s_ok != 0;
 }

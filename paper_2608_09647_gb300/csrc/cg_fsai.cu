@@ -270,7 +270,7 @@ __device__ bool fsai_start(const Ell<T>& G, const Ell<T>& GT, const FsaiVecs<T>&
 // The PCG loop from a start state (r in V.r0, p = G^T G r, rho = r.z, rr =
 // r.r) until sqrt(rr) <= stop_abs (kOk), maxit (kNotConverged), breakdown /
 // non-finite values, or a barrier timeout.  x += alpha p each iteration.
-template <int W, typename T>
+template <int W, typename T, int PRODUCT = kAsStored>
 __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, const FsaiVecs<T>& V, double rho,
                          double rr, double stop_abs, int maxit, int* iters, double* part, int pstride, Grid& g,
                          double* rho_last = nullptr) {
@@ -285,7 +285,7 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
   T* rc = V.r0;
   T* rn = V.r1;
   while (!done) {
-    double pq[1] = {spmv_phase<T, false>(S, V.p, V.q, g)};
+    double pq[1] = {spmv_phase<T, false, PRODUCT>(S, V.p, V.q, g)};
     const bool ok1 = kWords ? g.sum(pq, kKindPQ) : g.sum_parts(pq, part + kSlotPQ * (size_t)pstride);
     // the scalars once per CTA (an fp64 divide or square root in every
     // thread would load GB300's narrow fp64 pipe), shared through shared memory
@@ -298,9 +298,11 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
     __syncthreads();
     if (s_fl) { status = s_fl; break; }
     const T alpha = (T)s_sc[0];
-    // 1 / rho for this iteration's beta (beta_of), in warp 1 during the r update
+    // 1 / rho for this iteration's beta (beta_of), in warp 1 during the r update or, by
+    // partials, while thread 0 waits at the barrier after it
     __shared__ double s_inv_rho;
-    if (threadIdx.x == 32) s_inv_rho = 1.0 / rho;
+    const auto reciprocal = [&] { s_inv_rho = 1.0 / rho; };
+    if (kWords && threadIdx.x == 32) reciprocal();
     Acc<T> a_rho, a_rr;
     rows_x2(
         g, n,
@@ -319,7 +321,7 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
           V.x[i] = u.x;
         });
     double s2[2] = {a_rho.get(), a_rr.get()};
-    const bool ok2 = kWords ? g.sum(s2, kKindUpd) : g.sum_parts(s2, part + kSlotUpd * (size_t)pstride);
+    const bool ok2 = kWords ? g.sum(s2, kKindUpd) : g.sum_parts(s2, part + kSlotUpd * (size_t)pstride, reciprocal);
     if (threadIdx.x == 0) {
       s_sc[1] = beta_of(s2[0], rho, s_inv_rho);
       s_sc[2] = s2[0];
@@ -428,7 +430,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai64_kernel(FsaiParams F) {
 
 // fp32-inner / fp64-outer refinement (R6) with the inner M^-1 = G32^T G32 (R7);
 // CARRY: reliable updates (R8), the search direction survives each fp64 update.
-template <int W, bool CARRY>
+template <int W, bool CARRY, int PRODUCT>
 __global__ void __launch_bounds__(kBlock, 2) pcg_fsai_ir_kernel(FsaiParams F) {
   const SolveParams& P = F.P;
   Grid g(P.st, P.timeout_ns, P.skip_seq);
@@ -467,7 +469,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai_ir_kernel(FsaiParams F) {
     double rho = 0.0;
     if (!fsai_start<W, float>(F.G32, F.GT32, V, V.r0, n, P.part, P.pstride, g, &rho,
                               CARRY && outer > 0 ? rho_k : 0.0)) { status = kTimeout; break; }
-    const int st = fsai_loop<W, float>(P.S32, F.G32, F.GT32, V, rho, s3[2], P.tol_in * sqrt(s3[2]), P.maxit, &inner,
+    const int st = fsai_loop<W, float, PRODUCT>(P.S32, F.G32, F.GT32, V, rho, s3[2], P.tol_in * sqrt(s3[2]), P.maxit, &inner,
                                     P.part, P.pstride, g, &rho_k);
     if (st == kTimeout || st == kNumeric || st == kBreakdown) { status = st; break; }
     for (int64_t i = g.gtid; i < n; i += g.gstride) P.x[i] += (double)V.x[i];
@@ -859,8 +861,12 @@ const void* gf_spmv_for(int uw, bool dia) {
 template <bool COND>
 struct PickUpdP { template <int W> static const void* fn() { return (const void*)gf_upd_p<W, COND>; } };
 struct Pick64 { template <int W> static const void* fn() { return (const void*)pcg_fsai64_kernel<W>; } };
-template <bool CARRY>
-struct PickIr { template <int W> static const void* fn() { return (const void*)pcg_fsai_ir_kernel<W, CARRY>; } };
+template <bool CARRY, int PRODUCT>
+struct PickIr {
+  template <int W> static const void* fn() {  // (mirrored values: with the stencils' slots only)
+    return (const void*)pcg_fsai_ir_kernel<W, CARRY, (W > 0 ? PRODUCT : kAsStored)>;
+  }
+};
 
 // CTAs of the vector-phase kernels: one wave at the kernels' own residency,
 // bounded by the partial slots.
@@ -1489,8 +1495,8 @@ cg_status cgi::fsai_solve(cg_handle* h, const SolveParams& Pin, bool fp64, bool 
   const void* fn;
   const int sw = fsai_slots(f);
   if (fp64) fn = by_slots<Pick64>(sw);
-  else if (carry) fn = by_slots<PickIr<true>>(sw);
-  else fn = by_slots<PickIr<false>>(sw);
+  else if (Pin.S32.sym) fn = carry ? by_slots<PickIr<true, kMirrored>>(sw) : by_slots<PickIr<false, kMirrored>>(sw);
+  else fn = carry ? by_slots<PickIr<true, kAsStored>>(sw) : by_slots<PickIr<false, kAsStored>>(sw);
   int per_sm = 0;
   CGF_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, 0));
   const int G = std::max(1, std::min({grid, per_sm * h->sm_count, kXCtas}));

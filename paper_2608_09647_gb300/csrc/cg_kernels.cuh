@@ -67,9 +67,8 @@ struct Sell {
   int32_t uw;  // >= 0: every slice has width uw and no row is long (soff, lmask unread)
   int32_t dia;                // 1: sliced-diagonal layout, width uw = number of diagonals
   int32_t delta[kMaxDiag];    // diagonal offsets (dia only)
-  int32_t ring;               // > 0: spmv_phase_ring, on kRingBytes of dynamic shared memory;
-                              //      the allocated length of the vectors
-  int32_t sym;                // 1: dia, and slot m of row i is slot uw-1-m of row i + delta[m], bit for bit
+  int32_t ring;               // kStaged: the allocated length of the vectors
+  int32_t sym;                // 1: dia, and slot m of row i is slot uw-1-m of row i + delta[m], bit for bit (kMirrored)
   const int32_t* __restrict__ soff;
   const uint32_t* __restrict__ lmask;
   const int32_t* __restrict__ col;
@@ -177,7 +176,10 @@ struct Grid {
     x_init(xs, s, words, gridDim.x, blockIdx.x, blockIdx.x == 0 ? skip : 0u, to);
   }
   // a barrier; false: a wait gave up, leave the kernel
-  __device__ __forceinline__ bool sync() { return grid_barrier(st, G, timeout_ns, ++seq, skip_seq); }
+  template <class F = Nothing>
+  __device__ __forceinline__ bool sync(F meanwhile = F()) {
+    return grid_barrier(st, G, timeout_ns, ++seq, skip_seq, meanwhile);
+  }
   // a barrier that leaves the grid's sums of v in warp 0's v and says there whether
   // it succeeded; the caller's next __syncthreads() completes it for the other warps
   template <int NV>
@@ -194,8 +196,8 @@ struct Grid {
   // (27-point 160^3, 304 CTAs: 146.5 us an iteration against 148.7); a residual's sums,
   // up to four, cost one barrier.  A slot of part is written again only after another
   // barrier: a slower CTA may still be reading it until then.
-  template <int NV>
-  __device__ __forceinline__ bool sum_parts(double (&v)[NV], double* part);
+  template <int NV, class F = Nothing>
+  __device__ __forceinline__ bool sum_parts(double (&v)[NV], double* part, F meanwhile = F());
   // exchanges for up to 3 values of kinds `kind`, ..., the sums given to every thread
   // (the residual phases)
   template <int NV>
@@ -230,10 +232,10 @@ __device__ __forceinline__ void publish(double (&v)[NV], double* part, const Gri
   }
 }
 
-template <int NV>
-__device__ __forceinline__ bool Grid::sum_parts(double (&v)[NV], double* part) {
+template <int NV, class F>
+__device__ __forceinline__ bool Grid::sum_parts(double (&v)[NV], double* part, F meanwhile) {
   publish<NV>(v, part, *this);
-  if (!sync()) return false;
+  if (!sync(meanwhile)) return false;
   grid_sum<NV>(part, G, v);
   return true;
 }
@@ -821,21 +823,28 @@ __device__ __forceinline__ double spmv_phase_csr(const Sell<T>& S, const T* __re
   return dot.get();
 }
 
+// The product of a persistent fp32 kernel: from shared memory (spmv_phase_ring), from half
+// of a symmetric matrix's slices (kSym), or any layout as it lies.  A kernel each: with the
+// first two in the kernel of the third, not taken, every refinement that takes neither was
+// 3 to 4 % slower (33^3 rows, 7 points: 11.9 against 11.4 us an iteration, 80^3: 16.9
+// against 16.3), and the kernels that take them gain as much.
+constexpr int kAsStored = 0, kStaged = 1, kMirrored = 2;
+
 // a1 over the grid: q = A^ p and this thread's share of p.q.  Warps take
 // slices round-robin; long rows are summed by a warp each.  Uniform slices of
 // width 4, 6 or 8 go to the specialised loop.
-template <typename T, bool JAC, bool RING = false>
+template <typename T, bool JAC, int PRODUCT = kAsStored>
 __device__ __forceinline__ double spmv_phase(const Sell<T>& S, const T* __restrict__ p,
                                              T* __restrict__ q, Grid& g) {
+  static_assert(PRODUCT == kAsStored || sizeof(T) == 4, "fp32 forms");
+  if constexpr (PRODUCT == kStaged) return spmv_phase_ring<JAC>(S, p, q, g);
+  if constexpr (PRODUCT == kMirrored) {
+    if (S.uw == 4) return spmv_phase_w<T, JAC, 4, kSym>(S, p, q, g);
+    if (S.uw == 6) return spmv_phase_w<T, JAC, 6, kSym>(S, p, q, g);
+    return spmv_phase_w<T, JAC, 8, kSym>(S, p, q, g);
+  }
   if (S.csr) return spmv_phase_csr<T, JAC>(S, p, q, g);
   if (S.dia) {
-    if constexpr (sizeof(T) == 4 && RING)
-      if (S.ring) return spmv_phase_ring<JAC>(S, p, q, g);
-    if constexpr (sizeof(T) == 4) {
-      if (S.sym && S.uw == 4) return spmv_phase_w<T, JAC, 4, kSym>(S, p, q, g);
-      if (S.sym && S.uw == 6) return spmv_phase_w<T, JAC, 6, kSym>(S, p, q, g);
-      if (S.sym && S.uw == 8) return spmv_phase_w<T, JAC, 8, kSym>(S, p, q, g);
-    }
     if (S.uw == 4) return spmv_phase_w<T, JAC, 4, kDia>(S, p, q, g);
     if (S.uw == 6) return spmv_phase_w<T, JAC, 6, kDia>(S, p, q, g);
     if (S.uw == 8) return spmv_phase_w<T, JAC, 8, kDia>(S, p, q, g);
@@ -1034,7 +1043,7 @@ __device__ __forceinline__ void update_xp_phase(const Sell<T>& S, const LoopVecs
 // advances by the SpMVs done.  When an iteration ran, the caller's x is
 // written (out = scale x^, or out += fl64(scale x^) with OUT_ADD) before the
 // final grid barrier; otherwise out keeps its exact value.
-template <typename T, bool JAC, bool OUT_ADD>
+template <typename T, bool JAC, bool OUT_ADD, int PRODUCT = kAsStored>
 __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, double rr,
                        double stop_abs, int maxit, int* iters, double* rr_out, double* out,
                        double* part, int pstride, Grid& g, PhaseClock& clk, double* rho_last = nullptr) {
@@ -1051,7 +1060,7 @@ __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, doubl
   __shared__ int s_st, s_want, s_exact, s_conv;
   while (!done) {
     // a1: q = A^ p; p.q
-    double v1[1] = {spmv_phase<T, JAC, true>(S, V.p, V.q, g)};
+    double v1[1] = {spmv_phase<T, JAC, PRODUCT>(S, V.p, V.q, g)};
     clk.lap(g.st, 0);
     const bool ok1 = kWords ? g.sum(v1, kKindPQ) : g.sum_parts(v1, part + kSlotPQ * (size_t)pstride);
     clk.lap(g.st, 1);
@@ -1065,18 +1074,20 @@ __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, doubl
     if (s_st) { status = s_st; break; }
     const T alpha = (T)s_alpha;
     // a2: r^ -= alpha q; r.z, r.r (r.r only when the test needs it).  1 / rho for
-    // this iteration's beta (beta_of) in warp 1 meanwhile
+    // this iteration's beta (beta_of) in warp 1, meanwhile or, by partials, while thread
+    // 0 waits at the barrier
     const bool want_rr = s_want != 0;
-    if (threadIdx.x == 32) s_inv_rho = 1.0 / rho;
+    const auto reciprocal = [&] { s_inv_rho = 1.0 / rho; };
+    if (kWords && threadIdx.x == 32) reciprocal();
     double v2[2] = {0.0, 0.0};
     update_r_phase<T, JAC>(S, V, alpha, want_rr, v2[0], v2[1], g);
     clk.lap(g.st, 2);
     bool ok;
     if (JAC && (!kWords || want_rr)) {  // by partials one form for both: a second costs more than it saves
-      ok = kWords ? g.sum(v2, kKindUpd) : g.sum_parts(v2, part + kSlotUpd * (size_t)pstride);
+      ok = kWords ? g.sum(v2, kKindUpd) : g.sum_parts(v2, part + kSlotUpd * (size_t)pstride, reciprocal);
     } else {
       double w[1] = {v2[0]};
-      ok = kWords ? g.sum(w, kKindUpd) : g.sum_parts(w, part + kSlotUpd * (size_t)pstride);
+      ok = kWords ? g.sum(w, kKindUpd) : g.sum_parts(w, part + kSlotUpd * (size_t)pstride, reciprocal);
       v2[0] = v2[1] = w[0];  // plain CG: r.z is r.r
     }
     clk.lap(g.st, 3);
@@ -1230,11 +1241,11 @@ __global__ void __launch_bounds__(kBlock, 2) pcg64_kernel(SolveParams P) {
 // (reliable updates, R8): after each fp64 update the inner CG continues from
 // the replaced residual with its last search direction, p = r^' + (r^'.r^' /
 // rho_k) p_k, instead of restarting from p = r^'.
-template <bool JAC, bool CARRY>
+template <bool JAC, bool CARRY, int PRODUCT>
 __global__ void __launch_bounds__(kBlock, 2) pcg_ir_kernel(SolveParams P) {
   Grid g(P.st, P.timeout_ns, P.skip_seq);
   PhaseClock clk(P.timers != 0);
-  if (P.S32.ring) Ring().init();
+  if constexpr (PRODUCT == kStaged) Ring().init();
   const int64_t n = P.A.n;
   const LoopVecs<float>& V = P.V32;
   int status = kNotConverged, inner = 0, outer = 0;
@@ -1277,7 +1288,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_ir_kernel(SolveParams P) {
       for (int64_t i = g.gtid; i < n; i += g.gstride) V.p[i] = fma(beta, V.p[i], V.r[i]);
       if (!g.sync()) { status = kTimeout; break; }
     }
-    const int st = cg_loop<float, JAC, true>(P.S32, V, s4[2], s4[3], P.tol_in * sqrt(s4[3]),
+    const int st = cg_loop<float, JAC, true, PRODUCT>(P.S32, V, s4[2], s4[3], P.tol_in * sqrt(s4[3]),
                                              P.maxit, &inner, &rr32, P.x, P.part, P.pstride, g, clk, &rho_k);
     if (st == kTimeout || st == kNumeric || st == kBreakdown) { status = st; break; }
     ++outer;
