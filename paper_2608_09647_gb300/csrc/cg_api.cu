@@ -451,7 +451,7 @@ void residency(int dev, int sm_count, int* persistent, int* vectors) {
   std::lock_guard<std::mutex> lock(mu);
   int* k = known[dev < 0 || dev >= kMaxDevices ? 0 : dev];
   if (k[0] <= 0 || k[1] <= 0 || dev < 0 || dev >= kMaxDevices) {
-    int g = kXCtas;
+    int g = INT32_MAX;
     for (int r : {max_coresident(pcg64_kernel<true>, sm_count), max_coresident(pcg64_kernel<false>, sm_count)})
       g = std::min(g, r);
     for (int product : {kAsStored, kStaged, kMirrored})

@@ -416,7 +416,7 @@ __device__ __forceinline__ void grid_sum(const double* part, unsigned G, double 
 // exponent is exchanged first and the sum is formed again at that scale.
 constexpr int kXCtas = cg_exact::kMaxAddends;  // most CTAs of a grid that exchanges sums
 constexpr int kXVals = 2;                      // most sums per exchange
-constexpr int kXKinds = 8;                     // kinds of sums whose scales are kept
+constexpr int kXKinds = 7;                     // kinds of sums whose scales are kept
 
 // One word a 128-byte line: per set a plain counter (barriers without a sum) and
 // three limbs a value, each in kXSplit words that every kXSplit-th CTA adds to and that

@@ -252,8 +252,7 @@ __device__ bool fsai_start(const Ell<T>& G, const Ell<T>& GT, const FsaiVecs<T>&
         a.add(s, s);
       });
   double v[1] = {a.get()};
-  const bool ok = sizeof(T) == 8 ? g.sum_all(v, kKindStart) : g.sum_parts(v, part + kSlotStart * (size_t)pstride);
-  if (!ok) return false;
+  if (!g.sum_parts(v, part + kSlotStart * (size_t)pstride)) return false;
   *rho = v[0];
   const bool carry = rho_prev > 0.0;
   const T beta = carry ? (T)(v[0] / rho_prev) : T(0);
@@ -274,7 +273,6 @@ template <int W, typename T, int PRODUCT = kAsStored>
 __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, const FsaiVecs<T>& V, double rho,
                          double rr, double stop_abs, int maxit, int* iters, double* part, int pstride, Grid& g,
                          double* rho_last = nullptr) {
-  constexpr bool kWords = sizeof(T) == 8;  // sums by the exchange's words, else by partials
   const int64_t n = S.n;
   if (rho_last) *rho_last = rho;
   int k = *iters;
@@ -286,7 +284,7 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
   T* rn = V.r1;
   while (!done) {
     double pq[1] = {spmv_phase<T, false, PRODUCT>(S, V.p, V.q, g)};
-    const bool ok1 = kWords ? g.sum(pq, kKindPQ) : g.sum_parts(pq, part + kSlotPQ * (size_t)pstride);
+    const bool ok1 = g.sum_parts(pq, part + kSlotPQ * (size_t)pstride);
     // the scalars once per CTA (an fp64 divide or square root in every
     // thread would load GB300's narrow fp64 pipe), shared through shared memory
     __shared__ double s_sc[4];
@@ -298,11 +296,10 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
     __syncthreads();
     if (s_fl) { status = s_fl; break; }
     const T alpha = (T)s_sc[0];
-    // 1 / rho for this iteration's beta (beta_of), in warp 1 during the r update or, by
-    // partials, while thread 0 waits at the barrier after it
+    // 1 / rho for this iteration's beta (beta_of), while thread 0 waits at the barrier
+    // after the r update
     __shared__ double s_inv_rho;
     const auto reciprocal = [&] { s_inv_rho = 1.0 / rho; };
-    if (kWords && threadIdx.x == 32) reciprocal();
     Acc<T> a_rho, a_rr;
     rows_x2(
         g, n,
@@ -321,7 +318,7 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
           V.x[i] = u.x;
         });
     double s2[2] = {a_rho.get(), a_rr.get()};
-    const bool ok2 = kWords ? g.sum(s2, kKindUpd) : g.sum_parts(s2, part + kSlotUpd * (size_t)pstride, reciprocal);
+    const bool ok2 = g.sum_parts(s2, part + kSlotUpd * (size_t)pstride, reciprocal);
     if (threadIdx.x == 0) {
       s_sc[1] = beta_of(s2[0], rho, s_inv_rho);
       s_sc[2] = s2[0];
@@ -356,8 +353,7 @@ __device__ int fsai_loop(const Sell<T>& S, const Ell<T>& G, const Ell<T>& GT, co
 template <int W>
 __global__ void __launch_bounds__(kBlock, 2) pcg_fsai64_kernel(FsaiParams F) {
   const SolveParams& P = F.P;
-  __shared__ XState s_x;
-  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
+  Grid g(P.st, P.timeout_ns, P.skip_seq);
   const int64_t n = P.A.n;
   const FsaiVecs<double>& V = F.V64;
   int status = kNotConverged, k = 0, restarts = 0;
@@ -374,7 +370,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai64_kernel(FsaiParams F) {
       v[0] += ri * ri;
       v[1] += bi * bi;
     }
-    if (!g.sum_all(v)) { status = kTimeout; break; }
+    if (!g.sum_parts(v, P.part + kSlotRes * (size_t)P.pstride)) { status = kTimeout; break; }
     const double(&s2)[2] = v;
     const double rr_start = s2[0];
     if (first) {
@@ -413,7 +409,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg_fsai64_kernel(FsaiParams F) {
         const double ri = P.b[i] - V.q[i];
         w[0] += ri * ri;
       }
-      if (!g.sum_all(w)) { status = kTimeout; break; }
+      if (!g.sum_parts(w, P.part + kSlotRes * (size_t)P.pstride)) { status = kTimeout; break; }
       relres_true = sqrt(w[0]) / sqrt(bb);
       break;
     }
@@ -1499,7 +1495,7 @@ cg_status cgi::fsai_solve(cg_handle* h, const SolveParams& Pin, bool fp64, bool 
   else fn = carry ? by_slots<PickIr<true, kAsStored>>(sw) : by_slots<PickIr<false, kAsStored>>(sw);
   int per_sm = 0;
   CGF_CUDA(h, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kBlock, 0));
-  const int G = std::max(1, std::min({grid, per_sm * h->sm_count, kXCtas}));
+  const int G = std::max(1, std::min(grid, per_sm * h->sm_count));
   CGF_CUDA(h, cudaMemsetAsync(h->st, 0, kStBytes, h->stream));
   CGF_CUDA(h, cudaEventRecord(h->ev0, h->stream));
   CGF_CUDA(h, cudaLaunchCooperativeKernel(fn, dim3(G), dim3(kBlock), args, 0, h->stream));

@@ -150,75 +150,40 @@ struct SolveParams {
 constexpr int kParts = 8;
 constexpr int kSlotPQ = 0, kSlotRr = 1, kSlotUpd = 2, kSlotRes = 4, kSlotStart = kSlotRes + 3;
 
-// Kinds of the loops' sums (their scales are kept apart: two quantities of one kind would
+// Kinds of the exchanged sums (their scales are kept apart: two quantities of one kind would
 // find the other's scale, and a sum that does not suit the scale is formed anew, in two
-// more rounds).  The residual phase's up to three, and the start's r.z with FSAI.
-constexpr int kKindPQ = 0, kKindUpd = 1, kKindRr = 3, kKindRes = 4, kKindStart = 7;
+// more rounds).  The residual phase has three.
+constexpr int kKindPQ = 0, kKindUpd = 1, kKindRr = 3, kKindRes = 4;
 
-// Grid coordinates and the exchanges of one persistent launch.
+// Grid coordinates and the barriers of one persistent launch.
 struct Grid {
   unsigned G, cta;
   int64_t gtid, gstride;
   DevState* st;
-  XState* x;
   uint64_t timeout_ns;
   unsigned seq, skip_seq;
   unsigned fills;  // this warp's ring chunks so far (spmv_phase_ring)
   __device__ Grid() : G(gridDim.x), cta(blockIdx.x), gtid((int64_t)blockIdx.x * kBlock + threadIdx.x),
-        gstride((int64_t)gridDim.x * kBlock), st(nullptr), x(nullptr), timeout_ns(0), seq(0), skip_seq(0), fills(0) {}
+        gstride((int64_t)gridDim.x * kBlock), st(nullptr), timeout_ns(0), seq(0), skip_seq(0), fills(0) {}
   __device__ Grid(DevState* s, uint64_t to, unsigned skip) : Grid() {
     st = s;
     timeout_ns = to;
     skip_seq = skip;
-  }
-  __device__ Grid(DevState* s, XWord* words, XState* xs, uint64_t to, unsigned skip) : Grid(s, to, skip) {
-    x = xs;
-    x_init(xs, s, words, gridDim.x, blockIdx.x, blockIdx.x == 0 ? skip : 0u, to);
   }
   // a barrier; false: a wait gave up, leave the kernel
   template <class F = Nothing>
   __device__ __forceinline__ bool sync(F meanwhile = F()) {
     return grid_barrier(st, G, timeout_ns, ++seq, skip_seq, meanwhile);
   }
-  // a barrier that leaves the grid's sums of v in warp 0's v and says there whether
-  // it succeeded; the caller's next __syncthreads() completes it for the other warps
-  template <int NV>
-  __device__ __forceinline__ bool sum(double (&v)[NV], int kind) {
-    static_assert(NV <= kXVals, "values of one exchange");
-    const XSums r = grid_exchange<NV>(x, kind, v[0], NV > 1 ? v[NV - 1] : 0.0);
-    v[0] = r.v0;
-    if (NV > 1) v[NV - 1] = r.v1;
-    return r.ok;
-  }
-  // the same through per-CTA partials part[j G + cta] that every CTA adds up after a
-  // plain barrier, the sums in every thread: the fp32 kernels' form.  Their phases end
-  // more unevenly, and CTAs that poll an exchange's words slow the ones still at work
-  // (27-point 160^3, 304 CTAs: 146.5 us an iteration against 148.7); a residual's sums,
-  // up to four, cost one barrier.  A slot of part is written again only after another
+  // a barrier after which every thread has the grid's sums of v, through per-CTA partials
+  // part[j G + cta] that every CTA adds up.  (grid_exchange, one round trip instead of
+  // two, serves the one-CTA-an-SM forms.  Here phases end more unevenly, and CTAs that poll
+  // an exchange's words slow the ones still at work: refinement on 27 points, 160^3 rows,
+  // 304 CTAs, 148.7 us an iteration by exchanges, 146.5 so; fp64 on a power-law graph of
+  // 20,000 rows 18.3 and 16.4.)  A slot of part is written again only after another
   // barrier: a slower CTA may still be reading it until then.
   template <int NV, class F = Nothing>
   __device__ __forceinline__ bool sum_parts(double (&v)[NV], double* part, F meanwhile = F());
-  // exchanges for up to 3 values of kinds `kind`, ..., the sums given to every thread
-  // (the residual phases)
-  template <int NV>
-  __device__ __forceinline__ bool sum_all(double (&v)[NV], int kind = kKindRes) {
-    __shared__ double s_out[NV];
-#pragma unroll
-    for (int j = 0; j < NV; j += 2) {
-      const bool two = j + 1 < NV;
-      double w2[2] = {v[j], v[two ? j + 1 : j]}, w1[1] = {v[j]};
-      const bool ok = two ? sum<2>(w2, kind + j) : sum<1>(w1, kind + j);
-      if (threadIdx.x == 0) {
-        s_out[j] = two ? w2[0] : w1[0];
-        if (two) s_out[j + 1 < NV ? j + 1 : j] = w2[1];
-      }
-      if (!__syncthreads_and(ok)) return false;
-    }
-#pragma unroll
-    for (int j = 0; j < NV; ++j) v[j] = s_out[j];
-    __syncthreads();
-    return true;
-  }
 };
 
 // Write this CTA's block sums of v[0..NV) into part[j*G + cta] (v is
@@ -1047,7 +1012,6 @@ template <typename T, bool JAC, bool OUT_ADD, int PRODUCT = kAsStored>
 __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, double rr,
                        double stop_abs, int maxit, int* iters, double* rr_out, double* out,
                        double* part, int pstride, Grid& g, PhaseClock& clk, double* rho_last = nullptr) {
-  constexpr bool kWords = sizeof(T) == 8;  // sums by the exchange's words, else by partials
   if (rho_last) *rho_last = rho;  // r.z before the last step taken (reliable updates)
   int k = *iters;
   int status = kNotConverged;
@@ -1062,7 +1026,7 @@ __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, doubl
     // a1: q = A^ p; p.q
     double v1[1] = {spmv_phase<T, JAC, PRODUCT>(S, V.p, V.q, g)};
     clk.lap(g.st, 0);
-    const bool ok1 = kWords ? g.sum(v1, kKindPQ) : g.sum_parts(v1, part + kSlotPQ * (size_t)pstride);
+    const bool ok1 = g.sum_parts(v1, part + kSlotPQ * (size_t)pstride);
     clk.lap(g.st, 1);
     if (threadIdx.x == 0) {
       s_st = !ok1 ? kTimeout
@@ -1074,20 +1038,18 @@ __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, doubl
     if (s_st) { status = s_st; break; }
     const T alpha = (T)s_alpha;
     // a2: r^ -= alpha q; r.z, r.r (r.r only when the test needs it).  1 / rho for
-    // this iteration's beta (beta_of) in warp 1, meanwhile or, by partials, while thread
-    // 0 waits at the barrier
+    // this iteration's beta (beta_of) is formed while thread 0 waits at the barrier
     const bool want_rr = s_want != 0;
     const auto reciprocal = [&] { s_inv_rho = 1.0 / rho; };
-    if (kWords && threadIdx.x == 32) reciprocal();
     double v2[2] = {0.0, 0.0};
     update_r_phase<T, JAC>(S, V, alpha, want_rr, v2[0], v2[1], g);
     clk.lap(g.st, 2);
     bool ok;
-    if (JAC && (!kWords || want_rr)) {  // by partials one form for both: a second costs more than it saves
-      ok = kWords ? g.sum(v2, kKindUpd) : g.sum_parts(v2, part + kSlotUpd * (size_t)pstride, reciprocal);
+    if (JAC) {  // one form with r.r and without: a second costs more than it saves
+      ok = g.sum_parts(v2, part + kSlotUpd * (size_t)pstride, reciprocal);
     } else {
       double w[1] = {v2[0]};
-      ok = kWords ? g.sum(w, kKindUpd) : g.sum_parts(w, part + kSlotUpd * (size_t)pstride, reciprocal);
+      ok = g.sum_parts(w, part + kSlotUpd * (size_t)pstride, reciprocal);
       v2[0] = v2[1] = w[0];  // plain CG: r.z is r.r
     }
     clk.lap(g.st, 3);
@@ -1107,7 +1069,7 @@ __device__ int cg_loop(const Sell<T>& S, const LoopVecs<T>& V, double rho, doubl
     rho = s_rho;
     if (s_exact) {
       double v3[1] = {rr_phase<T>(S, V, g)};  // rho fell into the band early: exact r.r
-      const bool ok3 = kWords ? g.sum(v3, kKindRr) : g.sum_parts(v3, part + kSlotRr * (size_t)pstride);
+      const bool ok3 = g.sum_parts(v3, part + kSlotRr * (size_t)pstride);
       if (threadIdx.x == 0) {
         if (!ok3) s_st = kTimeout;
         s_rr = v3[0];
@@ -1158,8 +1120,7 @@ __device__ __forceinline__ void spmv_orig(const Csr<double>& A, const double* x,
 // restarts (readings R1-R5 of the method, see the oracle's header).
 template <bool JAC>
 __global__ void __launch_bounds__(kBlock, 2) pcg64_kernel(SolveParams P) {
-  __shared__ XState s_x;
-  Grid g(P.st, P.xs, &s_x, P.timeout_ns, P.skip_seq);
+  Grid g(P.st, P.timeout_ns, P.skip_seq);
   PhaseClock clk(P.timers != 0);
   const int64_t n = P.A.n;
   const LoopVecs<double>& V = P.V64;
@@ -1182,7 +1143,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg64_kernel(SolveParams P) {
       v[1] += ri * ri;
       v[2] += bi * bi;
     }
-    if (!g.sum_all(v)) { status = kTimeout; break; }
+    if (!g.sum_parts(v, P.part + kSlotRes * (size_t)P.pstride)) { status = kTimeout; break; }
     const double(&s3)[3] = v;
     if (first) {
       bb = s3[2];
@@ -1214,7 +1175,7 @@ __global__ void __launch_bounds__(kBlock, 2) pcg64_kernel(SolveParams P) {
         const double ri = P.b[i] - V.q[i];
         w[0] += ri * ri;
       }
-      if (!g.sum_all(w)) { status = kTimeout; break; }
+      if (!g.sum_parts(w, P.part + kSlotRes * (size_t)P.pstride)) { status = kTimeout; break; }
       relres_true = sqrt(w[0]) / sqrt(bb);
       break;
     }
