@@ -107,12 +107,10 @@ __device__ __forceinline__ double row_chain(const double* __restrict__ x, const 
 // consecutive rows' neighbours); longer rows, listed in s_med, by a warp each
 // (lanes stride over the row, a fixed xor tree joins them), so one long row
 // does not hold a warp of short ones.
+template <class Next>
 __device__ __forceinline__ void spmv_rowblock_fma(const Csr<double>& A, const double* __restrict__ x,
-                                                  double* __restrict__ y, int b, int* s_col, double* s_val,
-                                                  int* s_med, int* s_sort) {
-  // (the next block's bounds read ahead would spill at 6 CTAs per SM: 7 points, 150^3
-  // rows, 82.6 us a product against 76.7; 3 M rows of a power-law graph 109.7 against 105.6)
-  const BlockSpan B = block_span(A.rb, A.rowptr, b);
+                                                  double* __restrict__ y, const BlockSpan& B, int* s_col,
+                                                  double* s_val, int* s_med, int* s_sort, Next next) {
   const int r0 = B.r0, r1 = B.r1, k0 = B.k0, k1 = B.k1;
   const int t = threadIdx.x;
   if (k1 - k0 > kCapV) {  // long row (r1 == r0 + 1 by construction): strided FMA, fixed tree
@@ -121,6 +119,7 @@ __device__ __forceinline__ void spmv_rowblock_fma(const Csr<double>& A, const do
     double v[1] = {acc};
     block_sum<1>(v);
     if (t == 0) y[r0] = v[0];
+    next();
     return;
   }
   const int a0 = A.vec ? (k0 & ~3) : k0;
@@ -176,6 +175,7 @@ __device__ __forceinline__ void spmv_rowblock_fma(const Csr<double>& A, const do
   const int steps = __reduce_max_sync(0xffffffffu, mine), held = __reduce_add_sync(0xffffffffu, mine);
   const int live = __popc(__ballot_sync(0xffffffffu, i < r1 && !med));
   const bool uneven = __syncthreads_or(med || 4 * held < 3 * live * steps) != 0;
+  next();
   if (uneven) {
     // Rows of mixed lengths: a warp of 32 consecutive ones runs to its longest (GB300
     // issues an fp64 warp instruction in full whatever its active lanes: ~14 steps a
@@ -244,11 +244,27 @@ __device__ __forceinline__ void spmv_rowblock_fma(const Csr<double>& A, const do
 }
 
 // Row blocks cta, cta + stride, ... of y = A x by one CTA (static shared memory of the caller).
+// AHEAD: the next block's bounds are read while this one is summed, which two CTAs per SM
+// need (FSAI refinement, 1000^2 rows: 4.74 ms without, 4.55 with) and six have no registers
+// for (spmv_kernel spilled: 7 points, 150^3 rows, 82.6 us a product against 76.7).
+template <bool AHEAD>
 __device__ __forceinline__ void spmv_rowblocks(const Csr<double>& A, const double* x, double* y, int cta, int stride,
                                                int* s_col, double* s_val, int* s_med, int* s_sort) {
   if (threadIdx.x < 32) s_sort[threadIdx.x] = 0;
   __syncthreads();
-  for (int b = cta; b < A.nrb; b += stride) spmv_rowblock_fma(A, x, y, b, s_col, s_val, s_med, s_sort);
+  if constexpr (AHEAD) {
+    BlockSpan B{0, 0, 0, 0}, ahead{0, 0, 0, 0};
+    if (cta < A.nrb) B = block_span(A.rb, A.rowptr, cta);
+    for (int b = cta; b < A.nrb; b += stride) {
+      spmv_rowblock_fma(A, x, y, B, s_col, s_val, s_med, s_sort, [&] {
+        if (b + stride < A.nrb) ahead = block_span(A.rb, A.rowptr, b + stride);
+      });
+      B = ahead;
+    }
+  } else {
+    for (int b = cta; b < A.nrb; b += stride)
+      spmv_rowblock_fma(A, x, y, block_span(A.rb, A.rowptr, b), s_col, s_val, s_med, s_sort, [] {});
+  }
 }
 
 // Stand-alone y = A x over all row blocks (cg_spmv, the graph form's residuals);
@@ -261,7 +277,7 @@ __global__ void __launch_bounds__(kBlock, 6) spmv_kernel(Csr<T> A, const T* x, T
   __shared__ __align__(16) double s_val[kCap];
   __shared__ int s_med[kBlock];
   __shared__ int s_sort[32];
-  spmv_rowblocks(A, x, y, (int)blockIdx.x, (int)gridDim.x, s_col, s_val, s_med, s_sort);
+  spmv_rowblocks<false>(A, x, y, (int)blockIdx.x, (int)gridDim.x, s_col, s_val, s_med, s_sort);
 }
 
 }  // namespace cg

@@ -1113,7 +1113,7 @@ __device__ __forceinline__ void spmv_orig(const Csr<double>& A, const double* x,
   __shared__ __align__(16) double s_val[kCap];
   __shared__ int s_med[kBlock];
   __shared__ int s_sort[32];
-  spmv_rowblocks(A, x, q, (int)g.cta, (int)g.G, s_col, s_val, s_med, s_sort);
+  spmv_rowblocks<true>(A, x, q, (int)g.cta, (int)g.G, s_col, s_val, s_med, s_sort);
 }
 
 // fp64 (Jacobi-)PCG with true-residual check and residual-replacement
