@@ -81,7 +81,8 @@ typedef enum {
                                      16384 rows unless CG_OPT_GRID_CTAS, CG_OPT_DEBUG_SKIP_ARRIVAL
                                      or CG_OPT_PHASE_TIMERS is set; with the same exceptions form 1
                                      for stencil matrices whose vectors fit the SMs' shared memory
-                                     (about 10^6 rows); else graph from 2^18 rows; fp32
+                                     (about 10^6 rows; 385,000 with 27 points); else graph from
+                                     2^18 rows; fp32
                                      FSAI refinement: graph from 2^21 rows; else persistent),
                                      1 one persistent cooperative launch, 2 CUDA graph with a
                                      device-side WHILE node (nested WHILE nodes for fp32

@@ -310,6 +310,16 @@ const void* kernel_for(int uw, bool jac) {
 
 }  // namespace
 
+// The most bytes of a loop matrix streamed by this form.  Past them the matrix no longer
+// stays in the 126 MB L2 beside the vectors, and the 16 warps an SM that stream it are too
+// few.  Only matrices of more than 8 diagonals get there before their vectors outgrow shared
+// memory.  The line lies where the graph form overtakes, sooner for 27 points, whose 26
+// slots have a product of their own there.  fp64 Jacobi to 1e-12, ms, graph form and this:
+// 27 points 72^3 rows (78 MB) 5.74 and 5.56, 74^3 (84 MB) 6.06 and 6.32, 90^3 (152 MB) 9.41
+// and 10.9; 19 points 70^3 (49 MB) 6.44 and 4.78, 90^3 (105 MB) 10.2 and 9.48, 100^3
+// (144 MB) 12.3 and 12.2; 13 points 100^3 (96 MB) 10.4 and 9.42.
+int64_t streamed_max_bytes(int diagonals) { return diagonals == 26 ? 80000000 : 144000000; }
+
 cudaError_t cgi::resident_launch(const cg_handle* h, const SolveParams& P, bool jac, int* grid, bool* launched) {
   *launched = false;
   if (!h->dia || h->n < 1) return cudaSuccess;
@@ -317,6 +327,7 @@ cudaError_t cgi::resident_launch(const cg_handle* h, const SolveParams& P, bool 
   const int ctas = std::min(h->sm_count, 255);
   const int spc = (int)((h->nslices + ctas - 1) / ctas);
   for (int ms = 1; ms >= 0; --ms) {
+    if (!ms && (int64_t)sizeof(double) * h->sell_entries > streamed_max_bytes(h->uniform_w)) continue;
     const void* fn = ms ? kernel_for<true>(h->uniform_w, jac) : kernel_for<false>(h->uniform_w, jac);
     size_t limit = 0;
     if ((e = allow_dynamic_smem(fn, &limit)) != cudaSuccess) return e;
