@@ -72,7 +72,8 @@ typedef enum {
                                      residual reduction that triggers a reliable update (default 0.1) */
   CG_OPT_IR_MAX_OUTER = 4,        /* refinement steps / reliable updates cap (default 30) */
   CG_OPT_DEBUG_SKIP_ARRIVAL = 5,  /* fault injection: CTA 0 skips arrival at grid barrier #value
-                                     (cluster form: does not push exchange #value; 1-based; 0 = off),
+                                     (cluster form, and form 1 with the vectors in shared memory,
+                                     which auto then leaves out: exchange #value; 1-based; 0 = off),
                                      so every wait runs into its limit; 2^30 + k: in the fp32
                                      refinement of a 27-point matrix, a warp of CTA 0 does not start
                                      its k-th copy of values to shared memory */

@@ -1569,10 +1569,10 @@ cg_status solve_impl(cg_handle* h, const double* b, double* x, double tol, int32
   SolveParams P = make_solve_params(h, jac, b, x, tol, maxit, fp64, carry);
   if (fsai) return cgi::fsai_solve(h, P, fp64, carry, G, iters_out, relres_out);
   // stencil systems whose vectors the SMs' shared memory holds: one persistent launch
-  // that keeps them there (a grid size, the timers and the fault injection belong to
-  // the form below)
+  // that keeps them there (a grid size and the timers belong to the form below, the fault
+  // injection only with CG_OPT_LOOP_MODE 1 to this one)
   bool launched = false;
-  if (fp64 && h->loop_mode <= 1 && h->grid_opt == 0 && h->skip_seq == 0 && h->timers == 0)
+  if (fp64 && h->loop_mode <= 1 && h->grid_opt == 0 && (h->skip_seq == 0 || h->loop_mode == 1) && h->timers == 0)
     CG_CUDA(h, cgi::resident_launch(h, P, jac, &G, &launched));
   // auto: fp64 takes the graph form from kGraphMinRows rows; the refinement's
   // fp32 vector passes are short, so it stays in the persistent form

@@ -97,6 +97,7 @@ __global__ void __launch_bounds__(kThreads, 1) pcg64_resident_kernel(ResidentPar
     for (int k = t; k < ne; k += kThreads) ms[k] = __ldcs(vals + k);
     vals = ms;
   }
+  // (fault injection: CTA 0 does not add to exchange number skip_seq)
   x_init(&s_x, P.st, P.xs, gridDim.x, blockIdx.x, blockIdx.x == 0 ? P.skip_seq : 0u, P.timeout_ns);
   const Gather gp{(unsigned)__cvta_generic_to_shared(ps), pg, r0, nr, n - 1};
   // an exchange of sums whose CTAs hand over no global writes, and one that orders them
