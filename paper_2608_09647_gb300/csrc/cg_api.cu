@@ -420,6 +420,7 @@ std::vector<int32_t> build_row_blocks(const int32_t* rowptr, int64_t n, int64_t*
   return rb;
 }
 
+// Elements of an n-vector's place in a shared allocation (whole 256 bytes of fp32).
 size_t padded(int64_t n) { return ((size_t)std::max<int64_t>(n, 1) + 63) / 64 * 64; }
 
 const void* refinement_kernel(bool jac, bool carry, int product) {
@@ -579,8 +580,6 @@ cg_status cgi::ensure_offsets(cg_handle* h) {
 }
 
 namespace {
-
-// Elements of an n-vector's place in a shared allocation (whole 256 bytes of fp32).
 
 // sqrt(A_ii), 1/sqrt(A_ii) and the fp32 copies: one allocation, last step of the layout.
 cg_status ensure_diag_vectors(cg_handle* h) {

@@ -8,10 +8,12 @@
 // "long" block, which the CTA strides over and reduces).  spmv_rowblock_fma:
 // the block's column indices and values are copied to shared memory with
 // 16-byte loads (four indices, two pairs of values) starting at the 16-byte
-// boundary at or below the block's first nonzero; short rows (kThreadRow)
-// are summed by one thread each (storage order, fused multiply-adds: one fp64
-// FMA per nonzero), longer rows by a warp each, and a row beyond the block cap
-// by the whole CTA.  GB300's fp64 pipe issues 2 FMAs per clock per SM, so a
+// boundary at or below the block's first nonzero.  A block of even rows has them
+// summed by one thread each (storage order, fused multiply-adds: one fp64 FMA per
+// nonzero), or by two where it holds few long ones (27-point stencils); a block of
+// uneven rows has them sorted by length first, its rows of more than kThreadRow
+// entries summed by eight lanes each (long_row_sum); a row beyond the block cap is
+// summed by the whole CTA.  GB300's fp64 pipe issues 2 FMAs per clock per SM, so a
 // separate multiply and add per nonzero (two fp64 instructions) makes a
 // 7-point SpMV pipe-bound; with one FMA the kernel is HBM-bound.
 #pragma once
@@ -40,14 +42,12 @@ struct Csr {
 constexpr int kQuadPasses = 2;
 static_assert((kCapV + 3 + 3) / 4 <= kQuadPasses * kBlock, "a row block's window exceeds two quads per thread");
 constexpr int kRowUnroll = 4;  // a row's nonzeros whose gathers are in flight together
-// Rows with more nonzeros than a thread takes are summed by a warp each.  A
+// Rows with more nonzeros than a thread takes are summed by eight lanes each.  A
 // thread takes a row of up to kThreadRow entries; in the caller's CSR, when
 // more than kWideRows of a warp's 32 rows have kThreadRow + 1 .. kThreadRowWide
-// entries (a 27-point stencil) it takes those too: one
-// thread a row costs the warp one FMA step per entry, where a warp per row adds
-// a 5-level fp64 tree to every row (27 entries: ~0.84 fp64 warp instructions a
-// row against ~6); a few such rows among short ones go to warps, so they do not
-// hold a warp of short rows.
+// entries (a 27-point stencil) it takes those too: one thread a row costs the warp
+// one FMA step per entry, and no tree of fp64 additions per row; a few such rows
+// among short ones go to eight lanes, so they do not hold a warp of short rows.
 constexpr int kThreadRow = 16;
 constexpr int kThreadRowWide = 32;
 constexpr int kWideRows = 4;
@@ -122,12 +122,12 @@ __device__ __forceinline__ T long_row_sum(int len, Step step) {
 
 // One row block of y = A x with one fused multiply-add per nonzero (header
 // comment).  The block's column indices and values are copied with 16-byte
-// loads into s_col / s_val at their offset from the window start a0.  Rows of
-// at most kThreadRow nonzeros are then summed by their own thread, in storage
-// order, gathering x themselves (a warp's gathers for one term cover 32
-// consecutive rows' neighbours); longer rows, listed in s_med, by a warp each
-// (lanes stride over the row, a fixed xor tree joins them), so one long row
-// does not hold a warp of short ones.
+// loads into s_col / s_val at their offset from the window start a0.  In a block
+// of even rows thread t then sums row r0 + t, in storage order, gathering x itself
+// (a warp's gathers for one term cover 32 consecutive rows' neighbours), or two
+// threads a row sum its halves; in one of uneven rows s_med lists the rows by
+// descending length, the long ones first, which eight lanes each sum, the others
+// a thread each.
 template <class Next>
 __device__ __forceinline__ void spmv_rowblock_fma(const Csr<double>& A, const double* __restrict__ x,
                                                   double* __restrict__ y, const BlockSpan& B, int* s_col,

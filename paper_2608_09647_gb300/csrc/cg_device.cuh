@@ -414,7 +414,9 @@ __device__ __forceinline__ void grid_sum(const double* part, unsigned G, double 
 // whose sum does not fit (or is not finite) says so in the third word, and a total
 // far below the last one would lack bits: then, the same in every CTA, the largest
 // exponent is exchanged first and the sum is formed again at that scale.
-constexpr int kXCtas = cg_exact::kMaxAddends;  // most CTAs of a grid that exchanges sums
+template <int WARPS>                           // most CTAs, of WARPS warps, that exchange sums
+constexpr int kXCtas = cg_exact::kMaxSums / WARPS < cg_exact::kMaxAddends ? cg_exact::kMaxSums / WARPS
+                                                                          : cg_exact::kMaxAddends;
 constexpr int kXVals = 2;                      // most sums per exchange
 constexpr int kXKinds = 7;                     // kinds of sums whose scales are kept
 

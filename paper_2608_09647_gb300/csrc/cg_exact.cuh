@@ -191,12 +191,14 @@ CG_EXACT_HD i128 unpack(unsigned long long lo, unsigned long long hi, int* E, bo
 // ---- sums that many CTAs add up with 64-bit atomic adds
 //
 // An integer S in units of scale B travels as three addends of 43, 43 and 32 payload
-// bits (its two's complement modulo 2^118).  A CTA's up to 8 warps add theirs in shared
-// memory; the CTA's words carry one count each in their top 9 bits.  The sums of up to
-// 511 x 8 addends stay clear of the counts, and joining the payload sums modulo 2^118
-// gives the sum of the integers while that is below 2^117.  A warp whose sum cannot be
-// expressed at scale B marks its CTA an exception instead.
+// bits (its two's complement modulo 2^118).  A CTA's warps add theirs in shared memory;
+// the CTA's words carry one count each in their top 9 bits.  The sums of up to kMaxSums
+// addends (warps times CTAs) stay clear of the counts and of the exceptions, and joining
+// the payload sums modulo 2^118 gives the sum of the integers while that is below 2^117.
+// A warp whose sum cannot be expressed at scale B marks its CTA an exception instead.
 constexpr int kLimb = 43, kTop = 32, kExcAt = 45, kCountAt = 55, kMaxAddends = 511;
+constexpr int kMaxSums = 8 * kMaxAddends;
+static_assert(kMaxSums <= 1 << (kCountAt - kLimb) && kMaxSums <= 1 << (kExcAt - kTop), "limbs clear of the fields above");
 constexpr int kRoom = 20;  // a sum of exponent field e is exchanged at scale e - kRoom next time
 
 // Move the sum S at scale E to scale B; false where it does not fit.

@@ -30,7 +30,6 @@ constexpr int kRWarps = kThreads / 32;
 constexpr int kVecs = 4;       // x^, r^, q, p of a CTA's rows
 constexpr int kGroup = 4;      // rows of a thread together in the vector phases: a store to shared memory
                                // holds back the next row's loads (13.7 K clocks for 12 rows a thread)
-static_assert(kRWarps <= 16, "the exchange's limbs hold 16 warps' sums of at most 255 CTAs");
 
 struct ResidentParams {
   SolveParams P;
@@ -325,7 +324,7 @@ cudaError_t cgi::resident_launch(const cg_handle* h, const SolveParams& P, bool 
   *launched = false;
   if (!h->dia || h->n < 1) return cudaSuccess;
   cudaError_t e;
-  const int ctas = std::min(h->sm_count, 255);
+  const int ctas = std::min(h->sm_count, kXCtas<kRWarps>);
   const int spc = (int)((h->nslices + ctas - 1) / ctas);
   for (int ms = 1; ms >= 0; --ms) {
     if (!ms && (int64_t)sizeof(double) * h->sell_entries > streamed_max_bytes(h->uniform_w)) continue;
