@@ -1551,9 +1551,12 @@ cg_status cg_solve_batch(cg_handle* h, const double* const* b, double* const* x,
   CGB_CUDA(h, cudaMemcpyAsync(B->d_x, B->host_ptrs + ns, sizeof(void*) * ns, cudaMemcpyHostToDevice, h->stream));
   int G = 0, var = 0, teams = kSomeTeams;
   if (h->grid_opt > 0) {
-    // a forced grid runs on the variant with the most registers that can hold it
+    // a forced grid runs on the variant with the most registers that can hold it; with CTAs
+    // enough every system gets a team of its own, sized by its work (64 systems of up to
+    // 512^2 rows on 608 CTAs: 234 ms with 32 teams that take them in turn, 196 so)
     G = std::min(h->grid_opt, B->grid_max);
     while (var + 1 < kVariants && B->vmax[var] < G) ++var;
+    if (B->nsys <= kManyTeams && G >= 4 * B->nsys) teams = kManyTeams;
   } else {
     if (B->grid_tuned[sl] == 0) {
       const cg_status ts = autotune(h, jac, tol, maxit, f32, carry, tol_in);
